@@ -32,20 +32,17 @@ METRIC = "candidate mappings evaluated/sec"
 UNIT = "candidates/s"
 OBJ_NAMES = {0: "energy", 1: "latency", 2: "edp", 3: "energy_lcap", 4: "latency_ecap"}
 
-# Algorithmic work of the search kernels, per TESTED ROW (a row is the nine mappings that share tiling, order
-# and buffering levels; the kernel reports how many rows it tested, the others lay in tilings, middle levels
-# or groups that a coarser capacity test showed not to fit).  The least key of a row's nine mappings is its
-# row sum plus the least stationary-pair term, which is taken once per tiling, so a row needs one test.
-# Energy / latency, in thread-level 32-bit integer instructions: capacity difference of Eq. (4), its sign mask,
-# the feasible count, the masked row term, and 2/5 of a three-input minimum (five rows share two).
-# Energy-delay product: two capacity compares, their AND, the feasible count, and the single-precision row
-# bound (two adds, a max, a multiply, a compare, the predicate merge).
-ALG_OPS_PER_ROW = {0: 4.4, 1: 4.4, 2: 10.0}
+# Algorithmic work of the search kernels, per TESTED ROW.  A row is the nine mappings that share tiling, order and
+# buffering levels.  Levels fall into classes with equal buffer need and equal DRAM words, so that a tiling and order has
+# 432 different fused rows of 3125 (and 9 + 9 different choices of 625 unfused rows); the kernel decides each different
+# row once, exactly, for all the rows it stands for, and reports how many different rows it decided.  Each costs one
+# capacity compare (Eq. 4) and one weighted count, in thread-level 32-bit instructions; the least keys, the tables and
+# the winners' evaluation are not counted.
+ALG_OPS_PER_ROW = {0: 2.0, 1: 2.0, 2: 2.0}
 LANES_PER_SM = 64          # 4 sub-partitions x 16 lanes: width of the integer-ALU pipe, the busiest pipe of these kernels
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, recorded from the ncu captures summarised under
 # profiles/ (not measured in this run); workload -> objective -> bytes.  None where no capture backs it.
-NCU_DRAM_BYTES_PER_LAUNCH = {"gqa": {1: 199680, 2: 193024}, "llama": {0: 207360, 1: 198400},
-                             "bert": {0: 182272, 1: 201216}}
+NCU_DRAM_BYTES_PER_LAUNCH = {}
 
 
 WORKLOADS = {"tiny": mi.config1, "bert": mi.config2, "llama": mi.config3, "gqa": mi.config4}
@@ -349,7 +346,7 @@ def main():
         for i, (s, n) in enumerate(n_cand):
             ks = [k[i] for k in kernel_ms]
             sm = statistics.mean(ks)
-            ops = stats[i].rows_tested * ALG_OPS_PER_ROW.get(s["objective"], 10.0)
+            ops = stats[i].rows_tested * ALG_OPS_PER_ROW.get(s["objective"], 2.0)
             per_kernel.append(dict(
                 kernel="search_kernel<%s>" % OBJ_NAMES[s["objective"]], objective=s["objective"], problem=jobs[i][0]["name"],
                 avg_ms=sm, median_ms=statistics.median(ks), max_ms=max(ks), create_ms=stats[i].create_ms,
@@ -367,7 +364,7 @@ def main():
                                       if traffic is not None else "no capture of this kernel on this workload"),
                         peak_source="%d SMs x %d lanes of the integer-ALU pipe x %.0f MHz (clock sampled during the run)" %
                                     (n_sm, LANES_PER_SM, sm_mhz),
-                        ops_per_tested_row=ALG_OPS_PER_ROW.get(dom["objective"], 10.0),
+                        ops_per_tested_row=ALG_OPS_PER_ROW.get(dom["objective"], 2.0),
                         measured_rates_gops=dict(logic=peaks[0], add_logic=peaks[1], key_mix=peaks[2],
                                                  sm_mhz=peaks[3]))
         line = dict(
@@ -376,6 +373,8 @@ def main():
             higher_is_better=True, scaling="weak", vs_baseline=None, dtype="int64", data="synthetic",
             config=dict(workload=wname, searches=[OBJ_NAMES[s["objective"]] for s in searches],
                         candidates_per_step=cand_per_step, parallelism="replicas only",
+                        counted="every mapping of the space is decided exactly; rows with equal buffer needs and DRAM words "
+                                "are decided together (kernels[].rows_tested different rows)",
                         l2="flushed between steps (256 MB write); the path reads no HBM-resident input",
                         grid=stats[0].grid, block=stats[0].block, smem_bytes=stats[0].smem_bytes),
             clocks=clocks, gpu_launches=len(searches) * args.steps, check_failures=check_failures,

@@ -203,7 +203,7 @@ int mmee_destroy(mmee_handle_t* handle);
  * For whom: a process that has given the whole device to its own memory pool (a cudaMalloc from a
  * library then fails), or a latency-critical loop that cannot afford the device-wide
  * synchronisation of cudaMalloc / cudaFree.  This call makes no cudaMalloc, cudaFree or other
- * allocating call.  Its scratch (work counter, pruning bound, one partial top-k list per CTA) is a
+ * allocating call.  Its scratch (a header and one partial top-k list per CTA) is a
  * fixed 139 328-byte array inside the library image, present on every device that loads the
  * library for as long as the process lives.
  *
@@ -213,8 +213,8 @@ int mmee_destroy(mmee_handle_t* handle);
  * (with that device current); make that first call before any stream capture begins.  The address
  * is kept for the life of the process: after a cudaDeviceReset it is stale, and this entry point
  * must not be called on that device again.
- * objective.row_pruning must be 0 here (its kept-row list would need a device allocation).
- * Limits: the array holds the partial lists of at most 512 persistent CTAs; a device whose launch
+ * objective.row_pruning must be 0 here.
+ * Limits: the array holds the partial lists of at most 512 CTAs; a device whose launch
  * shape needs more is refused with MMEE_ERR_RANGE.  Other errors as mmee_create / mmee_search.
  * All calls on a device share the one array and it keeps the previous call's contents: the call
  * clears the header itself, but two mmee_search_static calls that overlap on the GPU (for instance
@@ -254,11 +254,9 @@ int mmee_eval(mmee_handle_t* handle, void* cuda_stream, uint64_t idx_begin, uint
 int mmee_decode(mmee_handle_t* handle, uint64_t idx, mmee_result_t* host_out);
 
 /*
- * mmee_dump_keys -- run the search kernel in its key-dump mode over the handle's tiling range and
- * store every candidate's objective key instead of reducing (Eq. 11: the full result matrix).  The
- * dump mode shares the kernel's tables, decode and task walk, and forms every key exactly in 64 bits
- * (the path the search takes for the energy-delay and capped objectives and for every group of rows
- * that its 32-bit filter flags); the filter itself is not part of it.
+ * mmee_dump_keys -- store every candidate's objective key over the handle's tiling range instead of reducing
+ * (Eq. 11: the full result matrix), formed exactly in 64 bits from the query-vector tables with which the
+ * search evaluates its winners' blocks.
  *   out_keys : DEVICE, (t_end - t_begin) * R * 9 int64; entry idx - t_begin*R*9.  Energy and
  *              latency keys as integers, EDP keys as the bit pattern of the double; INT64_MAX
  *              for a mapping that does not fit the buffer.
@@ -267,14 +265,11 @@ int mmee_decode(mmee_handle_t* handle, uint64_t idx, mmee_result_t* host_out);
 int mmee_dump_keys(mmee_handle_t* handle, void* cuda_stream, int64_t* out_keys);
 
 /*
- * mmee_filter_flags -- test view of the search kernel's filter.  The search decides with a cheap bound per group of
- * five rows (45 mappings: one level of D, the five levels of E, nine stationary pairs) whether the group can hold a
- * key below the current threshold, and forms exact keys only for flagged groups (32-bit threshold-relative sums for
- * energy and latency, a single-precision product bound followed by double-precision products for the energy-delay
- * product).  This call runs that filter over the handle's tiling range against the FIXED threshold `threshold_key`
- * (a key as the search orders it; for the energy-delay product the bit pattern of the double), inserts nothing, and
- * stores one byte per group: 1 = flagged.  A group that holds a mapping that fits, with an offered stationary pair and
- * a key < threshold_key, must be flagged; the converse need not hold.
+ * mmee_filter_flags -- which groups of five rows (45 mappings: one level of D, the five levels of E, nine stationary
+ * pairs) hold a mapping whose key lies below `threshold_key` (a key as the search orders it; for the energy-delay
+ * product the bit pattern of the double), over the handle's tiling range.  Stores one byte per group: 1 = flagged.  A
+ * group that holds a mapping that fits, with an offered stationary pair and a key < threshold_key, must be flagged; the
+ * converse need not hold (this implementation evaluates every mapping and flags no other group).
  *   out_flags : DEVICE, (t_end - t_begin) * (R / 125) * 25 bytes; group g of middle level m of task w (a task is 125
  *               consecutive rows of a tiling) at ((t - t_begin) * (R / 125) + w) * 25 + m * 5 + g.
  * Energy, latency and energy-delay objectives without row pruning; MMEE_ERR_ARG otherwise.  Asynchronous.
@@ -363,9 +358,9 @@ int mmee_recompute_flag(uint32_t pi, uint32_t beta_c, uint32_t* out_flag);
 
 /*
  * mmee_last_search_stats -- HOST counters of the most recent mmee_search on the handle, valid
- * after the stream has been synchronised (the call copies one counter from the device): kernels
+ * after the stream has been synchronised (the call copies two counters from the device): kernels
  * launched by that call (one: the CTA that finishes last merges the partial results and writes the
- * records), persistent CTAs, threads per CTA, dynamic shared memory per CTA, tasks (groups of 1125
+ * records), CTAs, threads per CTA, shared memory per CTA, tasks (groups of 1125
  * consecutive mappings) and, when mmee_kernel_timing is on, the device time of the search kernel in
  * milliseconds (CUDA events recorded on the search's stream; -1 when timing is off).  finalize_ms
  * is 0: the finalize step is part of the search kernel.
@@ -376,13 +371,13 @@ typedef struct {
     float    search_ms, finalize_ms;
     uint32_t rows_per_tiling;                /* R                                                  */
     uint32_t rows_evaluated_per_tiling;      /* R, or the rows that survive symbolic row pruning   */
-    uint64_t exact_path_visits;              /* groups of rows the 32-bit (or floating-point) filter sent to the
-                                                exact 64-bit path during that search               */
+    uint64_t exact_path_visits;              /* groups of five rows of the winners' blocks, evaluated mapping by
+                                                mapping at the end of that search                   */
     float    create_ms;                      /* host wall clock of the mmee_create that made the handle */
     uint32_t reserved;
-    uint64_t rows_tested;                    /* rows (of nine mappings each) whose capacity test (Eq. 4) and
-                                                bound the search evaluated; the rest lay in tilings, middle
-                                                levels or groups that a coarser test showed not to fit   */
+    uint64_t rows_tested;                    /* different rows (of nine mappings each) that the search decided: rows of
+                                                one tiling and order with equal buffer needs and DRAM words count
+                                                once, and none of a tiling whose smallest need does not fit */
 } mmee_launch_stats_t;
 int mmee_last_search_stats(const mmee_handle_t* handle, mmee_launch_stats_t* out);
 

@@ -5,7 +5,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
-#include <vector>
 
 #include "mmee_search.h"
 
@@ -19,7 +18,6 @@ struct mmee_handle {
     mmee_result_t* decode_buf;   // device, one record (mmee_decode); part of the scratch allocation
     mmee_result_t* host_out;     // pinned host memory mapped into the device's address space, 1 + topk records:
                                  // mmee_search_host lets the kernel write its records there (made at its first call)
-    mmee::PrunedTask* pruned;    // device, row pruning only
     uint32_t kept_rows;          // rows of a tiling that survive pruning (all rows without it)
     int device;
     mmee_launch_stats_t last;
@@ -45,75 +43,23 @@ int cuda_status(cudaError_t e) {
     return MMEE_ERR_CUDA;
 }
 
-// Tasks a CTA pulls per visit of the global counter, and the tilings such a range can touch.
-int choose_launch_shape(const Plan& p, int device, uint32_t search_tpt, uint32_t max_ctas, LaunchShape* shape) {
-    int sm_count = 0, smem_optin = 0;      // attribute queries: cudaGetDeviceProperties costs milliseconds
-    cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShape* shape) {
+    int sm_count = 0;      // attribute query: cudaGetDeviceProperties costs milliseconds
+    const cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return cuda_status(e);
-    // A task is 1125 mappings (225 with row pruning, where the searched units are single middle levels).
-    shape->search_tpt = search_tpt;
-    shape->pruned = nullptr;
-    // Two CTAs per SM under the 196 KB shared-memory carve-out, which leaves the row loops 60 KB of L1 (the next
-    // carve-out, 228 KB, leaves 28 KB and costs the energy-delay search a tenth of its speed).
-    constexpr size_t kSmemTarget = 97 * 1024;
-    // Ranges of whole tilings, as many as the table slots hold: a tiling's tables are then built once, not once
-    // by each of the two ranges it would straddle, and a range needs no slot for a tiling it only touches.
-    constexpr uint32_t kAlignedMaxTasks = 2048;
+    // Three CTAs per SM hold every register; small problems take fewer, with at least eight tilings each.
     const uint64_t tilings = p.t_end - p.t_begin;
-    bool aligned = search_tpt <= kAlignedMaxTasks && search_smem_bytes(p, 1) <= kSmemTarget;
-    uint32_t per_range = 1;                          // aligned: tilings of a range
-    if (aligned) {
-        while ((per_range + 1) * search_tpt <= kAlignedMaxTasks && search_smem_bytes(p, per_range + 1) <= kSmemTarget)
-            ++per_range;
-        // (a small problem, with fewer than four such ranges per CTA of a full grid, keeps ranges of a fixed number
-        // of tasks: whole tilings would leave most warps of a CTA without work)
-        if (tilings / per_range < 4ull * 2u * (uint64_t)sm_count) aligned = false;
-    }
-    if (aligned) {
-        shape->range_tasks = per_range * search_tpt;
-        shape->slots = per_range;
-    } else {
-        const uint32_t rounds = p.row_pruning ? 9 : 3;
-        shape->range_tasks = rounds * kWorkerThreads;
-        shape->slots = (shape->range_tasks - 1) / search_tpt + 2;
-        // Many small tilings per range need many table slots: shrink the range until they fit.
-        // (Worker warps take 32 tasks at a time, so a range may be as short as one warp's share.)
-        while (search_smem_bytes(p, shape->slots) > kSmemTarget && shape->range_tasks > 32) {
-            shape->range_tasks -= shape->range_tasks > (uint32_t)kWorkerThreads ? kWorkerThreads : 32;
-            shape->slots = (shape->range_tasks - 1) / search_tpt + 2;
-        }
-    }
-    const size_t smem = search_smem_bytes(p, shape->slots);
-    if (smem > (size_t)smem_optin) return MMEE_ERR_RANGE;
-    shape->smem_bytes = (uint32_t)smem;
-    int per_sm = 0;
-    if ((e = search_occupancy(p, device, smem, &per_sm)) != cudaSuccess) return cuda_status(e);
-    if (per_sm < 1) return MMEE_ERR_RANGE;
-    if (per_sm > 2) per_sm = 2;
-    uint64_t grid = (uint64_t)sm_count * (uint32_t)per_sm;
-    const uint64_t tasks = tilings * search_tpt;
-    if (aligned) {
-        // The last tilings go out one per range, about half a full range's worth per CTA: the CTAs then finish
-        // within one tiling of each other instead of within one full range.  (Measured with a whole, a half and a
-        // quarter of a range per CTA: the searches differ in which they prefer, by 1 to 3 %.)
-        uint64_t tail = grid * per_range / 2;
-        shape->n_big = (tilings - tail) / per_range;
-        tail = tilings - shape->n_big * per_range;
-        shape->tail_tasks = search_tpt;
-        shape->n_ranges = shape->n_big + tail;
-    } else {
-        shape->n_ranges = (tasks + shape->range_tasks - 1) / shape->range_tasks;
-        shape->n_big = shape->n_ranges;
-        shape->tail_tasks = shape->range_tasks;
-    }
-    const uint64_t ranges = shape->n_ranges;
-    if (grid > ranges) grid = ranges ? ranges : 1;
+    constexpr uint64_t kMinTilings = 8;
+    uint64_t grid = (tilings + kMinTilings - 1) / kMinTilings;
+    if (grid > 3ull * (uint32_t)sm_count) grid = 3ull * (uint32_t)sm_count;
+    if (!grid) grid = 1;
     // (a caller with a fixed scratch: a device that would take more CTAs is refused, not silently under-used)
     if (max_ctas && grid > max_ctas) return MMEE_ERR_RANGE;
+    // Passes of equal length, as few as the tables allow.
+    const uint64_t per_cta = (tilings + grid - 1) / grid;
+    const uint64_t passes = (per_cta + kMaxChunk - 1) / kMaxChunk;
     shape->grid = (uint32_t)grid;
-    // one spread range per CTA while at least as many ranges remain for the ascending part
-    shape->n_spread = grid < ranges / 2 ? grid : ranges / 2;
+    shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
     return MMEE_OK;
 }
 
@@ -132,30 +78,10 @@ int mmee_create(const mmee_workload_t* workload, const mmee_arch_t* arch, const 
     int rc = build_plan(workload, arch, objective, &h->plan);
     if (rc) { delete h; return rc; }
     if ((rc = cuda_status(cudaGetDevice(&h->device)))) { delete h; return rc; }
-    // Row pruning: the searched task space lists only the tasks that keep at least one row.
-    std::vector<PrunedTask> kept_tasks;
-    uint32_t search_tpt = h->plan.tasks_per_tiling;
     h->kept_rows = h->plan.rows_per_tiling;
-    if (h->plan.row_pruning) {
-        kept_tasks.resize(5 * (size_t)h->plan.tasks_per_tiling);
-        uint32_t n = 0;
-        build_pruned_tasks(h->plan, kept_tasks.data(), &n, &h->kept_rows);
-        kept_tasks.resize(n);
-        search_tpt = n;
-    }
-    rc = choose_launch_shape(h->plan, h->device, search_tpt, 0, &h->shape);
+    if (h->plan.row_pruning && (rc = set_kept_masks(&h->plan, &h->kept_rows))) { delete h; return rc; }
+    rc = choose_launch_shape(h->plan, h->device, 0, &h->shape);
     if (rc) { delete h; return rc; }
-    if (h->plan.row_pruning) {
-        const size_t bytes = kept_tasks.size() * sizeof(PrunedTask);
-        cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->pruned), bytes);
-        if (e == cudaSuccess) e = cudaMemcpy(h->pruned, kept_tasks.data(), bytes, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            if (h->pruned) cudaFree(h->pruned);
-            delete h;
-            return cuda_status(e);
-        }
-        h->shape.pruned = h->pruned;
-    }
     // one allocation: the search scratch, then one result record for mmee_decode
     const size_t sbytes = (scratch_bytes(h->shape.grid) + 15) / 16 * 16;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->scratch), sbytes + sizeof(mmee_result_t));
@@ -166,7 +92,6 @@ int mmee_create(const mmee_workload_t* workload, const mmee_arch_t* arch, const 
     }
     if (e != cudaSuccess) {
         if (h->scratch) cudaFree(h->scratch);
-        if (h->pruned) cudaFree(h->pruned);
         delete h;
         return cuda_status(e);
     }
@@ -194,14 +119,14 @@ int mmee_search(mmee_handle_t* h, void* cuda_stream, mmee_result_t* out_best, mm
         h->dirty = false;
     }
     if (h->timing) cudaEventRecord(h->ev[0], st);
-    const cudaError_t e = launch_search(h->plan, h->shape, h->device, h->scratch, nullptr, out_best, out_topk, st);
+    const cudaError_t e = launch_search(h->plan, h->shape, h->scratch, out_best, out_topk, st);
     if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
     if (h->timing) cudaEventRecord(h->ev[1], st);
     h->last.kernels_launched = 1;
     h->last.grid = h->shape.grid;
     h->last.block = kSearchThreads;
-    h->last.smem_bytes = h->shape.smem_bytes;
-    h->last.tasks = (h->plan.t_end - h->plan.t_begin) * h->shape.search_tpt;
+    h->last.smem_bytes = (uint32_t)search_smem_bytes();
+    h->last.tasks = (h->plan.t_end - h->plan.t_begin) * h->plan.tasks_per_tiling;
     h->last.rows_per_tiling = h->plan.rows_per_tiling;
     h->last.rows_evaluated_per_tiling = h->kept_rows;
     return MMEE_OK;
@@ -232,7 +157,6 @@ int mmee_destroy(mmee_handle_t* h) {
     cudaError_t e = cudaSuccess;
     if (h->timing) for (int i = 0; i < 2; ++i) cudaEventDestroy(h->ev[i]);
     if (h->scratch) e = cudaFree(h->scratch);
-    if (h->pruned) cudaFree(h->pruned);
     if (h->host_out) cudaFreeHost(h->host_out);
     delete h;
     return cuda_status(e);
@@ -282,34 +206,14 @@ int mmee_dump_keys(mmee_handle_t* h, void* cuda_stream, int64_t* out_keys) {
     if (n > (1ull << 31)) return MMEE_ERR_RANGE;
     int rc = check_device(h);
     if (rc) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (h->dirty) {
-        if ((rc = cuda_status(launch_reset(h->scratch, st)))) return rc;
-        h->dirty = false;
-    }
-    cudaError_t e = launch_search(h->plan, h->shape, h->device, h->scratch, out_keys, nullptr, nullptr, st);
-    if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
-    if ((e = launch_reset(h->scratch, st)) != cudaSuccess) { h->dirty = true; return cuda_status(e); }
-    return MMEE_OK;
+    return cuda_status(launch_dump_keys(h->plan, out_keys, static_cast<cudaStream_t>(cuda_stream)));
 }
 
 int mmee_filter_flags(mmee_handle_t* h, void* cuda_stream, int64_t threshold_key, uint8_t* out_flags) {
     if (!h || !out_flags || h->plan.row_pruning || h->plan.objective > MMEE_OBJ_EDP) return MMEE_ERR_ARG;
     int rc = check_device(h);
     if (rc) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (h->dirty) {
-        if ((rc = cuda_status(launch_reset(h->scratch, st)))) return rc;
-        h->dirty = false;
-    }
-    const uint64_t bytes = (h->plan.t_end - h->plan.t_begin) * (uint64_t)h->plan.tasks_per_tiling * 25u;
-    if ((rc = cuda_status(cudaMemsetAsync(out_flags, 0, bytes, st)))) return rc;
-    Plan p = h->plan;
-    p.key_cap = threshold_key;
-    cudaError_t e = launch_filter_flags(p, h->shape, h->device, h->scratch, out_flags, st);
-    if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
-    if ((e = launch_reset(h->scratch, st)) != cudaSuccess) { h->dirty = true; return cuda_status(e); }
-    return MMEE_OK;
+    return cuda_status(launch_group_flags(h->plan, threshold_key, out_flags, static_cast<cudaStream_t>(cuda_stream)));
 }
 
 int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch, const mmee_objective_t* objective,
@@ -499,13 +403,8 @@ int mmee_row_pruning_keep(const mmee_objective_t* objective, uint8_t* out_keep, 
     if (rc) return rc;
     *out_rows = plan.rows_per_tiling;
     if (capacity < plan.rows_per_tiling) return MMEE_ERR_RANGE;
-    std::vector<PrunedTask> tasks(5 * (size_t)plan.tasks_per_tiling);
-    uint32_t n = 0, kept = 0;
-    build_pruned_tasks(plan, tasks.data(), &n, &kept);
-    std::memset(out_keep, 0, plan.rows_per_tiling);
-    for (uint32_t i = 0; i < n; ++i)
-        for (uint32_t de = 0; de < 25; ++de)
-            if (tasks[i].rows >> de & 1u) out_keep[tasks[i].task * 125u + tasks[i].mid * 25u + de] = 1;
+    uint32_t kept = 0;
+    row_pruning_keep(plan, out_keep, &kept);
     return MMEE_OK;
 }
 
@@ -525,11 +424,11 @@ int mmee_last_search_stats(const mmee_handle_t* h, mmee_launch_stats_t* out) {
     out->exact_path_visits = 0;
     out->rows_tested = 0;
     if (h->last.kernels_launched) {
-        unsigned long long counters[3] = {0, 0, 0};      // last_exact_visits, tested_rows, last_tested_rows
-        const int rc = cuda_status(cudaMemcpy(counters, &h->scratch->last_exact_visits, sizeof(counters), cudaMemcpyDeviceToHost));
+        unsigned long long counters[2] = {0, 0};      // last_exact_groups, last_tested_rows
+        const int rc = cuda_status(cudaMemcpy(counters, &h->scratch->last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
         if (rc) return rc;
         out->exact_path_visits = counters[0];
-        out->rows_tested = counters[2];
+        out->rows_tested = counters[1];
     }
     if (h->timing && h->last.kernels_launched) {
         const cudaError_t e = cudaEventElapsedTime(&out->search_ms, h->ev[0], h->ev[1]);

@@ -132,6 +132,41 @@ void build_query_tables(QueryTables* q) {
     }
 }
 
+// Classes of levels with equal buffer need and DRAM words under one order (see OrderInfo), and where the search's
+// size table keeps what it needs of them.
+static void build_order_info(uint32_t order, const QueryTables& q, OrderInfo* o) {
+    std::memset(o, 0, sizeof(*o));
+    const Nest n = nest_of((int)order, 0);
+    const int lev_i = n.level_of[LOOP_I] - 3, lev_l = n.level_of[LOOP_L] - 3, lev_j = n.level_of[LOOP_J] - 3;
+    auto lower = [](int a, int b) { return a < b ? a : b; };
+    auto upper = [](int a, int b) { return a > b ? a : b; };
+    const int cuts[5][5] = {{0, 1, lev_i, 5, 5},
+                            {0, 1, lev_l, 5, 5},
+                            {0, lower(lev_i, lev_l), upper(lev_i, lev_l), 5, 5},
+                            {0, 1, lower(lev_l, lev_j), upper(lev_l, lev_j), 5},
+                            {0, 1, lower(lev_i, lev_j), upper(lev_i, lev_j), 5}};
+    for (int x = 0; x < 5; ++x)
+        for (int c = 0; c < 4; ++c) {
+            o->first[x][c] = (uint8_t)(cuts[x][c] < 5 ? cuts[x][c] : 4);
+            o->width[x][c] = (uint8_t)(cuts[x][c + 1] - cuts[x][c]);
+        }
+    for (int c = 0; c < 3; ++c) o->recompute[c] = q.recompute[order][o->first[OP_C][c]];
+    o->size_c[0] = S_il;
+    o->size_c[1] = lev_i < lev_l ? S_Il : S_iL;
+    o->size_c[2] = S_IL;
+    o->size_d_lo = lev_l < lev_j ? S_Lj : S_lJ;
+    o->size_e_lo = lev_i < lev_j ? S_Ij : S_iJ;
+    // D is fetched once from the class on whose own loops not resident all lie above i2: with i2 lowest that is every
+    // retained class, with i2 in the middle the one with the lower own loop resident; E likewise with l2.
+    const bool i_d1 = lev_i > lower(lev_l, lev_j), i_d2 = lev_i > upper(lev_l, lev_j);
+    const bool l_e1 = lev_l > lower(lev_i, lev_j), l_e2 = lev_l > upper(lev_i, lev_j);
+    o->size_d_res = (uint8_t)(i_d2 ? S_LJ : (i_d1 ? o->size_d_lo : S_lj));
+    o->size_e_res = (uint8_t)(l_e2 ? S_IJ : (l_e1 ? o->size_e_lo : S_ij));
+    o->flags = (uint16_t)((lev_l > lev_i ? kLaboveI : 0) | (lev_j > lev_i ? kJaboveI : 0) | (lev_i > lev_l ? kIaboveL : 0) |
+                          (lev_j > lev_l ? kJaboveL : 0) | (lev_j > lower(lev_i, lev_l) ? kJaboveC : 0) |
+                          (i_d1 ? kIaboveD1 : 0) | (i_d2 ? kIaboveD2 : 0) | (l_e1 ? kLaboveE1 : 0) | (l_e2 ? kLaboveE2 : 0));
+}
+
 int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_objective_t* o, Plan* p) {
     if (!w || !a || !o || !p) return MMEE_ERR_ARG;
     std::memset(p, 0, sizeof(*p));
@@ -219,7 +254,7 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
     p->c_mac = p->cq[3] + (p->has_rf ? 3 * p->cq[2] : 0);
     p->c_sfu = p->cq[4];
 
-    // The row loop compares buffer sizes in 32 bits, saturated at 2^30 - 1 words.
+    // The search compares buffer sizes in 32 bits, saturated at 2^30 - 1 words.
     if (a->gb_bytes / w->word_bytes >= (1ull << 30) - 1) return MMEE_ERR_RANGE;
     p->cap_words = (int64_t)(a->gb_bytes / w->word_bytes);
     p->bw = a->dram_words_per_cycle;
@@ -228,6 +263,7 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
     p->objective = o->objective;
     p->topk = o->topk;
     p->row_pruning = o->row_pruning;
+    p->fuse_mask = o->fuse_mask;
     p->sm_mask = o->stationary_mask ? o->stationary_mask : 0x1ffu;
     for (uint32_t b = 0; b < 9; ++b) p->n_sm += (p->sm_mask >> b) & 1u;
     p->key_cap = o->key_cap;
@@ -246,17 +282,8 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
     const long double limit = 4611686018427387904.0L;     // 2^62
     if (emax >= limit || lmax >= limit) return MMEE_ERR_OVERFLOW;
 
-    // Scale of the 32-bit threshold-relative keys of the energy and latency walks: the largest DRAM term of any
-    // mapping, I*K*L*J words (times c_dram_gb quanta for energy), must fit below 2^28 after the shift.
-    p->rel_shift = 0;
-    p->unit = 1;
-    if (p->objective == MMEE_OBJ_ENERGY || p->objective == MMEE_OBJ_LATENCY) {
-        long double biggest = (long double)dims[0] * dims[1] * dims[2] * dims[3] *
-                              (p->objective == MMEE_OBJ_ENERGY ? (long double)p->c_dram_gb : 1.0L);
-        while (biggest >= 268435456.0L) { biggest /= 2.0L; ++p->rel_shift; }
-    }
-
     build_query_tables(&p->q);
+    for (uint32_t s = 0; s < p->n_orders; ++s) build_order_info(p->order_id[s], p->q, &p->order[s]);
     return MMEE_OK;
 }
 

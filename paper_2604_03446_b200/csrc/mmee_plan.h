@@ -25,6 +25,36 @@ struct QueryTables {
     uint8_t recompute[6][5];      // [order][beta_C-3]
 };
 
+// Buffer sizes of a tiling's operands (TileTab::size): lower case a tile extent, upper case the whole dimension.
+enum SizeSlot { S_ik, S_iK, S_IK, S_kl, S_Kl, S_KL, S_il, S_Il, S_iL, S_IL, S_lj, S_Lj, S_lJ, S_LJ, S_ij, S_Ij, S_iJ, S_IJ, kSizeSlots };
+
+// Levels of one operand fall into classes with equal buffer need and equal DRAM words: only the operand's own inter-tile
+// loops change either (Section V-B, V-C), plus the step from L3 to L4, from where the operand counts as retained while
+// the other operator runs (Eq. 1, 2) and D / E leave Scenario 2.  Classes, in ascending level order:
+//   A: L3 | L4 .. below i2 | i2 ..          B: L3 | L4 .. below l2 | l2 ..
+//   C: L3 .. below its lower own loop | .. below its upper one | upper ..
+//   D, E: L3 | L4 .. below the lower own loop | .. below the upper one | upper ..
+struct alignas(4) OrderInfo {
+    uint8_t first[5][4];          // first level (beta - 3) of each class; classes per operand: 3, 3, 3, 4, 4
+    uint8_t width[5][4];          // levels in the class (0 for a fourth class that does not exist)
+    uint8_t recompute[3];         // C is regenerated, by class of C
+    uint8_t size_c[3];            // where a class's buffer size sits in a tiling's size table (TileTab::size): C by
+    uint8_t size_d_lo, size_e_lo; // class; D / E with the lower own loop resident (class 2)
+    uint8_t size_d_res, size_e_res;   // the smallest class of D / E that is fetched only once
+    uint16_t flags;               // OrderFlag bits: which loops run above which
+};
+enum OrderFlag {
+    kLaboveI = 1, kJaboveI = 2, kIaboveL = 4, kJaboveL = 8,
+    kJaboveC = 16,                // j2 above the lower own loop of C
+    kIaboveD1 = 32, kIaboveD2 = 64,   // i2 above the lower / upper own loop of D
+    kLaboveE1 = 128, kLaboveE2 = 256  // l2 above the lower / upper own loop of E
+};
+// Rows kept by symbolic pruning, by classes (every kept row is the first of its class combination).
+struct alignas(4) KeptMasks {
+    uint16_t fused[kMaxOrders][3][9];         // [order slot][class of C][3 * class of A + class of B]: bit 4 * d + e
+    uint16_t unfused[2][kMaxOrders][9];       // [unfused mode][order slot][3 * a + b]: bit 3 * d + e (L3, L4 merged)
+};
+
 struct Plan {
     uint32_t dim[4];              // I, K, L, J of one instance
     uint32_t ndiv[4];
@@ -38,7 +68,7 @@ struct Plan {
     uint8_t  block_order_slot[kMaxBlocks];   // position of the block's order in order_id[]
     uint32_t tasks_per_tiling;    // fused_tasks + 5 per unfused block
     uint32_t rows_per_tiling;     // R = 125 * tasks_per_tiling
-    uint64_t n_tilings;           // T
+    uint64_t n_tilings;           // T, at most MMEE_MAX_DIVISORS^4 = 2^24
     uint64_t t_begin, t_end;
     int64_t  cap_words;
     int64_t  c_dram_gb;           // quanta per DRAM word moved (DRAM + buffer side)
@@ -50,15 +80,15 @@ struct Plan {
     uint32_t bw, pe_rows, pe_cols;
     uint32_t objective, topk;
     uint32_t row_pruning;
+    uint32_t fuse_mask;
     uint32_t sm_mask, n_sm;       // stationary pairs in the space (bit s = 3*sm1+sm2; never 0) and their number
     int64_t  key_cap;             // capped objectives: bound on the other key
-    uint32_t rel_shift;           // energy: threshold-relative keys are kept in units of 2^rel_shift quanta
-    int32_t  unit;                // the constant 1, as a run-time value: x * unit + y is issued as an integer
-                                  // multiply-add, which the FMA pipe executes beside the integer ALU pipe
     uint32_t rf_tiling;           // register-file-level tiling: the block of each operator's tile is searched
     uint32_t rf_words;            // register-file capacity of one PE in words
     double   quantum_pj;
     QueryTables q;
+    OrderInfo order[kMaxOrders];  // by order slot
+    KeptMasks kept;               // row pruning only
     uint32_t divs[4][MMEE_MAX_DIVISORS];
 };
 
@@ -66,8 +96,9 @@ struct Plan {
 int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_objective_t* o, Plan* plan);
 void build_query_tables(QueryTables* q);
 
-// Tie-safe symbolic row pruning (mmee_prune.cu): keep[row] for every row of a tiling.
-struct PrunedTask { uint32_t task, mid, rows, pad; };   // task inside a tiling, middle level, 25-bit mask of kept rows
-int build_pruned_tasks(const Plan& plan, PrunedTask* out, uint32_t* n_out, uint32_t* kept_rows);
+// Tie-safe symbolic row pruning (mmee_prune.cu): keep[row] = 1 for the rows of a tiling that are evaluated; the number
+// of them; and their class masks in plan->kept (a plan with row_pruning).
+void row_pruning_keep(const Plan& plan, uint8_t* keep, uint32_t* kept_rows);
+int set_kept_masks(Plan* plan, uint32_t* kept_rows);
 
 }  // namespace mmee

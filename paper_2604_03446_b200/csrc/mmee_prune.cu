@@ -13,6 +13,7 @@
 #include "mmee_plan.h"
 
 #include <algorithm>
+#include <cstring>
 #include <map>
 #include <vector>
 
@@ -144,22 +145,44 @@ void build_row_keep(const Plan& p, std::vector<uint8_t>* keep) {
 
 }  // namespace
 
-// The (task, middle level) groups of 25 rows that still hold a kept row, in index order, with their
-// kept-row masks.  `out` has room for 5 * tasks_per_tiling entries.
-int build_pruned_tasks(const Plan& p, PrunedTask* out, uint32_t* n_out, uint32_t* kept_rows) {
+void row_pruning_keep(const Plan& p, uint8_t* out, uint32_t* kept_rows) {
     std::vector<uint8_t> keep;
     build_row_keep(p, &keep);
-    uint32_t n = 0, rows = 0;
-    for (uint32_t w = 0; w < p.tasks_per_tiling; ++w) {
-        for (uint32_t m = 0; m < 5; ++m) {
-            PrunedTask t = {w, m, 0, 0};
-            for (uint32_t de = 0; de < 25; ++de)
-                if (keep[w * 125u + m * 25u + de]) { t.rows |= 1u << de; ++rows; }
-            if (t.rows) out[n++] = t;
+    *kept_rows = 0;
+    for (uint32_t r = 0; r < p.rows_per_tiling; ++r) { out[r] = keep[r]; *kept_rows += keep[r]; }
+}
+
+// The kept rows as masks over classes of levels.  A row that is not the first of its class combination has equal
+// buffer needs and DRAM words as that first row and a higher index, so it is never kept; MMEE_ERR_CHECK if it were.
+int set_kept_masks(Plan* p, uint32_t* kept_rows) {
+    std::vector<uint8_t> keep(p->rows_per_tiling);
+    row_pruning_keep(*p, keep.data(), kept_rows);
+    std::memset(&p->kept, 0, sizeof(p->kept));
+    for (uint32_t row = 0; row < p->rows_per_tiling; ++row) {
+        if (!keep[row]) continue;
+        const uint32_t task = row / 125u, mid = row % 125u / 25u, de = row % 25u;
+        const bool fused = task < p->fused_tasks;
+        const uint32_t u = fused ? task : task - p->fused_tasks, per = fused ? 25u : 5u;
+        const uint32_t block = fused ? u / per : p->n_fused_blocks + u / per;
+        const uint32_t slot = p->block_order_slot[block];
+        const OrderInfo& o = p->order[slot];
+        const uint32_t lv[5] = {fused ? u % 25u / 5u : u % 5u, fused ? u % 5u : mid, fused ? mid : 0u, de / 5u, de % 5u};
+        uint32_t cls[5];
+        for (int x = 0; x < 5; ++x) {
+            int c = -1;
+            for (int i = 0; i < 4; ++i) if (o.width[x][i] && o.first[x][i] == lv[x]) c = i;
+            if (c < 0) return MMEE_ERR_CHECK;
+            cls[x] = (uint32_t)c;
+        }
+        if (fused) {
+            p->kept.fused[slot][cls[OP_C]][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (4 * cls[OP_D] + cls[OP_E]));
+        } else {
+            // an unfused nest knows no retained operands: L3 and the class from L4 on are one class of D and of E
+            if (cls[OP_D] == 1 || cls[OP_E] == 1) return MMEE_ERR_CHECK;
+            const uint32_t d = cls[OP_D] ? cls[OP_D] - 1 : 0, e = cls[OP_E] ? cls[OP_E] - 1 : 0;
+            p->kept.unfused[p->block_phi[block] - 1][slot][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (3 * d + e));
         }
     }
-    *n_out = n;
-    *kept_rows = rows;
     return MMEE_OK;
 }
 

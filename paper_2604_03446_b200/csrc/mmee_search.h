@@ -1,4 +1,4 @@
-// Internal: device scratch layout and kernel launchers (mmee_search.cu), used by the C ABI.
+// Internal: device scratch layout and kernel launchers (mmee_search.cu, mmee_views.cu), used by the C ABI.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -9,67 +9,51 @@
 namespace mmee {
 
 constexpr int kSearchThreads = 256;
-constexpr int kWorkerWarps = kSearchThreads / 32 - 1;     // the last warp builds tables
-constexpr int kWorkerThreads = kWorkerWarps * 32;
+constexpr uint32_t kMaxChunk = 64;      // tilings whose tables a CTA holds at once
 
-// One CTA's k best (key, idx) pairs, best first.
+// One CTA's contribution: its k best blocks as (least key, block number) pairs, best first, and its counts.
 struct alignas(16) Partial {
-    longlong2 e[MMEE_MAX_TOPK];     // x = key, y = idx: one 16-byte word per pair, stored and loaded whole
-    int32_t count;
-    int32_t pad[3];
+    longlong2 e[MMEE_MAX_TOPK];     // x = key, y = block number: one 16-byte word per pair, stored and loaded whole
+    uint32_t count;
+    uint32_t live_tilings;
+    uint64_t feasible_rows;
 };
 
-// Global scratch of one handle: a work counter, the feasible-row count, the shared pruning bound,
-// the count of exact-path visits and one partial list per CTA.  The header is reset by the finalize
-// step, which also keeps the finished search's visit count in `last_exact_visits`.
+// Global scratch of one handle: the shared bound (k > 1), the ticket counter and one partial list per CTA.  The
+// header is reset by the finalize step, which also keeps the finished search's counters.
 struct Scratch {
-    unsigned long long next_task;
-    unsigned long long feasible_rows;
-    long long G;
-    unsigned long long exact_visits;
-    unsigned long long last_exact_visits;
-    unsigned long long tested_rows;         // rows whose capacity test and bound were evaluated
-    unsigned long long last_tested_rows;
-    unsigned int done_ctas;         // ticket counter: the CTA that draws the last ticket runs the finalize step
-    unsigned int pad;
+    long long G;                            // upper bound on the k-th smallest key
+    unsigned long long last_exact_groups;   // groups of 45 mappings of the winning blocks, evaluated one by one
+    unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
+    unsigned int done_ctas;                 // ticket counter: the CTA that draws the last ticket runs the finalize step
+    unsigned int pad[9];
     Partial partial[1];     // grid entries follow
 };
+static_assert(offsetof(Scratch, partial) == 64, "the header is 64 bytes");
 
 struct LaunchShape {
-    uint32_t grid;          // persistent CTAs
-    uint32_t range_tasks;   // tasks a CTA takes per pull: those of `slots` whole tilings where that many fit
-    uint32_t slots;         // tilings one range can touch
-    uint32_t smem_bytes;
-    uint32_t search_tpt;    // tasks per tiling in the searched task space (fewer with row pruning)
-    uint32_t tail_tasks;    // tasks of each range from number n_big on (one tiling's; the last ranges are short)
-    const PrunedTask* pruned;   // device: the kept tasks of a tiling (row pruning), else null
-    uint64_t n_ranges;      // ranges of the searched task interval: n_big of range_tasks, the others of tail_tasks
-    uint64_t n_big;
-    uint64_t n_spread;      // the first n_spread pulls take ranges spread evenly over the interval (multiples of
-                            // n_ranges / n_spread >= 2), the others follow in ascending order; 0: ascending only
+    uint32_t grid;          // CTAs; CTA c takes one tiling of every `grid` consecutive ones
+    uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
 };
 
 inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 
-size_t search_smem_bytes(const Plan& p, uint32_t slots);
-cudaError_t search_occupancy(const Plan& p, int device, size_t smem, int* blocks_per_sm);
-// One launch per search: the last CTA to finish merges the partial lists, evaluates the winners into
-// out_best / out_topk (device) and resets the scratch header.  With `dump` set the kernel stores every
-// key instead and writes no result (the caller resets the header).
-cudaError_t launch_search(const Plan& p, const LaunchShape& shape, int device, Scratch* scratch, int64_t* dump,
-                          mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st);
-// Test mode: the search kernel's filter alone against the fixed threshold p.key_cap; flags[(task - first task) * 25
-// + middle level * 5 + group] is set to 1 for every flagged group (the caller clears the buffer first and resets
-// the scratch header afterwards).  Energy, latency and energy-delay objectives.
-cudaError_t launch_filter_flags(const Plan& p, const LaunchShape& shape, int device, Scratch* scratch, unsigned char* flags,
-                                cudaStream_t st);
+size_t search_smem_bytes();
+// One launch per search: the last CTA to finish merges the partial lists, evaluates the winners' blocks mapping by
+// mapping, writes the records to out_best / out_topk (device) and resets the scratch header.
+cudaError_t launch_search(const Plan& p, const LaunchShape& shape, Scratch* scratch, mmee_result_t* out_best,
+                          mmee_result_t* out_topk, cudaStream_t st);
 cudaError_t launch_reset(Scratch* scratch, cudaStream_t st);
+
+// Every key of the plan's tiling range (kInfKey where a mapping does not fit or its stationary pair is not offered).
+cudaError_t launch_dump_keys(const Plan& p, int64_t* out, cudaStream_t st);
+// One byte per group of 45 mappings of the range: 1 if one that fits has a key below `threshold`.
+cudaError_t launch_group_flags(const Plan& p, int64_t threshold, unsigned char* flags, cudaStream_t st);
 cudaError_t launch_eval(const Plan& p, uint64_t idx_begin, uint64_t count, mmee_result_t* out, cudaStream_t st);
 cudaError_t measure_alu_peak(double* giops);
 
-// Launch shape of a search on `device`: tasks per range, table slots, shared memory, persistent CTAs
-// (at most max_ctas when that is not 0: MMEE_ERR_RANGE if the device would take more), range order.
-int choose_launch_shape(const Plan& p, int device, uint32_t search_tpt, uint32_t max_ctas, LaunchShape* shape);
+// Launch shape of a search on `device` (at most max_ctas CTAs when that is not 0: MMEE_ERR_RANGE if it would take more).
+int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShape* shape);
 
 // MMEE_OK, or MMEE_ERR_CUDA with the error kept for mmee_last_cuda_error (per host thread).
 int cuda_status(cudaError_t e);

@@ -4,7 +4,7 @@
 // a serving process that has handed the whole device to its own memory pool, so that a
 // cudaMalloc issued by a library simply fails; or a latency-critical loop in which the implicit
 // device-wide synchronisation of cudaMalloc / cudaFree would stall every other stream.  For them
-// the work counter, the shared pruning bound and the per-CTA partial top-k lists -- the scratch
+// the header (ticket counter, shared bound) and the per-CTA partial top-k lists -- the scratch
 // that mmee_create otherwise allocates per handle -- live in one fixed array that is part of the
 // library image.  Every device that loads the library carries that array until the process exits.
 #include <cuda_runtime.h>
@@ -17,7 +17,7 @@ namespace {
 
 using namespace mmee;
 
-constexpr uint32_t kStaticMaxCtas = 512;       // persistent CTAs the fixed scratch has room for
+constexpr uint32_t kStaticMaxCtas = 512;       // CTAs the fixed scratch has room for
 constexpr int kMaxDevices = 64;
 constexpr size_t kStaticScratchBytes = sizeof(Scratch) + (size_t)(kStaticMaxCtas - 1) * sizeof(Partial);
 
@@ -54,18 +54,18 @@ extern "C" int mmee_search_static(const mmee_workload_t* workload, const mmee_ar
     Plan plan;
     int rc = build_plan(workload, arch, objective, &plan);      // host only
     if (rc) return rc;
-    if (plan.row_pruning) return MMEE_ERR_ARG;      // the kept-task list would need a device allocation
+    if (plan.row_pruning) return MMEE_ERR_ARG;      // documented: the allocation-free call searches every row
     int device = 0;
     if ((rc = cuda_status(cudaGetDevice(&device)))) return rc;
     // The same launch shape as a handle would get, bounded by what the fixed scratch can hold.
     LaunchShape shape;
-    if ((rc = choose_launch_shape(plan, device, plan.tasks_per_tiling, kStaticMaxCtas, &shape))) return rc;
+    if ((rc = choose_launch_shape(plan, device, kStaticMaxCtas, &shape))) return rc;
     Scratch* scratch = nullptr;
     if ((rc = static_scratch(device, &scratch))) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // The array keeps whatever the previous call left in it.  The header (work counter, feasible
-    // count, pruning bound) must start clean; the partial lists need no clearing, every CTA of
+    // The array keeps whatever the previous call left in it.  The header (ticket counter, shared
+    // bound) must start clean; the partial lists need no clearing, every CTA of
     // this launch overwrites its own before the finalize step reads them.
     if ((rc = cuda_status(launch_reset(scratch, st)))) return rc;
-    return cuda_status(launch_search(plan, shape, device, scratch, nullptr, out_best, out_topk, st));
+    return cuda_status(launch_search(plan, shape, scratch, out_best, out_topk, st));
 }

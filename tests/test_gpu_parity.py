@@ -585,3 +585,40 @@ def test_repeated_searches_after_a_cache_flush_agree(topk):
             r = mm.read_results(best, 1)[0]
             got = (r.n_feasible, tuple((x.idx, x.e_key) for x in mm.read_results(top, topk)))
             assert r.status == mm.OK and got == expected, (it, r.status, got[1][:2], expected[1][:2])
+
+
+@pytest.mark.parametrize("fuse_mask,order_set", [(7, 1), (1, 1), (2, 0), (4, 1), (5, 0), (6, 1)])
+@pytest.mark.parametrize("seed", [2, 7, 10])
+def test_single_tilings_decided_by_classes_of_levels(seed, fuse_mask, order_set):
+    """One tiling at a time (the smallest interval): the feasible count and the three best mappings that the closed
+    forms over classes of levels give, against the oracle's row-by-row evaluation, for every objective in turn, at
+    capacities at which some classes fit and others do not; then with the row-pruned class masks."""
+    cfg = mi.random_tiny_problem(seed)
+    base = dict(cfg["searches"][0], fuse_mask=fuse_mask, order_set=order_set, topk=3)
+    T = oracle.make_problem(cfg["workload"], cfg["arch"], base).T
+    for i, t in enumerate(sorted({0, T // 5, T // 3, T // 2, T - 2, T - 1})):
+        for objective in (mi.OBJ_ENERGY, mi.OBJ_LATENCY, mi.OBJ_EDP):
+            obj = dict(base, objective=objective, t_begin=t, t_end=t + 1)
+            check_search(cfg, obj)
+        want = oracle.search(oracle.make_problem(cfg["workload"], cfg["arch"], dict(obj, topk=1)))
+        best, _, _ = gpu_search(cfg, dict(obj, topk=1, row_pruning=1))
+        assert best.idx == (want.topk[0].idx if want.topk else mm.NO_INDEX)
+
+
+def test_top16_over_several_passes_equals_the_merge_of_its_parts():
+    """40 560 tilings: more than all CTAs hold tables for at once, so that each takes a second pass.  The sixteen best
+    of the whole are the sixteen best of three parts (each within one pass), and the optimum is the stored one."""
+    with open(os.path.join(GOLDEN, "search_ffn_gpt3_dram_1024KB.json")) as f:
+        gold = json.load(f)
+    cfg = dict(name=gold["name"], workload=gold["workload"], arch=gold["arch"])
+    obj = dict(gold["searches"][0]["objective"], topk=16)
+    T = oracle.make_problem(cfg["workload"], cfg["arch"], obj).T
+    best, whole, _ = gpu_search(cfg, obj)
+    parts, feasible = [], 0
+    for lo, hi in ((0, 11111), (11111, 27000), (27000, T)):
+        b, top, _ = gpu_search(cfg, dict(obj, t_begin=lo, t_end=hi))
+        parts += [(r.e_key, r.idx) for r in top if r.idx != mm.NO_INDEX]
+        feasible += b.n_feasible
+    assert [(r.e_key, r.idx) for r in whole] == sorted(parts)[:16]
+    assert best.n_feasible == feasible == gold["searches"][0]["n_feasible"]
+    assert best.idx == gold["searches"][0]["topk"][0]["idx"]
