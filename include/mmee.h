@@ -161,8 +161,9 @@ typedef struct mmee_handle mmee_handle_t;
  * the query vectors of every (order, operand, level) (Section V-E, Section VI-A "offline"
  * enumeration), quantises the energies and bounds the largest possible key.
  *   workload, arch, objective : HOST, read only during the call.
- *   out                       : HOST, receives the handle.  The handle owns a few KB of DEVICE
- *                               scratch on the device that is current at the call.
+ *   out                       : HOST, receives the handle.  The handle holds 0.13 MB of DEVICE scratch on the
+ *                               device that is current at the call and 6 KB of pinned host memory, taken from
+ *                               the library's idle workspaces (see mmee_trim) or allocated.
  * Errors: MMEE_ERR_ARG, _OVERFLOW, _QUANTUM, _RANGE (more than MMEE_MAX_DIVISORS divisors), _CUDA.
  */
 int mmee_create(const mmee_workload_t* workload, const mmee_arch_t* arch,
@@ -185,15 +186,25 @@ int mmee_search(mmee_handle_t* handle, void* cuda_stream, mmee_result_t* out_bes
 
 /*
  * mmee_search_host -- mmee_search on the default stream of the handle's device followed by the copy of
- * the records to HOST memory: the time to the optimal mapping of a planned search.  The first call on
- * a handle allocates 1 + topk records of pinned host memory that the kernel writes its records into;
- * later calls allocate nothing.  Synchronous.
+ * the records to HOST memory: the time to the optimal mapping of a planned search.  The kernel writes its
+ * records into the handle's pinned host memory; the call allocates nothing.  Synchronous.
  *   out_best : HOST, one record.   out_topk : HOST, objective.topk records, or NULL.
  * Returns MMEE_ERR_CHECK if the finalize step's self-check failed (the records are then not a result).
  */
 int mmee_search_host(mmee_handle_t* handle, mmee_result_t* out_best, mmee_result_t* out_topk);
 
+/*
+ * mmee_destroy -- release the handle; its workspace goes to the idle ones.  Waits for the handle's device when
+ * mmee_search was called on the handle.
+ */
 int mmee_destroy(mmee_handle_t* handle);
+
+/*
+ * mmee_trim -- free the idle workspaces.  Device scratch and pinned host memory of released handles and one-shot calls
+ * stay with the library for the next handle on the same device, at most eight of them (0.13 MB of device memory and
+ * 6 KB of pinned host memory each); no two handles or calls share one.  Handles in use are not affected.
+ */
+int mmee_trim(void);
 
 /*
  * mmee_search_static -- the same search as mmee_create + mmee_search + mmee_destroy, for callers

@@ -19,7 +19,7 @@ MAX_TOPK = 16
 NO_INDEX = 2 ** 64 - 1
 OK, ERR_ARG, ERR_OVERFLOW, ERR_QUANTUM, ERR_NO_FEASIBLE, ERR_CUDA, ERR_TIMEOUT, ERR_RANGE, ERR_CHECK = range(9)
 
-EXPORTS = ("mmee_create", "mmee_search", "mmee_search_host", "mmee_destroy", "mmee_search_static", "mmee_num_candidates", "mmee_num_tilings",
+EXPORTS = ("mmee_create", "mmee_search", "mmee_search_host", "mmee_destroy", "mmee_trim", "mmee_search_static", "mmee_num_candidates", "mmee_num_tilings",
            "mmee_num_rows", "mmee_strerror", "mmee_last_cuda_error", "mmee_eval", "mmee_decode", "mmee_dump_keys", "mmee_filter_flags", "mmee_solve_host", "mmee_pareto_front", "mmee_pareto_front_bs_da", "mmee_search_shapes",
            "mmee_query_vector", "mmee_recompute_flag", "mmee_row_pruning_keep", "mmee_last_search_stats", "mmee_kernel_timing",
            "mmee_alu_peak")
@@ -103,6 +103,7 @@ def library():
     L.mmee_search.argtypes = [H, C.c_void_p, C.c_void_p, C.c_void_p]
     L.mmee_search_host.argtypes = [H, C.POINTER(Result), C.POINTER(Result)]
     L.mmee_destroy.argtypes = [H]
+    L.mmee_trim.argtypes = []
     L.mmee_search_static.argtypes = [C.POINTER(Workload), C.POINTER(Arch), C.POINTER(Objective),
                                      C.c_void_p, C.c_void_p, C.c_void_p]
     for name in ("mmee_num_candidates", "mmee_num_tilings", "mmee_num_rows"):
@@ -162,6 +163,11 @@ def mmee_create(workload: dict, arch: dict, objective: dict) -> C.c_void_p:
 
 def mmee_destroy(handle) -> None:
     _check(library().mmee_destroy(handle), "mmee_destroy")
+
+
+def mmee_trim() -> None:
+    """Free the device scratch and pinned host memory that the library keeps of released handles."""
+    _check(library().mmee_trim(), "mmee_trim")
 
 
 def mmee_num_candidates(handle) -> int:

@@ -6,7 +6,7 @@
 #include <cstring>
 #include <new>
 
-#include "mmee_search.h"
+#include "mmee_workspace.h"
 
 static_assert(sizeof(mmee_result_t) == 336, "mmee_result_t is part of the ABI");
 static_assert(sizeof(mmee::Plan) <= 4096, "the plan travels as a kernel parameter");
@@ -14,15 +14,13 @@ static_assert(sizeof(mmee::Plan) <= 4096, "the plan travels as a kernel paramete
 struct mmee_handle {
     mmee::Plan plan;
     mmee::LaunchShape shape;
-    mmee::Scratch* scratch;      // device
-    mmee_result_t* decode_buf;   // device, one record (mmee_decode); part of the scratch allocation
-    mmee_result_t* host_out;     // pinned host memory mapped into the device's address space, 1 + topk records:
-                                 // mmee_search_host lets the kernel write its records there (made at its first call)
+    mmee::Workspace* ws;         // device scratch and pinned host records, from the kept workspaces
     uint32_t kept_rows;          // rows of a tiling that survive pruning (all rows without it)
     int device;
     mmee_launch_stats_t last;
     float create_ms;             // host wall clock of mmee_create
     bool dirty;                  // a launch failed half-way: the scratch header is reset before the next search
+    bool in_flight;              // a search was launched whose end this handle has not waited for
     bool timing;
     cudaEvent_t ev[2];           // before and after the search kernel
 };
@@ -43,15 +41,24 @@ int cuda_status(cudaError_t e) {
     return MMEE_ERR_CUDA;
 }
 
-int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShape* shape) {
+// Three CTAs per SM hold every register.
+int max_search_ctas(int device, uint32_t* out) {
     int sm_count = 0;      // attribute query: cudaGetDeviceProperties costs milliseconds
     const cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return cuda_status(e);
-    // Three CTAs per SM hold every register; small problems take fewer, with at least eight tilings each.
+    *out = 3u * (uint32_t)sm_count;
+    return MMEE_OK;
+}
+
+int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShape* shape) {
+    uint32_t most = 0;
+    const int rc = max_search_ctas(device, &most);
+    if (rc) return rc;
+    // Small problems take fewer CTAs, with at least eight tilings each.
     const uint64_t tilings = p.t_end - p.t_begin;
     constexpr uint64_t kMinTilings = 8;
     uint64_t grid = (tilings + kMinTilings - 1) / kMinTilings;
-    if (grid > 3ull * (uint32_t)sm_count) grid = 3ull * (uint32_t)sm_count;
+    if (grid > most) grid = most;
     if (!grid) grid = 1;
     // (a caller with a fixed scratch: a device that would take more CTAs is refused, not silently under-used)
     if (max_ctas && grid > max_ctas) return MMEE_ERR_RANGE;
@@ -82,19 +89,7 @@ int mmee_create(const mmee_workload_t* workload, const mmee_arch_t* arch, const 
     if (h->plan.row_pruning && (rc = set_kept_masks(&h->plan, &h->kept_rows))) { delete h; return rc; }
     rc = choose_launch_shape(h->plan, h->device, 0, &h->shape);
     if (rc) { delete h; return rc; }
-    // one allocation: the search scratch, then one result record for mmee_decode
-    const size_t sbytes = (scratch_bytes(h->shape.grid) + 15) / 16 * 16;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->scratch), sbytes + sizeof(mmee_result_t));
-    if (e == cudaSuccess) {
-        h->decode_buf = reinterpret_cast<mmee_result_t*>(reinterpret_cast<unsigned char*>(h->scratch) + sbytes);
-        e = launch_reset(h->scratch, 0);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-    }
-    if (e != cudaSuccess) {
-        if (h->scratch) cudaFree(h->scratch);
-        delete h;
-        return cuda_status(e);
-    }
+    if ((rc = workspace_acquire(h->device, &h->ws))) { delete h; return rc; }
     h->create_ms = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
     *out = h;
     return MMEE_OK;
@@ -109,17 +104,15 @@ static int check_device(const mmee_handle* h) {
     return cur == h->device ? MMEE_OK : MMEE_ERR_ARG;
 }
 
-int mmee_search(mmee_handle_t* h, void* cuda_stream, mmee_result_t* out_best, mmee_result_t* out_topk) {
-    if (!h || !out_best) return MMEE_ERR_ARG;
+static int search_on(mmee_handle* h, cudaStream_t st, mmee_result_t* out_best, mmee_result_t* out_topk) {
     int rc = check_device(h);
     if (rc) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (h->dirty) {        // an earlier launch on this handle failed: the header may hold a used work counter
-        if ((rc = cuda_status(launch_reset(h->scratch, st)))) return rc;
+    if (h->dirty) {        // an earlier launch on this handle failed: the header may hold a used ticket counter
+        if ((rc = cuda_status(launch_reset(h->ws->scratch, st)))) return rc;
         h->dirty = false;
     }
     if (h->timing) cudaEventRecord(h->ev[0], st);
-    const cudaError_t e = launch_search(h->plan, h->shape, h->scratch, out_best, out_topk, st);
+    const cudaError_t e = launch_search(h->plan, h->shape, h->ws->scratch, out_best, out_topk, st);
     if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
     if (h->timing) cudaEventRecord(h->ev[1], st);
     h->last.kernels_launched = 1;
@@ -132,35 +125,43 @@ int mmee_search(mmee_handle_t* h, void* cuda_stream, mmee_result_t* out_best, mm
     return MMEE_OK;
 }
 
+int mmee_search(mmee_handle_t* h, void* cuda_stream, mmee_result_t* out_best, mmee_result_t* out_topk) {
+    if (!h || !out_best) return MMEE_ERR_ARG;
+    h->in_flight = true;
+    return search_on(h, static_cast<cudaStream_t>(cuda_stream), out_best, out_topk);
+}
+
 int mmee_search_host(mmee_handle_t* h, mmee_result_t* out_best, mmee_result_t* out_topk) {
     if (!h || !out_best) return MMEE_ERR_ARG;
     const uint32_t k = h->plan.topk;
     int rc;
-    if (!h->host_out) {
-        // Pinned, mapped host memory: the kernel's last CTA writes the records straight into it, so that the
-        // host needs no copy call after the search, only the synchronisation.
-        rc = cuda_status(cudaHostAlloc(reinterpret_cast<void**>(&h->host_out), (size_t)(1 + k) * sizeof(mmee_result_t),
-                                       cudaHostAllocMapped));
-        if (rc) { h->host_out = nullptr; return rc; }
-    }
-    mmee_result_t* dev = nullptr;
-    if ((rc = cuda_status(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dev), h->host_out, 0)))) return rc;
-    if ((rc = mmee_search(h, nullptr, dev, dev + 1))) return rc;
-    if ((rc = cuda_status(cudaStreamSynchronize(nullptr)))) return rc;
-    std::memcpy(out_best, h->host_out, sizeof(mmee_result_t));
-    if (out_topk) std::memcpy(out_topk, h->host_out + 1, (size_t)k * sizeof(mmee_result_t));
+    if ((rc = search_on(h, nullptr, h->ws->host_dev, h->ws->host_dev + 1))) return rc;
+    if ((rc = cuda_status(cudaStreamSynchronize(nullptr)))) { h->in_flight = true; return rc; }
+    std::memcpy(out_best, h->ws->host, sizeof(mmee_result_t));
+    if (out_topk) std::memcpy(out_topk, h->ws->host + 1, (size_t)k * sizeof(mmee_result_t));
     return out_best->status == MMEE_ERR_CHECK ? MMEE_ERR_CHECK : MMEE_OK;
 }
 
 int mmee_destroy(mmee_handle_t* h) {
     if (!h) return MMEE_ERR_ARG;
-    cudaError_t e = cudaSuccess;
     if (h->timing) for (int i = 0; i < 2; ++i) cudaEventDestroy(h->ev[i]);
-    if (h->scratch) e = cudaFree(h->scratch);
-    if (h->host_out) cudaFreeHost(h->host_out);
+    int rc = MMEE_OK;
+    if (h->in_flight) {
+        // A search that the caller launched may still run: the workspace goes to the next handle only after it.  (Its
+        // stream may be gone; the wait is the one that freeing device memory implies.)
+        int cur = h->device;
+        cudaError_t e = cudaGetDevice(&cur);
+        if (e == cudaSuccess && cur != h->device) e = cudaSetDevice(h->device);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        if (cur != h->device) cudaSetDevice(cur);
+        rc = cuda_status(e);
+    }
+    const int rc2 = workspace_release(h->ws, rc == MMEE_OK && !h->dirty);
     delete h;
-    return cuda_status(e);
+    return rc ? rc : rc2;
 }
+
+int mmee_trim(void) { return workspace_trim(); }
 
 uint64_t mmee_num_candidates(const mmee_handle_t* h) {
     return h ? h->plan.n_tilings * (uint64_t)h->plan.rows_per_tiling * 9u : 0;
@@ -196,8 +197,10 @@ int mmee_decode(mmee_handle_t* h, uint64_t idx, mmee_result_t* host_out) {
     if (!h || !host_out || idx >= mmee_num_candidates(h)) return MMEE_ERR_ARG;
     int rc = check_device(h);
     if (rc) return rc;
-    if ((rc = cuda_status(launch_eval(h->plan, idx, 1, h->decode_buf, nullptr)))) return rc;
-    return cuda_status(cudaMemcpy(host_out, h->decode_buf, sizeof(mmee_result_t), cudaMemcpyDeviceToHost));
+    if ((rc = cuda_status(launch_eval(h->plan, idx, 1, h->ws->host_dev, nullptr)))) return rc;
+    if ((rc = cuda_status(cudaStreamSynchronize(nullptr)))) { h->in_flight = true; return rc; }
+    std::memcpy(host_out, h->ws->host, sizeof(mmee_result_t));
+    return MMEE_OK;
 }
 
 int mmee_dump_keys(mmee_handle_t* h, void* cuda_stream, int64_t* out_keys) {
@@ -223,20 +226,11 @@ int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch, co
     int rc = mmee_create(workload, arch, objective, &h);
     if (rc) return rc;
     const uint32_t k = h->plan.topk;
-    const size_t bytes = (size_t)(k + 1) * sizeof(mmee_result_t);
-    mmee_result_t* dev = nullptr;
-    if ((rc = cuda_status(cudaMalloc(reinterpret_cast<void**>(&dev), bytes)))) { mmee_destroy(h); return rc; }
-    rc = mmee_search(h, nullptr, dev, dev + 1);
-    if (rc == MMEE_OK) rc = cuda_status(cudaMemcpy(out_best, dev, sizeof(mmee_result_t), cudaMemcpyDeviceToHost));
-    if (rc == MMEE_OK && out_topk)
-        rc = cuda_status(cudaMemcpy(out_topk, dev + 1, (size_t)k * sizeof(mmee_result_t), cudaMemcpyDeviceToHost));
-    // the finalize step's self-check failed: the records are not a result
-    if (rc == MMEE_OK && out_best->status == MMEE_ERR_CHECK) rc = MMEE_ERR_CHECK;
+    rc = mmee_search_host(h, out_best, out_topk);
     // The plan (divisor lists, query vectors, coefficients) travels to the device as the kernels'
     // parameter block: once per launch.
     if (h2d_bytes) *h2d_bytes = 2ull * sizeof(mmee::Plan);
     if (d2h_bytes) *d2h_bytes = sizeof(mmee_result_t) * (uint64_t)(1 + (out_topk ? k : 0));
-    cudaFree(dev);
     const int rc2 = mmee_destroy(h);
     return rc ? rc : rc2;
 }
@@ -253,28 +247,23 @@ int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch, 
     if (rc) return rc;
     rc = mmee_create(workload, arch, &ol, &hl);
     if (rc) { mmee_destroy(he); return rc; }
-    mmee_result_t* dev = nullptr;
-    rc = cuda_status(cudaMalloc(reinterpret_cast<void**>(&dev), sizeof(mmee_result_t)));
     mmee_result_t r;
     int64_t latency_cap = INT64_MAX - 1;
     uint32_t n = 0;
     while (rc == MMEE_OK) {
         // least energy among the mappings that are still faster than the previous point
         he->plan.key_cap = latency_cap;
-        if ((rc = mmee_search(he, nullptr, dev, nullptr))) break;
-        if ((rc = cuda_status(cudaMemcpy(&r, dev, sizeof(r), cudaMemcpyDeviceToHost)))) break;
+        if ((rc = mmee_search_host(he, &r, nullptr))) break;
         if (r.idx == MMEE_NO_INDEX) break;                       // nothing faster is left
         // the fastest mapping at that energy: the point of the front, with its lowest index
         hl->plan.key_cap = r.e_key;
-        if ((rc = mmee_search(hl, nullptr, dev, nullptr))) break;
-        if ((rc = cuda_status(cudaMemcpy(&r, dev, sizeof(r), cudaMemcpyDeviceToHost)))) break;
+        if ((rc = mmee_search_host(hl, &r, nullptr))) break;
         if (r.idx == MMEE_NO_INDEX) { rc = MMEE_ERR_CHECK; break; }   // cannot happen: the previous optimum qualifies
         if (n < capacity) out_points[n] = r;
         ++n;
         if (r.l_key == 0) break;
         latency_cap = r.l_key - 1;
     }
-    if (dev) cudaFree(dev);
     mmee_destroy(he);
     mmee_destroy(hl);
     *n_points = n;
@@ -294,8 +283,6 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
     mmee_handle_t* h = nullptr;
     int rc = mmee_create(workload, &a, &o, &h);
     if (rc) return rc;
-    mmee_result_t* dev = nullptr;
-    rc = cuda_status(cudaMalloc(reinterpret_cast<void**>(&dev), sizeof(mmee_result_t)));
     mmee_result_t r, held;
     bool have = false;
     uint32_t n = 0;
@@ -303,9 +290,7 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
     // mapping needs; the next one allows one word less than that.  While the traffic stays the same the mapping
     // found needs less buffer for the same traffic; when it rises, the mapping held is a point of the front.
     while (rc == MMEE_OK) {
-        if ((rc = mmee_search(h, nullptr, dev, nullptr))) break;
-        if ((rc = cuda_status(cudaMemcpy(&r, dev, sizeof(r), cudaMemcpyDeviceToHost)))) break;
-        if (r.status == MMEE_ERR_CHECK) { rc = MMEE_ERR_CHECK; break; }
+        if ((rc = mmee_search_host(h, &r, nullptr))) break;
         const bool found = r.idx != MMEE_NO_INDEX;
         if (have && (!found || r.e_key != held.e_key)) {
             if (n < capacity) out_points[n] = held;
@@ -317,7 +302,6 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
         if (r.bs <= 0) { if (n < capacity) out_points[n] = held; ++n; break; }      // (cannot happen: tiles take words)
         h->plan.cap_words = r.bs - 1;
     }
-    if (dev) cudaFree(dev);
     mmee_destroy(h);
     *n_points = n;
     if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
@@ -332,35 +316,55 @@ int mmee_search_shapes(const mmee_workload_t* workload, const mmee_arch_t* arch,
     mmee_objective_t o = *objective;
     o.topk = 1;
     o.row_pruning = 0;
-    mmee_result_t* dev = nullptr;
-    int rc = cuda_status(cudaMalloc(reinterpret_cast<void**>(&dev), sizeof(mmee_result_t)));
+    int device = 0;
+    int rc = cuda_status(cudaGetDevice(&device));
     if (rc) return rc;
+    Workspace* ws = nullptr;
+    bool clean = true;
     bool have = false;
     int64_t best_key = 0;
-    for (uint32_t i = 0; i < n_shapes && rc == MMEE_OK; ++i) {
-        mmee_arch_t a = *arch;
-        a.pe_rows = shapes[2 * i];
-        a.pe_cols = shapes[2 * i + 1];
-        mmee_handle_t* h = nullptr;
-        if ((rc = mmee_create(workload, &a, &o, &h))) break;
-        rc = mmee_search(h, nullptr, dev, nullptr);
-        if (rc == MMEE_OK)
-            rc = cuda_status(cudaMemcpy(&out_per_shape[i], dev, sizeof(mmee_result_t), cudaMemcpyDeviceToHost));
-        if (rc == MMEE_OK && out_per_shape[i].status == MMEE_ERR_CHECK) rc = MMEE_ERR_CHECK;
-        const int rc2 = mmee_destroy(h);
-        if (rc == MMEE_OK) rc = rc2;
-        if (rc != MMEE_OK || out_per_shape[i].idx == MMEE_NO_INDEX) continue;
-        const mmee_result_t& r = out_per_shape[i];
-        // the key the search ordered by: energy, latency, or the bit pattern of the positive EDP product
-        int64_t key;
-        switch (o.objective) {
-            case MMEE_OBJ_ENERGY: case MMEE_OBJ_ENERGY_LCAP: key = r.e_key; break;
-            case MMEE_OBJ_LATENCY: case MMEE_OBJ_LATENCY_ECAP: key = r.l_key; break;
-            default: std::memcpy(&key, &r.edp_key, sizeof(key)); break;
+    // The shapes' searches follow one another on the stream, each with a record of its own; the host plans the next
+    // one meanwhile and waits once per kHostRecords of them.
+    for (uint32_t i0 = 0; i0 < n_shapes && rc == MMEE_OK; i0 += kHostRecords) {
+        const uint32_t n = n_shapes - i0 < kHostRecords ? n_shapes - i0 : kHostRecords;
+        for (uint32_t i = 0; i < n; ++i) {
+            mmee_arch_t a = *arch;
+            a.pe_rows = shapes[2 * (i0 + i)];
+            a.pe_cols = shapes[2 * (i0 + i) + 1];
+            Plan plan;
+            LaunchShape shape;
+            if ((rc = build_plan(workload, &a, &o, &plan))) break;
+            if ((rc = choose_launch_shape(plan, device, 0, &shape))) break;
+            if (!ws && (rc = workspace_acquire(device, &ws))) break;
+            if ((rc = cuda_status(launch_search(plan, shape, ws->scratch, ws->host_dev + i, nullptr, nullptr)))) {
+                clean = false;
+                break;
+            }
         }
-        if (!have || key < best_key) { have = true; best_key = key; *out_best_shape = i; }
+        if (!ws) break;
+        const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
+        if (rc2) clean = false;
+        if (rc == MMEE_OK) rc = rc2;
+        if (rc != MMEE_OK) break;
+        std::memcpy(out_per_shape + i0, ws->host, n * sizeof(mmee_result_t));
+        for (uint32_t i = i0; i < i0 + n; ++i) {
+            const mmee_result_t& r = out_per_shape[i];
+            if (r.status == MMEE_ERR_CHECK) rc = MMEE_ERR_CHECK;
+            if (rc != MMEE_OK || r.idx == MMEE_NO_INDEX) continue;
+            // the key the search ordered by: energy, latency, or the bit pattern of the positive EDP product
+            int64_t key;
+            switch (o.objective) {
+                case MMEE_OBJ_ENERGY: case MMEE_OBJ_ENERGY_LCAP: key = r.e_key; break;
+                case MMEE_OBJ_LATENCY: case MMEE_OBJ_LATENCY_ECAP: key = r.l_key; break;
+                default: std::memcpy(&key, &r.edp_key, sizeof(key)); break;
+            }
+            if (!have || key < best_key) { have = true; best_key = key; *out_best_shape = i; }
+        }
     }
-    cudaFree(dev);
+    if (ws) {
+        const int rc2 = workspace_release(ws, clean);
+        if (rc == MMEE_OK) rc = rc2;
+    }
     return rc;
 }
 
@@ -425,7 +429,7 @@ int mmee_last_search_stats(const mmee_handle_t* h, mmee_launch_stats_t* out) {
     out->rows_tested = 0;
     if (h->last.kernels_launched) {
         unsigned long long counters[2] = {0, 0};      // last_exact_groups, last_tested_rows
-        const int rc = cuda_status(cudaMemcpy(counters, &h->scratch->last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
+        const int rc = cuda_status(cudaMemcpy(counters, &h->ws->scratch->last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
         if (rc) return rc;
         out->exact_path_visits = counters[0];
         out->rows_tested = counters[1];

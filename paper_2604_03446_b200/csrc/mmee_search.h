@@ -52,6 +52,8 @@ cudaError_t launch_group_flags(const Plan& p, int64_t threshold, unsigned char* 
 cudaError_t launch_eval(const Plan& p, uint64_t idx_begin, uint64_t count, mmee_result_t* out, cudaStream_t st);
 cudaError_t measure_alu_peak(double* giops);
 
+// Most CTAs that a search on `device` takes.
+int max_search_ctas(int device, uint32_t* out);
 // Launch shape of a search on `device` (at most max_ctas CTAs when that is not 0: MMEE_ERR_RANGE if it would take more).
 int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShape* shape);
 

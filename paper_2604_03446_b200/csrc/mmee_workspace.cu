@@ -1,0 +1,106 @@
+// Workspaces kept between handles.
+//
+// A one-shot search takes 20 to 30 us on the device, but cudaMalloc and cudaFree of its scratch took about 700 us of
+// host time around it: with no other allocation of the library alive the driver maps and unmaps a 2 MB slab each time
+// (a search of 768 tilings through mmee_solve_host: 730 us).  So a workspace that is no longer in use stays in a list,
+// at most kMaxIdle of them (0.13 MB of device and 6 KB of pinned host memory each), for the next handle on its device.
+// A workspace belongs to one handle or call at a time, whatever thread or stream uses it; mmee_trim frees the idle ones.
+#include "mmee_workspace.h"
+
+#include <mutex>
+#include <new>
+
+namespace mmee {
+
+namespace {
+
+constexpr int kMaxIdle = 8;
+
+std::mutex g_mutex;
+Workspace* g_idle = nullptr;
+int g_n_idle = 0;
+
+int free_workspace(Workspace* ws) {
+    cudaError_t e = ws->scratch ? cudaFree(ws->scratch) : cudaSuccess;
+    if (ws->host) {
+        const cudaError_t e2 = cudaFreeHost(ws->host);
+        if (e == cudaSuccess) e = e2;
+    }
+    delete ws;
+    return cuda_status(e);
+}
+
+int make_workspace(int device, Workspace** out) {
+    Workspace* ws = new (std::nothrow) Workspace();
+    if (!ws) return MMEE_ERR_ARG;
+    ws->device = device;
+    int rc = max_search_ctas(device, &ws->max_ctas);
+    if (rc) { delete ws; return rc; }
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&ws->scratch), scratch_bytes(ws->max_ctas));
+    // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
+    // host needs no copy call after a search, only the synchronisation
+    if (e == cudaSuccess)
+        e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t),
+                          cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ws->host_dev), ws->host, 0);
+    if (e == cudaSuccess) e = launch_reset(ws->scratch, 0);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (e != cudaSuccess) {
+        free_workspace(ws);
+        return cuda_status(e);
+    }
+    *out = ws;
+    return MMEE_OK;
+}
+
+}  // namespace
+
+int workspace_acquire(int device, Workspace** out) {
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        for (Workspace** at = &g_idle; *at; at = &(*at)->next) {
+            if ((*at)->device != device) continue;
+            *out = *at;
+            *at = (*at)->next;
+            --g_n_idle;
+            return MMEE_OK;
+        }
+    }
+    const int rc = make_workspace(device, out);
+    if (rc != MMEE_ERR_CUDA) return rc;
+    workspace_trim();           // (another device's idle workspaces hold pinned host memory)
+    return make_workspace(device, out);
+}
+
+int workspace_release(Workspace* ws, bool clean) {
+    if (clean) {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (g_n_idle < kMaxIdle) {
+            ws->next = g_idle;
+            g_idle = ws;
+            ++g_n_idle;
+            return MMEE_OK;
+        }
+    }
+    return free_workspace(ws);
+}
+
+int workspace_trim() {
+    Workspace* list;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        list = g_idle;
+        g_idle = nullptr;
+        g_n_idle = 0;
+    }
+    int rc = MMEE_OK;
+    while (list) {
+        Workspace* ws = list;
+        list = list->next;
+        const int r = free_workspace(ws);
+        if (rc == MMEE_OK) rc = r;
+    }
+    return rc;
+}
+
+}  // namespace mmee

@@ -1,0 +1,28 @@
+// Internal: the memory a search needs -- device scratch and pinned host records -- kept between handles.
+#pragma once
+
+#include "mmee_search.h"
+
+namespace mmee {
+
+// One search's workspace.  Everything a search on the device needs fits it, whatever the problem.
+struct Workspace {
+    int device;
+    Scratch* scratch;               // device; its header is clean while the workspace is not in use
+    uint32_t max_ctas;              // partial lists the scratch has room for
+    mmee_result_t* host;            // pinned host memory: 1 + MMEE_MAX_TOPK records that kernels write into
+    mmee_result_t* host_dev;        // the same memory as the device addresses it
+    Workspace* next;
+};
+
+constexpr uint32_t kHostRecords = 1 + MMEE_MAX_TOPK;
+
+// A workspace on the current device (`device`), for the caller alone until it is given back.
+int workspace_acquire(int device, Workspace** out);
+// Gives it back.  `clean`: no work on it is in flight and its header is in its initial state; otherwise it is freed.
+// Returns the status of the free.
+int workspace_release(Workspace* ws, bool clean);
+// Frees every workspace that is not in use.
+int workspace_trim();
+
+}  // namespace mmee

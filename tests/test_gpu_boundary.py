@@ -311,3 +311,60 @@ def test_fronts_and_flags_on_a_problem_in_which_nothing_fits():
     with Handle(small, obj) as h:
         best, _ = mm.mmee_search_host(h)
     assert best.idx == mm.NO_INDEX and best.status == mm.ERR_NO_FEASIBLE and best.n_feasible == 0
+
+
+def test_workspaces_are_not_shared_between_live_handles_threads_or_streams():
+    """Released workspaces serve the next handle: one-shot calls from several threads, handles released while their
+    search is still in flight on a side stream, and more live handles than workspaces are kept, each with the oracle's
+    optimum; after mmee_trim everything works as before."""
+    import threading
+    cfgs = [mi.random_tiny_problem(s) for s in (2, 3, 5, 7)]
+    jobs = [(c, shrink_to(c, dict(c["searches"][0], topk=2), 2_000_000)) for c in cfgs]
+    want = [[r.idx for r in oracle.search(oracle.make_problem(c["workload"], c["arch"], o)).topk] for c, o in jobs]
+    found = lambda topk: [r.idx for r in topk if r.idx != mm.NO_INDEX]
+
+    errors = []
+
+    def worker(i):
+        try:
+            torch.cuda.set_device(0)
+            for n in range(40):
+                c, o = jobs[(i + n) % len(jobs)]
+                assert found(mm.mmee_solve_host(c["workload"], c["arch"], o)[1]) == want[(i + n) % len(jobs)]
+        except Exception as e:                       # noqa: BLE001 (reported by the main thread)
+            errors.append(e)
+
+    threads = [threading.Thread(target=worker, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    pending = []
+    for n in range(60):                              # released while in flight, the next handle at once
+        c, o = jobs[n % len(jobs)]
+        st = streams[n % len(streams)]
+        top = mm.result_buffer(2)
+        st.wait_stream(torch.cuda.current_stream())
+        h = mm.mmee_create(c["workload"], c["arch"], o)
+        mm.mmee_search(h, mm.result_buffer(1), top, stream=st)
+        mm.mmee_destroy(h)
+        pending.append((top, n % len(jobs)))
+    torch.cuda.synchronize()
+    for top, j in pending:
+        assert found(mm.read_results(top, 2)) == want[j]
+
+    handles = [mm.mmee_create(c["workload"], c["arch"], o) for c, o in jobs * 4]     # more than are kept
+    tops = [mm.result_buffer(2) for _ in handles]
+    best = [mm.result_buffer(1) for _ in handles]
+    for h, b, t in zip(handles, best, tops):
+        mm.mmee_search(h, b, t)
+    for h in handles:
+        mm.mmee_destroy(h)
+    mm.mmee_trim()
+    for i, t in enumerate(tops):
+        assert found(mm.read_results(t, 2)) == want[i % len(jobs)]
+    c, o = jobs[0]
+    assert found(mm.mmee_solve_host(c["workload"], c["arch"], o)[1]) == want[0]
