@@ -127,7 +127,7 @@ struct Shared {
     uint32_t last_cta, check_failed;
     union {
         TileTab tile[kMaxChunk];
-        BlockTab block[MMEE_MAX_TOPK];
+        BlockTab block[kWarps];
     };
 };
 
@@ -186,64 +186,76 @@ __device__ __forceinline__ void best_of_block(const Plan& p, const Shared& sh, i
     warp_min_pair(ek, ei);
 }
 
-// The k best mappings of the first n_found blocks in sh.block, none above `bound`: every warp takes its share of the
-// blocks' class combinations in ascending order and keeps a list of mappings.
+// The mappings of block `j` of sh.block that precede the running k-th pair (lk, li), none above `bound`, into the warps'
+// lists.  Every warp takes its share of the block's class combinations best first, so that a list is full after one or
+// two of them (the rows of a combination share their keys) and the others are only compared with its last entry: taken
+// in index order instead, with all blocks in one pass, this took 53 us of a top-16 search whose best keys tie.
 template <int OBJ>
-__device__ __forceinline__ void best_of_blocks(const Plan& p, const Shared& sh, int n_blocks, int64_t bound, int k, int lane,
-                                               int64_t& ek, uint64_t& ei) {
-    ek = kInfKey;
-    ei = UINT64_MAX;
-    const uint32_t total = (uint32_t)n_blocks * kFusedReps;
-    for (uint32_t r0 = threadIdx.x - lane; r0 < total; r0 += kSearchThreads) {
-        const uint32_t mine = r0 + lane;
-        int64_t least = kInfKey;
-        uint64_t first = UINT64_MAX;
-        if (mine < total) {
-            const BlockTab& bt = sh.block[mine / kFusedReps];
-            const uint32_t r = mine % kFusedReps;
-            const bool fused = bt.phi == 0;
-            if (fused || r < kUnfusedReps) {
-                const Rep q = decode_rep(sh.order[bt.slot], fused, r);
-                const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
-                if (t.fits) {
-                    for (int s = 0; s < 9; ++s)
-                        if ((p.sm_mask >> s) & 1u) least = min64(least, mapping_key<OBJ>(p, bt, t, s));
-                    first = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u;
-                }
-            }
-        }
-        bool todo = least <= bound && least != kInfKey;
-        while (true) {
-            int64_t lk = __shfl_sync(kFull, ek, k - 1);
-            uint64_t li = __shfl_sync(kFull, ei, k - 1);
-            const unsigned m = __ballot_sync(kFull, todo && pair_less(least, first, lk, li));
-            if (!m) break;
-            // one class combination at a time: all of its rows, all stationary pairs, across the lanes
-            const int src = __ffs(m) - 1;
-            if (lane == src) todo = false;
-            const BlockTab& bt = sh.block[(r0 + src) / kFusedReps];
-            const bool fused = bt.phi == 0;
-            const Rep q = decode_rep(sh.order[bt.slot], fused, (r0 + src) % kFusedReps);
-            const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
-            const uint32_t n = (uint32_t)(q.width[0] * q.width[1] * q.width[2] * q.width[3] * q.width[4]) * 9u;
-            for (uint32_t i0 = 0; i0 < n; i0 += 32) {
-                const uint32_t i = i0 + lane;
-                uint32_t u = i / 9u;
-                const int s = (int)(i - u * 9u);
-                int lv[5];
+__device__ __forceinline__ void best_of_block_multi(const Plan& p, const Shared& sh, int j, int64_t bound, int k, int lane,
+                                                    int64_t lk, uint64_t li, int64_t& ek, uint64_t& ei) {
+    const BlockTab& bt = sh.block[j];
+    const OrderInfo& o = sh.order[bt.slot];
+    const bool fused = bt.phi == 0;
+    const uint32_t n_reps = fused ? kFusedReps : kUnfusedReps;
+    constexpr int kShare = (int)((kFusedReps + kSearchThreads - 1) / kSearchThreads);
+    int64_t least[kShare];
+    uint64_t first[kShare];
 #pragma unroll
-                for (int x = 4; x >= 0; --x) {
-                    const uint32_t w = (uint32_t)q.width[x], v = u / w;
-                    lv[x] = q.lv[x] + (int)(u - v * w);
-                    u = v;
-                }
-                const int64_t key = mapping_key<OBJ>(p, bt, t, s);
-                const uint64_t idx = bt.first_idx + row_of(fused, lv[0], lv[1], lv[2], lv[3], lv[4]) * 9u + (uint32_t)s;
-                lk = __shfl_sync(kFull, ek, k - 1);
-                li = __shfl_sync(kFull, ei, k - 1);
-                const bool pend = i < n && ((p.sm_mask >> s) & 1u) && key <= bound && pair_less(key, idx, lk, li);
-                warp_offer(ek, ei, k, key, idx, pend, lane);
+    for (int i = 0; i < kShare; ++i) {
+        least[i] = kInfKey;
+        first[i] = UINT64_MAX;
+        const uint32_t r = threadIdx.x + (uint32_t)i * kSearchThreads;
+        if (r >= n_reps) continue;
+        const Rep q = decode_rep(o, fused, r);
+        const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        if (!t.fits) continue;
+        int64_t m = kInfKey;
+        for (int s = 0; s < 9; ++s)
+            if ((p.sm_mask >> s) & 1u) m = min64(m, mapping_key<OBJ>(p, bt, t, s));
+        if (m > bound) continue;
+        least[i] = m;
+        first[i] = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u;
+    }
+    while (true) {
+        // the best combination not yet taken, and the pair it has to precede
+        int64_t bk = least[0];
+        uint64_t bi = first[0];
+#pragma unroll
+        for (int i = 1; i < kShare; ++i)
+            if (pair_less(least[i], first[i], bk, bi)) { bk = least[i]; bi = first[i]; }
+        warp_min_pair(bk, bi);
+        const int64_t ok = __shfl_sync(kFull, ek, k - 1);
+        const uint64_t oi = __shfl_sync(kFull, ei, k - 1);
+        if (pair_less(ok, oi, lk, li)) { lk = ok; li = oi; }
+        if (!pair_less(bk, bi, lk, li)) break;
+        uint32_t r = 0;
+#pragma unroll
+        for (int i = 0; i < kShare; ++i)
+            if (first[i] == bi) { r = threadIdx.x + (uint32_t)i * kSearchThreads + 1u; least[i] = kInfKey; first[i] = UINT64_MAX; }
+        r = __reduce_max_sync(kFull, r) - 1u;
+        // all of its rows and stationary pairs, in index order across the lanes
+        const Rep q = decode_rep(o, fused, r);
+        const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        const uint32_t n = (uint32_t)(q.width[0] * q.width[1] * q.width[2] * q.width[3] * q.width[4]) * 9u;
+        for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+            const uint32_t i = i0 + lane;
+            uint32_t u = i / 9u;
+            const int s = (int)(i - u * 9u);
+            int lv[5];
+#pragma unroll
+            for (int x = 4; x >= 0; --x) {
+                const uint32_t w = (uint32_t)q.width[x], v = u / w;
+                lv[x] = q.lv[x] + (int)(u - v * w);
+                u = v;
             }
+            const int64_t key = mapping_key<OBJ>(p, bt, t, s);
+            const uint64_t idx = bt.first_idx + row_of(fused, lv[0], lv[1], lv[2], lv[3], lv[4]) * 9u + (uint32_t)s;
+            const int64_t tk = __shfl_sync(kFull, ek, k - 1);
+            const uint64_t ti = __shfl_sync(kFull, ei, k - 1);
+            const bool pend = i < n && ((p.sm_mask >> s) & 1u) && key <= bound && pair_less(key, idx, lk, li) && pair_less(key, idx, tk, ti);
+            // (later rows repeat the same keys at higher indices)
+            if (!__any_sync(kFull, pend)) break;
+            warp_offer(ek, ei, k, key, idx, pend, lane);
         }
     }
 }
@@ -323,17 +335,21 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
         sh.feasible_rows[warp] = rows;
         sh.live_tilings[warp] = (uint32_t)live;
     }
-    int n_blocks, found;
+    int found;
+    uint32_t n_groups = 0;         // groups of five rows of the blocks evaluated mapping by mapping
     int64_t bound;
     if (!MULTI) {
         warp_min_pair(ek, ei);
         min_over_warps(sh, lane, warp, ek, ei);
-        found = n_blocks = ek != kInfKey ? 1 : 0;
+        found = ek != kInfKey ? 1 : 0;
         bound = ek;
         // ---- the winning block, mapping by mapping
-        if (n_blocks && tid < kBlockItems) block_item(p, (uint32_t)ei, tid, &sh.block[0]);
+        if (found && tid < kBlockItems) block_item(p, (uint32_t)ei, tid, &sh.block[0]);
         __syncthreads();
-        if (n_blocks) best_of_block<OBJ>(p, sh, bound, ek, ei);
+        if (found) {
+            n_groups = block_rows(sh.block[0]) / 5u;
+            best_of_block<OBJ>(p, sh, bound, ek, ei);
+        }
         min_over_warps(sh, lane, warp, ek, ei);
     } else {
         merge_warps(sh, k, lane, warp, ek, ei);
@@ -346,14 +362,46 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
             if (j < lane && other == e.y) fresh = false;
         }
         unsigned m = __ballot_sync(kFull, fresh);
-        n_blocks = __popc(m);
-        for (int j = 0; m; m &= m - 1, ++j) {
-            const uint32_t id = (uint32_t)__shfl_sync(kFull, e.y, __ffs(m) - 1);
-            if (j % kWarps == warp) block_item(p, id, lane, &sh.block[j]);
+        const int n_fresh = __popc(m);
+        ek = kInfKey;
+        ei = UINT64_MAX;
+        int64_t lk = kInfKey;           // the k-th best mapping so far
+        uint64_t li = UINT64_MAX;
+        __syncthreads();                // sh.tops has been read
+        // ---- the winning blocks, mapping by mapping, best block first; once a block's (least key, first index) does
+        // not precede the k-th mapping, neither does a later one's
+        for (int j0 = 0; j0 < n_fresh; j0 += kWarps) {
+            int64_t bk[kWarps];
+#pragma unroll
+            for (int j = 0; j < kWarps; ++j) {
+                const int src = m ? __ffs(m) - 1 : 0;
+                bk[j] = m ? (int64_t)__shfl_sync(kFull, e.x, src) : kInfKey;
+                const uint32_t id = (uint32_t)__shfl_sync(kFull, e.y, src);
+                if (m && j == warp) block_item(p, id, lane, &sh.block[j]);
+                m &= m - 1;
+            }
+            __syncthreads();
+            bool more = true;
+#pragma unroll 1
+            for (int j = 0; j < kWarps && j0 + j < n_fresh; ++j) {
+                int64_t key = bk[0];
+#pragma unroll
+                for (int i = 1; i < kWarps; ++i) key = i == j ? bk[i] : key;
+                more = pair_less(key, sh.block[j].first_idx, lk, li);
+                if (!more) break;
+                n_groups += block_rows(sh.block[j]) / 5u;
+                best_of_block_multi<OBJ>(p, sh, j, bound, k, lane, lk, li, ek, ei);
+                merge_warps(sh, k, lane, warp, ek, ei);
+                const longlong2 last = sh.tops[0][k - 1];
+                lk = last.x;
+                li = (uint64_t)last.y;
+                if (warp) { ek = kInfKey; ei = UINT64_MAX; }        // (warp 0 goes on with the merged list)
+                __syncthreads();
+            }
+            if (!more) break;
         }
+        if (!n_fresh && lane < kTopK && warp == 0) sh.tops[0][lane] = make_longlong2(kInfKey, -1ll);
         __syncthreads();
-        best_of_blocks<OBJ>(p, sh, n_blocks, bound, k, lane, ek, ei);
-        merge_warps(sh, k, lane, warp, ek, ei);
     }
 
     // ---- every winner evaluated in full, one warp per record (the parts of a record on different lanes); the key it
@@ -387,16 +435,15 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
     }
     __syncthreads();
     if (tid == 0) {
-        unsigned long long all_rows = 0, all_live = 0, groups = 0;
+        unsigned long long all_rows = 0, all_live = 0;
         for (int w = 0; w < kWarps; ++w) { all_rows += sh.feasible_rows[w]; all_live += sh.live_tilings[w]; }
-        for (int j = 0; j < n_blocks; ++j) groups += block_rows(sh.block[j]) / 5u;
         first.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
         first.n_feasible = all_rows * (uint64_t)p.n_sm;
         if (sh.check_failed) first.status = MMEE_ERR_CHECK;
         *out_best = first;
         // ready for the next search on this scratch
         scratch->G = kInfKey - 1;
-        scratch->last_exact_groups = groups;
+        scratch->last_exact_groups = n_groups;
         const uint32_t unfused_modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
         scratch->last_tested_rows = all_live * p.n_orders * ((p.fuse_mask & 1u ? kFusedReps : 0u) + (unfused_modes ? 18u : 0u));
         scratch->done_ctas = 0;
