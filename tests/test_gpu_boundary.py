@@ -368,3 +368,51 @@ def test_workspaces_are_not_shared_between_live_handles_threads_or_streams():
         assert found(mm.read_results(t, 2)) == want[i % len(jobs)]
     c, o = jobs[0]
     assert found(mm.mmee_solve_host(c["workload"], c["arch"], o)[1]) == want[0]
+
+
+def test_searches_that_follow_one_another_on_a_stream():
+    """A search starts while the kernel before it on the stream ends: alternating searches of different problems and
+    list lengths into the same buffers, each followed by copies of its records on the same stream, without any wait
+    between; an empty tiling range among them; then the same from a captured graph."""
+    cfgs = [mi.random_tiny_problem(s) for s in (3, 5, 9)]
+    jobs = [(c, shrink_to(c, dict(c["searches"][0], topk=k), 2_000_000)) for c, k in zip(cfgs, (1, 16, 3))]
+    want = [[(r.idx, r.e_key) for r in oracle.search(oracle.make_problem(c["workload"], c["arch"], o)).topk] for c, o in jobs]
+    empty = (cfgs[1], dict(jobs[1][1], t_begin=3, t_end=3))
+    want.append([])
+    handles = [mm.mmee_create(c["workload"], c["arch"], o) for c, o in jobs + [empty]]
+    ks = [1, 16, 3, 16]
+    best, top = mm.result_buffer(1), mm.result_buffer(16)
+
+    def one_round():
+        out = []
+        for h, k in zip(handles, ks):
+            mm.mmee_search(h, best, top)
+            out.append((best.clone(), top.clone()))
+        return out
+
+    def check(rounds):
+        for b, (j, k) in zip(rounds, [(j, ks[j]) for j in range(4)] * (len(rounds) // 4)):
+            got = [(r.idx, r.e_key) for r in mm.read_results(b[1], k) if r.idx != mm.NO_INDEX]
+            assert got == want[j] and mm.read_results(b[0], 1)[0].idx == (want[j][0][0] if want[j] else mm.NO_INDEX)
+
+    try:
+        rounds = []
+        for _ in range(50):
+            rounds += one_round()
+        for _ in range(30):                      # no copies between: the last search's records stay
+            for h in handles[:3]:
+                mm.mmee_search(h, best, top)
+        rounds_end = (best.clone(), top.clone())
+        torch.cuda.synchronize()
+        check(rounds)
+        assert [(r.idx, r.e_key) for r in mm.read_results(rounds_end[1], 3) if r.idx != mm.NO_INDEX] == want[2]
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            captured = one_round()
+        for _ in range(5):
+            graph.replay()
+        torch.cuda.synchronize()
+        check(captured)
+    finally:
+        for h in handles:
+            mm.mmee_destroy(h)
