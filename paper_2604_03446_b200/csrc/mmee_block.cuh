@@ -25,14 +25,14 @@ __device__ __forceinline__ void stationary_terms(const Plan& p, const uint32_t b
     int64_t w, cy;
     uint32_t blk[3];
     tile_array_terms(p, b, op, sm, w, cy, blk);
-    const TilingCounts c = tiling_counts(p, b);
-    if (op == 0) {
-        P = p.c_br * (c.t1 * w + c.carry1) + p.c_mac * c.ikl + p.c_sfu * c.il;
-        Q = c.t1 * cy * (int64_t)p.bw;
-    } else {
-        P = p.c_br * (c.t2 * w + c.carry2) + p.c_mac * c.ilj;
-        Q = c.t2 * cy * (int64_t)p.bw;
-    }
+    // tile invocations; partial sums carried between the steps of the reduction; MACs (see tiling_counts)
+    const int64_t il = (int64_t)b[LOOP_I] * b[LOOP_L];
+    const int64_t outer = op == 0 ? il : (int64_t)b[LOOP_I] * b[LOOP_J];
+    const int64_t calls = il * (op == 0 ? b[LOOP_K] : b[LOOP_J]);
+    const int64_t carried = (calls - outer) * b[4 + LOOP_I] * (op == 0 ? b[4 + LOOP_L] : b[4 + LOOP_J]);
+    const int64_t elements = (int64_t)p.dim[LOOP_I] * p.dim[LOOP_L];
+    P = p.c_br * (calls * w + carried) + p.c_mac * (elements * (op == 0 ? p.dim[LOOP_K] : p.dim[LOOP_J])) + (op == 0 ? p.c_sfu * elements : 0);
+    Q = calls * cy * (int64_t)p.bw;
 }
 
 // Item `item` (0 .. kBlockItems - 1) of the tables of block `id` = tiling * n_blocks + block.

@@ -29,7 +29,7 @@ constexpr int64_t kNoRow = INT64_C(1) << 62;   // DRAM words of "no row fits"; s
 struct TileTab {
     int32_t  size[kSizeSlots];      // buffer words, saturated to kSizeCap
     uint32_t t;                     // tiling index
-    uint32_t iD, lD, jD;            // inter-tile bounds
+    uint32_t b[8];                  // bounds i_D, k_D, l_D, j_D, i_G, k_G, l_G, j_G
     // Stationary-pair terms, linear in the recomputation factor rho of C (j_D or 1):
     //   energy P1[sm1] * rho + P2[sm2] (buffer<->PE words, MACs, softmax), compute words Q1[sm1] * rho + Q2[sm2]
     int64_t  P1[3], P2[3], Q1[3], Q2[3];
@@ -43,12 +43,19 @@ MMEE_HD int sat_add(int a, int b) { const int s = a + b; return s < kSizeCap ? s
 MMEE_HD int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 MMEE_HD int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
 
-// Slot i of a tiling's size table.
-MMEE_HD uint64_t size_words(const uint32_t dim[4], const uint32_t g[4], int slot) {
-    // dimension pair of the slot and which of the two is whole: bits 0-1 / 2-3 the dimensions, bits 4 / 5 whole
+// Words of size slot `slot` of a tiling with tile extents g.  Six bits a slot: the two dimensions (bits 0-1, 2-3) and which
+// of them is whole (bits 4, 5); ten slots to a word, so that lanes with different slots look nothing up.
+constexpr uint64_t size_codes(int first) {
     constexpr uint8_t code[kSizeSlots] = {
         0x04, 0x24, 0x34, 0x09, 0x19, 0x39, 0x08, 0x18, 0x28, 0x38, 0x0e, 0x1e, 0x2e, 0x3e, 0x0c, 0x1c, 0x2c, 0x3c};
-    const uint32_t c = code[slot], x = c & 3u, y = (c >> 2) & 3u;
+    uint64_t w = 0;
+    for (int i = first; i < first + 10 && i < kSizeSlots; ++i) w |= (uint64_t)code[i] << (6 * (i - first));
+    return w;
+}
+MMEE_HD uint64_t size_words(const uint32_t dim[4], const uint32_t g[4], int slot) {
+    constexpr uint64_t lo = size_codes(0), hi = size_codes(10);
+    const uint32_t c = (uint32_t)(slot < 10 ? lo >> (6 * slot) : hi >> (6 * (slot - 10)));
+    const uint32_t x = c & 3u, y = (c >> 2) & 3u;
     return (uint64_t)((c & 16u) ? dim[x] : g[x]) * ((c & 32u) ? dim[y] : g[y]);
 }
 
@@ -69,13 +76,13 @@ MMEE_HD void fused_class(const TileTab& tb, const OrderInfo& oi, const DimWords&
     const uint32_t f = oi.flags;
     const bool rc = oi.recompute[c] != 0;
     // DRAM words (Section V-C).  A: fetched again for every l2 (and, when C is regenerated, every j2) above its blocker.
-    const int64_t rho = rc ? (int64_t)tb.jD : 1;
-    const int64_t gA[3] = {dw.ik * tb.lD * rho,
-                           dw.ik * ((f & kLaboveI) ? tb.lD : 1u) * ((f & kJaboveI) ? rho : 1), dw.ik};
-    const int64_t gB[3] = {dw.kl * tb.iD * rho,
-                           dw.kl * ((f & kIaboveL) ? tb.iD : 1u) * ((f & kJaboveL) ? rho : 1), dw.kl};
+    const int64_t rho = rc ? (int64_t)tb.b[LOOP_J] : 1;
+    const int64_t gA[3] = {dw.ik * tb.b[LOOP_L] * rho,
+                           dw.ik * ((f & kLaboveI) ? tb.b[LOOP_L] : 1u) * ((f & kJaboveI) ? rho : 1), dw.ik};
+    const int64_t gB[3] = {dw.kl * tb.b[LOOP_I] * rho,
+                           dw.kl * ((f & kIaboveL) ? tb.b[LOOP_I] : 1u) * ((f & kJaboveL) ? rho : 1), dw.kl};
     // D and E: (both at L3), (one held, the other at L3: the larger and the smaller sum), (both held)
-    const int64_t d_l3 = dw.lj * tb.iD, e_l3 = dw.ij * tb.lD;
+    const int64_t d_l3 = dw.lj * tb.b[LOOP_I], e_l3 = dw.ij * tb.b[LOOP_L];
     const int64_t y_held = dw.lj + dw.ij, y_none = d_l3 + e_l3, y_d = dw.lj + e_l3, y_e = d_l3 + dw.ij;
     const bool d_first = y_d <= y_e;            // holding D saves more
     const int64_t y_best = d_first ? y_d : y_e, y_next = d_first ? y_e : y_d;
@@ -157,10 +164,10 @@ MMEE_HD void unfused_nests(const TileTab& tb, const OrderInfo& oi, const DimWord
     const int B[3] = {tb.size[S_kl], tb.size[S_Kl], tb.size[S_KL]};
     const int D[3] = {tb.size[S_lj], tb.size[oi.size_d_lo], tb.size[S_LJ]};
     const int E[3] = {tb.size[S_ij], tb.size[oi.size_e_lo], tb.size[S_IJ]};
-    const int64_t gA[3] = {dw.ik * tb.lD, dw.ik * ((f & kLaboveI) ? tb.lD : 1u), dw.ik};
-    const int64_t gB[3] = {dw.kl * tb.iD, dw.kl * ((f & kIaboveL) ? tb.iD : 1u), dw.kl};
-    const int64_t gD[3] = {dw.lj * ((f & kIaboveD1) ? tb.iD : 1u), dw.lj * ((f & kIaboveD2) ? tb.iD : 1u), dw.lj};
-    const int64_t gE[3] = {dw.ij * ((f & kLaboveE1) ? tb.lD : 1u), dw.ij * ((f & kLaboveE2) ? tb.lD : 1u), dw.ij};
+    const int64_t gA[3] = {dw.ik * tb.b[LOOP_L], dw.ik * ((f & kLaboveI) ? tb.b[LOOP_L] : 1u), dw.ik};
+    const int64_t gB[3] = {dw.kl * tb.b[LOOP_I], dw.kl * ((f & kIaboveL) ? tb.b[LOOP_I] : 1u), dw.kl};
+    const int64_t gD[3] = {dw.lj * ((f & kIaboveD1) ? tb.b[LOOP_I] : 1u), dw.lj * ((f & kIaboveD2) ? tb.b[LOOP_I] : 1u), dw.lj};
+    const int64_t gE[3] = {dw.ij * ((f & kLaboveE1) ? tb.b[LOOP_L] : 1u), dw.ij * ((f & kLaboveE2) ? tb.b[LOOP_L] : 1u), dw.ij};
     uint32_t n1 = 0, n2 = 0, m1 = 0, m2 = 0;
     int64_t x1 = kNoRow, x2 = kNoRow;
 #pragma unroll
@@ -183,7 +190,7 @@ MMEE_HD void unfused_nests(const TileTab& tb, const OrderInfo& oi, const DimWord
     rows = n1 * n2;
     const bool some = x1 < kNoRow && x2 < kNoRow;
     words1 = some ? x1 + dw.il : kNoRow;
-    words2 = some ? x2 + dw.il * ((f & kJaboveC) ? tb.jD : 1u) : kNoRow;
+    words2 = some ? x2 + dw.il * ((f & kJaboveC) ? tb.b[LOOP_J] : 1u) : kNoRow;
 }
 
 MMEE_HD int64_t edp_bits(int64_t e, int64_t l) {       // ordered by the bit pattern of the positive product
@@ -223,7 +230,7 @@ MMEE_HD int64_t unfused_key(int64_t x1, int64_t x2, int64_t pass, int64_t P1, in
 // latency separate into the operators' own minima.
 template <int OBJ>
 MMEE_HD int64_t fused_least_key(const TileTab& tb, int64_t x, bool rc, uint32_t sm_mask, int64_t c_dram, int64_t cap) {
-    const int64_t rho = rc ? (int64_t)tb.jD : 1;
+    const int64_t rho = rc ? (int64_t)tb.b[LOOP_J] : 1;
     if ((OBJ == MMEE_OBJ_ENERGY || OBJ == MMEE_OBJ_LATENCY) && sm_mask == 0x1ffu) {
         const int64_t* u = OBJ == MMEE_OBJ_ENERGY ? tb.P1 : tb.Q1;
         const int64_t* v = OBJ == MMEE_OBJ_ENERGY ? tb.P2 : tb.Q2;

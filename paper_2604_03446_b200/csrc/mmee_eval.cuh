@@ -15,67 +15,75 @@ __device__ __forceinline__ int64_t monomial(uint32_t q, const uint32_t b[8]) {
     return v;
 }
 
-// Ceiling of a / b for 32-bit operands (tile extents and array sizes), widened for the products.
-__device__ __forceinline__ int64_t ceil_div(uint32_t a, uint32_t b) { return (int64_t)((a + b - 1u) / b); }
-
-// Compute cycles of one (m x r) * (r x n) tile on a rows x cols array.
-// 0 weight stationary: r x n weights folded onto the array, m inputs streamed per fold;
-// 1 input stationary:  m x r inputs folded, n weight columns streamed;
-// 2 output stationary: m x n outputs folded, r reduction steps streamed.
-__device__ __forceinline__ int64_t tile_cycles(int sm, uint32_t m, uint32_t r, uint32_t n, uint32_t rows, uint32_t cols) {
-    if (sm == 0) return ceil_div(r, rows) * ceil_div(n, cols) * (int64_t)m;
-    if (sm == 1) return ceil_div(m, rows) * ceil_div(r, cols) * (int64_t)n;
-    return ceil_div(m, rows) * ceil_div(n, cols) * (int64_t)r;
+// Words moved between the global buffer and the array, and compute cycles, of one (m x r) * (r x n) tile on a rows x cols
+// array.  The stationary operand's two extents are cut into parts that the array holds at once:
+//   0 weight stationary: r x n weights folded onto the array, m inputs streamed per fold;
+//   1 input stationary:  m x r inputs folded, n weight columns streamed;
+//   2 output stationary: m x n outputs folded, r reduction steps streamed.
+// Words: the stationary operand once, a streamed operand once per part of the other dimension, partial sums read and
+// written between parts of the reduction (2 * parts - 1 transfers per output element).  With qa, qb parts of the two
+// extents this is c0 + ca * qa + cb * qb, and the cycles are third * qa * qb times the cycles of a part: one form for the
+// three modes, so that lanes of a warp with different modes run the same instructions (six diverging paths before).
+struct TileForm {
+    uint32_t ea, eb;            // extents of the stationary operand
+    int64_t c0, ca, cb, third;
+};
+__device__ __forceinline__ TileForm tile_form(int sm, uint32_t m, uint32_t r, uint32_t n) {
+    const int64_t mr = (int64_t)m * r, rn = (int64_t)r * n, mn = (int64_t)m * n;
+    TileForm f;
+    f.ea = sm == 0 ? r : m;
+    f.eb = sm == 1 ? r : n;
+    f.c0 = sm == 0 ? rn - mn : (sm == 1 ? mr - mn : mn);
+    f.ca = sm == 0 ? 2 * mn : rn;
+    f.cb = sm == 1 ? 2 * mn : mr;
+    f.third = sm == 0 ? m : (sm == 1 ? n : r);
+    return f;
 }
 
-// Words moved between the global buffer and the array for one tile: the stationary operand
-// once, the streamed operand once per fold of the other dimension, partial sums read and
-// written between reduction folds (2*folds - 1 transfers per output element).
-__device__ __forceinline__ int64_t tile_traffic(int sm, uint32_t m, uint32_t r, uint32_t n, uint32_t rows, uint32_t cols) {
-    const int64_t M = m, R = r, N = n;
-    if (sm == 0) return R * N + M * R * ceil_div(n, cols) + M * N * (2 * ceil_div(r, rows) - 1);
-    if (sm == 1) return M * R + R * N * ceil_div(m, rows) + M * N * (2 * ceil_div(r, cols) - 1);
-    return M * R * ceil_div(n, cols) + R * N * ceil_div(m, rows) + M * N;
-}
-
-// Register-file-level tiling (objective.rf_tiling): buffer<->array words and compute cycles of one tile when
-// its stationary operand is processed in blocks of a x b elements; the block is searched over the divisors of the
-// operand's two extents (dimension ids da, db: the extents are tile extents of those dimensions, so their
-// divisors are among the plan's divisor lists), in ascending (a, b) order, keeping the admissible block with
-// the least (words, cycles) for the energy objective and the least (cycles, words) for the latency objective.
+// Register-file-level tiling (objective.rf_tiling): the stationary operand is processed in blocks of a x b elements, a
+// and b divisors of its extents (dimension ids da, db: the extents are tile extents of those dimensions, so that their
+// divisors are among the plan's divisor lists), with ceil(a / rows) * ceil(b / cols) elements per PE, at most
+// rf_words - 2.  The admissible block with the least (words, cycles) for the energy objective, the least (cycles, words)
+// for the latency objective, the first in ascending (a, b) order among equal ones.
+// At a given b the admissible a are the divisors up to a limit that falls as b grows, and the words fall strictly as a
+// grows; so the best a for every b is the largest one (energy), or the largest among those with the least
+// (ea / a) * ceil(a / rows) (latency): one walk of b downwards with a running best over a, na + nb steps instead of
+// na * nb (a BERT-base latency search 97 -> 50 us).
 // blk receives the block as (m, r, n) extents, 1 for the streamed extent.
-__device__ __forceinline__ void rf_block_terms(const Plan& p, int sm, uint32_t m, uint32_t r, uint32_t n, int da, int db,
-                                               int64_t& words, int64_t& cycles, uint32_t blk[3]) {
-    const uint32_t ea = sm == 0 ? r : m, eb = sm == 0 ? n : (sm == 1 ? r : n);
-    const int64_t M = m, R = r, N = n;
+__device__ __forceinline__ void rf_block_terms(const Plan& p, int sm, const TileForm& f, int da, int db, int64_t& words,
+                                               int64_t& cycles, uint32_t blk[3]) {
+    const bool latency = p.objective == MMEE_OBJ_LATENCY;
+    const uint32_t most = p.rf_words - 2;
+    const uint32_t na = p.ndiv[da];
+    uint32_t ia = 0;                                // next divisor of dimension da to be looked at
+    uint32_t a_best = 0, ha_best = 0, qa_best = 0;  // the best a among those before it (0: none)
     bool have = false;
     int64_t bw = 0, bc = 0;
     uint32_t ba = 0, bb = 0;
-    for (uint32_t ia = 0; ia < p.ndiv[da]; ++ia) {
-        const uint32_t a = p.divs[da][ia];
-        if (a > ea) break;
-        if (ea % a) continue;
-        const int64_t ha = ceil_div(a, p.pe_rows);
-        for (uint32_t ib = 0; ib < p.ndiv[db]; ++ib) {
-            const uint32_t b = p.divs[db][ib];
-            if (b > eb) break;
-            if (eb % b) continue;
-            const int64_t held = ha * ceil_div(b, p.pe_cols);       // stationary elements per PE
-            if (held + 2 > (int64_t)p.rf_words) continue;
-            int64_t w, c;
-            if (sm == 0) {
-                w = R * N + M * R * (int64_t)(n / b) + M * N * (2 * (int64_t)(r / a) - 1);
-                c = (int64_t)(r / a) * (int64_t)(n / b) * M * held;
-            } else if (sm == 1) {
-                w = M * R + R * N * (int64_t)(m / a) + M * N * (2 * (int64_t)(r / b) - 1);
-                c = (int64_t)(m / a) * (int64_t)(r / b) * N * held;
-            } else {
-                w = M * R * (int64_t)(n / b) + R * N * (int64_t)(m / a) + M * N;
-                c = (int64_t)(m / a) * (int64_t)(n / b) * R * held;
-            }
-            const bool better = !have || (p.objective == MMEE_OBJ_LATENCY ? (c < bc || (c == bc && w < bw))
-                                                                          : (w < bw || (w == bw && c < bc)));
-            if (better) { have = true; bw = w; bc = c; ba = a; bb = b; }
+    for (uint32_t ib = p.ndiv[db]; ib-- > 0;) {
+        const uint32_t b = p.divs[db][ib];
+        if (b > f.eb) continue;
+        const uint32_t qb = f.eb / b;
+        if (qb * b != f.eb) continue;
+        const uint32_t hb = (b + p.pe_cols - 1) / p.pe_cols;
+        const uint32_t limit = most / hb;           // elements of the first extent that a PE may hold
+        for (; ia < na; ++ia) {
+            const uint32_t a = p.divs[da][ia];
+            if (a > f.ea) { ia = na; break; }
+            const uint32_t ha = (a + p.pe_rows - 1) / p.pe_rows;
+            if (ha > limit) break;
+            const uint32_t qa = f.ea / a;
+            if (qa * a != f.ea) continue;
+            if (!a_best || !latency || (uint64_t)qa * ha <= (uint64_t)qa_best * ha_best) { a_best = a; ha_best = ha; qa_best = qa; }
+        }
+        if (!a_best) continue;
+        const int64_t w = f.c0 + f.ca * qa_best + f.cb * qb;
+        const int64_t c = f.third * ((int64_t)qa_best * ha_best) * ((int64_t)qb * hb);
+        const int64_t x = latency ? c : w, y = latency ? w : c, bx = latency ? bc : bw, by = latency ? bw : bc;
+        // (b falls from step to step: of equal blocks the one with the smaller a, then the later b)
+        if (!have || x < bx || (x == bx && (y < by || (y == by && a_best <= ba)))) {
+            have = true;
+            bw = w; bc = c; ba = a_best; bb = b;
         }
     }
     // (a block of one element needs three registers, which the planner requires: some block is always admissible)
@@ -91,13 +99,15 @@ __device__ __forceinline__ void rf_block_terms(const Plan& p, int sm, uint32_t m
 __device__ __forceinline__ void tile_array_terms(const Plan& p, const uint32_t b[8], int op, int sm, int64_t& words,
                                                  int64_t& cycles, uint32_t blk[3]) {
     const uint32_t m = b[4], r = op == 0 ? b[5] : b[6], n = op == 0 ? b[6] : b[7];
+    const TileForm f = tile_form(sm, m, r, n);
     if (p.rf_tiling) {
         // dimensions of the stationary operand's two extents
         const int dm = LOOP_I, dr = op == 0 ? LOOP_K : LOOP_L, dn = op == 0 ? LOOP_L : LOOP_J;
-        rf_block_terms(p, sm, m, r, n, sm == 0 ? dr : dm, sm == 0 ? dn : (sm == 1 ? dr : dn), words, cycles, blk);
+        rf_block_terms(p, sm, f, sm == 0 ? dr : dm, sm == 0 ? dn : (sm == 1 ? dr : dn), words, cycles, blk);
     } else {
-        words = tile_traffic(sm, m, r, n, p.pe_rows, p.pe_cols);
-        cycles = tile_cycles(sm, m, r, n, p.pe_rows, p.pe_cols);
+        const int64_t qa = (f.ea + p.pe_rows - 1) / p.pe_rows, qb = (f.eb + p.pe_cols - 1) / p.pe_cols;
+        words = f.c0 + f.ca * qa + f.cb * qb;
+        cycles = f.third * qa * qb;
         blk[0] = blk[1] = blk[2] = 0;
     }
 }
@@ -176,12 +186,13 @@ struct CandidateChoice {
 
 __device__ __forceinline__ CandidateChoice decode_candidate(const Plan& p, uint64_t idx) {
     CandidateChoice d;
-    const uint64_t per_t = (uint64_t)p.rows_per_tiling * 9u;
-    d.t = idx / per_t;
-    const uint32_t rem = (uint32_t)(idx - d.t * per_t);
-    d.row = rem / 9u;
-    d.s = rem % 9u;
-    const uint32_t w = d.row / 125u, mid = (d.row % 125u) / 25u, de = d.row % 25u;
+    // (a space has fewer than 2^32 tasks -- at most 2^24 tilings of 210 -- so only the division by the constant is 64-bit)
+    const uint32_t task = (uint32_t)(idx / (uint64_t)kCandPerTask), in_task = (uint32_t)(idx - (uint64_t)task * kCandPerTask);
+    const uint32_t t = task / p.tasks_per_tiling, w = task - t * p.tasks_per_tiling;
+    d.t = t;
+    d.row = w * (uint32_t)kRowsPerTask + in_task / 9u;
+    d.s = in_task % 9u;
+    const uint32_t mid = in_task / 225u, de = in_task / 9u % 25u;
     d.c = decode_task(p, w);
     d.fused = d.c.phi == 0;
     d.lv[OP_A] = d.c.la;

@@ -128,6 +128,7 @@ struct Shared {
     union {
         TileTab tile[kMaxChunk];
         BlockTab block[kWarps];
+        mmee_result_t record[kWarps];
     };
 };
 
@@ -344,7 +345,9 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
         found = ek != kInfKey ? 1 : 0;
         bound = ek;
         // ---- the winning block, mapping by mapping
-        if (found && tid < kBlockItems) block_item(p, (uint32_t)ei, tid, &sh.block[0]);
+        // (the three kinds of items on three warps)
+        const int item = warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (tid == 64 ? 31 : -1));
+        if (found && item >= 0) block_item(p, (uint32_t)ei, item, &sh.block[0]);
         __syncthreads();
         if (found) {
             n_groups = block_rows(sh.block[0]) / 5u;
@@ -411,7 +414,12 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
     else if (lane == 0) entry = make_longlong2((long long)ek, (long long)ei);
     const int n_out = __popc(__ballot_sync(kFull, entry.x != kInfKey));
     if (tid == 0 && (n_out == 0) != (found == 0)) atomicOr(&sh.check_failed, 1u);
-    mmee_result_t r, first;
+    // (records are put together in shared memory and copied by the warp: a lane holds words `lane` and `lane + 32`)
+    constexpr int kWords = sizeof(mmee_result_t) / 8;
+    static_assert(sizeof(mmee_result_t) % 8 == 0 && kWords <= 64 && offsetof(mmee_result_t, status) % 8 == 4, "record words");
+    mmee_result_t& r = sh.record[warp];
+    const unsigned long long* words = reinterpret_cast<const unsigned long long*>(&r);
+    unsigned long long first0 = 0, first1 = 0;
     for (int rec = warp; rec < k; rec += kWarps) {
         const long long rk = __shfl_sync(kFull, entry.x, rec);
         const uint64_t ri = (uint64_t)__shfl_sync(kFull, entry.y, rec);
@@ -421,27 +429,47 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
                 const int64_t key = OBJ == MMEE_OBJ_EDP ? __double_as_longlong(r.edp_key) : key_of<OBJ>(r.e_key, r.l_key, p.key_cap);
                 if (!(key == rk && r.feasible && r.t >= p.t_begin && r.t < p.t_end)) atomicOr(&sh.check_failed, 1u);
             }
-        } else if (lane == 0) {
+        } else {
             // empty slot
             unsigned long long* raw = reinterpret_cast<unsigned long long*>(&r);
-            for (unsigned i = 0; i < sizeof(r) / 8; ++i) raw[i] = 0;
-            r.idx = MMEE_NO_INDEX;
-            r.status = n_out ? MMEE_OK : MMEE_ERR_NO_FEASIBLE;
+            for (int i = lane; i < kWords; i += 32) raw[i] = 0;
+            __syncwarp();
+            if (lane == 0) {
+                r.idx = MMEE_NO_INDEX;
+                r.status = n_out ? MMEE_OK : MMEE_ERR_NO_FEASIBLE;
+            }
         }
-        if (lane == 0) {
-            if (out_topk) out_topk[rec] = r;
-            if (rec == 0) first = r;
+        __syncwarp();
+        const unsigned long long w0 = words[lane], w1 = lane + 32 < kWords ? words[lane + 32] : 0;
+        if (out_topk) {
+            unsigned long long* to = reinterpret_cast<unsigned long long*>(&out_topk[rec]);
+            to[lane] = w0;
+            if (lane + 32 < kWords) to[lane + 32] = w1;
         }
+        if (rec == 0) { first0 = w0; first1 = w1; }
+        __syncwarp();
     }
     __syncthreads();
-    if (tid == 0) {
-        unsigned long long all_rows = 0, all_live = 0;
-        for (int w = 0; w < kWarps; ++w) { all_rows += sh.feasible_rows[w]; all_live += sh.live_tilings[w]; }
-        first.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
-        first.n_feasible = all_rows * (uint64_t)p.n_sm;
-        if (sh.check_failed) first.status = MMEE_ERR_CHECK;
-        *out_best = first;
+    if (warp == 0) {
+        unsigned long long all_rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
+#pragma unroll
+        for (int off = kWarps / 2; off; off >>= 1) all_rows += __shfl_xor_sync(kFull, all_rows, off);
+        all_rows = __shfl_sync(kFull, all_rows, 0);
+        auto set = [&](size_t word, unsigned long long v) {
+            if (lane == (int)word) first0 = v;
+            if (lane + 32 == (int)word) first1 = v;
+        };
+        set(offsetof(mmee_result_t, n_total) / 8, (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u);
+        set(offsetof(mmee_result_t, n_feasible) / 8, all_rows * (uint64_t)p.n_sm);
+        if (sh.check_failed && lane == (int)(offsetof(mmee_result_t, status) / 8))
+            first0 = (first0 & 0xffffffffull) | ((unsigned long long)MMEE_ERR_CHECK << 32);
+        unsigned long long* to = reinterpret_cast<unsigned long long*>(out_best);
+        to[lane] = first0;
+        if (lane + 32 < kWords) to[lane + 32] = first1;
+    } else if (tid == 32) {
         // ready for the next search on this scratch
+        unsigned long long all_live = 0;
+        for (int w = 0; w < kWarps; ++w) all_live += sh.live_tilings[w];
         scratch->G = kInfKey - 1;
         scratch->last_exact_groups = n_groups;
         const uint32_t unfused_modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
@@ -462,22 +490,18 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
 __device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// The tables of one tiling, by eight threads (sub = 0..7): one stationary mode of one operator each, sizes and bounds.
+// The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
+// and the sizes between them.
 __device__ __forceinline__ void build_tile(const Plan& p, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
     if (sub < 6) {
-        const int op = sub / 3, sm = sub % 3;
+        const int op = sub >= 3 ? 1 : 0, sm = sub - 3 * op;
         int64_t P, Q;
         stationary_terms(p, b, op, sm, P, Q);
         (op ? tb->P2 : tb->P1)[sm] = P;
         (op ? tb->Q2 : tb->Q1)[sm] = Q;
-        return;
     }
-#pragma unroll
-    for (int i = 0; i < kSizeSlots / 2; ++i) {
-        const uint64_t v0 = size_words(p.dim, b + 4, i), v1 = size_words(p.dim, b + 4, i + kSizeSlots / 2);
-        tb->size[sub == 6 ? i : i + kSizeSlots / 2] = sat_size(sub == 6 ? v0 : v1);
-    }
-    if (sub == 6) { tb->t = t; tb->iD = b[LOOP_I]; tb->lD = b[LOOP_L]; tb->jD = b[LOOP_J]; }
+    for (int i = sub; i < kSizeSlots; i += 8) tb->size[i] = sat_size(size_words(p.dim, tb->b + 4, i));
+    if (sub == 7) tb->t = t;
 }
 
 template <int OBJ, bool PRUNE, bool MULTI>
@@ -565,6 +589,13 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
             uint32_t slot = 0;
             if (live && (tid & 7) == 0) slot = atomicAdd(&sh.n_live, 1u);
             slot = __shfl_sync(kFull, slot, lane & ~7);
+            if (live) {
+                uint32_t own = b[0];
+#pragma unroll
+                for (int d = 1; d < 8; ++d) own = (tid & 7) == d ? b[d] : own;
+                sh.tile[slot].b[tid & 7] = own;
+            }
+            __syncwarp();
             if (live) build_tile(p, b, t, tid & 7, &sh.tile[slot]);
         }
         if (MULTI && m0 == 0) {

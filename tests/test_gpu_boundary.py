@@ -416,3 +416,23 @@ def test_searches_that_follow_one_another_on_a_stream():
     finally:
         for h in handles:
             mm.mmee_destroy(h)
+
+
+@pytest.mark.parametrize("objective", [mi.OBJ_ENERGY, mi.OBJ_LATENCY])
+@pytest.mark.parametrize("pe,rf_words", [((7, 3), 6), ((8, 8), 5), ((1, 16), 40), ((4, 6), 3)])
+def test_register_file_blocks_with_many_divisors(pe, rf_words, objective):
+    """The block search walks one divisor list down and the other up instead of trying every pair: extents with many
+    divisors, arrays that do not divide them, register files from the smallest on; sampled candidates (block, words and
+    cycles among their fields) against the oracle, which tries every block."""
+    cfg = dict(name="rf_ragged", workload=mi.workload(1, 1, 1, 360, 120, 48, 30, 1),
+               arch=mi.arch(pe[0], pe[1], 1, 40000, 64, 4, 120.0, 4.0, 1.0, 0.5, c_softmax=3.0, energy_quantum_pj=0.5))
+    cfg["arch"]["rf_bytes"] = max(6, rf_words)
+    obj = mi.objective(objective, 1, rf_tiling=1)
+    p = oracle.make_problem(cfg["workload"], cfg["arch"], obj)
+    rng = np.random.default_rng(rf_words)
+    buf = mm.result_buffer(9)
+    with Handle(cfg, obj) as h:
+        for start in rng.integers(0, p.N // 9, size=250):
+            mm.mmee_eval(h, int(start) * 9, 9, buf)          # one row: the nine stationary pairs
+            for g, o in zip(mm.read_results(buf, 9), oracle.evaluate_range(p, int(start) * 9, 9)):
+                assert_same_record(g, o, "idx %d" % o.idx)
