@@ -21,10 +21,11 @@ struct BlockTab {
 constexpr int kBlockItems = 32;
 
 // Stationary-mode terms of one operator of one tiling: its energy and compute words at rho = 1 (see TileTab).
-__device__ __forceinline__ void stationary_terms(const Plan& p, const uint32_t b[8], int op, int sm, int64_t& P, int64_t& Q) {
+template <class Divisors>
+__device__ __forceinline__ void stationary_terms(const Plan& p, const Divisors& dv, const uint32_t b[8], int op, int sm, int64_t& P, int64_t& Q) {
     int64_t w, cy;
     uint32_t blk[3];
-    tile_array_terms(p, b, op, sm, w, cy, blk);
+    tile_array_terms(p, dv, b, op, sm, w, cy, blk);
     // tile invocations; partial sums carried between the steps of the reduction; MACs (see tiling_counts)
     const int64_t il = (int64_t)b[LOOP_I] * b[LOOP_L];
     const int64_t outer = op == 0 ? il : (int64_t)b[LOOP_I] * b[LOOP_J];
@@ -36,7 +37,8 @@ __device__ __forceinline__ void stationary_terms(const Plan& p, const uint32_t b
 }
 
 // Item `item` (0 .. kBlockItems - 1) of the tables of block `id` = tiling * n_blocks + block.
-__device__ __forceinline__ void block_item(const Plan& p, uint32_t id, int item, BlockTab* bt) {
+template <class Divisors>
+__device__ __forceinline__ void block_item(const Plan& p, const Divisors& dv, uint32_t id, int item, BlockTab* bt) {
     const uint32_t t = id / p.n_blocks, block = id - t * p.n_blocks;
     const uint32_t phi = p.block_phi[block], slot = p.block_order_slot[block], order = p.order_id[slot];
     uint32_t b[8];
@@ -52,7 +54,7 @@ __device__ __forceinline__ void block_item(const Plan& p, uint32_t id, int item,
     } else if (item < 31) {
         const int op = (item - 25) / 3, sm = (item - 25) % 3;
         int64_t P, Q;
-        stationary_terms(p, b, op, sm, P, Q);
+        stationary_terms(p, dv, b, op, sm, P, Q);
         (op ? bt->P2 : bt->P1)[sm] = P;
         (op ? bt->Q2 : bt->Q1)[sm] = Q;
     } else {

@@ -40,6 +40,15 @@ __device__ __forceinline__ TileForm tile_form(int sm, uint32_t m, uint32_t r, ui
     return f;
 }
 
+// Divisors of dimension d in ascending order, and how often one has to be folded onto the array's rows / columns: read from
+// the plan (here) or from a CTA's shared copy.
+struct PlanDivisors {
+    const Plan& p;
+    __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return p.divs[d][i]; }
+    __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_rows - 1) / p.pe_rows; }
+    __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_cols - 1) / p.pe_cols; }
+};
+
 // Register-file-level tiling (objective.rf_tiling): the stationary operand is processed in blocks of a x b elements, a
 // and b divisors of its extents (dimension ids da, db: the extents are tile extents of those dimensions, so that their
 // divisors are among the plan's divisor lists), with ceil(a / rows) * ceil(b / cols) elements per PE, at most
@@ -50,8 +59,9 @@ __device__ __forceinline__ TileForm tile_form(int sm, uint32_t m, uint32_t r, ui
 // (ea / a) * ceil(a / rows) (latency): one walk of b downwards with a running best over a, na + nb steps instead of
 // na * nb (a BERT-base latency search 97 -> 50 us).
 // blk receives the block as (m, r, n) extents, 1 for the streamed extent.
-__device__ __forceinline__ void rf_block_terms(const Plan& p, int sm, const TileForm& f, int da, int db, int64_t& words,
-                                               int64_t& cycles, uint32_t blk[3]) {
+template <class Divisors>
+__device__ __forceinline__ void rf_block_terms(const Plan& p, const Divisors& dv, int sm, const TileForm& f, int da, int db,
+                                               int64_t& words, int64_t& cycles, uint32_t blk[3]) {
     const bool latency = p.objective == MMEE_OBJ_LATENCY;
     const uint32_t most = p.rf_words - 2;
     const uint32_t na = p.ndiv[da];
@@ -61,24 +71,23 @@ __device__ __forceinline__ void rf_block_terms(const Plan& p, int sm, const Tile
     int64_t bw = 0, bc = 0;
     uint32_t ba = 0, bb = 0;
     for (uint32_t ib = p.ndiv[db]; ib-- > 0;) {
-        const uint32_t b = p.divs[db][ib];
+        const uint32_t b = dv.div(db, ib);
         if (b > f.eb) continue;
         const uint32_t qb = f.eb / b;
         if (qb * b != f.eb) continue;
-        const uint32_t hb = (b + p.pe_cols - 1) / p.pe_cols;
-        const uint32_t limit = most / hb;           // elements of the first extent that a PE may hold
+        const uint64_t hb = dv.col_folds(db, ib);
         for (; ia < na; ++ia) {
-            const uint32_t a = p.divs[da][ia];
+            const uint32_t a = dv.div(da, ia);
             if (a > f.ea) { ia = na; break; }
-            const uint32_t ha = (a + p.pe_rows - 1) / p.pe_rows;
-            if (ha > limit) break;
+            const uint32_t ha = dv.row_folds(da, ia);
+            if (ha * hb > most) break;
             const uint32_t qa = f.ea / a;
             if (qa * a != f.ea) continue;
             if (!a_best || !latency || (uint64_t)qa * ha <= (uint64_t)qa_best * ha_best) { a_best = a; ha_best = ha; qa_best = qa; }
         }
         if (!a_best) continue;
         const int64_t w = f.c0 + f.ca * qa_best + f.cb * qb;
-        const int64_t c = f.third * ((int64_t)qa_best * ha_best) * ((int64_t)qb * hb);
+        const int64_t c = f.third * ((int64_t)qa_best * ha_best) * (int64_t)(qb * hb);
         const int64_t x = latency ? c : w, y = latency ? w : c, bx = latency ? bc : bw, by = latency ? bw : bc;
         // (b falls from step to step: of equal blocks the one with the smaller a, then the later b)
         if (!have || x < bx || (x == bx && (y < by || (y == by && a_best <= ba)))) {
@@ -96,14 +105,15 @@ __device__ __forceinline__ void rf_block_terms(const Plan& p, int sm, const Tile
 
 // Words and cycles of one tile of operator `op` (0: (i_G x k_G)(k_G x l_G), 1: (i_G x l_G)(l_G x j_G)) under
 // stationary mode sm: one array fold per pass, or the register-file block search.
-__device__ __forceinline__ void tile_array_terms(const Plan& p, const uint32_t b[8], int op, int sm, int64_t& words,
+template <class Divisors>
+__device__ __forceinline__ void tile_array_terms(const Plan& p, const Divisors& dv, const uint32_t b[8], int op, int sm, int64_t& words,
                                                  int64_t& cycles, uint32_t blk[3]) {
     const uint32_t m = b[4], r = op == 0 ? b[5] : b[6], n = op == 0 ? b[6] : b[7];
     const TileForm f = tile_form(sm, m, r, n);
     if (p.rf_tiling) {
         // dimensions of the stationary operand's two extents
         const int dm = LOOP_I, dr = op == 0 ? LOOP_K : LOOP_L, dn = op == 0 ? LOOP_L : LOOP_J;
-        rf_block_terms(p, sm, f, sm == 0 ? dr : dm, sm == 0 ? dn : (sm == 1 ? dr : dn), words, cycles, blk);
+        rf_block_terms(p, dv, sm, f, sm == 0 ? dr : dm, sm == 0 ? dn : (sm == 1 ? dr : dn), words, cycles, blk);
     } else {
         const int64_t qa = (f.ea + p.pe_rows - 1) / p.pe_rows, qb = (f.eb + p.pe_cols - 1) / p.pe_cols;
         words = f.c0 + f.ca * qa + f.cb * qb;
@@ -218,11 +228,12 @@ __device__ __forceinline__ void operand_terms(const Plan& p, const CandidateChoi
 
 // Array-level terms of one operator (0: C = A*B, 1: E = C*D) under one stationary mode: buffer<->PE words
 // including the carried partial sums, and compute cycles.
-__device__ __forceinline__ void operator_array_terms(const Plan& p, const uint32_t b[8], const TilingCounts& c, int op,
+template <class Divisors>
+__device__ __forceinline__ void operator_array_terms(const Plan& p, const Divisors& dv, const uint32_t b[8], const TilingCounts& c, int op,
                                                      int sm, bool recompute, int64_t& words, int64_t& cycles,
                                                      uint32_t blk[3]) {
     int64_t w, cy;
-    tile_array_terms(p, b, op, sm, w, cy, blk);
+    tile_array_terms(p, dv, b, op, sm, w, cy, blk);
     if (op == 0) {
         const int64_t rho = recompute ? (int64_t)b[3] : 1;
         const int64_t t1 = rho * c.t1;
@@ -309,14 +320,15 @@ __device__ inline void evaluate_candidate(const Plan& p, uint64_t idx, mmee_resu
     for (int x = 0; x < 5; ++x) operand_terms(p, d, b, x, bs[x], da[x]);
     int64_t w1, c1, w2, c2;
     uint32_t blk1[3], blk2[3];
-    operator_array_terms(p, b, tt, 0, d.sm1, d.rc != 0, w1, c1, blk1);
-    operator_array_terms(p, b, tt, 1, d.sm2, d.rc != 0, w2, c2, blk2);
+    operator_array_terms(p, PlanDivisors{p}, b, tt, 0, d.sm1, d.rc != 0, w1, c1, blk1);
+    operator_array_terms(p, PlanDivisors{p}, b, tt, 1, d.sm2, d.rc != 0, w2, c2, blk2);
     assemble_record(p, idx, d, b, tt, bs, da, w1, c1, w2, c2, blk1, blk2, o);
 }
 
 // The same by one warp (all 32 lanes call it converged): lanes 0..4 take one operand each, lanes 5 and 6 one
 // operator's array-level terms each; lane 0 gathers the parts and holds the record on return.
-__device__ inline void evaluate_candidate_warp(const Plan& p, uint64_t idx, int lane, mmee_result_t& o) {
+template <class Divisors>
+__device__ inline void evaluate_candidate_warp(const Plan& p, const Divisors& dv, uint64_t idx, int lane, mmee_result_t& o) {
     const CandidateChoice d = decode_candidate(p, idx);
     uint32_t b[8];
     tiling_bounds(p, d.t, b);
@@ -324,7 +336,7 @@ __device__ inline void evaluate_candidate_warp(const Plan& p, uint64_t idx, int 
     int64_t v0 = 0, v1 = 0;
     uint32_t blk[3] = {0, 0, 0};
     if (lane < 5) operand_terms(p, d, b, lane, v0, v1);
-    else if (lane < 7) operator_array_terms(p, b, tt, lane - 5, lane == 5 ? d.sm1 : d.sm2, d.rc != 0, v0, v1, blk);
+    else if (lane < 7) operator_array_terms(p, dv, b, tt, lane - 5, lane == 5 ? d.sm1 : d.sm2, d.rc != 0, v0, v1, blk);
     int64_t part0[7], part1[7];
 #pragma unroll
     for (int i = 0; i < 7; ++i) {

@@ -118,6 +118,7 @@ struct Shared {
     OrderInfo order[kMaxOrders];
     KeptMasks kept;
     uint32_t divs[4][MMEE_MAX_DIVISORS];
+    uint32_t row_folds[4][MMEE_MAX_DIVISORS], col_folds[4][MMEE_MAX_DIVISORS];      // register-file tiling only
     alignas(16) longlong2 tops[kWarps][MMEE_MAX_TOPK];
     long long G;                    // k > 1: upper bound on the k-th smallest key
     unsigned long long feasible_rows[kWarps];
@@ -130,6 +131,13 @@ struct Shared {
         BlockTab block[kWarps];
         mmee_result_t record[kWarps];
     };
+};
+
+struct SharedDivisors {       // see PlanDivisors
+    const Shared& sh;
+    __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
+    __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return sh.row_folds[d][i]; }
+    __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return sh.col_folds[d][i]; }
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -347,7 +355,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
         // ---- the winning block, mapping by mapping
         // (the three kinds of items on three warps)
         const int item = warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (tid == 64 ? 31 : -1));
-        if (found && item >= 0) block_item(p, (uint32_t)ei, item, &sh.block[0]);
+        if (found && item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)ei, item, &sh.block[0]);
         __syncthreads();
         if (found) {
             n_groups = block_rows(sh.block[0]) / 5u;
@@ -380,7 +388,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
                 const int src = m ? __ffs(m) - 1 : 0;
                 bk[j] = m ? (int64_t)__shfl_sync(kFull, e.x, src) : kInfKey;
                 const uint32_t id = (uint32_t)__shfl_sync(kFull, e.y, src);
-                if (m && j == warp) block_item(p, id, lane, &sh.block[j]);
+                if (m && j == warp) block_item(p, SharedDivisors{sh}, id, lane, &sh.block[j]);
                 m &= m - 1;
             }
             __syncthreads();
@@ -424,7 +432,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
         const long long rk = __shfl_sync(kFull, entry.x, rec);
         const uint64_t ri = (uint64_t)__shfl_sync(kFull, entry.y, rec);
         if (rec < n_out) {
-            evaluate_candidate_warp(p, ri, lane, r);
+            evaluate_candidate_warp(p, SharedDivisors{sh}, ri, lane, r);
             if (lane == 0) {
                 const int64_t key = OBJ == MMEE_OBJ_EDP ? __double_as_longlong(r.edp_key) : key_of<OBJ>(r.e_key, r.l_key, p.key_cap);
                 if (!(key == rk && r.feasible && r.t >= p.t_begin && r.t < p.t_end)) atomicOr(&sh.check_failed, 1u);
@@ -492,11 +500,11 @@ __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepco
 
 // The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
 // and the sizes between them.
-__device__ __forceinline__ void build_tile(const Plan& p, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
+__device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
     if (sub < 6) {
         const int op = sub >= 3 ? 1 : 0, sm = sub - 3 * op;
         int64_t P, Q;
-        stationary_terms(p, b, op, sm, P, Q);
+        stationary_terms(p, SharedDivisors{sh}, b, op, sm, P, Q);
         (op ? tb->P2 : tb->P1)[sm] = P;
         (op ? tb->Q2 : tb->Q1)[sm] = Q;
     }
@@ -516,7 +524,15 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
     if (PRUNE)
         for (int i = tid; i < (int)(sizeof(KeptMasks) / 4); i += kSearchThreads)
             reinterpret_cast<uint32_t*>(&sh.kept)[i] = reinterpret_cast<const uint32_t*>(&p.kept)[i];
-    if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) sh.divs[tid >> 6][tid & 63] = p.divs[tid >> 6][tid & 63];
+    static_assert(kSearchThreads == 4 * MMEE_MAX_DIVISORS, "one thread per divisor");
+    if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) {
+        const int d = tid >> 6, i = tid & 63;
+        sh.divs[d][i] = p.divs[d][i];
+        if (p.rf_tiling) {
+            sh.row_folds[d][i] = PlanDivisors{p}.row_folds(d, i);
+            sh.col_folds[d][i] = PlanDivisors{p}.col_folds(d, i);
+        }
+    }
     if (tid == 0) {
         sh.n_live = 0;
         sh.cursor = 0;
@@ -596,7 +612,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
                 sh.tile[slot].b[tid & 7] = own;
             }
             __syncwarp();
-            if (live) build_tile(p, b, t, tid & 7, &sh.tile[slot]);
+            if (live) build_tile(p, sh, b, t, tid & 7, &sh.tile[slot]);
         }
         if (MULTI && m0 == 0) {
             // (k > 1 shares a bound through the scratch while it works on the items)

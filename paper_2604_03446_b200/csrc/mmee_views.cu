@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(kViewThreads) dump_kernel(const __grid_constan
     const uint32_t first = (uint32_t)p.t_begin * p.n_blocks, last = (uint32_t)p.t_end * p.n_blocks;
     const uint64_t origin = p.t_begin * p.rows_per_tiling * 9u;
     for (uint32_t id = first + blockIdx.x; id < last; id += gridDim.x) {
-        if (threadIdx.x < kBlockItems) block_item(p, id, (int)threadIdx.x, &bt);
+        if (threadIdx.x < kBlockItems) block_item(p, PlanDivisors{p}, id, (int)threadIdx.x, &bt);
         __syncthreads();
         const uint32_t n = block_rows(bt) * 9u;
         int64_t* o = out + (bt.first_idx - origin);
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(kViewThreads) flags_kernel(const __grid_consta
     const uint32_t first = (uint32_t)p.t_begin * p.n_blocks, last = (uint32_t)p.t_end * p.n_blocks;
     const uint64_t origin = p.t_begin * p.rows_per_tiling * 9u;
     for (uint32_t id = first + blockIdx.x; id < last; id += gridDim.x) {
-        if (threadIdx.x < kBlockItems) block_item(p, id, (int)threadIdx.x, &bt);
+        if (threadIdx.x < kBlockItems) block_item(p, PlanDivisors{p}, id, (int)threadIdx.x, &bt);
         __syncthreads();
         unsigned char* o = flags + (bt.first_idx - origin) / 45u;
         for (uint32_t i = threadIdx.x; i < block_rows(bt) / 5u; i += kViewThreads) {
