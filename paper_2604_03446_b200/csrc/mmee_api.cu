@@ -68,11 +68,54 @@ int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShap
     const uint64_t per_cta = (tilings + grid - 1) / grid;
     const uint64_t passes = (per_cta + kMaxChunk - 1) / kMaxChunk;
     shape->grid = (uint32_t)grid;
+    shape->chain = shape->chain_read = false;
     shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
     return MMEE_OK;
 }
 
 }  // namespace mmee
+
+namespace {
+
+// Searches chained on the device (see LaunchShape::chain), step i with plans[i % n_plans], until one finds nothing: their
+// records in order, through `take` (which returns false to stop), and their number.  The host waits for a batch of them at a time, first
+// `first_batch`, then twice as many as before; what is launched beyond the last one ends at once.
+template <class Take>
+int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found, Take take) {
+    int device = 0;
+    int rc = cuda_status(cudaGetDevice(&device));
+    if (rc) return rc;
+    LaunchShape shape;
+    if ((rc = choose_launch_shape(plans[0], device, 0, &shape))) return rc;
+    Workspace* ws = nullptr;
+    if ((rc = workspace_acquire(device, &ws))) return rc;
+    bool clean = true, more = true;
+    *n_found = 0;
+    uint32_t step = 0;
+    for (uint32_t batch = first_batch; more && rc == MMEE_OK; batch = 2 * batch < kHostRecords ? 2 * batch : kHostRecords) {
+        uint32_t n = 0;
+        for (; n < batch && rc == MMEE_OK; ++n) {
+            shape.chain = true;
+            shape.chain_read = step + n > 0;
+            rc = cuda_status(launch_search(plans[(step + n) % (uint32_t)n_plans], shape, ws->scratch, ws->host_dev + n, nullptr, nullptr));
+            if (rc) clean = false;
+        }
+        const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
+        if (rc2) clean = false;
+        if (rc == MMEE_OK) rc = rc2;
+        for (uint32_t i = 0; i < n && more && rc == MMEE_OK; ++i) {
+            const mmee_result_t& r = ws->host[i];
+            if (r.status == MMEE_ERR_CHECK) { rc = MMEE_ERR_CHECK; break; }
+            more = r.idx != MMEE_NO_INDEX;
+            if (more) { ++*n_found; more = take(r, step + i); }
+        }
+        step += n;
+    }
+    const int rc2 = workspace_release(ws, clean);
+    return rc ? rc : rc2;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -241,33 +284,26 @@ int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch, 
                       mmee_result_t* out_points, uint32_t capacity, uint32_t* n_points) {
     if (!objective || !n_points || (!out_points && capacity)) return MMEE_ERR_ARG;
     *n_points = 0;
-    mmee_objective_t oe = *objective, ol = *objective;
-    oe.objective = MMEE_OBJ_ENERGY_LCAP;  oe.topk = 1; oe.row_pruning = 0; oe.key_cap = INT64_MAX - 1;
-    ol.objective = MMEE_OBJ_LATENCY_ECAP; ol.topk = 1; ol.row_pruning = 0; ol.key_cap = INT64_MAX - 1;
-    mmee_handle_t *he = nullptr, *hl = nullptr;
-    int rc = mmee_create(workload, arch, &oe, &he);
-    if (rc) return rc;
-    rc = mmee_create(workload, arch, &ol, &hl);
-    if (rc) { mmee_destroy(he); return rc; }
-    mmee_result_t r;
-    int64_t latency_cap = INT64_MAX - 1;
-    uint32_t n = 0;
-    while (rc == MMEE_OK) {
-        // least energy among the mappings that are still faster than the previous point
-        he->plan.key_cap = latency_cap;
-        if ((rc = mmee_search_host(he, &r, nullptr))) break;
-        if (r.idx == MMEE_NO_INDEX) break;                       // nothing faster is left
-        // the fastest mapping at that energy: the point of the front, with its lowest index
-        hl->plan.key_cap = r.e_key;
-        if ((rc = mmee_search_host(hl, &r, nullptr))) break;
-        if (r.idx == MMEE_NO_INDEX) { rc = MMEE_ERR_CHECK; break; }   // cannot happen: the previous optimum qualifies
-        if (n < capacity) out_points[n] = r;
-        ++n;
-        if (r.l_key == 0) break;
-        latency_cap = r.l_key - 1;
-    }
-    mmee_destroy(he);
-    mmee_destroy(hl);
+    mmee_objective_t o = *objective;
+    o.topk = 1; o.row_pruning = 0; o.key_cap = INT64_MAX - 1;
+    Plan plans[2];
+    int rc;
+    o.objective = MMEE_OBJ_ENERGY_LCAP;
+    if ((rc = build_plan(workload, arch, &o, &plans[0]))) return rc;
+    o.objective = MMEE_OBJ_LATENCY_ECAP;
+    if ((rc = build_plan(workload, arch, &o, &plans[1]))) return rc;
+    uint32_t n = 0, n_found = 0;
+    // Even steps: the least energy among the mappings that are still faster than the previous point (none: the front is
+    // complete).  Odd steps: the fastest mapping at that energy, the point of the front, with its lowest index.
+    rc = run_chain(plans, 2, 4, &n_found, [&](const mmee_result_t& r, uint32_t step) {
+        if (step % 2) {
+            if (n < capacity) out_points[n] = r;
+            ++n;
+        }
+        return true;
+    });
+    // (an even step's optimum qualifies for the odd one)
+    if (rc == MMEE_OK && n_found % 2) rc = MMEE_ERR_CHECK;
     *n_points = n;
     if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
     return rc;
@@ -282,29 +318,29 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
     a.e_dram_pj = 1.0; a.e_gb_pj = a.e_rf_pj = a.e_mac_pj = 0.0; a.c_softmax = 0.0; a.energy_quantum_pj = 1.0;
     mmee_objective_t o = *objective;
     o.objective = MMEE_OBJ_ENERGY; o.topk = 1; o.row_pruning = 0; o.key_cap = 0;
-    mmee_handle_t* h = nullptr;
-    int rc = mmee_create(workload, &a, &o, &h);
+    Plan plan;
+    int rc = build_plan(workload, &a, &o, &plan);
     if (rc) return rc;
-    mmee_result_t r, held;
+    mmee_result_t held = {};
     bool have = false;
-    uint32_t n = 0;
+    uint32_t n = 0, n_found = 0;
     // Searches with a shrinking buffer: each returns the least DRAM traffic that fits, with the buffer words its
     // mapping needs; the next one allows one word less than that.  While the traffic stays the same the mapping
     // found needs less buffer for the same traffic; when it rises, the mapping held is a point of the front.
-    while (rc == MMEE_OK) {
-        if ((rc = mmee_search_host(h, &r, nullptr))) break;
-        const bool found = r.idx != MMEE_NO_INDEX;
-        if (have && (!found || r.e_key != held.e_key)) {
+    rc = run_chain(&plan, 1, 8, &n_found, [&](const mmee_result_t& r, uint32_t) {
+        if (have && r.e_key != held.e_key) {
             if (n < capacity) out_points[n] = held;
             ++n;
         }
-        if (!found) break;
         held = r;
         have = true;
-        if (r.bs <= 0) { if (n < capacity) out_points[n] = held; ++n; break; }      // (cannot happen: tiles take words)
-        h->plan.cap_words = r.bs - 1;
+        plan.cap_words = r.bs - 1;      // (for the tables of the next batch: tilings that cannot fit are left out)
+        return plan.cap_words >= 0;
+    });
+    if (rc == MMEE_OK && have) {
+        if (n < capacity) out_points[n] = held;
+        ++n;
     }
-    mmee_destroy(h);
     *n_points = n;
     if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
     return rc;

@@ -20,6 +20,10 @@ struct BlockTab {
 
 constexpr int kBlockItems = 32;
 
+// The bounds of a search: the plan's, or one of them set by the search before it (see LaunchShape::chain).
+struct Limits { int64_t cap_words, key_cap; };
+
+
 // Stationary-mode terms of one operator of one tiling: its energy and compute words at rho = 1 (see TileTab).
 template <class Divisors>
 __device__ __forceinline__ void stationary_terms(const Plan& p, const Divisors& dv, const uint32_t b[8], int op, int sm, int64_t& P, int64_t& Q) {
@@ -77,7 +81,7 @@ struct RowTerms {
     int64_t x1, x2;             // DRAM words of A and B, of D and E (unfused: C's write-back and read-back included)
     int64_t rho;                // recomputation factor of C
 };
-__device__ __forceinline__ RowTerms row_terms(const Plan& p, const BlockTab& bt, int a, int b, int c, int d, int e) {
+__device__ __forceinline__ RowTerms row_terms(const Plan& p, const Limits& lim, const BlockTab& bt, int a, int b, int c, int d, int e) {
     RowTerms r;
     const int64_t A = bt.size[0][a], B = bt.size[1][b], C = bt.size[2][c], D = bt.size[3][d], E = bt.size[4][e];
     int64_t need1 = A + B + C, need2 = C + D + E;
@@ -87,7 +91,7 @@ __device__ __forceinline__ RowTerms row_terms(const Plan& p, const BlockTab& bt,
         need2 += (a ? A : 0) + (b ? B : 0);
         rc = p.q.recompute[p.order_id[bt.slot]][c];
     }
-    r.fits = max64(need1, need2) <= p.cap_words;
+    r.fits = max64(need1, need2) <= lim.cap_words;
     r.rho = rc ? (int64_t)bt.jD : 1;
     r.x1 = bt.g[0][a][rc] + bt.g[1][b][rc];
     r.x2 = bt.g[3][d][0] + bt.g[4][e][0];
@@ -96,17 +100,17 @@ __device__ __forceinline__ RowTerms row_terms(const Plan& p, const BlockTab& bt,
 }
 
 template <int OBJ>
-__device__ __forceinline__ int64_t mapping_key(const Plan& p, const BlockTab& bt, const RowTerms& r, int s) {
+__device__ __forceinline__ int64_t mapping_key(const Plan& p, const Limits& lim, const BlockTab& bt, const RowTerms& r, int s) {
     const int u = s / 3, v = s - 3 * u;
-    return bt.phi == 0 ? fused_key<OBJ>(r.x1 + r.x2, r.rho, bt.P1[u], bt.P2[v], bt.Q1[u], bt.Q2[v], p.c_dram_gb, p.key_cap)
-                       : unfused_key<OBJ>(r.x1, r.x2, bt.pass, bt.P1[u], bt.P2[v], bt.Q1[u], bt.Q2[v], p.c_dram_gb, p.key_cap);
+    return bt.phi == 0 ? fused_key<OBJ>(r.x1 + r.x2, r.rho, bt.P1[u], bt.P2[v], bt.Q1[u], bt.Q2[v], p.c_dram_gb, lim.key_cap)
+                       : unfused_key<OBJ>(r.x1, r.x2, bt.pass, bt.P1[u], bt.P2[v], bt.Q1[u], bt.Q2[v], p.c_dram_gb, lim.key_cap);
 }
 
 // Row `row` of the block by its levels; the number of rows of the block.
-__device__ __forceinline__ RowTerms block_row(const Plan& p, const BlockTab& bt, uint32_t row) {
+__device__ __forceinline__ RowTerms block_row(const Plan& p, const Limits& lim, const BlockTab& bt, uint32_t row) {
     const int e = (int)(row % 5u), d = (int)(row / 5u % 5u);
-    if (bt.phi == 0) return row_terms(p, bt, (int)(row / 625u), (int)(row / 125u % 5u), (int)(row / 25u % 5u), d, e);
-    return row_terms(p, bt, (int)(row / 125u), (int)(row / 25u % 5u), 0, d, e);
+    if (bt.phi == 0) return row_terms(p, lim, bt, (int)(row / 625u), (int)(row / 125u % 5u), (int)(row / 25u % 5u), d, e);
+    return row_terms(p, lim, bt, (int)(row / 125u), (int)(row / 25u % 5u), 0, d, e);
 }
 __device__ __forceinline__ uint32_t block_rows(const BlockTab& bt) { return bt.phi == 0 ? 3125u : 625u; }
 

@@ -251,7 +251,8 @@ __device__ __forceinline__ void operator_array_terms(const Plan& p, const Diviso
 __device__ __forceinline__ void assemble_record(const Plan& p, uint64_t idx, const CandidateChoice& d, const uint32_t b[8],
                                                 const TilingCounts& tt, const int64_t bs[5], const int64_t da_in[5],
                                                 int64_t words1, int64_t cyc1, int64_t words2, int64_t cyc2,
-                                                const uint32_t blk1[3], const uint32_t blk2[3], mmee_result_t& o) {
+                                                const uint32_t blk1[3], const uint32_t blk2[3], int64_t cap_words,
+                                                mmee_result_t& o) {
     const uint32_t* lv = d.lv;
     o.idx = idx; o.t = d.t; o.row = d.row;
     for (int i = 0; i < 8; ++i) o.bound[i] = b[i];
@@ -300,7 +301,7 @@ __device__ __forceinline__ void assemble_record(const Plan& p, uint64_t idx, con
     o.n[0] = n_dram; o.n[1] = n_gb; o.n[2] = n_rf; o.n[3] = n_mac; o.n[4] = n_sfu;
     o.e_key = e_key; o.l_key = l_key;
     o.recompute = (uint8_t)d.rc;
-    o.feasible = (uint8_t)(o.bs <= p.cap_words && ((p.sm_mask >> d.s) & 1u));
+    o.feasible = (uint8_t)(o.bs <= cap_words && ((p.sm_mask >> d.s) & 1u));
     o.edp_key = __dmul_rn((double)e_key, (double)l_key);
     o.energy_pj = __dmul_rn(__dmul_rn((double)e_key, p.quantum_pj), (double)p.instances);
     const uint32_t waves = (p.instances + p.n_arrays - 1) / p.n_arrays;
@@ -322,13 +323,14 @@ __device__ inline void evaluate_candidate(const Plan& p, uint64_t idx, mmee_resu
     uint32_t blk1[3], blk2[3];
     operator_array_terms(p, PlanDivisors{p}, b, tt, 0, d.sm1, d.rc != 0, w1, c1, blk1);
     operator_array_terms(p, PlanDivisors{p}, b, tt, 1, d.sm2, d.rc != 0, w2, c2, blk2);
-    assemble_record(p, idx, d, b, tt, bs, da, w1, c1, w2, c2, blk1, blk2, o);
+    assemble_record(p, idx, d, b, tt, bs, da, w1, c1, w2, c2, blk1, blk2, p.cap_words, o);
 }
 
 // The same by one warp (all 32 lanes call it converged): lanes 0..4 take one operand each, lanes 5 and 6 one
 // operator's array-level terms each; lane 0 gathers the parts and holds the record on return.
 template <class Divisors>
-__device__ inline void evaluate_candidate_warp(const Plan& p, const Divisors& dv, uint64_t idx, int lane, mmee_result_t& o) {
+__device__ inline void evaluate_candidate_warp(const Plan& p, const Divisors& dv, uint64_t idx, int64_t cap_words, int lane,
+                                               mmee_result_t& o) {
     const CandidateChoice d = decode_candidate(p, idx);
     uint32_t b[8];
     tiling_bounds(p, d.t, b);
@@ -349,7 +351,8 @@ __device__ inline void evaluate_candidate_warp(const Plan& p, const Divisors& dv
         blk1[i] = __shfl_sync(0xffffffffu, blk[i], 5);
         blk2[i] = __shfl_sync(0xffffffffu, blk[i], 6);
     }
-    if (lane == 0) assemble_record(p, idx, d, b, tt, part0, part1, part0[5], part1[5], part0[6], part1[6], blk1, blk2, o);
+    if (lane == 0) assemble_record(p, idx, d, b, tt, part0, part1, part0[5], part1[5], part0[6], part1[6], blk1, blk2,
+                                   cap_words, o);
 }
 
 }  // namespace mmee

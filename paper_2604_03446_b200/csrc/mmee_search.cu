@@ -28,6 +28,8 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = kSearchThreads / 32;
 constexpr int kTopK = (int)MMEE_MAX_TOPK;
+// One optimum; one optimum over the rows kept by symbolic pruning; the k best; one optimum of a chain of searches.
+constexpr int kModeSingle = 0, kModePrune = 1, kModeMulti = 2, kModeChain = 3;
 
 // ------------------------------------------------------------------------------------------------
 // (key, number) pairs
@@ -175,7 +177,7 @@ __device__ __forceinline__ uint32_t row_of(bool fused, int a, int b, int c, int 
 // combination precedes its other rows, so only those are looked at).  All threads of the CTA; the pair ends up in every
 // lane of every warp's own share, to be reduced over the warps.
 template <int OBJ>
-__device__ __forceinline__ void best_of_block(const Plan& p, const Shared& sh, int64_t key, int64_t& ek, uint64_t& ei) {
+__device__ __forceinline__ void best_of_block(const Plan& p, const Limits& lim, const Shared& sh, int64_t key, int64_t& ek, uint64_t& ei) {
     const BlockTab& bt = sh.block[0];
     const OrderInfo& o = sh.order[bt.slot];
     const bool fused = bt.phi == 0;
@@ -183,12 +185,12 @@ __device__ __forceinline__ void best_of_block(const Plan& p, const Shared& sh, i
     ei = UINT64_MAX;
     for (uint32_t r = threadIdx.x; r < (fused ? kFusedReps : kUnfusedReps); r += kSearchThreads) {
         const Rep q = decode_rep(o, fused, r);
-        const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
         if (!t.fits) continue;
         uint32_t at = 9;
 #pragma unroll
         for (int s = 8; s >= 0; --s)
-            if (((p.sm_mask >> s) & 1u) && mapping_key<OBJ>(p, bt, t, s) == key) at = (uint32_t)s;
+            if (((p.sm_mask >> s) & 1u) && mapping_key<OBJ>(p, lim, bt, t, s) == key) at = (uint32_t)s;
         const uint64_t idx = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u + at;
         if (at < 9u && idx < ei) { ek = key; ei = idx; }
     }
@@ -200,7 +202,7 @@ __device__ __forceinline__ void best_of_block(const Plan& p, const Shared& sh, i
 // two of them (the rows of a combination share their keys) and the others are only compared with its last entry: taken
 // in index order instead, with all blocks in one pass, this took 53 us of a top-16 search whose best keys tie.
 template <int OBJ>
-__device__ __forceinline__ void best_of_block_multi(const Plan& p, const Shared& sh, int j, int64_t bound, int k, int lane,
+__device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits& lim, const Shared& sh, int j, int64_t bound, int k, int lane,
                                                     int64_t lk, uint64_t li, int64_t& ek, uint64_t& ei) {
     const BlockTab& bt = sh.block[j];
     const OrderInfo& o = sh.order[bt.slot];
@@ -216,11 +218,11 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Shared&
         const uint32_t r = threadIdx.x + (uint32_t)i * kSearchThreads;
         if (r >= n_reps) continue;
         const Rep q = decode_rep(o, fused, r);
-        const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
         if (!t.fits) continue;
         int64_t m = kInfKey;
         for (int s = 0; s < 9; ++s)
-            if ((p.sm_mask >> s) & 1u) m = min64(m, mapping_key<OBJ>(p, bt, t, s));
+            if ((p.sm_mask >> s) & 1u) m = min64(m, mapping_key<OBJ>(p, lim, bt, t, s));
         if (m > bound) continue;
         least[i] = m;
         first[i] = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u;
@@ -244,7 +246,7 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Shared&
         r = __reduce_max_sync(kFull, r) - 1u;
         // all of its rows and stationary pairs, in index order across the lanes
         const Rep q = decode_rep(o, fused, r);
-        const RowTerms t = row_terms(p, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
         const uint32_t n = (uint32_t)(q.width[0] * q.width[1] * q.width[2] * q.width[3] * q.width[4]) * 9u;
         for (uint32_t i0 = 0; i0 < n; i0 += 32) {
             const uint32_t i = i0 + lane;
@@ -257,7 +259,7 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Shared&
                 lv[x] = q.lv[x] + (int)(u - v * w);
                 u = v;
             }
-            const int64_t key = mapping_key<OBJ>(p, bt, t, s);
+            const int64_t key = mapping_key<OBJ>(p, lim, bt, t, s);
             const uint64_t idx = bt.first_idx + row_of(fused, lv[0], lv[1], lv[2], lv[3], lv[4]) * 9u + (uint32_t)s;
             const int64_t tk = __shfl_sync(kFull, ek, k - 1);
             const uint64_t ti = __shfl_sync(kFull, ei, k - 1);
@@ -295,10 +297,11 @@ __device__ __forceinline__ void min_over_warps(Shared& sh, int lane, int warp, i
 }
 
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
-template <int OBJ, bool MULTI>
-__device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* __restrict__ scratch, int n_partials,
+template <int OBJ, int MODE>
+__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, Scratch* __restrict__ scratch, int n_partials,
                                            mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr bool MULTI = MODE == kModeMulti;
     const int k = MULTI ? (int)p.topk : 1;
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
@@ -359,7 +362,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
         __syncthreads();
         if (found) {
             n_groups = block_rows(sh.block[0]) / 5u;
-            best_of_block<OBJ>(p, sh, bound, ek, ei);
+            best_of_block<OBJ>(p, lim, sh, bound, ek, ei);
         }
         min_over_warps(sh, lane, warp, ek, ei);
     } else {
@@ -401,7 +404,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
                 more = pair_less(key, sh.block[j].first_idx, lk, li);
                 if (!more) break;
                 n_groups += block_rows(sh.block[j]) / 5u;
-                best_of_block_multi<OBJ>(p, sh, j, bound, k, lane, lk, li, ek, ei);
+                best_of_block_multi<OBJ>(p, lim, sh, j, bound, k, lane, lk, li, ek, ei);
                 merge_warps(sh, k, lane, warp, ek, ei);
                 const longlong2 last = sh.tops[0][k - 1];
                 lk = last.x;
@@ -432,9 +435,9 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
         const long long rk = __shfl_sync(kFull, entry.x, rec);
         const uint64_t ri = (uint64_t)__shfl_sync(kFull, entry.y, rec);
         if (rec < n_out) {
-            evaluate_candidate_warp(p, SharedDivisors{sh}, ri, lane, r);
+            evaluate_candidate_warp(p, SharedDivisors{sh}, ri, lim.cap_words, lane, r);
             if (lane == 0) {
-                const int64_t key = OBJ == MMEE_OBJ_EDP ? __double_as_longlong(r.edp_key) : key_of<OBJ>(r.e_key, r.l_key, p.key_cap);
+                const int64_t key = OBJ == MMEE_OBJ_EDP ? __double_as_longlong(r.edp_key) : key_of<OBJ>(r.e_key, r.l_key, lim.key_cap);
                 if (!(key == rk && r.feasible && r.t >= p.t_begin && r.t < p.t_end)) atomicOr(&sh.check_failed, 1u);
             }
         } else {
@@ -454,7 +457,14 @@ __device__ __noinline__ void finalize_step(const Plan& p, Shared& sh, Scratch* _
             to[lane] = w0;
             if (lane + 32 < kWords) to[lane + 32] = w1;
         }
-        if (rec == 0) { first0 = w0; first1 = w1; }
+        if (rec == 0) {
+            first0 = w0;
+            first1 = w1;
+            if (MODE == kModeChain && lane == 0) {
+                // the next search's bound: one word less of buffer / this energy / one word less of latency
+                scratch->chain_bound = n_out == 0 ? -1 : (OBJ == MMEE_OBJ_ENERGY ? r.bs - 1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? r.e_key : r.l_key - 1));
+            }
+        }
         __syncwarp();
     }
     __syncthreads();
@@ -512,10 +522,11 @@ __device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, cons
     if (sub == 7) tb->t = t;
 }
 
-template <int OBJ, bool PRUNE, bool MULTI>
+template <int OBJ, int MODE>
 __global__ void __launch_bounds__(kSearchThreads, 3)
 search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* __restrict__ scratch,
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
+    constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     release_next_kernel();
@@ -543,11 +554,14 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
     const int k = MULTI ? (int)p.topk : 1;
     const int64_t I = p.dim[0], K = p.dim[1], L = p.dim[2], J = p.dim[3];
     const DimWords dw = {I * K, K * L, L * J, I * J, I * L};
-    const int capc = (int)p.cap_words;
+    // (a chained search: the bound that the search before it left, read before the items)
+    Limits lim = {p.cap_words, p.key_cap};
+    int capc = (int)p.cap_words;
     const uint32_t grid = gridDim.x, n_tilings = (uint32_t)(p.t_end - p.t_begin);
     const uint32_t n_orders = p.n_orders;
     auto any = [](bool v) { return __any_sync(kFull, v) != 0; };
 
+    bool ended = false;
     // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
@@ -619,7 +633,19 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
             wait_previous_kernel();
             if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&scratch->G);
         }
+        if (CHAIN && shape.chain_read && m0 == 0) {
+            wait_previous_kernel();
+            const int64_t bound = __ldcg(&scratch->chain_bound);
+            if (OBJ == MMEE_OBJ_ENERGY) {
+                lim.cap_words = bound;
+                capc = (int)bound;
+            } else {
+                lim.key_cap = bound;
+            }
+            ended = bound < 0;
+        }
         __syncthreads();
+        if (CHAIN && ended) break;       // the search before found nothing: neither does this one
 
         const uint32_t per_class = sh.n_live * n_orders;
         if (tid == 0) my_live += sh.n_live;
@@ -654,7 +680,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
                 if (valid) my_rows += rows;
                 const bool some = valid && x < kNoRow;
                 if (any(some)) {
-                    const int64_t key = fused_least_key<OBJ>(tb, some ? x : 0, oi.recompute[c] != 0, p.sm_mask, p.c_dram_gb, p.key_cap);
+                    const int64_t key = fused_least_key<OBJ>(tb, some ? x : 0, oi.recompute[c] != 0, p.sm_mask, p.c_dram_gb, lim.key_cap);
                     offer(key, id, some);
                 }
             } else {
@@ -674,7 +700,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
                             if ((fit1 >> ab) & 1u) rows += (uint32_t)__popc(fit2 & sh.kept.unfused[phi - 1][os][ab]);
                     }
                     if (some) my_rows += rows;
-                    const int64_t key = unfused_least_key<OBJ>(tb, y1, y2, phi == 2 ? 2 * dw.il : 0, p.sm_mask, p.c_dram_gb, p.key_cap);
+                    const int64_t key = unfused_least_key<OBJ>(tb, y1, y2, phi == 2 ? 2 * dw.il : 0, p.sm_mask, p.c_dram_gb, lim.key_cap);
                     offer(key, id + block, some);
                     block += n_orders;
                 }
@@ -727,7 +753,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
     __syncthreads();
     if (sh.last_cta) {
         __threadfence();
-        finalize_step<OBJ, MULTI>(p, sh, scratch, (int)grid, out_best, out_topk);
+        finalize_step<OBJ, MODE>(p, lim, sh, scratch, (int)grid, out_best, out_topk);
     }
 }
 
@@ -736,11 +762,17 @@ __global__ void reset_kernel(Scratch* scratch) {
     scratch->done_ctas = 0;
 }
 
+// (only the objectives of the Pareto fronts are chained)
+template <int OBJ>
+constexpr int chain_mode() { return OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? kModeSingle : kModeChain; }
+
 template <int OBJ>
 cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, Scratch* scratch, mmee_result_t* out_best,
                             mmee_result_t* out_topk, cudaStream_t st) {
-    auto* kernel = p.row_pruning ? search_kernel<OBJ, true, false>
-                                 : (p.topk > 1 ? search_kernel<OBJ, false, true> : search_kernel<OBJ, false, false>);
+    auto* kernel = shape.chain ? (OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? nullptr : search_kernel<OBJ, chain_mode<OBJ>()>)
+                   : p.row_pruning ? search_kernel<OBJ, kModePrune>
+                   : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
+    if (!kernel) return cudaErrorInvalidValue;
     cudaLaunchAttribute overlap;
     overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     overlap.val.programmaticStreamSerializationAllowed = 1;

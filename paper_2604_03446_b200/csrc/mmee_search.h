@@ -9,7 +9,7 @@
 namespace mmee {
 
 constexpr int kSearchThreads = 256;
-constexpr uint32_t kMaxChunk = 64;      // tilings whose tables a CTA holds at once
+constexpr uint32_t kMaxChunk = 96;      // tilings whose tables a CTA holds at once
 
 // One CTA's contribution: its k best blocks as (least key, block number) pairs, best first, and its counts.
 struct alignas(16) Partial {
@@ -25,8 +25,9 @@ struct Scratch {
     long long G;                            // upper bound on the k-th smallest key
     unsigned long long last_exact_groups;   // groups of 45 mappings of the winning blocks, evaluated one by one
     unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
+    long long chain_bound;                  // what a chained search leaves to the next one; -1: it found nothing
     unsigned int done_ctas;                 // ticket counter: the CTA that draws the last ticket runs the finalize step
-    unsigned int pad[9];
+    unsigned int pad[7];
     Partial partial[1];     // grid entries follow
 };
 static_assert(offsetof(Scratch, partial) == 64, "the header is 64 bytes");
@@ -34,7 +35,13 @@ static_assert(offsetof(Scratch, partial) == 64, "the header is 64 bytes");
 struct LaunchShape {
     uint32_t grid;          // CTAs; CTA c takes one tiling of every `grid` consecutive ones
     uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
+    bool chain;             // one of a chain of searches:
+    bool chain_read;        // ... not the first
 };
+// Chained searches (k = 1, no row pruning; the Pareto fronts): each takes a bound from what the one before it on the
+// stream found, on the device, so that the host waits once for several: the buffer words (energy) or the bound on the
+// other key (capped objectives) come from the scratch instead of the plan (and are not above the plan's), and the bound
+// for the next search is left there.  After a search that found nothing the others end at once.
 
 inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 

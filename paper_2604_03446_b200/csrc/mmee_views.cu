@@ -15,6 +15,7 @@ constexpr int kViewThreads = 256;
 template <int OBJ>
 __global__ void __launch_bounds__(kViewThreads) dump_kernel(const __grid_constant__ Plan p, int64_t* __restrict__ out) {
     __shared__ BlockTab bt;
+    const Limits lim = {p.cap_words, p.key_cap};
     const uint32_t first = (uint32_t)p.t_begin * p.n_blocks, last = (uint32_t)p.t_end * p.n_blocks;
     const uint64_t origin = p.t_begin * p.rows_per_tiling * 9u;
     for (uint32_t id = first + blockIdx.x; id < last; id += gridDim.x) {
@@ -24,8 +25,8 @@ __global__ void __launch_bounds__(kViewThreads) dump_kernel(const __grid_constan
         int64_t* o = out + (bt.first_idx - origin);
         for (uint32_t i = threadIdx.x; i < n; i += kViewThreads) {
             const uint32_t row = i / 9u, s = i - row * 9u;
-            const RowTerms r = block_row(p, bt, row);
-            o[i] = r.fits && ((p.sm_mask >> s) & 1u) ? mapping_key<OBJ>(p, bt, r, (int)s) : kInfKey;
+            const RowTerms r = block_row(p, lim, bt, row);
+            o[i] = r.fits && ((p.sm_mask >> s) & 1u) ? mapping_key<OBJ>(p, lim, bt, r, (int)s) : kInfKey;
         }
         __syncthreads();
     }
@@ -35,6 +36,7 @@ template <int OBJ>
 __global__ void __launch_bounds__(kViewThreads) flags_kernel(const __grid_constant__ Plan p, int64_t threshold,
                                                              unsigned char* __restrict__ flags) {
     __shared__ BlockTab bt;
+    const Limits lim = {p.cap_words, p.key_cap};
     const uint32_t first = (uint32_t)p.t_begin * p.n_blocks, last = (uint32_t)p.t_end * p.n_blocks;
     const uint64_t origin = p.t_begin * p.rows_per_tiling * 9u;
     for (uint32_t id = first + blockIdx.x; id < last; id += gridDim.x) {
@@ -44,9 +46,9 @@ __global__ void __launch_bounds__(kViewThreads) flags_kernel(const __grid_consta
         for (uint32_t i = threadIdx.x; i < block_rows(bt) / 5u; i += kViewThreads) {
             bool below = false;
             for (uint32_t e = 0; e < 5; ++e) {
-                const RowTerms r = block_row(p, bt, i * 5u + e);
+                const RowTerms r = block_row(p, lim, bt, i * 5u + e);
                 for (int s = 0; s < 9; ++s)
-                    below |= r.fits && ((p.sm_mask >> s) & 1u) && mapping_key<OBJ>(p, bt, r, s) < threshold;
+                    below |= r.fits && ((p.sm_mask >> s) & 1u) && mapping_key<OBJ>(p, lim, bt, r, s) < threshold;
             }
             o[i] = below ? 1 : 0;
         }
