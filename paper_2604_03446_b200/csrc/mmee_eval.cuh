@@ -326,33 +326,35 @@ __device__ inline void evaluate_candidate(const Plan& p, uint64_t idx, mmee_resu
     assemble_record(p, idx, d, b, tt, bs, da, w1, c1, w2, c2, blk1, blk2, p.cap_words, o);
 }
 
-// The same by one warp (all 32 lanes call it converged): lanes 0..4 take one operand each, lanes 5 and 6 one
-// operator's array-level terms each; lane 0 gathers the parts and holds the record on return.
-template <class Divisors>
-__device__ inline void evaluate_candidate_warp(const Plan& p, const Divisors& dv, uint64_t idx, int64_t cap_words, int lane,
-                                               mmee_result_t& o) {
+// The same by WIDTH lanes (32, or 16: the halves of a warp with a mapping each; all 32 lanes call it converged): lanes 0..4
+// take one operand each, lanes 5 and 6 one operator's array-level terms each; lane 0 gathers the parts and, with `write`
+// set, puts the record together.
+template <int WIDTH, class Divisors>
+__device__ inline void evaluate_candidate_lanes(const Plan& p, const Divisors& dv, uint64_t idx, int64_t cap_words, int lane,
+                                                bool write, mmee_result_t& o) {
     const CandidateChoice d = decode_candidate(p, idx);
     uint32_t b[8];
     tiling_bounds(p, d.t, b);
     const TilingCounts tt = tiling_counts(p, b);
+    const int l = lane & (WIDTH - 1);
     int64_t v0 = 0, v1 = 0;
     uint32_t blk[3] = {0, 0, 0};
-    if (lane < 5) operand_terms(p, d, b, lane, v0, v1);
-    else if (lane < 7) operator_array_terms(p, dv, b, tt, lane - 5, lane == 5 ? d.sm1 : d.sm2, d.rc != 0, v0, v1, blk);
+    if (l < 5) operand_terms(p, d, b, l, v0, v1);
+    else if (l < 7) operator_array_terms(p, dv, b, tt, l - 5, l == 5 ? d.sm1 : d.sm2, d.rc != 0, v0, v1, blk);
     int64_t part0[7], part1[7];
 #pragma unroll
     for (int i = 0; i < 7; ++i) {
-        part0[i] = __shfl_sync(0xffffffffu, v0, i);
-        part1[i] = __shfl_sync(0xffffffffu, v1, i);
+        part0[i] = __shfl_sync(0xffffffffu, v0, i, WIDTH);
+        part1[i] = __shfl_sync(0xffffffffu, v1, i, WIDTH);
     }
     uint32_t blk1[3], blk2[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        blk1[i] = __shfl_sync(0xffffffffu, blk[i], 5);
-        blk2[i] = __shfl_sync(0xffffffffu, blk[i], 6);
+        blk1[i] = __shfl_sync(0xffffffffu, blk[i], 5, WIDTH);
+        blk2[i] = __shfl_sync(0xffffffffu, blk[i], 6, WIDTH);
     }
-    if (lane == 0) assemble_record(p, idx, d, b, tt, part0, part1, part0[5], part1[5], part0[6], part1[6], blk1, blk2,
-                                   cap_words, o);
+    if (l == 0 && write)
+        assemble_record(p, idx, d, b, tt, part0, part1, part0[5], part1[5], part0[6], part1[6], blk1, blk2, cap_words, o);
 }
 
 }  // namespace mmee

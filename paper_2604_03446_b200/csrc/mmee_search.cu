@@ -122,6 +122,7 @@ struct Shared {
     uint32_t divs[4][MMEE_MAX_DIVISORS];
     uint32_t row_folds[4][MMEE_MAX_DIVISORS], col_folds[4][MMEE_MAX_DIVISORS];      // register-file tiling only
     alignas(16) longlong2 tops[kWarps][MMEE_MAX_TOPK];
+    longlong2 kth[kWarps];          // finalize, k > 1: the k-th pair of each warp's list (kInfKey: not full)
     long long G;                    // k > 1: upper bound on the k-th smallest key
     unsigned long long feasible_rows[kWarps];
     uint32_t live_tilings[kWarps];
@@ -131,7 +132,7 @@ struct Shared {
     union {
         TileTab tile[kMaxChunk];
         BlockTab block[kWarps];
-        mmee_result_t record[kWarps];
+        mmee_result_t record[MMEE_MAX_TOPK];
     };
 };
 
@@ -197,61 +198,54 @@ __device__ __forceinline__ void best_of_block(const Plan& p, const Limits& lim, 
     warp_min_pair(ek, ei);
 }
 
+__device__ __forceinline__ longlong2 ld_volatile(const longlong2* a) {
+    longlong2 v;
+    asm volatile("ld.volatile.shared.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"((uint32_t)__cvta_generic_to_shared(a)));
+    return v;
+}
+
 // The mappings of block `j` of sh.block that precede the running k-th pair (lk, li), none above `bound`, into the warps'
-// lists.  Every warp takes its share of the block's class combinations best first, so that a list is full after one or
-// two of them (the rows of a combination share their keys) and the others are only compared with its last entry: taken
-// in index order instead, with all blocks in one pass, this took 53 us of a top-16 search whose best keys tie.
+// lists.  A lane holds one class combination and walks its mappings in (key, index) order: the stationary pairs of its
+// least key over its rows, then those of the next larger key; the warp takes the smallest of its lanes' next mappings
+// until it has k of them or the next one does not precede what a full list of any warp ends with.  (Taking whole
+// combinations one after the other, each sorted into the list, needed a dozen of them per warp where all mappings tie:
+// 24 us of a Llama top-16 search instead of 16.)
 template <int OBJ>
-__device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits& lim, const Shared& sh, int j, int64_t bound, int k, int lane,
+__device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits& lim, Shared& sh, int j, int64_t bound, int k, int lane,
                                                     int64_t lk, uint64_t li, int64_t& ek, uint64_t& ei) {
     const BlockTab& bt = sh.block[j];
     const OrderInfo& o = sh.order[bt.slot];
     const bool fused = bt.phi == 0;
     const uint32_t n_reps = fused ? kFusedReps : kUnfusedReps;
-    constexpr int kShare = (int)((kFusedReps + kSearchThreads - 1) / kSearchThreads);
-    int64_t least[kShare];
-    uint64_t first[kShare];
-#pragma unroll
-    for (int i = 0; i < kShare; ++i) {
-        least[i] = kInfKey;
-        first[i] = UINT64_MAX;
-        const uint32_t r = threadIdx.x + (uint32_t)i * kSearchThreads;
-        if (r >= n_reps) continue;
-        const Rep q = decode_rep(o, fused, r);
+#pragma unroll 1
+    for (uint32_t r = threadIdx.x; r - lane < n_reps; r += kSearchThreads) {
+        const Rep q = decode_rep(o, fused, r < n_reps ? r : 0u);
         const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
-        if (!t.fits) continue;
-        int64_t m = kInfKey;
-        for (int s = 0; s < 9; ++s)
-            if ((p.sm_mask >> s) & 1u) m = min64(m, mapping_key<OBJ>(p, lim, bt, t, s));
-        if (m > bound) continue;
-        least[i] = m;
-        first[i] = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u;
-    }
-    while (true) {
-        // the best combination not yet taken, and the pair it has to precede
-        int64_t bk = least[0];
-        uint64_t bi = first[0];
-#pragma unroll
-        for (int i = 1; i < kShare; ++i)
-            if (pair_less(least[i], first[i], bk, bi)) { bk = least[i]; bi = first[i]; }
-        warp_min_pair(bk, bi);
-        const int64_t ok = __shfl_sync(kFull, ek, k - 1);
-        const uint64_t oi = __shfl_sync(kFull, ei, k - 1);
-        if (pair_less(ok, oi, lk, li)) { lk = ok; li = oi; }
-        if (!pair_less(bk, bi, lk, li)) break;
-        uint32_t r = 0;
-#pragma unroll
-        for (int i = 0; i < kShare; ++i)
-            if (first[i] == bi) { r = threadIdx.x + (uint32_t)i * kSearchThreads + 1u; least[i] = kInfKey; first[i] = UINT64_MAX; }
-        r = __reduce_max_sync(kFull, r) - 1u;
-        // all of its rows and stationary pairs, in index order across the lanes
-        const Rep q = decode_rep(o, fused, r);
-        const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
-        const uint32_t n = (uint32_t)(q.width[0] * q.width[1] * q.width[2] * q.width[3] * q.width[4]) * 9u;
-        for (uint32_t i0 = 0; i0 < n; i0 += 32) {
-            const uint32_t i = i0 + lane;
-            uint32_t u = i / 9u;
-            const int s = (int)(i - u * 9u);
+        const uint32_t n_rows = (uint32_t)(q.width[0] * q.width[1] * q.width[2] * q.width[3] * q.width[4]);
+        int64_t hk = -1;                        // the lane's next mapping: key, index, row of the combination
+        uint64_t hi = UINT64_MAX;
+        uint32_t row = 0, pairs = 0, left = 0;  // stationary pairs with that key, those left of the row
+        auto next = [&]() {
+            left &= left - 1u;
+            if (!left) {
+                if (pairs && row + 1 < n_rows) {
+                    ++row;
+                } else {                        // the next larger key
+                    const int64_t last = hk;
+                    hk = kInfKey;
+                    pairs = 0;
+                    for (int s = 0; s < 9; ++s) {
+                        const int64_t key = mapping_key<OBJ>(p, lim, bt, t, s);
+                        if (!((p.sm_mask >> s) & 1u) || key <= last || key > hk) continue;
+                        pairs = key < hk ? 1u << s : pairs | 1u << s;
+                        hk = key;
+                    }
+                    row = 0;
+                    if (hk > bound) { hk = kInfKey; hi = UINT64_MAX; return; }
+                }
+                left = pairs;
+            }
+            uint32_t u = row;
             int lv[5];
 #pragma unroll
             for (int x = 4; x >= 0; --x) {
@@ -259,15 +253,28 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits&
                 lv[x] = q.lv[x] + (int)(u - v * w);
                 u = v;
             }
-            const int64_t key = mapping_key<OBJ>(p, lim, bt, t, s);
-            const uint64_t idx = bt.first_idx + row_of(fused, lv[0], lv[1], lv[2], lv[3], lv[4]) * 9u + (uint32_t)s;
-            const int64_t tk = __shfl_sync(kFull, ek, k - 1);
-            const uint64_t ti = __shfl_sync(kFull, ei, k - 1);
-            const bool pend = i < n && ((p.sm_mask >> s) & 1u) && key <= bound && pair_less(key, idx, lk, li) && pair_less(key, idx, tk, ti);
-            // (later rows repeat the same keys at higher indices)
-            if (!__any_sync(kFull, pend)) break;
-            warp_offer(ek, ei, k, key, idx, pend, lane);
+            hi = bt.first_idx + row_of(fused, lv[0], lv[1], lv[2], lv[3], lv[4]) * 9u + (uint32_t)(__ffs(left) - 1);
+        };
+        if (r < n_reps && t.fits) next();
+        else hk = kInfKey;
+        // (every warp's k-th pair bounds the block's: a torn view is impossible, a pair is one 16-byte word)
+        const longlong2 other = ld_volatile(&sh.kth[lane & (kWarps - 1)]);
+        int64_t ok = other.x, nk = kInfKey;
+        uint64_t oi = (uint64_t)other.y, ni = UINT64_MAX;
+        warp_min_pair(ok, oi);
+        if (pair_less(ok, oi, lk, li)) { lk = ok; li = oi; }
+#pragma unroll 1
+        for (int i = 0; i < k; ++i) {
+            int64_t bk = hk;
+            uint64_t bi = hi;
+            warp_min_pair(bk, bi);
+            if (!pair_less(bk, bi, lk, li)) break;
+            if (lane == i) { nk = bk; ni = bi; }
+            if (hi == bi) next();
         }
+        reg_merge(ek, ei, k, nk, ni, lane);
+        if (lane == k - 1) sh.kth[threadIdx.x >> 5] = make_longlong2((long long)ek, (long long)ei);
+        __syncwarp();
     }
 }
 
@@ -294,6 +301,11 @@ __device__ __forceinline__ void min_over_warps(Shared& sh, int lane, int warp, i
     ek = v.x;
     ei = (uint64_t)v.y;
     warp_min_pair(ek, ei);
+}
+
+// The items of a block's tables (block_item), their three kinds on three warps.
+__device__ __forceinline__ int split_item(int warp, int lane) {
+    return warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (warp == 2 && lane == 0 ? 31 : -1));
 }
 
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
@@ -356,8 +368,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         found = ek != kInfKey ? 1 : 0;
         bound = ek;
         // ---- the winning block, mapping by mapping
-        // (the three kinds of items on three warps)
-        const int item = warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (tid == 64 ? 31 : -1));
+        const int item = split_item(warp, lane);
         if (found && item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)ei, item, &sh.block[0]);
         __syncthreads();
         if (found) {
@@ -383,21 +394,26 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         uint64_t li = UINT64_MAX;
         __syncthreads();                // sh.tops has been read
         // ---- the winning blocks, mapping by mapping, best block first; once a block's (least key, first index) does
-        // not precede the k-th mapping, neither does a later one's
-        for (int j0 = 0; j0 < n_fresh; j0 += kWarps) {
+        // not precede the k-th mapping, neither does a later one's.  (Usually the first block is the only one: its
+        // tables are built by three warps, the others' one block to a warp.)
+        bool more = true;
+        for (int j0 = 0; more && j0 < n_fresh; j0 += j0 ? kWarps : 1) {
+            const int n_batch = j0 ? min(kWarps, n_fresh - j0) : 1;
             int64_t bk[kWarps];
 #pragma unroll
             for (int j = 0; j < kWarps; ++j) {
-                const int src = m ? __ffs(m) - 1 : 0;
-                bk[j] = m ? (int64_t)__shfl_sync(kFull, e.x, src) : kInfKey;
-                const uint32_t id = (uint32_t)__shfl_sync(kFull, e.y, src);
-                if (m && j == warp) block_item(p, SharedDivisors{sh}, id, lane, &sh.block[j]);
+                if (j >= n_batch) continue;
+                const int src = __ffs(m) - 1;
                 m &= m - 1;
+                bk[j] = __shfl_sync(kFull, e.x, src);
+                const uint32_t id = (uint32_t)__shfl_sync(kFull, e.y, src);
+                const int item = j0 ? (j == warp ? lane : -1) : split_item(warp, lane);
+                if (item >= 0) block_item(p, SharedDivisors{sh}, id, item, &sh.block[j]);
             }
+            if (lane == 0) sh.kth[warp] = make_longlong2(kInfKey, -1ll);
             __syncthreads();
-            bool more = true;
 #pragma unroll 1
-            for (int j = 0; j < kWarps && j0 + j < n_fresh; ++j) {
+            for (int j = 0; j < n_batch; ++j) {
                 int64_t key = bk[0];
 #pragma unroll
                 for (int i = 1; i < kWarps; ++i) key = i == j ? bk[i] : key;
@@ -412,78 +428,71 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
                 if (warp) { ek = kInfKey; ei = UINT64_MAX; }        // (warp 0 goes on with the merged list)
                 __syncthreads();
             }
-            if (!more) break;
         }
         if (!n_fresh && lane < kTopK && warp == 0) sh.tops[0][lane] = make_longlong2(kInfKey, -1ll);
         __syncthreads();
     }
 
-    // ---- every winner evaluated in full, one warp per record (the parts of a record on different lanes); the key it
-    // was ranked by must be the key of that evaluation, or the records are marked as no result
-    longlong2 entry = make_longlong2(kInfKey, -1ll);
-    if (MULTI) { if (lane < k) entry = sh.tops[0][lane]; }
-    else if (lane == 0) entry = make_longlong2((long long)ek, (long long)ei);
-    const int n_out = __popc(__ballot_sync(kFull, entry.x != kInfKey));
-    if (tid == 0 && (n_out == 0) != (found == 0)) atomicOr(&sh.check_failed, 1u);
-    // (records are put together in shared memory and copied by the warp: a lane holds words `lane` and `lane + 32`)
+    // ---- every winner evaluated in full by its lanes (a warp, or half a warp per record when there are several); the
+    // key it was ranked by must be the key of that evaluation, or the records are marked as no result
+    constexpr int kLanes = MULTI ? 16 : 32;
     constexpr int kWords = sizeof(mmee_result_t) / 8;
-    static_assert(sizeof(mmee_result_t) % 8 == 0 && kWords <= 64 && offsetof(mmee_result_t, status) % 8 == 4, "record words");
-    mmee_result_t& r = sh.record[warp];
-    const unsigned long long* words = reinterpret_cast<const unsigned long long*>(&r);
-    unsigned long long first0 = 0, first1 = 0;
-    for (int rec = warp; rec < k; rec += kWarps) {
-        const long long rk = __shfl_sync(kFull, entry.x, rec);
-        const uint64_t ri = (uint64_t)__shfl_sync(kFull, entry.y, rec);
-        if (rec < n_out) {
-            evaluate_candidate_warp(p, SharedDivisors{sh}, ri, lim.cap_words, lane, r);
-            if (lane == 0) {
+    static_assert(sizeof(mmee_result_t) % 8 == 0 && MMEE_MAX_TOPK == 2 * kWarps, "two records to a warp");
+    const int rec = MULTI ? 2 * warp + (lane >> 4) : 0, l = lane & (kLanes - 1);
+    longlong2 entry = make_longlong2(kInfKey, -1ll);
+    if (MULTI && lane < k) entry = sh.tops[0][lane];
+    const int n_out = MULTI ? __popc(__ballot_sync(kFull, entry.x != kInfKey)) : (ek != kInfKey ? 1 : 0);
+    if (tid == 0 && (n_out == 0) != (found == 0)) atomicOr(&sh.check_failed, 1u);
+    if (MULTI ? 2 * warp < k : warp == 0) {
+        mmee_result_t& r = sh.record[rec];          // put together in shared memory and copied from there
+        const int64_t rk = MULTI ? (int64_t)__shfl_sync(kFull, entry.x, rec) : ek;
+        uint64_t ri = MULTI ? (uint64_t)__shfl_sync(kFull, entry.y, rec) : ei;
+        const uint64_t other = MULTI ? (uint64_t)__shfl_sync(kFull, entry.y, 2 * warp) : ei;
+        const bool full = rec < n_out;
+        if (!full) ri = other;                      // (a half without a record goes along with the other)
+        if ((MULTI ? 2 * warp : 0) < n_out)
+            evaluate_candidate_lanes<kLanes>(p, SharedDivisors{sh}, ri, lim.cap_words, lane, full, r);
+        if (full) {
+            if (l == 0) {
                 const int64_t key = OBJ == MMEE_OBJ_EDP ? __double_as_longlong(r.edp_key) : key_of<OBJ>(r.e_key, r.l_key, lim.key_cap);
                 if (!(key == rk && r.feasible && r.t >= p.t_begin && r.t < p.t_end)) atomicOr(&sh.check_failed, 1u);
             }
         } else {
             // empty slot
             unsigned long long* raw = reinterpret_cast<unsigned long long*>(&r);
-            for (int i = lane; i < kWords; i += 32) raw[i] = 0;
-            __syncwarp();
-            if (lane == 0) {
+            for (int i = l; i < kWords; i += kLanes) raw[i] = 0;
+            __syncwarp(MULTI ? 0xffffu << (lane & 16) : kFull);
+            if (l == 0) {
                 r.idx = MMEE_NO_INDEX;
                 r.status = n_out ? MMEE_OK : MMEE_ERR_NO_FEASIBLE;
             }
         }
         __syncwarp();
-        const unsigned long long w0 = words[lane], w1 = lane + 32 < kWords ? words[lane + 32] : 0;
-        if (out_topk) {
+        if (out_topk && rec < k) {
+            const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
             unsigned long long* to = reinterpret_cast<unsigned long long*>(&out_topk[rec]);
-            to[lane] = w0;
-            if (lane + 32 < kWords) to[lane + 32] = w1;
+            for (int i = l; i < kWords; i += kLanes) to[i] = from[i];
         }
-        if (rec == 0) {
-            first0 = w0;
-            first1 = w1;
-            if (MODE == kModeChain && lane == 0) {
-                // the next search's bound: one word less of buffer / this energy / one word less of latency
-                scratch->chain_bound = n_out == 0 ? -1 : (OBJ == MMEE_OBJ_ENERGY ? r.bs - 1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? r.e_key : r.l_key - 1));
-            }
+        if (MODE == kModeChain && tid == 0) {
+            // the next search's bound: one word less of buffer / this energy / one word less of latency
+            scratch->chain_bound = n_out == 0 ? -1 : (OBJ == MMEE_OBJ_ENERGY ? r.bs - 1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? r.e_key : r.l_key - 1));
         }
-        __syncwarp();
     }
     __syncthreads();
     if (warp == 0) {
         unsigned long long all_rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
 #pragma unroll
         for (int off = kWarps / 2; off; off >>= 1) all_rows += __shfl_xor_sync(kFull, all_rows, off);
-        all_rows = __shfl_sync(kFull, all_rows, 0);
-        auto set = [&](size_t word, unsigned long long v) {
-            if (lane == (int)word) first0 = v;
-            if (lane + 32 == (int)word) first1 = v;
-        };
-        set(offsetof(mmee_result_t, n_total) / 8, (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u);
-        set(offsetof(mmee_result_t, n_feasible) / 8, all_rows * (uint64_t)p.n_sm);
-        if (sh.check_failed && lane == (int)(offsetof(mmee_result_t, status) / 8))
-            first0 = (first0 & 0xffffffffull) | ((unsigned long long)MMEE_ERR_CHECK << 32);
+        mmee_result_t& best = sh.record[0];
+        if (lane == 0) {
+            best.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
+            best.n_feasible = all_rows * (uint64_t)p.n_sm;
+            if (sh.check_failed) best.status = MMEE_ERR_CHECK;
+        }
+        __syncwarp();
+        const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&best);
         unsigned long long* to = reinterpret_cast<unsigned long long*>(out_best);
-        to[lane] = first0;
-        if (lane + 32 < kWords) to[lane + 32] = first1;
+        for (int i = lane; i < kWords; i += 32) to[i] = from[i];
     } else if (tid == 32) {
         // ready for the next search on this scratch
         unsigned long long all_live = 0;
