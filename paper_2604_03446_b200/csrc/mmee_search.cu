@@ -209,7 +209,7 @@ __device__ __forceinline__ longlong2 ld_volatile(const longlong2* a) {
 // least key over its rows, then those of the next larger key; the warp takes the smallest of its lanes' next mappings
 // until it has k of them or the next one does not precede what a full list of any warp ends with.  (Taking whole
 // combinations one after the other, each sorted into the list, needed a dozen of them per warp where all mappings tie:
-// 24 us of a Llama top-16 search instead of 16.)
+// 24 us of a Llama top-16 search instead of 12.)
 template <int OBJ>
 __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits& lim, Shared& sh, int j, int64_t bound, int k, int lane,
                                                     int64_t lk, uint64_t li, int64_t& ek, uint64_t& ei) {
@@ -221,16 +221,31 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits&
     for (uint32_t r = threadIdx.x; r - lane < n_reps; r += kSearchThreads) {
         const Rep q = decode_rep(o, fused, r < n_reps ? r : 0u);
         const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
-        const uint32_t n_rows = (uint32_t)(q.width[0] * q.width[1] * q.width[2] * q.width[3] * q.width[4]);
-        int64_t hk = -1;                        // the lane's next mapping: key, index, row of the combination
+        const uint32_t first_row = row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        int64_t hk = -1;                        // the lane's next mapping: key, index
         uint64_t hi = UINT64_MAX;
-        uint32_t row = 0, pairs = 0, left = 0;  // stationary pairs with that key, those left of the row
+        uint32_t pairs = 0, left = 0;           // stationary pairs with that key, those left of the row
+        uint32_t row = 0;                       // the row, and where its levels stand within their classes
+        int at[5] = {0, 0, 0, 0, 0};
         auto next = [&]() {
             left &= left - 1u;
             if (!left) {
-                if (pairs && row + 1 < n_rows) {
-                    ++row;
-                } else {                        // the next larger key
+                bool more = pairs != 0;
+                if (more) {
+                    more = false;               // the next row of the combination: its levels count up, E's fastest
+                    int stride = 1;
+#pragma unroll
+                    for (int x = 4; x >= 0; --x) {
+                        if (!fused && x == OP_C) continue;
+                        if (!more) {
+                            more = ++at[x] < q.width[x];
+                            row += (uint32_t)(more ? stride : -stride * (q.width[x] - 1));
+                            if (!more) at[x] = 0;
+                        }
+                        stride *= 5;
+                    }
+                }
+                if (!more) {                    // the next larger key
                     const int64_t last = hk;
                     hk = kInfKey;
                     pairs = 0;
@@ -240,20 +255,12 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits&
                         pairs = key < hk ? 1u << s : pairs | 1u << s;
                         hk = key;
                     }
-                    row = 0;
+                    row = first_row;
                     if (hk > bound) { hk = kInfKey; hi = UINT64_MAX; return; }
                 }
                 left = pairs;
             }
-            uint32_t u = row;
-            int lv[5];
-#pragma unroll
-            for (int x = 4; x >= 0; --x) {
-                const uint32_t w = (uint32_t)q.width[x], v = u / w;
-                lv[x] = q.lv[x] + (int)(u - v * w);
-                u = v;
-            }
-            hi = bt.first_idx + row_of(fused, lv[0], lv[1], lv[2], lv[3], lv[4]) * 9u + (uint32_t)(__ffs(left) - 1);
+            hi = bt.first_idx + row * 9u + (uint32_t)(__ffs(left) - 1);
         };
         if (r < n_reps && t.fits) next();
         else hk = kInfKey;
@@ -381,11 +388,8 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         const longlong2 e = lane < kTopK ? sh.tops[0][lane] : make_longlong2(kInfKey, -1ll);
         found = __popc(__ballot_sync(kFull, e.x != kInfKey));
         bound = found == k ? (int64_t)__shfl_sync(kFull, e.x, k - 1) : kInfKey - 1;     // k items hold k mappings
-        bool fresh = e.x != kInfKey;            // the first item of its block
-        for (int j = 0; j < kTopK; ++j) {
-            const long long other = __shfl_sync(kFull, e.y, j);
-            if (j < lane && other == e.y) fresh = false;
-        }
+        const unsigned same = __match_any_sync(kFull, (unsigned long long)e.y);      // (by all lanes, whatever they hold)
+        const bool fresh = e.x != kInfKey && __ffs(same) - 1 == lane;                 // the first item of its block
         unsigned m = __ballot_sync(kFull, fresh);
         const int n_fresh = __popc(m);
         ek = kInfKey;
