@@ -40,10 +40,12 @@ __device__ __forceinline__ TileForm tile_form(int sm, uint32_t m, uint32_t r, ui
     return f;
 }
 
-// Divisors of dimension d in ascending order, and how often one has to be folded onto the array's rows / columns: read from
+// The array's rows and columns, the divisors of dimension d in ascending order, and how often one has to be folded onto the array's rows / columns: read from
 // the plan (here) or from a CTA's shared copy.
 struct PlanDivisors {
     const Plan& p;
+    __device__ __forceinline__ uint32_t rows() const { return p.pe_rows; }
+    __device__ __forceinline__ uint32_t cols() const { return p.pe_cols; }
     __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return p.divs[d][i]; }
     __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_rows - 1) / p.pe_rows; }
     __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_cols - 1) / p.pe_cols; }
@@ -115,7 +117,7 @@ __device__ __forceinline__ void tile_array_terms(const Plan& p, const Divisors& 
         const int dm = LOOP_I, dr = op == 0 ? LOOP_K : LOOP_L, dn = op == 0 ? LOOP_L : LOOP_J;
         rf_block_terms(p, dv, sm, f, sm == 0 ? dr : dm, sm == 0 ? dn : (sm == 1 ? dr : dn), words, cycles, blk);
     } else {
-        const int64_t qa = (f.ea + p.pe_rows - 1) / p.pe_rows, qb = (f.eb + p.pe_cols - 1) / p.pe_cols;
+        const int64_t qa = (f.ea + dv.rows() - 1) / dv.rows(), qb = (f.eb + dv.cols() - 1) / dv.cols();
         words = f.c0 + f.ca * qa + f.cb * qb;
         cycles = f.third * qa * qb;
         blk[0] = blk[1] = blk[2] = 0;

@@ -120,6 +120,7 @@ struct Shared {
     OrderInfo order[kMaxOrders];
     KeptMasks kept;
     uint32_t divs[4][MMEE_MAX_DIVISORS];
+    uint32_t pe_rows, pe_cols;      // the array's logical shape
     uint32_t row_folds[4][MMEE_MAX_DIVISORS], col_folds[4][MMEE_MAX_DIVISORS];      // register-file tiling only
     alignas(16) longlong2 tops[kWarps][MMEE_MAX_TOPK];
     longlong2 kth[kWarps];          // finalize, k > 1: the k-th pair of each warp's list (kInfKey: not full)
@@ -138,6 +139,8 @@ struct Shared {
 
 struct SharedDivisors {       // see PlanDivisors
     const Shared& sh;
+    __device__ __forceinline__ uint32_t rows() const { return sh.pe_rows; }
+    __device__ __forceinline__ uint32_t cols() const { return sh.pe_cols; }
     __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
     __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return sh.row_folds[d][i]; }
     __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return sh.col_folds[d][i]; }
@@ -317,7 +320,8 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
 
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
 template <int OBJ, int MODE>
-__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, Scratch* __restrict__ scratch, int n_partials,
+__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, SearchHeader* __restrict__ head,
+                                           const Partial* __restrict__ partials, int n_partials,
                                            mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr bool MULTI = MODE == kModeMulti;
@@ -329,21 +333,21 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
     // ---- the k best items of all CTAs (loads bypass the L1 cache, all of a thread's in flight at once)
     for (int c0 = 0; c0 < n_partials; c0 += kSearchThreads) {
         const int c = c0 + tid;
-        longlong2 head = make_longlong2(kInfKey, -1ll), tail = make_longlong2(0, 0);
+        longlong2 first = make_longlong2(kInfKey, -1ll), tail = make_longlong2(0, 0);
         if (c < n_partials) {
-            head = __ldcg(&scratch->partial[c].e[0]);
-            tail = __ldcg(reinterpret_cast<const longlong2*>(&scratch->partial[c].count));
+            first = __ldcg(&partials[c].e[0]);
+            tail = __ldcg(reinterpret_cast<const longlong2*>(&partials[c].count));
         }
         const uint32_t count = (uint32_t)tail.x;
         live += (uint64_t)tail.x >> 32;
         rows += (unsigned long long)tail.y;
         if (!MULTI) {
-            if (count && pair_less(head.x, (uint64_t)head.y, ek, ei)) { ek = head.x; ei = (uint64_t)head.y; }
+            if (count && pair_less(first.x, (uint64_t)first.y, ek, ei)) { ek = first.x; ei = (uint64_t)first.y; }
         } else {
             // the lists of this warp's lanes, best heads first: once a head does not precede the k-th entry, no
             // other list adds anything
-            int64_t hk = count ? head.x : kInfKey;
-            uint64_t hi = count ? (uint64_t)head.y : UINT64_MAX;
+            int64_t hk = count ? first.x : kInfKey;
+            uint64_t hi = count ? (uint64_t)first.y : UINT64_MAX;
             while (true) {
                 int64_t bk = hk;
                 uint64_t bi = hi;
@@ -352,7 +356,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
                 const int src = __ffs(__ballot_sync(kFull, hk == bk && hi == bi && count)) - 1;
                 const int n = (int)__shfl_sync(kFull, count, src);
                 longlong2 theirs = make_longlong2(kInfKey, -1ll);
-                if (lane < n) theirs = __ldcg(&scratch->partial[c0 + warp * 32 + src].e[lane]);
+                if (lane < n) theirs = __ldcg(&partials[c0 + warp * 32 + src].e[lane]);
                 reg_merge(ek, ei, k, theirs.x, (uint64_t)theirs.y, lane);
                 if (lane == src) { hk = kInfKey; hi = UINT64_MAX; }
             }
@@ -479,7 +483,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         }
         if (MODE == kModeChain && tid == 0) {
             // the next search's bound: one word less of buffer / this energy / one word less of latency
-            scratch->chain_bound = n_out == 0 ? -1 : (OBJ == MMEE_OBJ_ENERGY ? r.bs - 1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? r.e_key : r.l_key - 1));
+            head->chain_bound = n_out == 0 ? -1 : (OBJ == MMEE_OBJ_ENERGY ? r.bs - 1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? r.e_key : r.l_key - 1));
         }
     }
     __syncthreads();
@@ -501,11 +505,11 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         // ready for the next search on this scratch
         unsigned long long all_live = 0;
         for (int w = 0; w < kWarps; ++w) all_live += sh.live_tilings[w];
-        scratch->G = kInfKey - 1;
-        scratch->last_exact_groups = n_groups;
+        head->G = kInfKey - 1;
+        head->last_exact_groups = n_groups;
         const uint32_t unfused_modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
-        scratch->last_tested_rows = all_live * p.n_orders * ((p.fuse_mask & 1u ? kFusedReps : 0u) + (unfused_modes ? 18u : 0u));
-        scratch->done_ctas = 0;
+        head->last_tested_rows = all_live * p.n_orders * ((p.fuse_mask & 1u ? kFusedReps : 0u) + (unfused_modes ? 18u : 0u));
+        head->done_ctas = 0;
     }
 }
 
@@ -537,30 +541,35 @@ __device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, cons
 
 template <int OBJ, int MODE>
 __global__ void __launch_bounds__(kSearchThreads, 3)
-search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* __restrict__ scratch,
+search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ heads, Partial* __restrict__ partials,
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    SearchHeader* head = heads + blockIdx.y;
     release_next_kernel();
     for (int i = tid; i < (int)(sizeof(sh.order) / 4); i += kSearchThreads)
         reinterpret_cast<uint32_t*>(sh.order)[i] = reinterpret_cast<const uint32_t*>(p.order)[i];
     if (PRUNE)
         for (int i = tid; i < (int)(sizeof(KeptMasks) / 4); i += kSearchThreads)
             reinterpret_cast<uint32_t*>(&sh.kept)[i] = reinterpret_cast<const uint32_t*>(&p.kept)[i];
+    const uint32_t pe_rows = shape.n_arrays ? shape.array[blockIdx.y][0] : p.pe_rows;
+    const uint32_t pe_cols = shape.n_arrays ? shape.array[blockIdx.y][1] : p.pe_cols;
     static_assert(kSearchThreads == 4 * MMEE_MAX_DIVISORS, "one thread per divisor");
     if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) {
         const int d = tid >> 6, i = tid & 63;
         sh.divs[d][i] = p.divs[d][i];
         if (p.rf_tiling) {
-            sh.row_folds[d][i] = PlanDivisors{p}.row_folds(d, i);
-            sh.col_folds[d][i] = PlanDivisors{p}.col_folds(d, i);
+            sh.row_folds[d][i] = (p.divs[d][i] + pe_rows - 1) / pe_rows;
+            sh.col_folds[d][i] = (p.divs[d][i] + pe_cols - 1) / pe_cols;
         }
     }
     if (tid == 0) {
         sh.n_live = 0;
         sh.cursor = 0;
         sh.check_failed = 0;
+        sh.pe_rows = pe_rows;
+        sh.pe_cols = pe_cols;
     }
     __syncthreads();
 
@@ -594,7 +603,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
         // a full list bounds the k-th smallest key for everybody
         if (lane == k - 1 && ek < *reinterpret_cast<volatile long long*>(&sh.G)) {
             atomicMin(&sh.G, (long long)ek);
-            atomicMin(&scratch->G, (long long)ek);
+            atomicMin(&head->G, (long long)ek);
         }
     };
 
@@ -644,11 +653,11 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
         if (MULTI && m0 == 0) {
             // (k > 1 shares a bound through the scratch while it works on the items)
             wait_previous_kernel();
-            if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&scratch->G);
+            if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
         }
         if (CHAIN && shape.chain_read && m0 == 0) {
             wait_previous_kernel();
-            const int64_t bound = __ldcg(&scratch->chain_bound);
+            const int64_t bound = __ldcg(&head->chain_bound);
             if (OBJ == MMEE_OBJ_ENERGY) {
                 lim.cap_words = bound;
                 capc = (int)bound;
@@ -671,7 +680,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
             g = __shfl_sync(kFull, g, 0);
             if (g >= groups) break;
             long long g_seen = 0;       // k > 1: the other CTAs' bound, used after this item
-            if (MULTI && lane == 0) g_seen = *reinterpret_cast<volatile long long*>(&scratch->G);
+            if (MULTI && lane == 0) g_seen = *reinterpret_cast<volatile long long*>(&head->G);
             const bool fused = g < fused_groups;
             uint32_t i = (fused ? g : g - fused_groups) * 32u + (uint32_t)lane;
             const uint32_t n_items = fused ? fused_items : per_class;
@@ -734,11 +743,11 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
     }
     wait_previous_kernel();     // from here on the scratch and the result records are touched
     if (warp == 0) {
-        Partial* out = &scratch->partial[blockIdx.x];
+        Partial* out = &partials[blockIdx.y * grid + blockIdx.x];
         uint32_t count;
         if (MULTI) {
             // an entry above the bound (some full list's last key) is not among the k best
-            long long g_end = lane == 0 ? *reinterpret_cast<volatile long long*>(&scratch->G) : 0;
+            long long g_end = lane == 0 ? *reinterpret_cast<volatile long long*>(&head->G) : 0;
             g_end = __shfl_sync(kFull, g_end, 0);
             count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey && ek <= g_end));
             if (lane < (int)max(count, 1u)) out->e[lane] = make_longlong2((long long)ek, (long long)ei);
@@ -761,18 +770,18 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, Scratch* 
         // draws the last one knows that all lists are there and runs the finalize step.
         __threadfence();
         __syncwarp();
-        if (lane == 0) sh.last_cta = atomicAdd(&scratch->done_ctas, 1u) == grid - 1 ? 1u : 0u;
+        if (lane == 0) sh.last_cta = atomicAdd(&head->done_ctas, 1u) == grid - 1 ? 1u : 0u;
     }
     __syncthreads();
     if (sh.last_cta) {
         __threadfence();
-        finalize_step<OBJ, MODE>(p, lim, sh, scratch, (int)grid, out_best, out_topk);
+        finalize_step<OBJ, MODE>(p, lim, sh, head, partials + blockIdx.y * grid, (int)grid, out_best + blockIdx.y, out_topk);
     }
 }
 
-__global__ void reset_kernel(Scratch* scratch) {
-    scratch->G = kInfKey - 1;
-    scratch->done_ctas = 0;
+__global__ void reset_kernel(SearchHeader* heads) {
+    heads[threadIdx.x].G = kInfKey - 1;
+    heads[threadIdx.x].done_ctas = 0;
 }
 
 // (only the objectives of the Pareto fronts are chained)
@@ -780,8 +789,8 @@ template <int OBJ>
 constexpr int chain_mode() { return OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? kModeSingle : kModeChain; }
 
 template <int OBJ>
-cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, Scratch* scratch, mmee_result_t* out_best,
-                            mmee_result_t* out_topk, cudaStream_t st) {
+cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
+                            mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
     auto* kernel = shape.chain ? (OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? nullptr : search_kernel<OBJ, chain_mode<OBJ>()>)
                    : p.row_pruning ? search_kernel<OBJ, kModePrune>
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
@@ -790,31 +799,31 @@ cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, Scratch* sc
     overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     overlap.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(shape.grid);
+    cfg.gridDim = dim3(shape.grid, shape.n_arrays ? shape.n_arrays : 1u);
     cfg.blockDim = dim3(kSearchThreads);
     cfg.stream = st;
     cfg.attrs = &overlap;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p, shape, scratch, out_best, out_topk);
+    return cudaLaunchKernelEx(&cfg, kernel, p, shape, heads, partials, out_best, out_topk);
 }
 
 }  // namespace
 
 size_t search_smem_bytes() { return sizeof(Shared); }
 
-cudaError_t launch_search(const Plan& p, const LaunchShape& shape, Scratch* scratch, mmee_result_t* out_best,
-                          mmee_result_t* out_topk, cudaStream_t st) {
+cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
+                          mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
     switch (p.objective) {
-        case MMEE_OBJ_ENERGY: return launch_search_t<MMEE_OBJ_ENERGY>(p, shape, scratch, out_best, out_topk, st);
-        case MMEE_OBJ_LATENCY: return launch_search_t<MMEE_OBJ_LATENCY>(p, shape, scratch, out_best, out_topk, st);
-        case MMEE_OBJ_EDP: return launch_search_t<MMEE_OBJ_EDP>(p, shape, scratch, out_best, out_topk, st);
-        case MMEE_OBJ_ENERGY_LCAP: return launch_search_t<MMEE_OBJ_ENERGY_LCAP>(p, shape, scratch, out_best, out_topk, st);
-        default: return launch_search_t<MMEE_OBJ_LATENCY_ECAP>(p, shape, scratch, out_best, out_topk, st);
+        case MMEE_OBJ_ENERGY: return launch_search_t<MMEE_OBJ_ENERGY>(p, shape, heads, partials, out_best, out_topk, st);
+        case MMEE_OBJ_LATENCY: return launch_search_t<MMEE_OBJ_LATENCY>(p, shape, heads, partials, out_best, out_topk, st);
+        case MMEE_OBJ_EDP: return launch_search_t<MMEE_OBJ_EDP>(p, shape, heads, partials, out_best, out_topk, st);
+        case MMEE_OBJ_ENERGY_LCAP: return launch_search_t<MMEE_OBJ_ENERGY_LCAP>(p, shape, heads, partials, out_best, out_topk, st);
+        default: return launch_search_t<MMEE_OBJ_LATENCY_ECAP>(p, shape, heads, partials, out_best, out_topk, st);
     }
 }
 
-cudaError_t launch_reset(Scratch* scratch, cudaStream_t st) {
-    reset_kernel<<<1, 1, 0, st>>>(scratch);
+cudaError_t launch_reset(SearchHeader* heads, int n, cudaStream_t st) {
+    reset_kernel<<<1, n, 0, st>>>(heads);
     return cudaGetLastError();
 }
 

@@ -19,22 +19,31 @@ struct alignas(16) Partial {
     uint64_t feasible_rows;
 };
 
-// Global scratch of one handle: the shared bound (k > 1), the ticket counter and one partial list per CTA.  The
-// header is reset by the finalize step, which also keeps the finished search's counters.
-struct Scratch {
+// What one search's CTAs share: the bound (k > 1) and the ticket counter, reset by the finalize step, which also keeps the
+// finished search's counters.
+struct SearchHeader {
     long long G;                            // upper bound on the k-th smallest key
     unsigned long long last_exact_groups;   // groups of 45 mappings of the winning blocks, evaluated one by one
     unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
     long long chain_bound;                  // what a chained search leaves to the next one; -1: it found nothing
     unsigned int done_ctas;                 // ticket counter: the CTA that draws the last ticket runs the finalize step
     unsigned int pad[7];
+};
+static_assert(sizeof(SearchHeader) == 64, "the header is 64 bytes");
+
+// Global scratch of one handle: a header and one partial list per CTA.
+struct Scratch {
+    SearchHeader head;
     Partial partial[1];     // grid entries follow
 };
-static_assert(offsetof(Scratch, partial) == 64, "the header is 64 bytes");
+
+constexpr uint32_t kMaxArrays = MMEE_MAX_TOPK + 1;
 
 struct LaunchShape {
     uint32_t grid;          // CTAs; CTA c takes one tiling of every `grid` consecutive ones
     uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
+    uint32_t n_arrays;      // logical array shapes searched by one launch (blockIdx.y), 0: the plan's own
+    uint32_t array[kMaxArrays][2];      // their PE rows and columns
     bool chain;             // one of a chain of searches:
     bool chain_read;        // ... not the first
 };
@@ -48,9 +57,11 @@ inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(g
 size_t search_smem_bytes();
 // One launch per search: the last CTA to finish merges the partial lists, evaluates the winners' blocks mapping by
 // mapping, writes the records to out_best / out_topk (device) and resets the scratch header.
-cudaError_t launch_search(const Plan& p, const LaunchShape& shape, Scratch* scratch, mmee_result_t* out_best,
-                          mmee_result_t* out_topk, cudaStream_t st);
-cudaError_t launch_reset(Scratch* scratch, cudaStream_t st);
+// With shape.n_arrays set: that many searches (k = 1), each with a header of its own, partial lists in a row and one
+// record in out_best.
+cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
+                          mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st);
+cudaError_t launch_reset(SearchHeader* heads, int n, cudaStream_t st);
 
 // Every key of the plan's tiling range (kInfKey where a mapping does not fit or its stationary pair is not offered).
 cudaError_t launch_dump_keys(const Plan& p, int64_t* out, cudaStream_t st);
@@ -61,8 +72,9 @@ cudaError_t measure_alu_peak(double* giops);
 
 // Most CTAs that a search on `device` takes.
 int max_search_ctas(int device, uint32_t* out);
-// Launch shape of a search on `device` (at most max_ctas CTAs when that is not 0: MMEE_ERR_RANGE if it would take more).
-int choose_launch_shape(const Plan& p, int device, uint32_t max_ctas, LaunchShape* shape);
+// Launch shape of a search on `device` that shares it with `sharing` - 1 others (at most max_ctas CTAs when that is not 0:
+// MMEE_ERR_RANGE if it would take more).
+int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t max_ctas, LaunchShape* shape);
 
 // MMEE_OK, or MMEE_ERR_CUDA with the error kept for mmee_last_cuda_error (per host thread).
 int cuda_status(cudaError_t e);

@@ -21,7 +21,7 @@ Workspace* g_idle = nullptr;
 int g_n_idle = 0;
 
 int free_workspace(Workspace* ws) {
-    cudaError_t e = ws->scratch ? cudaFree(ws->scratch) : cudaSuccess;
+    cudaError_t e = ws->heads ? cudaFree(ws->heads) : cudaSuccess;
     if (ws->host) {
         const cudaError_t e2 = cudaFreeHost(ws->host);
         if (e == cudaSuccess) e = e2;
@@ -36,14 +36,18 @@ int make_workspace(int device, Workspace** out) {
     ws->device = device;
     int rc = max_search_ctas(device, &ws->max_ctas);
     if (rc) { delete ws; return rc; }
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&ws->scratch), scratch_bytes(ws->max_ctas));
+    // one allocation: the headers of sharing searches, then the scratch (whose own header comes first)
+    unsigned char* mem = nullptr;
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), kMaxArrays * sizeof(SearchHeader) + scratch_bytes(ws->max_ctas));
+    ws->heads = reinterpret_cast<SearchHeader*>(mem);
+    if (e == cudaSuccess) ws->scratch = reinterpret_cast<Scratch*>(mem + kMaxArrays * sizeof(SearchHeader));
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t),
                           cudaHostAllocMapped | cudaHostAllocPortable);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ws->host_dev), ws->host, 0);
-    if (e == cudaSuccess) e = launch_reset(ws->scratch, 0);
+    if (e == cudaSuccess) e = launch_reset(ws->heads, (int)kMaxArrays + 1, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         free_workspace(ws);

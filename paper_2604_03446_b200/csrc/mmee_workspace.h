@@ -8,14 +8,16 @@ namespace mmee {
 // One search's workspace.  Everything a search on the device needs fits it, whatever the problem.
 struct Workspace {
     int device;
-    Scratch* scratch;               // device; its header is clean while the workspace is not in use
+    Scratch* scratch;               // device; its headers are clean while the workspace is not in use
     uint32_t max_ctas;              // partial lists the scratch has room for
+    SearchHeader* heads;            // device, kMaxArrays: headers of searches that share the partial lists; clean as well
     mmee_result_t* host;            // pinned host memory: 1 + MMEE_MAX_TOPK records that kernels write into
     mmee_result_t* host_dev;        // the same memory as the device addresses it
     Workspace* next;
 };
 
 constexpr uint32_t kHostRecords = 1 + MMEE_MAX_TOPK;
+static_assert(kMaxArrays <= kHostRecords, "one record per array shape");
 
 // A workspace on the current device (`device`), for the caller alone until it is given back.
 int workspace_acquire(int device, Workspace** out);

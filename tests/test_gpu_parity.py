@@ -220,6 +220,25 @@ def test_search_shapes_picks_the_best_logical_array():
     assert best_key["shape_flow"] <= best_key["flow"] <= best_key["fixed"]
 
 
+@pytest.mark.parametrize("objective,n_shapes", [(mi.OBJ_EDP, 17), (mi.OBJ_ENERGY, 18), (mi.OBJ_LATENCY, 40)])
+def test_search_shapes_in_several_launches(objective, n_shapes):
+    """Up to 17 shapes share a launch and its CTAs: a full launch, one shape more, and three launches; every shape's
+    record equals the one-shot call on that shape, the first of equal best shapes is reported."""
+    cfg = mi.random_tiny_problem(9)
+    obj = dict(shrink(cfg, dict(cfg["searches"][0], objective=objective, topk=1), 3_000_000), row_pruning=0)
+    shapes = [(1 + (7 * i) % 11, 1 + (5 * i) % 7) for i in range(n_shapes)]
+    per_shape, best = mm.mmee_search_shapes(cfg["workload"], cfg["arch"], obj, shapes)
+    keys = []
+    for (r, c), got in zip(shapes, per_shape):
+        alone = mm.mmee_solve_host(cfg["workload"], dict(cfg["arch"], pe_rows=r, pe_cols=c), obj)[0]
+        assert bytes(got) == bytes(alone)
+        keys.append({mi.OBJ_EDP: got.edp_key, mi.OBJ_ENERGY: got.e_key, mi.OBJ_LATENCY: got.l_key}[objective])
+    assert best == keys.index(min(keys))
+    with pytest.raises(mm.MmeeError) as e:
+        mm.mmee_search_shapes(cfg["workload"], cfg["arch"], obj, [(2, 2), (0, 4)])
+    assert e.value.code == mm.ERR_ARG
+
+
 def test_config1_full_search():
     cfg = mi.config1()
     best, _ = check_search(cfg, cfg["searches"][0])
