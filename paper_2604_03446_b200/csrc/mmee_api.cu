@@ -22,6 +22,7 @@ struct mmee_handle {
     bool dirty;                  // a launch failed half-way: the scratch header is reset before the next search
     bool in_flight;              // a search was launched whose end this handle has not waited for
     bool timing;
+    int flip;                    // the scratch of the last search
     cudaEvent_t ev[2];           // before and after the search kernel
 };
 
@@ -40,6 +41,14 @@ int cuda_status(cudaError_t e) {
     g_last_cuda_error = e;
     return MMEE_ERR_CUDA;
 }
+
+// Searches of at most this many tilings (and those for the k best, which would otherwise wait before their items) wait for
+// the kernel before them in their finalize step only (see mmee_search.cu).  The next search then starts while this one
+// finalizes, not earlier: better while the finalize step is the longer part, worse once the items are.  One energy search
+// after the other, early / late start (us): 4 900 tilings 11.3 / 10.4, 5 929 11.2 / 10.2, 7 056 11.0 to 12.5 / 9.6 to 13.8
+// (edge accelerator at S = 2048, ragged S = 96 on the edge), 8 064 11.5 / 12.1, 10 816 13.5 / 15.4, 18 496 11.4 / 12.2.
+// With register-file tiling the tables take longest: 23.5 / 26.5.
+constexpr uint64_t kLateTilings = 6000;
 
 // Three CTAs per SM hold every register.  One slot is left free: a search that follows another starts while that one's
 // last CTA finalizes, and a CTA that had to wait for its slot would begin its work only then (BERT energy, one search
@@ -70,6 +79,8 @@ int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t ma
     const uint64_t passes = (per_cta + kMaxChunk - 1) / kMaxChunk;
     shape->grid = (uint32_t)grid;
     shape->n_arrays = 0;
+    shape->overlap = true;
+    shape->late = p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling);
     shape->chain = shape->chain_read = false;
     shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
     return MMEE_OK;
@@ -98,8 +109,9 @@ int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found,
         uint32_t n = 0;
         for (; n < batch && rc == MMEE_OK; ++n) {
             shape.chain = true;
+            shape.late = false;
             shape.chain_read = step + n > 0;
-            rc = cuda_status(launch_search(plans[(step + n) % (uint32_t)n_plans], shape, &ws->scratch->head, ws->scratch->partial,
+            rc = cuda_status(launch_search(plans[(step + n) % (uint32_t)n_plans], shape, &ws->scratch[0]->head, ws->scratch[0]->partial,
                                            ws->host_dev + n, nullptr, nullptr));
             if (rc) clean = false;
         }
@@ -155,12 +167,17 @@ static int check_device(const mmee_handle* h) {
 static int search_on(mmee_handle* h, cudaStream_t st, mmee_result_t* out_best, mmee_result_t* out_topk) {
     int rc = check_device(h);
     if (rc) return rc;
-    if (h->dirty) {        // an earlier launch on this handle failed: the header may hold a used ticket counter
-        if ((rc = cuda_status(launch_reset(&h->ws->scratch->head, 1, st)))) return rc;
+    LaunchShape shape = h->shape;
+    if (h->dirty) {        // an earlier launch on this handle failed: a header may hold a used ticket counter
+        for (int i = 0; i < 2; ++i)
+            if ((rc = cuda_status(launch_reset(&h->ws->scratch[i]->head, 1, st)))) return rc;
         h->dirty = false;
+        shape.overlap = false;          // (its CTAs touch the headers: not before the resets have ended)
     }
+    h->flip ^= 1;
+    Scratch* scratch = h->ws->scratch[h->flip];
     if (h->timing) cudaEventRecord(h->ev[0], st);
-    const cudaError_t e = launch_search(h->plan, h->shape, &h->ws->scratch->head, h->ws->scratch->partial, out_best, out_topk, st);
+    const cudaError_t e = launch_search(h->plan, shape, &scratch->head, scratch->partial, out_best, out_topk, st);
     if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
     if (h->timing) cudaEventRecord(h->ev[1], st);
     h->last.kernels_launched = 1;
@@ -381,7 +398,7 @@ int mmee_search_shapes(const mmee_workload_t* workload, const mmee_arch_t* arch,
         if ((rc = choose_launch_shape(plan, device, n, 0, &shape))) break;
         shape.n_arrays = n;
         std::memcpy(shape.array, shapes + 2 * i0, n * sizeof(shape.array[0]));
-        if ((rc = cuda_status(launch_search(plan, shape, ws->heads, ws->scratch->partial, ws->host_dev, nullptr, nullptr)))) clean = false;
+        if ((rc = cuda_status(launch_search(plan, shape, ws->heads, ws->scratch[0]->partial, ws->host_dev, nullptr, nullptr)))) clean = false;
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc2) clean = false;
         if (rc == MMEE_OK) rc = rc2;
@@ -466,7 +483,7 @@ int mmee_last_search_stats(const mmee_handle_t* h, mmee_launch_stats_t* out) {
     out->rows_tested = 0;
     if (h->last.kernels_launched) {
         unsigned long long counters[2] = {0, 0};      // last_exact_groups, last_tested_rows
-        const int rc = cuda_status(cudaMemcpy(counters, &h->ws->scratch->head.last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
+        const int rc = cuda_status(cudaMemcpy(counters, &h->ws->scratch[h->flip]->head.last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
         if (rc) return rc;
         out->exact_path_visits = counters[0];
         out->rows_tested = counters[1];

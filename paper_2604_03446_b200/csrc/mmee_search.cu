@@ -517,11 +517,15 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
 // the search kernel
 // ------------------------------------------------------------------------------------------------
 
-// Searches launched one after the other overlap (programmatic dependent launch): a search's CTAs start as soon as those
-// of the kernel before it on the stream leave room, which is while its last CTA finalizes, and wait for its end before
-// they touch anything but their parameters and shared memory.  A kernel that is not launched this way follows a search
-// as usual, and a search follows one as usual.  Searches one after the other, without and with this (us each): smallest
-// configuration 20.5 and 13.1, BERT energy 22.9 and 18.8, GQA latency 28.7 and 22.7.
+// Searches launched one after the other overlap (programmatic dependent launch), in one of two ways.
+//   early: a search lets the next one start at once; that one's CTAs move in as this one's leave, and wait for its end
+//          before they publish (k > 1, chained: before their items), since it may still use their scratch;
+//   late:  only the CTA that finalizes waits for the kernel before, and lets the next search start after that wait.  The
+//          CTAs then publish while the search before finalizes, into the other one of the handle's two scratches: the
+//          search that used theirs last had ended before the one before them let them start.
+// A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  Searches one after
+// the other, without and with this (us each): smallest configuration 20.5 and 8.9, BERT energy 22.9 and 10.4, GQA latency
+// 28.7 and 13.7, convolution chain top-16 133 and 58 (other changes between them included).
 __device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -547,7 +551,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     SearchHeader* head = heads + blockIdx.y;
-    release_next_kernel();
+    const bool late = shape.late;
+    if (!late) release_next_kernel();
     for (int i = tid; i < (int)(sizeof(sh.order) / 4); i += kSearchThreads)
         reinterpret_cast<uint32_t*>(sh.order)[i] = reinterpret_cast<const uint32_t*>(p.order)[i];
     if (PRUNE)
@@ -652,7 +657,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         }
         if (MULTI && m0 == 0) {
             // (k > 1 shares a bound through the scratch while it works on the items)
-            wait_previous_kernel();
+            if (!late) wait_previous_kernel();
             if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
         }
         if (CHAIN && shape.chain_read && m0 == 0) {
@@ -741,7 +746,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)ek, (long long)ei);
         __syncthreads();
     }
-    wait_previous_kernel();     // from here on the scratch and the result records are touched
+    if (!late) wait_previous_kernel();      // from here on the scratch is touched
     if (warp == 0) {
         Partial* out = &partials[blockIdx.y * grid + blockIdx.x];
         uint32_t count;
@@ -774,6 +779,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     }
     __syncthreads();
     if (sh.last_cta) {
+        if (late) {
+            wait_previous_kernel();         // from here on the result records are touched
+            release_next_kernel();
+        }
         __threadfence();
         finalize_step<OBJ, MODE>(p, lim, sh, head, partials + blockIdx.y * grid, (int)grid, out_best + blockIdx.y, out_topk);
     }
@@ -803,7 +812,7 @@ cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeade
     cfg.blockDim = dim3(kSearchThreads);
     cfg.stream = st;
     cfg.attrs = &overlap;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = shape.overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, p, shape, heads, partials, out_best, out_topk);
 }
 

@@ -44,6 +44,8 @@ struct LaunchShape {
     uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
     uint32_t n_arrays;      // logical array shapes searched by one launch (blockIdx.y), 0: the plan's own
     uint32_t array[kMaxArrays][2];      // their PE rows and columns
+    bool overlap;           // may start before the kernel before it on the stream has ended (see mmee_search.cu)
+    bool late;              // ... and its CTAs wait for that end in the finalize step only
     bool chain;             // one of a chain of searches:
     bool chain_read;        // ... not the first
 };

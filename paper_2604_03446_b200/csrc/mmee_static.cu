@@ -60,6 +60,7 @@ extern "C" int mmee_search_static(const mmee_workload_t* workload, const mmee_ar
     // The same launch shape as a handle would get, bounded by what the fixed scratch can hold.
     LaunchShape shape;
     if ((rc = choose_launch_shape(plan, device, 1, kStaticMaxCtas, &shape))) return rc;
+    shape.overlap = false;      // its CTAs touch the scratch without a wait for the reset below
     Scratch* scratch = nullptr;
     if ((rc = static_scratch(device, &scratch))) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
