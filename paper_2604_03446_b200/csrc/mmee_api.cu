@@ -50,14 +50,15 @@ int cuda_status(cudaError_t e) {
 // With register-file tiling the tables take longest: 23.5 / 26.5.
 constexpr uint64_t kLateTilings = 6000;
 
-// Three CTAs per SM hold every register.  One slot is left free: a search that follows another starts while that one's
+// Two CTAs per SM (118 registers a thread, no spills) beat three (80, spilled) and four (64): GQA latency 13.0, 13.7 and
+// 15.1 us, BERT energy 9.4, 10.4 and 12.6, convolution chain top-16 52, 58 and 65.  One slot is left free: a search that follows another starts while that one's
 // last CTA finalizes, and a CTA that had to wait for its slot would begin its work only then (BERT energy, one search
 // after the other: 16.4 us with all slots taken, 11.6 us with one left; GQA latency 20.1 and 13.7).
 int max_search_ctas(int device, uint32_t* out) {
     int sm_count = 0;      // attribute query: cudaGetDeviceProperties costs milliseconds
     const cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return cuda_status(e);
-    *out = 3u * (uint32_t)sm_count - 1u;
+    *out = 2u * (uint32_t)sm_count - 1u;
     return MMEE_OK;
 }
 

@@ -544,7 +544,7 @@ __device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, cons
 }
 
 template <int OBJ, int MODE>
-__global__ void __launch_bounds__(kSearchThreads, 3)
+__global__ void __launch_bounds__(kSearchThreads, 2)
 search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ heads, Partial* __restrict__ partials,
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;

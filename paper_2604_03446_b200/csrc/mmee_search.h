@@ -9,7 +9,7 @@
 namespace mmee {
 
 constexpr int kSearchThreads = 256;
-constexpr uint32_t kMaxChunk = 96;      // tilings whose tables a CTA holds at once
+constexpr uint32_t kMaxChunk = 144;     // tilings whose tables a CTA holds at once
 
 // One CTA's contribution: its k best blocks as (least key, block number) pairs, best first, and its counts.
 struct alignas(16) Partial {
