@@ -46,7 +46,7 @@ __device__ __forceinline__ void block_item(const Plan& p, const Divisors& dv, ui
     const uint32_t t = id / p.n_blocks, block = id - t * p.n_blocks;
     const uint32_t phi = p.block_phi[block], slot = p.block_order_slot[block], order = p.order_id[slot];
     uint32_t b[8];
-    tiling_bounds(p, t, b);
+    tiling_bounds(p, dv, t, b);
     if (item < 25) {
         const int x = item / 5, l = item % 5;
         bt->size[x][l] = sat_size((uint64_t)monomial(p.q.bs[order][x][l], b));

@@ -47,6 +47,7 @@ struct PlanDivisors {
     __device__ __forceinline__ uint32_t rows() const { return p.pe_rows; }
     __device__ __forceinline__ uint32_t cols() const { return p.pe_cols; }
     __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return p.divs[d][i]; }
+    __device__ __forceinline__ uint32_t cofactor(int d, uint32_t i) const { return p.dim[d] / p.divs[d][i]; }
     __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_rows - 1) / p.pe_rows; }
     __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_cols - 1) / p.pe_cols; }
 };
@@ -145,16 +146,16 @@ __device__ __forceinline__ TilingCounts tiling_counts(const Plan& p, const uint3
 }
 
 // Tiling index -> boundary vector b (one column of the boundary matrix, Section VI-A).
-__device__ __forceinline__ void tiling_bounds(const Plan& p, uint64_t t64, uint32_t b[8]) {
+template <class Divisors>
+__device__ __forceinline__ void tiling_bounds(const Plan& p, const Divisors& dv, uint64_t t64, uint32_t b[8]) {
     uint32_t t = (uint32_t)t64;                 // at most MMEE_MAX_DIVISORS^4 = 2^24 tilings
 #pragma unroll
     for (int d = 3; d >= 0; --d) {
-        const uint32_t q = t / p.ndiv[d];
+        const uint32_t q = p.ndiv_inv[d] ? __umulhi(t, p.ndiv_inv[d]) : t;        // t / ndiv
         const uint32_t a = t - q * p.ndiv[d];
         t = q;
-        const uint32_t g = p.divs[d][a];
-        b[4 + d] = g;
-        b[d] = p.dim[d] / g;
+        b[4 + d] = dv.div(d, a);
+        b[d] = dv.cofactor(d, a);
     }
 }
 
@@ -317,7 +318,7 @@ __device__ __forceinline__ void assemble_record(const Plan& p, uint64_t idx, con
 __device__ inline void evaluate_candidate(const Plan& p, uint64_t idx, mmee_result_t& o) {
     const CandidateChoice d = decode_candidate(p, idx);
     uint32_t b[8];
-    tiling_bounds(p, d.t, b);
+    tiling_bounds(p, PlanDivisors{p}, d.t, b);
     const TilingCounts tt = tiling_counts(p, b);
     int64_t bs[5], da[5];
     for (int x = 0; x < 5; ++x) operand_terms(p, d, b, x, bs[x], da[x]);
@@ -336,7 +337,7 @@ __device__ inline void evaluate_candidate_lanes(const Plan& p, const Divisors& d
                                                 bool write, mmee_result_t& o) {
     const CandidateChoice d = decode_candidate(p, idx);
     uint32_t b[8];
-    tiling_bounds(p, d.t, b);
+    tiling_bounds(p, dv, d.t, b);
     const TilingCounts tt = tiling_counts(p, b);
     const int l = lane & (WIDTH - 1);
     int64_t v0 = 0, v1 = 0;

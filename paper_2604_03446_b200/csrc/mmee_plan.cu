@@ -211,6 +211,10 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
         for (uint32_t i = 0; i < nlo; ++i) p->divs[d][n++] = lo[i];
         for (uint32_t i = nhi; i-- > 0;) p->divs[d][n++] = hi[i];
         p->ndiv[d] = n;
+        // (u * ceil(2^32 / n) / 2^32 exceeds u / n by less than 2^24 / 2^32 < 1 / n for n <= MMEE_MAX_DIVISORS, so that
+        // the integer part is the quotient)
+        p->ndiv_inv[d] = n > 1 ? (uint32_t)((((uint64_t)1 << 32) + n - 1) / n) : 0u;
+        if ((uint64_t)p->divs[d][0] * p->divs[d][n - 1] == dims[d]) p->mirrored |= 1u << d;
         p->n_tilings *= n;
     }
 

@@ -58,6 +58,8 @@ struct alignas(4) KeptMasks {
 struct Plan {
     uint32_t dim[4];              // I, K, L, J of one instance
     uint32_t ndiv[4];
+    uint32_t ndiv_inv[4];         // ceil(2^32 / ndiv), for quotients by ndiv of numbers below 2^24 (0 when ndiv is 1)
+    uint32_t mirrored;            // bit d: the divisor list of dimension d holds all divisors: cofactors in descending order
     uint32_t instances, n_arrays;
     uint32_t n_orders;            // orders in the search, in row order
     uint32_t order_id[kMaxOrders];

@@ -120,6 +120,7 @@ struct Shared {
     OrderInfo order[kMaxOrders];
     KeptMasks kept;
     uint32_t divs[4][MMEE_MAX_DIVISORS];
+    uint32_t cofactors[4][MMEE_MAX_DIVISORS];       // dimension / divisor
     uint32_t pe_rows, pe_cols;      // the array's logical shape
     uint32_t row_folds[4][MMEE_MAX_DIVISORS], col_folds[4][MMEE_MAX_DIVISORS];      // register-file tiling only
     alignas(16) longlong2 tops[kWarps][MMEE_MAX_TOPK];
@@ -142,6 +143,7 @@ struct SharedDivisors {       // see PlanDivisors
     __device__ __forceinline__ uint32_t rows() const { return sh.pe_rows; }
     __device__ __forceinline__ uint32_t cols() const { return sh.pe_cols; }
     __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
+    __device__ __forceinline__ uint32_t cofactor(int d, uint32_t i) const { return sh.cofactors[d][i]; }
     __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return sh.row_folds[d][i]; }
     __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return sh.col_folds[d][i]; }
 };
@@ -564,6 +566,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) {
         const int d = tid >> 6, i = tid & 63;
         sh.divs[d][i] = p.divs[d][i];
+        sh.cofactors[d][i] = (p.mirrored >> d) & 1u ? p.divs[d][p.ndiv[d] - 1 - i] : p.dim[d] / p.divs[d][i];
         if (p.rf_tiling) {
             sh.row_folds[d][i] = (p.divs[d][i] + pe_rows - 1) / pe_rows;
             sh.col_folds[d][i] = (p.divs[d][i] + pe_cols - 1) / pe_cols;
@@ -629,15 +632,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             bool live = mine && rel < n_tilings;
             if (live) {
                 t = (uint32_t)(p.t_begin + rel);
-                uint32_t u = t;
-#pragma unroll
-                for (int d = 3; d >= 0; --d) {
-                    const uint32_t v = u / p.ndiv[d];
-                    const uint32_t g = sh.divs[d][u - v * p.ndiv[d]];
-                    u = v;
-                    b[4 + d] = g;
-                    b[d] = p.dim[d] / g;
-                }
+                tiling_bounds(p, SharedDivisors{sh}, t, b);
                 // With every operand at L3 the buffer need is smallest: max(A+B+C, C+D+E) tiles (Eq. 1-4).
                 const uint64_t ta = (uint64_t)b[4] * b[5], tbb = (uint64_t)b[5] * b[6], tc = (uint64_t)b[4] * b[6];
                 const uint64_t td = (uint64_t)b[6] * b[7], te = (uint64_t)b[4] * b[7];
