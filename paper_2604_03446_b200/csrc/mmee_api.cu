@@ -83,6 +83,7 @@ int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t ma
     shape->overlap = true;
     shape->late = p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling);
     shape->chain = shape->chain_read = false;
+    shape->chain_to = nullptr;
     shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
     return MMEE_OK;
 }
@@ -92,7 +93,7 @@ int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t ma
 namespace {
 
 // Searches chained on the device (see LaunchShape::chain), step i with plans[i % n_plans], until one finds nothing: their
-// records in order, through `take` (which returns false to stop), and their number.  The host waits for a batch of them at a time, first
+// optima in order, through `take` (which returns false to stop), and their number.  The host waits for a batch of them at a time, first
 // `first_batch`, then twice as many as before; what is launched beyond the last one ends at once.
 template <class Take>
 int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found, Take take) {
@@ -112,10 +113,12 @@ int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found,
             shape.chain = true;
             shape.late = false;
             shape.chain_read = step + n > 0;
+            shape.chain_to = ws->chain + n;
             rc = cuda_status(launch_search(plans[(step + n) % (uint32_t)n_plans], shape, &ws->scratch[0]->head, ws->scratch[0]->partial,
-                                           ws->host_dev + n, nullptr, nullptr));
-            if (rc) clean = false;
+                                           nullptr, nullptr, nullptr));
         }
+        if (rc == MMEE_OK) rc = cuda_status(launch_resolve(plans[n_plans - 1], ws->chain, n, step, n_plans > 1, ws->host_dev, nullptr));
+        if (rc) clean = false;
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc2) clean = false;
         if (rc == MMEE_OK) rc = rc2;

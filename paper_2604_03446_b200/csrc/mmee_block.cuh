@@ -112,6 +112,15 @@ __device__ __forceinline__ RowTerms block_row(const Plan& p, const Limits& lim, 
     if (bt.phi == 0) return row_terms(p, lim, bt, (int)(row / 625u), (int)(row / 125u % 5u), (int)(row / 25u % 5u), d, e);
     return row_terms(p, lim, bt, (int)(row / 125u), (int)(row / 25u % 5u), 0, d, e);
 }
+// Buffer words that row `row` of the block needs (Eq. 4).  Exact for a row that fits.
+__device__ __forceinline__ int64_t block_need(const BlockTab& bt, uint32_t row) {
+    const int e = (int)(row % 5u), d = (int)(row / 5u % 5u);
+    const bool fused = bt.phi == 0;
+    const int c = fused ? (int)(row / 25u % 5u) : 0, a = (int)(fused ? row / 625u : row / 125u), b = (int)(fused ? row / 125u % 5u : row / 25u % 5u);
+    const int64_t A = bt.size[0][a], B = bt.size[1][b], C = bt.size[2][c], D = bt.size[3][d], E = bt.size[4][e];
+    if (!fused) return max64(A + B + C, C + D + E);
+    return max64(A + B + C + (d ? D : 0) + (e ? E : 0), C + D + E + (a ? A : 0) + (b ? B : 0));
+}
 __device__ __forceinline__ uint32_t block_rows(const BlockTab& bt) { return bt.phi == 0 ? 3125u : 625u; }
 
 }  // namespace mmee

@@ -315,6 +315,31 @@ __device__ __forceinline__ void min_over_warps(Shared& sh, int lane, int warp, i
     warp_min_pair(ek, ei);
 }
 
+// What the kernels look up in shared memory, by all threads of a CTA (the caller synchronises).
+template <bool PRUNE>
+__device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uint32_t pe_cols, Shared& sh) {
+    const int tid = threadIdx.x;
+    for (int i = tid; i < (int)(sizeof(sh.order) / 4); i += kSearchThreads)
+        reinterpret_cast<uint32_t*>(sh.order)[i] = reinterpret_cast<const uint32_t*>(p.order)[i];
+    if (PRUNE)
+        for (int i = tid; i < (int)(sizeof(KeptMasks) / 4); i += kSearchThreads)
+            reinterpret_cast<uint32_t*>(&sh.kept)[i] = reinterpret_cast<const uint32_t*>(&p.kept)[i];
+    static_assert(kSearchThreads == 4 * MMEE_MAX_DIVISORS, "one thread per divisor");
+    if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) {
+        const int d = tid >> 6, i = tid & 63;
+        sh.divs[d][i] = p.divs[d][i];
+        sh.cofactors[d][i] = (p.mirrored >> d) & 1u ? p.divs[d][p.ndiv[d] - 1 - i] : p.dim[d] / p.divs[d][i];
+        if (p.rf_tiling) {
+            sh.row_folds[d][i] = (p.divs[d][i] + pe_rows - 1) / pe_rows;
+            sh.col_folds[d][i] = (p.divs[d][i] + pe_cols - 1) / pe_cols;
+        }
+    }
+    if (tid == 0) {
+        sh.pe_rows = pe_rows;
+        sh.pe_cols = pe_cols;
+    }
+}
+
 // The items of a block's tables (block_item), their three kinds on three warps.
 __device__ __forceinline__ int split_item(int warp, int lane) {
     return warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (warp == 2 && lane == 0 ? 31 : -1));
@@ -322,7 +347,7 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
 
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
 template <int OBJ, int MODE>
-__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, SearchHeader* __restrict__ head,
+__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to, SearchHeader* __restrict__ head,
                                            const Partial* __restrict__ partials, int n_partials,
                                            mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -380,6 +405,16 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         min_over_warps(sh, lane, warp, ek, ei);
         found = ek != kInfKey ? 1 : 0;
         bound = ek;
+        constexpr bool kBlockOnly = MODE == kModeChain && OBJ != MMEE_OBJ_ENERGY;
+        if (MODE == kModeChain && tid == 0) {
+            unsigned long long fit = 0;
+            for (int w = 0; w < kWarps; ++w) fit += sh.feasible_rows[w];
+            *chain_to = {(long long)ek, (unsigned long long)ei, fit * p.n_sm, (long long)(kBlockOnly ? lim.key_cap : lim.cap_words)};
+            // the next search's bound: this energy / one word less of latency
+            if (kBlockOnly || !found) head->chain_bound = !found ? -1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? ek : ek - 1);
+            head->done_ctas = 0;
+        }
+        if (kBlockOnly) return;
         // ---- the winning block, mapping by mapping
         const int item = split_item(warp, lane);
         if (found && item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)ei, item, &sh.block[0]);
@@ -389,6 +424,14 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
             best_of_block<OBJ>(p, lim, sh, bound, ek, ei);
         }
         min_over_warps(sh, lane, warp, ek, ei);
+        if (MODE == kModeChain) {
+            // energy: the mapping itself, and one word of buffer less than it needs for the next search
+            if (tid == 0 && found) {
+                chain_to->where = ei;
+                head->chain_bound = block_need(sh.block[0], (uint32_t)((ei - sh.block[0].first_idx) / 9u)) - 1;
+            }
+            return;
+        }
     } else {
         merge_warps(sh, k, lane, warp, ek, ei);
         const longlong2 e = lane < kTopK ? sh.tops[0][lane] : make_longlong2(kInfKey, -1ll);
@@ -483,10 +526,6 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
             unsigned long long* to = reinterpret_cast<unsigned long long*>(&out_topk[rec]);
             for (int i = l; i < kWords; i += kLanes) to[i] = from[i];
         }
-        if (MODE == kModeChain && tid == 0) {
-            // the next search's bound: one word less of buffer / this energy / one word less of latency
-            head->chain_bound = n_out == 0 ? -1 : (OBJ == MMEE_OBJ_ENERGY ? r.bs - 1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? r.e_key : r.l_key - 1));
-        }
     }
     __syncthreads();
     if (warp == 0) {
@@ -555,29 +594,12 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     SearchHeader* head = heads + blockIdx.y;
     const bool late = shape.late;
     if (!late) release_next_kernel();
-    for (int i = tid; i < (int)(sizeof(sh.order) / 4); i += kSearchThreads)
-        reinterpret_cast<uint32_t*>(sh.order)[i] = reinterpret_cast<const uint32_t*>(p.order)[i];
-    if (PRUNE)
-        for (int i = tid; i < (int)(sizeof(KeptMasks) / 4); i += kSearchThreads)
-            reinterpret_cast<uint32_t*>(&sh.kept)[i] = reinterpret_cast<const uint32_t*>(&p.kept)[i];
-    const uint32_t pe_rows = shape.n_arrays ? shape.array[blockIdx.y][0] : p.pe_rows;
-    const uint32_t pe_cols = shape.n_arrays ? shape.array[blockIdx.y][1] : p.pe_cols;
-    static_assert(kSearchThreads == 4 * MMEE_MAX_DIVISORS, "one thread per divisor");
-    if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) {
-        const int d = tid >> 6, i = tid & 63;
-        sh.divs[d][i] = p.divs[d][i];
-        sh.cofactors[d][i] = (p.mirrored >> d) & 1u ? p.divs[d][p.ndiv[d] - 1 - i] : p.dim[d] / p.divs[d][i];
-        if (p.rf_tiling) {
-            sh.row_folds[d][i] = (p.divs[d][i] + pe_rows - 1) / pe_rows;
-            sh.col_folds[d][i] = (p.divs[d][i] + pe_cols - 1) / pe_cols;
-        }
-    }
+    load_shared<PRUNE>(p, shape.n_arrays ? shape.array[blockIdx.y][0] : p.pe_rows,
+                       shape.n_arrays ? shape.array[blockIdx.y][1] : p.pe_cols, sh);
     if (tid == 0) {
         sh.n_live = 0;
         sh.cursor = 0;
         sh.check_failed = 0;
-        sh.pe_rows = pe_rows;
-        sh.pe_cols = pe_cols;
     }
     __syncthreads();
 
@@ -591,7 +613,6 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     const uint32_t n_orders = p.n_orders;
     auto any = [](bool v) { return __any_sync(kFull, v) != 0; };
 
-    bool ended = false;
     // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
@@ -664,10 +685,12 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             } else {
                 lim.key_cap = bound;
             }
-            ended = bound < 0;
+            if (bound < 0) {            // the search before found nothing: neither does this one, nor the next
+                if (blockIdx.x == 0 && tid == 0) *shape.chain_to = {kInfKey, 0, 0, -1};
+                return;
+            }
         }
         __syncthreads();
-        if (CHAIN && ended) break;       // the search before found nothing: neither does this one
 
         const uint32_t per_class = sh.n_live * n_orders;
         if (tid == 0) my_live += sh.n_live;
@@ -779,7 +802,56 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             release_next_kernel();
         }
         __threadfence();
-        finalize_step<OBJ, MODE>(p, lim, sh, head, partials + blockIdx.y * grid, (int)grid, out_best + blockIdx.y, out_topk);
+        finalize_step<OBJ, MODE>(p, lim, sh, shape.chain_to, head, partials + blockIdx.y * grid, (int)grid, out_best + blockIdx.y, out_topk);
+    }
+}
+
+template <int OBJ>
+__global__ void __launch_bounds__(kSearchThreads, 2)
+resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* __restrict__ chain, uint32_t first_step, bool odd_only,
+               mmee_result_t* __restrict__ out) {
+    __shared__ Shared sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const ChainRecord c = chain[blockIdx.x];
+    const bool full = c.key != kInfKey && (!odd_only || ((first_step + blockIdx.x) & 1u));
+    mmee_result_t& r = sh.record[0];
+    if (full) {
+        load_shared<false>(p, p.pe_rows, p.pe_cols, sh);
+        __syncthreads();
+        const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
+        int64_t ek = c.key;
+        uint64_t ei = c.where;
+        if (OBJ != MMEE_OBJ_ENERGY) {
+            const int item = split_item(warp, lane);
+            if (item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)c.where, item, &sh.block[0]);
+            __syncthreads();
+            best_of_block<OBJ>(p, lim, sh, c.key, ek, ei);
+            min_over_warps(sh, lane, warp, ek, ei);
+        }
+        if (warp == 0) {
+            const bool have = ek == c.key;
+            evaluate_candidate_lanes<32>(p, SharedDivisors{sh}, have ? ei : 0, lim.cap_words, lane, lane == 0, r);
+            if (lane == 0) {
+                r.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
+                r.n_feasible = c.n_feasible;
+                if (!(have && key_of<OBJ>(r.e_key, r.l_key, lim.key_cap) == c.key && r.feasible && r.t >= p.t_begin && r.t < p.t_end))
+                    r.status = MMEE_ERR_CHECK;
+            }
+        }
+    } else if (warp == 0) {
+        unsigned long long* raw = reinterpret_cast<unsigned long long*>(&r);
+        for (int i = lane; i < (int)(sizeof(r) / 8); i += 32) raw[i] = 0;
+        __syncwarp();
+        if (lane == 0 && c.key == kInfKey) {
+            r.idx = MMEE_NO_INDEX;
+            r.status = MMEE_ERR_NO_FEASIBLE;
+        }
+    }
+    if (warp == 0) {
+        __syncwarp();
+        const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
+        unsigned long long* to = reinterpret_cast<unsigned long long*>(&out[blockIdx.x]);
+        for (int i = lane; i < (int)(sizeof(r) / 8); i += 32) to[i] = from[i];
     }
 }
 
@@ -824,6 +896,16 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
         case MMEE_OBJ_ENERGY_LCAP: return launch_search_t<MMEE_OBJ_ENERGY_LCAP>(p, shape, heads, partials, out_best, out_topk, st);
         default: return launch_search_t<MMEE_OBJ_LATENCY_ECAP>(p, shape, heads, partials, out_best, out_topk, st);
     }
+}
+
+cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, uint32_t first_step, bool odd_only,
+                           mmee_result_t* out, cudaStream_t st) {
+    switch (p.objective) {
+        case MMEE_OBJ_ENERGY: resolve_kernel<MMEE_OBJ_ENERGY><<<n, kSearchThreads, 0, st>>>(p, chain, first_step, odd_only, out); break;
+        case MMEE_OBJ_LATENCY_ECAP: resolve_kernel<MMEE_OBJ_LATENCY_ECAP><<<n, kSearchThreads, 0, st>>>(p, chain, first_step, odd_only, out); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_reset(SearchHeader* heads, int n, cudaStream_t st) {

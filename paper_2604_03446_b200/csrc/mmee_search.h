@@ -39,6 +39,15 @@ struct Scratch {
 
 constexpr uint32_t kMaxArrays = MMEE_MAX_TOPK + 1;
 
+// What a chained search leaves of its optimum: the key (kInfKey: nothing fits), the mapping's index (energy) or the block
+// that holds it (capped objectives), the mappings that fit, and the bound it was found under.
+struct ChainRecord {
+    long long key;
+    unsigned long long where;
+    unsigned long long n_feasible;
+    long long bound;
+};
+
 struct LaunchShape {
     uint32_t grid;          // CTAs; CTA c takes one tiling of every `grid` consecutive ones
     uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
@@ -48,11 +57,14 @@ struct LaunchShape {
     bool late;              // ... and its CTAs wait for that end in the finalize step only
     bool chain;             // one of a chain of searches:
     bool chain_read;        // ... not the first
+    ChainRecord* chain_to;  // device: where it leaves its optimum
 };
 // Chained searches (k = 1, no row pruning; the Pareto fronts): each takes a bound from what the one before it on the
 // stream found, on the device, so that the host waits once for several: the buffer words (energy) or the bound on the
 // other key (capped objectives) come from the scratch instead of the plan (and are not above the plan's), and the bound
-// for the next search is left there.  After a search that found nothing the others end at once.
+// for the next search is left there.  After a search that found nothing the others end at once.  A chained search writes
+// no record but a ChainRecord: the next one has to wait for its end, and the records of all can be made side by side
+// afterwards (launch_resolve).
 
 inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 
@@ -63,6 +75,10 @@ size_t search_smem_bytes();
 // record in out_best.
 cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
                           mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st);
+// Full records of the optima that n chained searches left, one CTA each; those with an odd number only (`odd_only`; the
+// others' records say no more than whether something was found).
+cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, uint32_t first_step, bool odd_only,
+                           mmee_result_t* out, cudaStream_t st);
 cudaError_t launch_reset(SearchHeader* heads, int n, cudaStream_t st);
 
 // Every key of the plan's tiling range (kInfKey where a mapping does not fit or its stationary pair is not offered).

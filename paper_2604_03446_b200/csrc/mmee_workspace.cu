@@ -36,11 +36,13 @@ int make_workspace(int device, Workspace** out) {
     ws->device = device;
     int rc = max_search_ctas(device, &ws->max_ctas);
     if (rc) { delete ws; return rc; }
-    // one allocation: the headers of sharing searches, then the two scratches
-    const size_t heads = kMaxArrays * sizeof(SearchHeader), bytes = scratch_bytes(ws->max_ctas);
+    // one allocation: the headers of sharing searches and the chained searches' optima, then the two scratches
+    static_assert(sizeof(ChainRecord) == 32, "a multiple of 16 bytes keeps the scratches aligned");
+    const size_t heads = kMaxArrays * sizeof(SearchHeader) + kHostRecords * sizeof(ChainRecord), bytes = scratch_bytes(ws->max_ctas);
     unsigned char* mem = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), heads + 2 * bytes);
     ws->heads = reinterpret_cast<SearchHeader*>(mem);
+    ws->chain = reinterpret_cast<ChainRecord*>(mem + kMaxArrays * sizeof(SearchHeader));
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + heads + i * bytes);
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation

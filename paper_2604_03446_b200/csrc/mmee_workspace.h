@@ -11,6 +11,7 @@ struct Workspace {
     Scratch* scratch[2];            // device; headers are clean while the workspace is not in use.  Two, for a search that
                                     // publishes while the one before it on the handle still finalizes
     uint32_t max_ctas;              // partial lists a scratch has room for
+    ChainRecord* chain;             // device, kHostRecords: what chained searches left
     SearchHeader* heads;            // device, kMaxArrays: headers of searches that share the partial lists; clean as well
     mmee_result_t* host;            // pinned host memory: 1 + MMEE_MAX_TOPK records that kernels write into
     mmee_result_t* host_dev;        // the same memory as the device addresses it
