@@ -40,6 +40,14 @@ __device__ __forceinline__ void stationary_terms(const Plan& p, const Divisors& 
     Q = calls * cy * (int64_t)p.bw;
 }
 
+// Index of the first mapping of block `id` = tiling * n_blocks + block.
+__device__ __forceinline__ uint64_t block_first_idx(const Plan& p, uint32_t id) {
+    const uint32_t t = id / p.n_blocks, block = id - t * p.n_blocks;
+    const uint32_t fused_rows = p.n_fused_blocks * 3125u;
+    const uint32_t row0 = block < p.n_fused_blocks ? block * 3125u : fused_rows + (block - p.n_fused_blocks) * 625u;
+    return ((uint64_t)t * p.rows_per_tiling + row0) * 9u;
+}
+
 // Item `item` (0 .. kBlockItems - 1) of the tables of block `id` = tiling * n_blocks + block.
 template <class Divisors>
 __device__ __forceinline__ void block_item(const Plan& p, const Divisors& dv, uint32_t id, int item, BlockTab* bt) {
@@ -69,9 +77,7 @@ __device__ __forceinline__ void block_item(const Plan& p, const Divisors& dv, ui
         bt->jD = b[LOOP_J];
         bt->c_write = il;
         bt->pass = phi == 2 ? 2 * il : 0;
-        const uint32_t fused_rows = p.n_fused_blocks * 3125u;
-        const uint32_t row0 = block < p.n_fused_blocks ? block * 3125u : fused_rows + (block - p.n_fused_blocks) * 625u;
-        bt->first_idx = ((uint64_t)t * p.rows_per_tiling + row0) * 9u;
+        bt->first_idx = block_first_idx(p, id);
     }
 }
 

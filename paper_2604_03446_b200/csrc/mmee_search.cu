@@ -227,62 +227,71 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits&
         const Rep q = decode_rep(o, fused, r < n_reps ? r : 0u);
         const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
         const uint32_t first_row = row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
-        int64_t hk = -1;                        // the lane's next mapping: key, index
-        uint64_t hi = UINT64_MAX;
+        int64_t hk = -1;                        // the lane's next mapping: key, index relative to the block's first
+        uint32_t off = 0;
         uint32_t pairs = 0, left = 0;           // stationary pairs with that key, those left of the row
         uint32_t row = 0;                       // the row, and where its levels stand within their classes
         int at[5] = {0, 0, 0, 0, 0};
-        auto next = [&]() {
-            left &= left - 1u;
-            if (!left) {
-                bool more = pairs != 0;
-                if (more) {
-                    more = false;               // the next row of the combination: its levels count up, E's fastest
-                    int stride = 1;
-#pragma unroll
-                    for (int x = 4; x >= 0; --x) {
-                        if (!fused && x == OP_C) continue;
-                        if (!more) {
-                            more = ++at[x] < q.width[x];
-                            row += (uint32_t)(more ? stride : -stride * (q.width[x] - 1));
-                            if (!more) at[x] = 0;
-                        }
-                        stride *= 5;
-                    }
-                }
-                if (!more) {                    // the next larger key
-                    const int64_t last = hk;
-                    hk = kInfKey;
-                    pairs = 0;
-                    for (int s = 0; s < 9; ++s) {
-                        const int64_t key = mapping_key<OBJ>(p, lim, bt, t, s);
-                        if (!((p.sm_mask >> s) & 1u) || key <= last || key > hk) continue;
-                        pairs = key < hk ? 1u << s : pairs | 1u << s;
-                        hk = key;
-                    }
-                    row = first_row;
-                    if (hk > bound) { hk = kInfKey; hi = UINT64_MAX; return; }
-                }
-                left = pairs;
-            }
-            hi = bt.first_idx + row * 9u + (uint32_t)(__ffs(left) - 1);
-        };
-        if (r < n_reps && t.fits) next();
-        else hk = kInfKey;
         // (every warp's k-th pair bounds the block's: a torn view is impossible, a pair is one 16-byte word)
         const longlong2 other = ld_volatile(&sh.kth[lane & (kWarps - 1)]);
         int64_t ok = other.x, nk = kInfKey;
         uint64_t oi = (uint64_t)other.y, ni = UINT64_MAX;
         warp_min_pair(ok, oi);
         if (pair_less(ok, oi, lk, li)) { lk = ok; li = oi; }
+        bool advance = r < n_reps && t.fits;
+        if (!advance) hk = kInfKey;
+        int64_t level = -1;                     // the key whose mappings are being taken
 #pragma unroll 1
-        for (int i = 0; i < k; ++i) {
-            int64_t bk = hk;
-            uint64_t bi = hi;
-            warp_min_pair(bk, bi);
-            if (!pair_less(bk, bi, lk, li)) break;
-            if (lane == i) { nk = bk; ni = bi; }
-            if (hi == bi) next();
+        for (int i = 0; i < k;) {
+            if (advance) {
+                left &= left - 1u;
+                if (!left) {
+                    bool more = false;
+                    if (pairs) {                // the next row of the combination: its levels count up, E's fastest
+                        int stride = 1;
+#pragma unroll
+                        for (int x = 4; x >= 0; --x) {
+                            if (!fused && x == OP_C) continue;
+                            if (!more) {
+                                more = ++at[x] < q.width[x];
+                                row += (uint32_t)(more ? stride : -stride * (q.width[x] - 1));
+                                if (!more) at[x] = 0;
+                            }
+                            stride *= 5;
+                        }
+                    }
+                    if (!more) {                // the next larger key
+                        const int64_t last = hk;
+                        hk = kInfKey;
+                        pairs = 0;
+                        for (int s = 0; s < 9; ++s) {
+                            const int64_t key = mapping_key<OBJ>(p, lim, bt, t, s);
+                            if (!((p.sm_mask >> s) & 1u) || key <= last || key > hk) continue;
+                            pairs = key < hk ? 1u << s : pairs | 1u << s;
+                            hk = key;
+                        }
+                        row = first_row;
+                        if (hk > bound) hk = kInfKey;
+                    }
+                    left = pairs;
+                }
+                off = row * 9u + (uint32_t)(__ffs(left) - 1);
+            }
+            // the lowest index among the lanes whose next mapping has the current key; without one, the next key
+            uint32_t mine = hk == level ? off : 0xffffffffu;
+            uint32_t least = __reduce_min_sync(kFull, mine);
+            if (least == 0xffffffffu) {
+                const uint32_t kh = __reduce_min_sync(kFull, (uint32_t)((uint64_t)hk >> 32));
+                const uint32_t kl = __reduce_min_sync(kFull, (uint32_t)((uint64_t)hk >> 32) == kh ? (uint32_t)hk : 0xffffffffu);
+                level = (int64_t)(((uint64_t)kh << 32) | kl);
+                if (level == kInfKey) break;
+                mine = hk == level ? off : 0xffffffffu;
+                least = __reduce_min_sync(kFull, mine);
+            }
+            if (!pair_less(level, bt.first_idx + least, lk, li)) break;
+            if (lane == i) { nk = level; ni = bt.first_idx + least; }
+            advance = mine == least;
+            ++i;
         }
         reg_merge(ek, ei, k, nk, ni, lane);
         if (lane == k - 1) sh.kth[threadIdx.x >> 5] = make_longlong2((long long)ek, (long long)ei);
@@ -452,6 +461,10 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         bool more = true;
         for (int j0 = 0; more && j0 < n_fresh; j0 += j0 ? kWarps : 1) {
             const int n_batch = j0 ? min(kWarps, n_fresh - j0) : 1;
+            const int next = __ffs(m) - 1;
+            const int64_t next_key = __shfl_sync(kFull, e.x, next);
+            const uint32_t next_id = (uint32_t)__shfl_sync(kFull, e.y, next);
+            if (!pair_less(next_key, block_first_idx(p, next_id), lk, li)) break;
             int64_t bk[kWarps];
 #pragma unroll
             for (int j = 0; j < kWarps; ++j) {
