@@ -62,7 +62,7 @@ int max_search_ctas(int device, uint32_t* out) {
     return MMEE_OK;
 }
 
-int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t max_ctas, LaunchShape* shape) {
+int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape) {
     uint32_t most = 0;
     const int rc = max_search_ctas(device, &most);
     if (rc) return rc;
@@ -70,18 +70,18 @@ int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t ma
     const uint64_t tilings = p.t_end - p.t_begin;
     constexpr uint64_t kMinTilings = 8;
     uint64_t grid = (tilings + kMinTilings - 1) / kMinTilings;
-    if (sharing > 1 && most > sharing) most /= sharing;
     if (grid > most) grid = most;
     if (!grid) grid = 1;
     // (a caller with a fixed scratch: a device that would take more CTAs is refused, not silently under-used)
     if (max_ctas && grid > max_ctas) return MMEE_ERR_RANGE;
     // Passes of equal length, as few as the tables allow.
     const uint64_t per_cta = (tilings + grid - 1) / grid;
-    const uint64_t passes = (per_cta + kMaxChunk - 1) / kMaxChunk;
+    const uint32_t chunk = search_chunk(n_arrays);
+    const uint64_t passes = (per_cta + chunk - 1) / chunk;
     shape->grid = (uint32_t)grid;
-    shape->n_arrays = 0;
+    shape->n_arrays = n_arrays;
     shape->overlap = true;
-    shape->late = p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling);
+    shape->late = n_arrays == 0 && (p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling));
     shape->chain = shape->chain_read = false;
     shape->chain_to = nullptr;
     shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
@@ -101,7 +101,7 @@ int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found,
     int rc = cuda_status(cudaGetDevice(&device));
     if (rc) return rc;
     LaunchShape shape;
-    if ((rc = choose_launch_shape(plans[0], device, 1, 0, &shape))) return rc;
+    if ((rc = choose_launch_shape(plans[0], device, 0, 0, &shape))) return rc;
     Workspace* ws = nullptr;
     if ((rc = workspace_acquire(device, &ws))) return rc;
     bool clean = true, more = true;
@@ -151,7 +151,7 @@ int mmee_create(const mmee_workload_t* workload, const mmee_arch_t* arch, const 
     if ((rc = cuda_status(cudaGetDevice(&h->device)))) { delete h; return rc; }
     h->kept_rows = h->plan.rows_per_tiling;
     if (h->plan.row_pruning && (rc = set_kept_masks(&h->plan, &h->kept_rows))) { delete h; return rc; }
-    rc = choose_launch_shape(h->plan, h->device, 1, 0, &h->shape);
+    rc = choose_launch_shape(h->plan, h->device, 0, 0, &h->shape);
     if (rc) { delete h; return rc; }
     if ((rc = workspace_acquire(h->device, &h->ws))) { delete h; return rc; }
     h->create_ms = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -174,7 +174,7 @@ static int search_on(mmee_handle* h, cudaStream_t st, mmee_result_t* out_best, m
     LaunchShape shape = h->shape;
     if (h->dirty) {        // an earlier launch on this handle failed: a header may hold a used ticket counter
         for (int i = 0; i < 2; ++i)
-            if ((rc = cuda_status(launch_reset(&h->ws->scratch[i]->head, 1, st)))) return rc;
+            if ((rc = cuda_status(launch_reset(&h->ws->scratch[i]->head, st)))) return rc;
         h->dirty = false;
         shape.overlap = false;          // (its CTAs touch the headers: not before the resets have ended)
     }
@@ -387,9 +387,9 @@ int mmee_search_shapes(const mmee_workload_t* workload, const mmee_arch_t* arch,
     int64_t best_key = 0;
     for (uint32_t i = 0; i < n_shapes; ++i)
         if (!shapes[2 * i] || !shapes[2 * i + 1]) return MMEE_ERR_ARG;
-    // Shapes differ in nothing but the array's rows and columns: up to kMaxArrays of them are searched by one launch,
-    // each on its share of the CTAs, so that they merge and evaluate their winners at the same time.  (One launch per
-    // shape: 180 us for eleven shapes of the BERT-base chain, each waiting for the one before; now 103 us.)
+    // Shapes differ in nothing but the array's rows and columns, so that which rows fit and what they fetch is found once
+    // for up to kMaxArrays of them; only the stationary-pair terms and the keys are formed per shape.  (Eleven shapes of
+    // the BERT-base chain: one launch per shape 180 us, one launch with a share of the CTAs for each 94 us, this 57 us.)
     mmee_arch_t a = *arch;
     a.pe_rows = shapes[0];
     a.pe_cols = shapes[1];
@@ -400,9 +400,8 @@ int mmee_search_shapes(const mmee_workload_t* workload, const mmee_arch_t* arch,
         const uint32_t n = n_shapes - i0 < kMaxArrays ? n_shapes - i0 : kMaxArrays;
         LaunchShape shape;
         if ((rc = choose_launch_shape(plan, device, n, 0, &shape))) break;
-        shape.n_arrays = n;
         std::memcpy(shape.array, shapes + 2 * i0, n * sizeof(shape.array[0]));
-        if ((rc = cuda_status(launch_search(plan, shape, ws->heads, ws->scratch[0]->partial, ws->host_dev, nullptr, nullptr)))) clean = false;
+        if ((rc = cuda_status(launch_search_arrays(plan, shape, ws->scratch[0]->partial, ws->host_dev, nullptr)))) clean = false;
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc2) clean = false;
         if (rc == MMEE_OK) rc = rc2;

@@ -25,14 +25,18 @@ namespace mmee {
 constexpr int kSizeCap = (1 << 30) - 1;        // buffer sizes saturate here, above every admissible capacity
 constexpr int64_t kNoRow = INT64_C(1) << 62;   // DRAM words of "no row fits"; sums of words stay below 2^62
 
+// Stationary-pair terms of one tiling, linear in the recomputation factor rho of C (j_D or 1): energy P1[sm1] * rho + P2[sm2]
+// (buffer<->PE words, MACs, softmax), compute words Q1[sm1] * rho + Q2[sm2].
+struct StatTerms {
+    int64_t P1[3], P2[3], Q1[3], Q2[3];
+};
+
 // What a CTA keeps of one tiling, shared by its orders and classes.
 struct TileTab {
     int32_t  size[kSizeSlots];      // buffer words, saturated to kSizeCap
     uint32_t t;                     // tiling index
     uint32_t b[8];                  // bounds i_D, k_D, l_D, j_D, i_G, k_G, l_G, j_G
-    // Stationary-pair terms, linear in the recomputation factor rho of C (j_D or 1):
-    //   energy P1[sm1] * rho + P2[sm2] (buffer<->PE words, MACs, softmax), compute words Q1[sm1] * rho + Q2[sm2]
-    int64_t  P1[3], P2[3], Q1[3], Q2[3];
+    StatTerms st;
 };
 
 // Whole operands, the same for every tiling.
@@ -229,33 +233,32 @@ MMEE_HD int64_t unfused_key(int64_t x1, int64_t x2, int64_t pass, int64_t P1, in
 // Least key over the offered stationary pairs (sm_mask bit 3 * sm1 + sm2).  With all nine offered the energy and the
 // latency separate into the operators' own minima.
 template <int OBJ>
-MMEE_HD int64_t fused_least_key(const TileTab& tb, int64_t x, bool rc, uint32_t sm_mask, int64_t c_dram, int64_t cap) {
-    const int64_t rho = rc ? (int64_t)tb.b[LOOP_J] : 1;
+MMEE_HD int64_t fused_least_key(const StatTerms& st, int64_t x, int64_t rho, uint32_t sm_mask, int64_t c_dram, int64_t cap) {
     if ((OBJ == MMEE_OBJ_ENERGY || OBJ == MMEE_OBJ_LATENCY) && sm_mask == 0x1ffu) {
-        const int64_t* u = OBJ == MMEE_OBJ_ENERGY ? tb.P1 : tb.Q1;
-        const int64_t* v = OBJ == MMEE_OBJ_ENERGY ? tb.P2 : tb.Q2;
+        const int64_t* u = OBJ == MMEE_OBJ_ENERGY ? st.P1 : st.Q1;
+        const int64_t* v = OBJ == MMEE_OBJ_ENERGY ? st.P2 : st.Q2;
         const int64_t w = min64(u[0], min64(u[1], u[2])) * rho + min64(v[0], min64(v[1], v[2]));
         return OBJ == MMEE_OBJ_ENERGY ? c_dram * x + w : max64(x, w);
     }
     int64_t best = kInfKey;
 #pragma unroll
     for (int s = 0; s < 9; ++s) {
-        const int64_t k = fused_key<OBJ>(x, rho, tb.P1[s / 3], tb.P2[s % 3], tb.Q1[s / 3], tb.Q2[s % 3], c_dram, cap);
+        const int64_t k = fused_key<OBJ>(x, rho, st.P1[s / 3], st.P2[s % 3], st.Q1[s / 3], st.Q2[s % 3], c_dram, cap);
         best = ((sm_mask >> s) & 1u) ? min64(best, k) : best;
     }
     return best;
 }
 template <int OBJ>
-MMEE_HD int64_t unfused_least_key(const TileTab& tb, int64_t x1, int64_t x2, int64_t pass, uint32_t sm_mask, int64_t c_dram,
+MMEE_HD int64_t unfused_least_key(const StatTerms& st, int64_t x1, int64_t x2, int64_t pass, uint32_t sm_mask, int64_t c_dram,
                                   int64_t cap) {
     if (OBJ == MMEE_OBJ_ENERGY && sm_mask == 0x1ffu)
-        return c_dram * (x1 + x2 + pass) + min64(tb.P1[0], min64(tb.P1[1], tb.P1[2])) + min64(tb.P2[0], min64(tb.P2[1], tb.P2[2]));
+        return c_dram * (x1 + x2 + pass) + min64(st.P1[0], min64(st.P1[1], st.P1[2])) + min64(st.P2[0], min64(st.P2[1], st.P2[2]));
     if (OBJ == MMEE_OBJ_LATENCY && sm_mask == 0x1ffu)
-        return max64(x1, min64(tb.Q1[0], min64(tb.Q1[1], tb.Q1[2]))) + pass + max64(x2, min64(tb.Q2[0], min64(tb.Q2[1], tb.Q2[2])));
+        return max64(x1, min64(st.Q1[0], min64(st.Q1[1], st.Q1[2]))) + pass + max64(x2, min64(st.Q2[0], min64(st.Q2[1], st.Q2[2])));
     int64_t best = kInfKey;
 #pragma unroll
     for (int s = 0; s < 9; ++s) {
-        const int64_t k = unfused_key<OBJ>(x1, x2, pass, tb.P1[s / 3], tb.P2[s % 3], tb.Q1[s / 3], tb.Q2[s % 3], c_dram, cap);
+        const int64_t k = unfused_key<OBJ>(x1, x2, pass, st.P1[s / 3], st.P2[s % 3], st.Q1[s / 3], st.Q2[s % 3], c_dram, cap);
         best = ((sm_mask >> s) & 1u) ? min64(best, k) : best;
     }
     return best;

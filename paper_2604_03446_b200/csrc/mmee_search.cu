@@ -28,8 +28,9 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = kSearchThreads / 32;
 constexpr int kTopK = (int)MMEE_MAX_TOPK;
-// One optimum; one optimum over the rows kept by symbolic pruning; the k best; one optimum of a chain of searches.
-constexpr int kModeSingle = 0, kModePrune = 1, kModeMulti = 2, kModeChain = 3;
+// One optimum; one optimum over the rows kept by symbolic pruning; the k best; one optimum of a chain of searches;
+// one optimum for each of several array shapes.
+constexpr int kModeSingle = 0, kModePrune = 1, kModeMulti = 2, kModeChain = 3, kModeArrays = 4;
 
 // ------------------------------------------------------------------------------------------------
 // (key, number) pairs
@@ -324,6 +325,16 @@ __device__ __forceinline__ void min_over_warps(Shared& sh, int lane, int warp, i
     warp_min_pair(ek, ei);
 }
 
+struct ArrayDivisors {        // the same with another array's rows and columns
+    const Shared& sh;
+    uint32_t pe_rows, pe_cols;
+    __device__ __forceinline__ uint32_t rows() const { return pe_rows; }
+    __device__ __forceinline__ uint32_t cols() const { return pe_cols; }
+    __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
+    __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return (sh.divs[d][i] + pe_rows - 1) / pe_rows; }
+    __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return (sh.divs[d][i] + pe_cols - 1) / pe_cols; }
+};
+
 // What the kernels look up in shared memory, by all threads of a CTA (the caller synchronises).
 template <bool PRUNE>
 __device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uint32_t pe_cols, Shared& sh) {
@@ -585,13 +596,14 @@ __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepco
 
 // The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
 // and the sizes between them.
+template <bool TERMS>
 __device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
-    if (sub < 6) {
+    if (TERMS && sub < 6) {
         const int op = sub >= 3 ? 1 : 0, sm = sub - 3 * op;
         int64_t P, Q;
         stationary_terms(p, SharedDivisors{sh}, b, op, sm, P, Q);
-        (op ? tb->P2 : tb->P1)[sm] = P;
-        (op ? tb->Q2 : tb->Q1)[sm] = Q;
+        (op ? tb->st.P2 : tb->st.P1)[sm] = P;
+        (op ? tb->st.Q2 : tb->st.Q1)[sm] = Q;
     }
     for (int i = sub; i < kSizeSlots; i += 8) tb->size[i] = sat_size(size_words(p.dim, tb->b + 4, i));
     if (sub == 7) tb->t = t;
@@ -599,16 +611,19 @@ __device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, cons
 
 template <int OBJ, int MODE>
 __global__ void __launch_bounds__(kSearchThreads, 2)
-search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ heads, Partial* __restrict__ partials,
+search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ head, Partial* __restrict__ partials,
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
+    constexpr bool ARRAYS = MODE == kModeArrays;
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    SearchHeader* head = heads + blockIdx.y;
     const bool late = shape.late;
     if (!late) release_next_kernel();
-    load_shared<PRUNE>(p, shape.n_arrays ? shape.array[blockIdx.y][0] : p.pe_rows,
-                       shape.n_arrays ? shape.array[blockIdx.y][1] : p.pe_cols, sh);
+    load_shared<PRUNE>(p, p.pe_rows, p.pe_cols, sh);
+    // Array shapes: the stationary-pair terms of shape y and tiling slot i at [y * chunk + i], behind the tilings' tables;
+    // the warps' best items of shape y in sh.tops[.][y].
+    StatTerms* terms = reinterpret_cast<StatTerms*>(&sh.tile[shape.chunk]);
+    if (ARRAYS && tid < kWarps * (int)MMEE_MAX_TOPK) sh.tops[tid / (int)MMEE_MAX_TOPK][tid % (int)MMEE_MAX_TOPK] = make_longlong2(kInfKey, -1ll);
     if (tid == 0) {
         sh.n_live = 0;
         sh.cursor = 0;
@@ -649,6 +664,21 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         }
     };
 
+    // The same for every array shape, one after the other: key_of_terms(terms) is the item's least key.
+    auto offer_arrays = [&](auto key_of_terms, uint32_t slot, uint32_t id, bool valid) {
+        for (uint32_t y = 0; y < shape.n_arrays; ++y) {
+            const int64_t key = key_of_terms(terms[y * shape.chunk + slot]);
+            const longlong2 own = sh.tops[warp][y];
+            const bool better = valid && pair_less(key, id, own.x, (uint64_t)own.y);
+            if (!any(better)) continue;
+            int64_t nk = better ? key : kInfKey;
+            uint64_t ni = better ? id : UINT64_MAX;
+            warp_min_pair(nk, ni);
+            if (lane == 0) sh.tops[warp][y] = make_longlong2((long long)nk, (long long)ni);
+            __syncwarp();
+        }
+    };
+
     // Tiling number m of this CTA is one of the m-th `grid` consecutive ones, a different one in every round (a fixed
     // one would be the same divisor of the last dimension again and again).
     for (uint32_t m0 = 0; (uint64_t)m0 * grid < n_tilings; m0 += shape.chunk) {
@@ -682,7 +712,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 sh.tile[slot].b[tid & 7] = own;
             }
             __syncwarp();
-            if (live) build_tile(p, sh, b, t, tid & 7, &sh.tile[slot]);
+            if (live) build_tile<!ARRAYS>(p, sh, b, t, tid & 7, &sh.tile[slot]);
         }
         if (MULTI && m0 == 0) {
             // (k > 1 shares a bound through the scratch while it works on the items)
@@ -704,6 +734,19 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             }
         }
         __syncthreads();
+        if (ARRAYS) {
+            const uint32_t n_live = sh.n_live;
+            for (uint32_t i = tid; i < n_live * 6u * shape.n_arrays; i += kSearchThreads) {
+                const uint32_t y = i / (n_live * 6u), u = i - y * n_live * 6u, slot = u / 6u;
+                const int op = u - slot * 6u >= 3u ? 1 : 0, sm = (int)(u - slot * 6u) - 3 * op;
+                StatTerms& st = terms[y * shape.chunk + slot];
+                int64_t P, Q;
+                stationary_terms(p, ArrayDivisors{sh, shape.array[y][0], shape.array[y][1]}, sh.tile[slot].b, op, sm, P, Q);
+                (op ? st.P2 : st.P1)[sm] = P;
+                (op ? st.Q2 : st.Q1)[sm] = Q;
+            }
+            __syncthreads();
+        }
 
         const uint32_t per_class = sh.n_live * n_orders;
         if (tid == 0) my_live += sh.n_live;
@@ -738,8 +781,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 if (valid) my_rows += rows;
                 const bool some = valid && x < kNoRow;
                 if (any(some)) {
-                    const int64_t key = fused_least_key<OBJ>(tb, some ? x : 0, oi.recompute[c] != 0, p.sm_mask, p.c_dram_gb, lim.key_cap);
-                    offer(key, id, some);
+                    const int64_t y = some ? x : 0, rho = oi.recompute[c] != 0 ? (int64_t)tb.b[LOOP_J] : 1;
+                    auto key = [&](const StatTerms& t) { return fused_least_key<OBJ>(t, y, rho, p.sm_mask, p.c_dram_gb, lim.key_cap); };
+                    if (ARRAYS) offer_arrays(key, slot, id, some);
+                    else offer(key(tb.st), id, some);
                 }
             } else {
                 uint32_t fit1, fit2, rows;
@@ -758,8 +803,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                             if ((fit1 >> ab) & 1u) rows += (uint32_t)__popc(fit2 & sh.kept.unfused[phi - 1][os][ab]);
                     }
                     if (some) my_rows += rows;
-                    const int64_t key = unfused_least_key<OBJ>(tb, y1, y2, phi == 2 ? 2 * dw.il : 0, p.sm_mask, p.c_dram_gb, lim.key_cap);
-                    offer(key, id + block, some);
+                    const int64_t pass = phi == 2 ? 2 * dw.il : 0;
+                    auto key = [&](const StatTerms& t) { return unfused_least_key<OBJ>(t, y1, y2, pass, p.sm_mask, p.c_dram_gb, lim.key_cap); };
+                    if (ARRAYS) offer_arrays(key, slot, id + block, some);
+                    else offer(key(tb.st), id + block, some);
                     block += n_orders;
                 }
             }
@@ -772,14 +819,32 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     if (lane == 0) sh.feasible_rows[warp] = my_rows;
     if (MULTI) {
         merge_warps(sh, k, lane, warp, ek, ei);
-    } else {
+    } else if (!ARRAYS) {
         warp_min_pair(ek, ei);
         if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)ek, (long long)ei);
         __syncthreads();
     }
     if (!late) wait_previous_kernel();      // from here on the scratch is touched
+    if (ARRAYS) {
+        // the best item of every shape; the kernel that follows merges them (resolve_arrays_kernel)
+        __syncthreads();
+        Partial* out = &partials[blockIdx.x];
+        for (uint32_t y = warp; y < shape.n_arrays; y += kWarps) {
+            const longlong2 v = sh.tops[lane & (kWarps - 1)][y];
+            int64_t nk = v.x;
+            uint64_t ni = (uint64_t)v.y;
+            warp_min_pair(nk, ni);
+            if (lane == 0) out->e[y] = make_longlong2((long long)nk, (long long)ni);
+        }
+        if (tid == 0) {
+            unsigned long long rows = 0;
+            for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
+            out->feasible_rows = rows;
+        }
+        return;
+    }
     if (warp == 0) {
-        Partial* out = &partials[blockIdx.y * grid + blockIdx.x];
+        Partial* out = &partials[blockIdx.x];
         uint32_t count;
         if (MULTI) {
             // an entry above the bound (some full list's last key) is not among the k best
@@ -815,7 +880,60 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             release_next_kernel();
         }
         __threadfence();
-        finalize_step<OBJ, MODE>(p, lim, sh, shape.chain_to, head, partials + blockIdx.y * grid, (int)grid, out_best + blockIdx.y, out_topk);
+        finalize_step<OBJ, MODE>(p, lim, sh, shape.chain_to, head, partials, (int)grid, out_best, out_topk);
+    }
+}
+
+__global__ void reset_kernel(SearchHeader* head) {
+    head->G = kInfKey - 1;
+    head->done_ctas = 0;
+}
+
+// The full record of an optimum, by one CTA: mapping `where`, or (IN_BLOCK) the first mapping with key `key` of block
+// `where`.  key kInfKey: nothing fits.
+template <int OBJ, bool IN_BLOCK>
+__device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim, uint32_t pe_rows, uint32_t pe_cols, Shared& sh,
+                                               int64_t key, uint64_t where, unsigned long long n_feasible, mmee_result_t* out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    mmee_result_t& r = sh.record[0];
+    if (key != kInfKey) {
+        load_shared<false>(p, pe_rows, pe_cols, sh);
+        __syncthreads();
+        int64_t ek = key;
+        uint64_t ei = where;
+        if (IN_BLOCK) {
+            const int item = split_item(warp, lane);
+            if (item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)where, item, &sh.block[0]);
+            __syncthreads();
+            best_of_block<OBJ>(p, lim, sh, key, ek, ei);
+            min_over_warps(sh, lane, warp, ek, ei);
+        }
+        if (warp == 0) {
+            const bool have = ek == key;
+            evaluate_candidate_lanes<32>(p, SharedDivisors{sh}, have ? ei : 0, lim.cap_words, lane, lane == 0, r);
+            if (lane == 0) {
+                const int64_t own = OBJ == MMEE_OBJ_EDP ? __double_as_longlong(r.edp_key) : key_of<OBJ>(r.e_key, r.l_key, lim.key_cap);
+                if (!(have && own == key && r.feasible && r.t >= p.t_begin && r.t < p.t_end)) r.status = MMEE_ERR_CHECK;
+            }
+        }
+    } else if (warp == 0) {
+        unsigned long long* raw = reinterpret_cast<unsigned long long*>(&r);
+        for (int i = lane; i < (int)(sizeof(r) / 8); i += 32) raw[i] = 0;
+        __syncwarp();
+        if (lane == 0) {
+            r.idx = MMEE_NO_INDEX;
+            r.status = MMEE_ERR_NO_FEASIBLE;
+        }
+    }
+    if (warp == 0) {
+        if (lane == 0) {
+            r.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
+            r.n_feasible = n_feasible;
+        }
+        __syncwarp();
+        const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
+        unsigned long long* to = reinterpret_cast<unsigned long long*>(out);
+        for (int i = lane; i < (int)(sizeof(r) / 8); i += 32) to[i] = from[i];
     }
 }
 
@@ -824,53 +942,41 @@ __global__ void __launch_bounds__(kSearchThreads, 2)
 resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* __restrict__ chain, uint32_t first_step, bool odd_only,
                mmee_result_t* __restrict__ out) {
     __shared__ Shared sh;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const ChainRecord c = chain[blockIdx.x];
-    const bool full = c.key != kInfKey && (!odd_only || ((first_step + blockIdx.x) & 1u));
-    mmee_result_t& r = sh.record[0];
-    if (full) {
-        load_shared<false>(p, p.pe_rows, p.pe_cols, sh);
-        __syncthreads();
-        const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
-        int64_t ek = c.key;
-        uint64_t ei = c.where;
-        if (OBJ != MMEE_OBJ_ENERGY) {
-            const int item = split_item(warp, lane);
-            if (item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)c.where, item, &sh.block[0]);
-            __syncthreads();
-            best_of_block<OBJ>(p, lim, sh, c.key, ek, ei);
-            min_over_warps(sh, lane, warp, ek, ei);
+    if (c.key != kInfKey && odd_only && !((first_step + blockIdx.x) & 1u)) {
+        if (threadIdx.x == 0) {         // (the host asks of this one only whether something was found)
+            out[blockIdx.x].idx = 0;
+            out[blockIdx.x].status = MMEE_OK;
         }
-        if (warp == 0) {
-            const bool have = ek == c.key;
-            evaluate_candidate_lanes<32>(p, SharedDivisors{sh}, have ? ei : 0, lim.cap_words, lane, lane == 0, r);
-            if (lane == 0) {
-                r.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
-                r.n_feasible = c.n_feasible;
-                if (!(have && key_of<OBJ>(r.e_key, r.l_key, lim.key_cap) == c.key && r.feasible && r.t >= p.t_begin && r.t < p.t_end))
-                    r.status = MMEE_ERR_CHECK;
-            }
-        }
-    } else if (warp == 0) {
-        unsigned long long* raw = reinterpret_cast<unsigned long long*>(&r);
-        for (int i = lane; i < (int)(sizeof(r) / 8); i += 32) raw[i] = 0;
-        __syncwarp();
-        if (lane == 0 && c.key == kInfKey) {
-            r.idx = MMEE_NO_INDEX;
-            r.status = MMEE_ERR_NO_FEASIBLE;
-        }
+        return;
     }
-    if (warp == 0) {
-        __syncwarp();
-        const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
-        unsigned long long* to = reinterpret_cast<unsigned long long*>(&out[blockIdx.x]);
-        for (int i = lane; i < (int)(sizeof(r) / 8); i += 32) to[i] = from[i];
-    }
+    const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
+    resolve_record<OBJ, OBJ != MMEE_OBJ_ENERGY>(p, lim, p.pe_rows, p.pe_cols, sh, c.key, c.where, c.n_feasible, out + blockIdx.x);
 }
 
-__global__ void reset_kernel(SearchHeader* heads) {
-    heads[threadIdx.x].G = kInfKey - 1;
-    heads[threadIdx.x].done_ctas = 0;
+// Merge of the CTAs' best items of array shape blockIdx.x, and the record of the optimum.
+template <int OBJ>
+__global__ void __launch_bounds__(kSearchThreads, 2)
+resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, const Partial* __restrict__ partials,
+                      mmee_result_t* __restrict__ out) {
+    __shared__ Shared sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t ek = kInfKey;
+    uint64_t ei = UINT64_MAX;
+    unsigned long long rows = 0;
+    for (uint32_t c = tid; c < shape.grid; c += kSearchThreads) {
+        const longlong2 v = partials[c].e[blockIdx.x];
+        rows += partials[c].feasible_rows;
+        if (pair_less(v.x, (uint64_t)v.y, ek, ei)) { ek = v.x; ei = (uint64_t)v.y; }
+    }
+    for (int off = 16; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+    if (lane == 0) sh.feasible_rows[warp] = rows;
+    warp_min_pair(ek, ei);
+    min_over_warps(sh, lane, warp, ek, ei);
+    rows = 0;
+    for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
+    resolve_record<OBJ, true>(p, Limits{p.cap_words, p.key_cap}, shape.array[blockIdx.x][0], shape.array[blockIdx.x][1], sh, ek, ei,
+                              rows * p.n_sm, out + blockIdx.x);
 }
 
 // (only the objectives of the Pareto fronts are chained)
@@ -878,9 +984,10 @@ template <int OBJ>
 constexpr int chain_mode() { return OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? kModeSingle : kModeChain; }
 
 template <int OBJ>
-cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
+cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials,
                             mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
-    auto* kernel = shape.chain ? (OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? nullptr : search_kernel<OBJ, chain_mode<OBJ>()>)
+    auto* kernel = shape.n_arrays ? search_kernel<OBJ, kModeArrays>
+                   : shape.chain ? (OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? nullptr : search_kernel<OBJ, chain_mode<OBJ>()>)
                    : p.row_pruning ? search_kernel<OBJ, kModePrune>
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
     if (!kernel) return cudaErrorInvalidValue;
@@ -888,26 +995,26 @@ cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeade
     overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     overlap.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(shape.grid, shape.n_arrays ? shape.n_arrays : 1u);
+    cfg.gridDim = dim3(shape.grid);
     cfg.blockDim = dim3(kSearchThreads);
     cfg.stream = st;
     cfg.attrs = &overlap;
     cfg.numAttrs = shape.overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, p, shape, heads, partials, out_best, out_topk);
+    return cudaLaunchKernelEx(&cfg, kernel, p, shape, head, partials, out_best, out_topk);
 }
 
 }  // namespace
 
 size_t search_smem_bytes() { return sizeof(Shared); }
 
-cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
+cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials,
                           mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
     switch (p.objective) {
-        case MMEE_OBJ_ENERGY: return launch_search_t<MMEE_OBJ_ENERGY>(p, shape, heads, partials, out_best, out_topk, st);
-        case MMEE_OBJ_LATENCY: return launch_search_t<MMEE_OBJ_LATENCY>(p, shape, heads, partials, out_best, out_topk, st);
-        case MMEE_OBJ_EDP: return launch_search_t<MMEE_OBJ_EDP>(p, shape, heads, partials, out_best, out_topk, st);
-        case MMEE_OBJ_ENERGY_LCAP: return launch_search_t<MMEE_OBJ_ENERGY_LCAP>(p, shape, heads, partials, out_best, out_topk, st);
-        default: return launch_search_t<MMEE_OBJ_LATENCY_ECAP>(p, shape, heads, partials, out_best, out_topk, st);
+        case MMEE_OBJ_ENERGY: return launch_search_t<MMEE_OBJ_ENERGY>(p, shape, head, partials, out_best, out_topk, st);
+        case MMEE_OBJ_LATENCY: return launch_search_t<MMEE_OBJ_LATENCY>(p, shape, head, partials, out_best, out_topk, st);
+        case MMEE_OBJ_EDP: return launch_search_t<MMEE_OBJ_EDP>(p, shape, head, partials, out_best, out_topk, st);
+        case MMEE_OBJ_ENERGY_LCAP: return launch_search_t<MMEE_OBJ_ENERGY_LCAP>(p, shape, head, partials, out_best, out_topk, st);
+        default: return launch_search_t<MMEE_OBJ_LATENCY_ECAP>(p, shape, head, partials, out_best, out_topk, st);
     }
 }
 
@@ -921,8 +1028,26 @@ cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_reset(SearchHeader* heads, int n, cudaStream_t st) {
-    reset_kernel<<<1, n, 0, st>>>(heads);
+uint32_t search_chunk(uint32_t n_arrays) {
+    return (uint32_t)(kMaxChunk * sizeof(TileTab) / (sizeof(TileTab) + n_arrays * sizeof(StatTerms)));
+}
+
+cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partial* partials, mmee_result_t* out, cudaStream_t st) {
+    const cudaError_t e = launch_search(p, shape, nullptr, partials, nullptr, nullptr, st);
+    if (e != cudaSuccess) return e;
+    const unsigned n = shape.n_arrays;
+    switch (p.objective) {
+        case MMEE_OBJ_ENERGY: resolve_arrays_kernel<MMEE_OBJ_ENERGY><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
+        case MMEE_OBJ_LATENCY: resolve_arrays_kernel<MMEE_OBJ_LATENCY><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
+        case MMEE_OBJ_EDP: resolve_arrays_kernel<MMEE_OBJ_EDP><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
+        case MMEE_OBJ_ENERGY_LCAP: resolve_arrays_kernel<MMEE_OBJ_ENERGY_LCAP><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
+        default: resolve_arrays_kernel<MMEE_OBJ_LATENCY_ECAP><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reset(SearchHeader* head, cudaStream_t st) {
+    reset_kernel<<<1, 1, 0, st>>>(head);
     return cudaGetLastError();
 }
 

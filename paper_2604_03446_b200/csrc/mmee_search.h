@@ -37,7 +37,7 @@ struct Scratch {
     Partial partial[1];     // grid entries follow
 };
 
-constexpr uint32_t kMaxArrays = MMEE_MAX_TOPK + 1;
+constexpr uint32_t kMaxArrays = MMEE_MAX_TOPK;      // one entry of a partial list each
 
 // What a chained search leaves of its optimum: the key (kInfKey: nothing fits), the mapping's index (energy) or the block
 // that holds it (capped objectives), the mappings that fit, and the bound it was found under.
@@ -51,7 +51,7 @@ struct ChainRecord {
 struct LaunchShape {
     uint32_t grid;          // CTAs; CTA c takes one tiling of every `grid` consecutive ones
     uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
-    uint32_t n_arrays;      // logical array shapes searched by one launch (blockIdx.y), 0: the plan's own
+    uint32_t n_arrays;      // logical array shapes searched by one launch, 0: the plan's own
     uint32_t array[kMaxArrays][2];      // their PE rows and columns
     bool overlap;           // may start before the kernel before it on the stream has ended (see mmee_search.cu)
     bool late;              // ... and its CTAs wait for that end in the finalize step only
@@ -69,17 +69,19 @@ struct LaunchShape {
 inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 
 size_t search_smem_bytes();
+// Tilings whose tables a CTA holds at once, with the stationary-pair terms of n_arrays array shapes.
+uint32_t search_chunk(uint32_t n_arrays);
 // One launch per search: the last CTA to finish merges the partial lists, evaluates the winners' blocks mapping by
 // mapping, writes the records to out_best / out_topk (device) and resets the scratch header.
-// With shape.n_arrays set: that many searches (k = 1), each with a header of its own, partial lists in a row and one
-// record in out_best.
-cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* heads, Partial* partials,
+cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials,
                           mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st);
+// The same search (k = 1) on each of shape.n_arrays logical arrays, one record each in `out`: two launches.
+cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partial* partials, mmee_result_t* out, cudaStream_t st);
 // Full records of the optima that n chained searches left, one CTA each; those with an odd number only (`odd_only`; the
 // others' records say no more than whether something was found).
 cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, uint32_t first_step, bool odd_only,
                            mmee_result_t* out, cudaStream_t st);
-cudaError_t launch_reset(SearchHeader* heads, int n, cudaStream_t st);
+cudaError_t launch_reset(SearchHeader* head, cudaStream_t st);
 
 // Every key of the plan's tiling range (kInfKey where a mapping does not fit or its stationary pair is not offered).
 cudaError_t launch_dump_keys(const Plan& p, int64_t* out, cudaStream_t st);
@@ -90,9 +92,9 @@ cudaError_t measure_alu_peak(double* giops);
 
 // Most CTAs that a search on `device` takes.
 int max_search_ctas(int device, uint32_t* out);
-// Launch shape of a search on `device` that shares it with `sharing` - 1 others (at most max_ctas CTAs when that is not 0:
-// MMEE_ERR_RANGE if it would take more).
-int choose_launch_shape(const Plan& p, int device, uint32_t sharing, uint32_t max_ctas, LaunchShape* shape);
+// Launch shape of a search of n_arrays array shapes (0: the plan's own) on `device` (at most max_ctas CTAs when that is not
+// 0: MMEE_ERR_RANGE if it would take more).
+int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape);
 
 // MMEE_OK, or MMEE_ERR_CUDA with the error kept for mmee_last_cuda_error (per host thread).
 int cuda_status(cudaError_t e);

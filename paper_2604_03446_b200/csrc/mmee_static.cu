@@ -59,7 +59,7 @@ extern "C" int mmee_search_static(const mmee_workload_t* workload, const mmee_ar
     if ((rc = cuda_status(cudaGetDevice(&device)))) return rc;
     // The same launch shape as a handle would get, bounded by what the fixed scratch can hold.
     LaunchShape shape;
-    if ((rc = choose_launch_shape(plan, device, 1, kStaticMaxCtas, &shape))) return rc;
+    if ((rc = choose_launch_shape(plan, device, 0, kStaticMaxCtas, &shape))) return rc;
     shape.overlap = false;      // its CTAs touch the scratch without a wait for the reset below
     Scratch* scratch = nullptr;
     if ((rc = static_scratch(device, &scratch))) return rc;
@@ -67,6 +67,6 @@ extern "C" int mmee_search_static(const mmee_workload_t* workload, const mmee_ar
     // The array keeps whatever the previous call left in it.  The header (ticket counter, shared
     // bound) must start clean; the partial lists need no clearing, every CTA of
     // this launch overwrites its own before the finalize step reads them.
-    if ((rc = cuda_status(launch_reset(&scratch->head, 1, st)))) return rc;
+    if ((rc = cuda_status(launch_reset(&scratch->head, st)))) return rc;
     return cuda_status(launch_search(plan, shape, &scratch->head, scratch->partial, out_best, out_topk, st));
 }

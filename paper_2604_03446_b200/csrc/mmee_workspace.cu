@@ -21,7 +21,7 @@ Workspace* g_idle = nullptr;
 int g_n_idle = 0;
 
 int free_workspace(Workspace* ws) {
-    cudaError_t e = ws->heads ? cudaFree(ws->heads) : cudaSuccess;
+    cudaError_t e = ws->chain ? cudaFree(ws->chain) : cudaSuccess;
     if (ws->host) {
         const cudaError_t e2 = cudaFreeHost(ws->host);
         if (e == cudaSuccess) e = e2;
@@ -36,22 +36,20 @@ int make_workspace(int device, Workspace** out) {
     ws->device = device;
     int rc = max_search_ctas(device, &ws->max_ctas);
     if (rc) { delete ws; return rc; }
-    // one allocation: the headers of sharing searches and the chained searches' optima, then the two scratches
+    // one allocation: the chained searches' optima, then the two scratches
     static_assert(sizeof(ChainRecord) == 32, "a multiple of 16 bytes keeps the scratches aligned");
-    const size_t heads = kMaxArrays * sizeof(SearchHeader) + kHostRecords * sizeof(ChainRecord), bytes = scratch_bytes(ws->max_ctas);
+    const size_t chain = kHostRecords * sizeof(ChainRecord), bytes = scratch_bytes(ws->max_ctas);
     unsigned char* mem = nullptr;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), heads + 2 * bytes);
-    ws->heads = reinterpret_cast<SearchHeader*>(mem);
-    ws->chain = reinterpret_cast<ChainRecord*>(mem + kMaxArrays * sizeof(SearchHeader));
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + heads + i * bytes);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), chain + 2 * bytes);
+    ws->chain = reinterpret_cast<ChainRecord*>(mem);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + chain + i * bytes);
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t),
                           cudaHostAllocMapped | cudaHostAllocPortable);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ws->host_dev), ws->host, 0);
-    if (e == cudaSuccess) e = launch_reset(ws->heads, (int)kMaxArrays, 0);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = launch_reset(&ws->scratch[i]->head, 1, 0);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = launch_reset(&ws->scratch[i]->head, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         free_workspace(ws);

@@ -12,7 +12,6 @@ struct Workspace {
                                     // publishes while the one before it on the handle still finalizes
     uint32_t max_ctas;              // partial lists a scratch has room for
     ChainRecord* chain;             // device, kHostRecords: what chained searches left
-    SearchHeader* heads;            // device, kMaxArrays: headers of searches that share the partial lists; clean as well
     mmee_result_t* host;            // pinned host memory: 1 + MMEE_MAX_TOPK records that kernels write into
     mmee_result_t* host_dev;        // the same memory as the device addresses it
     Workspace* next;
