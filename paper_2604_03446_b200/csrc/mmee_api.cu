@@ -45,9 +45,9 @@ int cuda_status(cudaError_t e) {
 // Searches of at most this many tilings (and those for the k best, which would otherwise wait before their items) wait for
 // the kernel before them in their finalize step only (see mmee_search.cu).  The next search then starts while this one
 // finalizes, not earlier: better while the finalize step is the longer part, worse once the items are.  One energy search
-// after the other, early / late start (us): 4 900 tilings 11.3 / 10.4, 5 929 11.2 / 10.2, 7 056 11.0 to 12.5 / 9.6 to 13.8
-// (edge accelerator at S = 2048, ragged S = 96 on the edge), 8 064 11.5 / 12.1, 10 816 13.5 / 15.4, 18 496 11.4 / 12.2.
-// With register-file tiling the tables take longest: 23.5 / 26.5.
+// after the other, early / late start (us): 4 900 tilings 9.7 / 8.8, 5 929 9.6 / 8.9, 7 056 9.3 / 8.5 (edge accelerator,
+// S = 2048) and 10.6 / 11.4 (ragged S = 96), 8 064 10.4 / 10.9, 10 816 12.0 / 13.4, 18 496 9.9 / 10.5.  With register-file
+// tiling the tables take longest: 23.5 / 26.5 at 4 900.
 constexpr uint64_t kLateTilings = 6000;
 
 // Two CTAs per SM (118 registers a thread, no spills) beat three (80, spilled) and four (64): GQA latency 13.0, 13.7 and

@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <vector>
 
 namespace mmee {
@@ -154,7 +155,7 @@ void row_pruning_keep(const Plan& p, uint8_t* out, uint32_t* kept_rows) {
 
 // The kept rows as masks over classes of levels.  A row that is not the first of its class combination has equal
 // buffer needs and DRAM words as that first row and a higher index, so it is never kept; MMEE_ERR_CHECK if it were.
-int set_kept_masks(Plan* p, uint32_t* kept_rows) {
+static int find_kept_masks(Plan* p, uint32_t* kept_rows) {
     std::vector<uint8_t> keep(p->rows_per_tiling);
     row_pruning_keep(*p, keep.data(), kept_rows);
     std::memset(&p->kept, 0, sizeof(p->kept));
@@ -184,6 +185,26 @@ int set_kept_masks(Plan* p, uint32_t* kept_rows) {
         }
     }
     return MMEE_OK;
+}
+
+// The masks depend on the orders and the fusion modes alone, not on the problem: like the paper's offline pruning they are
+// found once for each of the 14 choices (13 ms of host time) and kept.
+int set_kept_masks(Plan* p, uint32_t* kept_rows) {
+    struct Entry {
+        std::once_flag once;
+        int status = MMEE_OK;
+        uint32_t rows = 0;
+        KeptMasks masks = {};
+    };
+    static Entry entries[2][8];
+    Entry& e = entries[p->n_orders == kMaxOrders ? 1 : 0][p->fuse_mask & 7u];
+    std::call_once(e.once, [&] {
+        e.status = find_kept_masks(p, &e.rows);
+        e.masks = p->kept;
+    });
+    p->kept = e.masks;
+    *kept_rows = e.rows;
+    return e.status;
 }
 
 }  // namespace mmee
