@@ -300,9 +300,9 @@ int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch,
  * mmee_pareto_front -- the energy-latency trade-off of the whole mapping space (Section VII-E): every
  * pair (e_key, l_key) of a feasible mapping that no other feasible mapping improves in one key without
  * losing in the other, by increasing energy / decreasing latency, each with the lowest-index mapping
- * that attains it.  Computed by alternating capped searches on the device (least energy under a latency
- * bound, then least latency at that energy): two searches per point, each taking its bound from the
- * record of the one before it on the device.  objective.objective, .topk,
+ * that attains it.  Computed by device searches under a shrinking latency bound (least energy, then least
+ * latency at that energy): one search per point, each taking its bound from the point before it on the
+ * device.  objective.objective, .topk,
  * .row_pruning and .key_cap are ignored.  Synchronous.
  *   out_points : HOST, `capacity` records; *n_points receives the number of points of the front, also
  *                when it exceeds capacity (then MMEE_ERR_RANGE is returned and the first `capacity`

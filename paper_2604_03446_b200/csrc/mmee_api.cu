@@ -92,20 +92,19 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
 
 namespace {
 
-// Searches chained on the device (see LaunchShape::chain), step i with plans[i % n_plans], until one finds nothing: their
-// optima in order, through `take` (which returns false to stop), and their number.  The host waits for a batch of them at a time, first
-// `first_batch`, then twice as many as before; what is launched beyond the last one ends at once.
+// Searches chained on the device (see LaunchShape::chain) until one finds nothing: their optima in order, through `take`
+// (which returns false to stop).  The host waits for a batch of them at a time, first `first_batch`, then twice as many as
+// before; what is launched beyond the last one ends at once.  The records are made with the plan `records`.
 template <class Take>
-int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found, Take take) {
+int run_chain(const Plan& plan, const Plan& records, uint32_t first_batch, Take take) {
     int device = 0;
     int rc = cuda_status(cudaGetDevice(&device));
     if (rc) return rc;
     LaunchShape shape;
-    if ((rc = choose_launch_shape(plans[0], device, 0, 0, &shape))) return rc;
+    if ((rc = choose_launch_shape(plan, device, 0, 0, &shape))) return rc;
     Workspace* ws = nullptr;
     if ((rc = workspace_acquire(device, &ws))) return rc;
     bool clean = true, more = true;
-    *n_found = 0;
     uint32_t step = 0;
     for (uint32_t batch = first_batch; more && rc == MMEE_OK; batch = 2 * batch < kHostRecords ? 2 * batch : kHostRecords) {
         uint32_t n = 0;
@@ -114,10 +113,10 @@ int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found,
             shape.late = false;
             shape.chain_read = step + n > 0;
             shape.chain_to = ws->chain + n;
-            rc = cuda_status(launch_search(plans[(step + n) % (uint32_t)n_plans], shape, &ws->scratch[0]->head, ws->scratch[0]->partial,
+            rc = cuda_status(launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial,
                                            nullptr, nullptr, nullptr));
         }
-        if (rc == MMEE_OK) rc = cuda_status(launch_resolve(plans[n_plans - 1], ws->chain, n, step, n_plans > 1, ws->host_dev, nullptr));
+        if (rc == MMEE_OK) rc = cuda_status(launch_resolve(records, ws->chain, n, ws->host_dev, nullptr));
         if (rc) clean = false;
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc2) clean = false;
@@ -125,8 +124,7 @@ int run_chain(Plan* plans, int n_plans, uint32_t first_batch, uint32_t* n_found,
         for (uint32_t i = 0; i < n && more && rc == MMEE_OK; ++i) {
             const mmee_result_t& r = ws->host[i];
             if (r.status == MMEE_ERR_CHECK) { rc = MMEE_ERR_CHECK; break; }
-            more = r.idx != MMEE_NO_INDEX;
-            if (more) { ++*n_found; more = take(r, step + i); }
+            more = r.idx != MMEE_NO_INDEX && take(r);
         }
         step += n;
     }
@@ -310,24 +308,20 @@ int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch, 
     *n_points = 0;
     mmee_objective_t o = *objective;
     o.topk = 1; o.row_pruning = 0; o.key_cap = INT64_MAX - 1;
-    Plan plans[2];
+    Plan plan, records;
     int rc;
     o.objective = MMEE_OBJ_ENERGY_LCAP;
-    if ((rc = build_plan(workload, arch, &o, &plans[0]))) return rc;
+    if ((rc = build_plan(workload, arch, &o, &plan))) return rc;
     o.objective = MMEE_OBJ_LATENCY_ECAP;
-    if ((rc = build_plan(workload, arch, &o, &plans[1]))) return rc;
-    uint32_t n = 0, n_found = 0;
-    // Even steps: the least energy among the mappings that are still faster than the previous point (none: the front is
-    // complete).  Odd steps: the fastest mapping at that energy, the point of the front, with its lowest index.
-    rc = run_chain(plans, 2, 4, &n_found, [&](const mmee_result_t& r, uint32_t step) {
-        if (step % 2) {
-            if (n < capacity) out_points[n] = r;
-            ++n;
-        }
+    if ((rc = build_plan(workload, arch, &o, &records))) return rc;
+    uint32_t n = 0;
+    // Each search finds the least energy among the mappings that are still faster than the previous point, and the least
+    // latency at that energy: the next point of the front, with its lowest index.  None: the front is complete.
+    rc = run_chain(plan, records, 3, [&](const mmee_result_t& r) {
+        if (n < capacity) out_points[n] = r;
+        ++n;
         return true;
     });
-    // (an even step's optimum qualifies for the odd one)
-    if (rc == MMEE_OK && n_found % 2) rc = MMEE_ERR_CHECK;
     *n_points = n;
     if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
     return rc;
@@ -347,11 +341,11 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
     if (rc) return rc;
     mmee_result_t held = {};
     bool have = false;
-    uint32_t n = 0, n_found = 0;
+    uint32_t n = 0;
     // Searches with a shrinking buffer: each returns the least DRAM traffic that fits, with the buffer words its
     // mapping needs; the next one allows one word less than that.  While the traffic stays the same the mapping
     // found needs less buffer for the same traffic; when it rises, the mapping held is a point of the front.
-    rc = run_chain(&plan, 1, 8, &n_found, [&](const mmee_result_t& r, uint32_t) {
+    rc = run_chain(plan, plan, 8, [&](const mmee_result_t& r) {
         if (have && r.e_key != held.e_key) {
             if (n < capacity) out_points[n] = held;
             ++n;

@@ -99,17 +99,31 @@ __device__ __forceinline__ void warp_offer(int64_t& ek, uint64_t& ei, int k, int
     }
 }
 
-// Smallest pair of the warp, in every lane, by 32-bit warp minima (keys are non-negative).
+// Smallest of the non-negative numbers of the lanes with `in` set (UINT64_MAX if there is none), by 32-bit warp minima;
+// `in` becomes whether this lane holds it.
+__device__ __forceinline__ uint64_t warp_min_u64(uint64_t v, bool& in) {
+    const uint32_t hi = __reduce_min_sync(kFull, in ? (uint32_t)(v >> 32) : 0xffffffffu);
+    in = in && (uint32_t)(v >> 32) == hi;
+    const uint32_t lo = __reduce_min_sync(kFull, in ? (uint32_t)v : 0xffffffffu);
+    in = in && (uint32_t)v == lo;
+    return ((uint64_t)hi << 32) | lo;
+}
+
+// Smallest pair of the warp, in every lane (keys are non-negative).
 __device__ __forceinline__ void warp_min_pair(int64_t& k, uint64_t& i) {
-    const uint32_t kh = __reduce_min_sync(kFull, (uint32_t)((uint64_t)k >> 32));
-    const bool m1 = (uint32_t)((uint64_t)k >> 32) == kh;
-    const uint32_t kl = __reduce_min_sync(kFull, m1 ? (uint32_t)k : 0xffffffffu);
-    const bool m2 = m1 && (uint32_t)k == kl;
-    const uint32_t ih = __reduce_min_sync(kFull, m2 ? (uint32_t)(i >> 32) : 0xffffffffu);
-    const bool m3 = m2 && (uint32_t)(i >> 32) == ih;
-    const uint32_t il = __reduce_min_sync(kFull, m3 ? (uint32_t)i : 0xffffffffu);
-    k = (int64_t)(((uint64_t)kh << 32) | kl);
-    i = ((uint64_t)ih << 32) | il;
+    bool in = true;
+    k = (int64_t)warp_min_u64((uint64_t)k, in);
+    i = warp_min_u64(i, in);
+}
+// ... by key, then second key, then number.
+__device__ __forceinline__ void warp_min_triple(int64_t& k, int64_t& k2, uint64_t& i) {
+    bool in = true;
+    k = (int64_t)warp_min_u64((uint64_t)k, in);
+    k2 = (int64_t)warp_min_u64((uint64_t)k2, in);
+    i = warp_min_u64(i, in);
+}
+__device__ __forceinline__ bool triple_less(int64_t ka, int64_t la, uint64_t ia, int64_t kb, int64_t lb, uint64_t ib) {
+    return ka < kb || (ka == kb && (la < lb || (la == lb && ia < ib)));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -365,6 +379,43 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
     return warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (warp == 2 && lane == 0 ? 31 : -1));
 }
 
+// The end of one search of the energy-latency front, by all threads of the last CTA: the least (energy, latency, block) of
+// all CTAs is the next point of the front.  It is left as a latency optimum under that energy, which is what
+// launch_resolve looks for in the block; the next search allows one word less of latency.
+__device__ __noinline__ void finalize_front(const Plan& p, Shared& sh, ChainRecord* chain_to, SearchHeader* __restrict__ head,
+                                            const Partial* __restrict__ partials, int n_partials) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t ek = kInfKey, el = kInfKey;
+    uint64_t ei = UINT64_MAX;
+    unsigned long long rows = 0;
+    for (int c = tid; c < n_partials; c += kSearchThreads) {
+        const longlong2 v = __ldcg(&partials[c].e[0]), w = __ldcg(&partials[c].e[1]);
+        rows += __ldcg(&partials[c].feasible_rows);
+        if (triple_less(v.x, v.y, (uint64_t)w.x, ek, el, ei)) { ek = v.x; el = v.y; ei = (uint64_t)w.x; }
+    }
+    for (int off = 16; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+    warp_min_triple(ek, el, ei);
+    if (lane == 0) {
+        sh.feasible_rows[warp] = rows;
+        sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
+        sh.tops[warp][1] = make_longlong2((long long)ei, 0);
+    }
+    __syncthreads();
+    if (warp) return;
+    rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
+    for (int off = kWarps / 2; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+    ek = sh.tops[lane & (kWarps - 1)][0].x;
+    el = sh.tops[lane & (kWarps - 1)][0].y;
+    ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
+    warp_min_triple(ek, el, ei);
+    if (lane == 0) {
+        const bool found = ek != kInfKey;
+        *chain_to = {(long long)(found ? el : kInfKey), (unsigned long long)ei, rows * p.n_sm, (long long)ek};
+        head->chain_bound = found ? el - 1 : -1;
+        head->done_ctas = 0;
+    }
+}
+
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
 template <int OBJ, int MODE>
 __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to, SearchHeader* __restrict__ head,
@@ -425,16 +476,13 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         min_over_warps(sh, lane, warp, ek, ei);
         found = ek != kInfKey ? 1 : 0;
         bound = ek;
-        constexpr bool kBlockOnly = MODE == kModeChain && OBJ != MMEE_OBJ_ENERGY;
         if (MODE == kModeChain && tid == 0) {
             unsigned long long fit = 0;
             for (int w = 0; w < kWarps; ++w) fit += sh.feasible_rows[w];
-            *chain_to = {(long long)ek, (unsigned long long)ei, fit * p.n_sm, (long long)(kBlockOnly ? lim.key_cap : lim.cap_words)};
-            // the next search's bound: this energy / one word less of latency
-            if (kBlockOnly || !found) head->chain_bound = !found ? -1 : (OBJ == MMEE_OBJ_ENERGY_LCAP ? ek : ek - 1);
+            *chain_to = {(long long)ek, (unsigned long long)ei, fit * p.n_sm, (long long)lim.cap_words};
+            if (!found) head->chain_bound = -1;
             head->done_ctas = 0;
         }
-        if (kBlockOnly) return;
         // ---- the winning block, mapping by mapping
         const int item = split_item(warp, lane);
         if (found && item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)ei, item, &sh.block[0]);
@@ -615,6 +663,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
     constexpr bool ARRAYS = MODE == kModeArrays;
+    constexpr bool FRONT = CHAIN && OBJ == MMEE_OBJ_ENERGY_LCAP;      // least (energy, latency) under a bound on the latency
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool late = shape.late;
@@ -644,6 +693,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
+    int64_t el = kInfKey;           // FRONT: its latency
     unsigned long long my_rows = 0;
     uint32_t my_live = 0;
 
@@ -662,6 +712,20 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             atomicMin(&sh.G, (long long)ek);
             atomicMin(&head->G, (long long)ek);
         }
+    };
+
+    // FRONT: the item's least (energy, latency) over the stationary pairs; pair(s, e, l) forms those of pair s.
+    auto offer_front = [&](auto pair, uint32_t id, bool valid) {
+        int64_t be = kInfKey, bl = kInfKey;
+#pragma unroll
+        for (int s = 0; s < 9; ++s) {
+            int64_t e, l;
+            pair(s, e, l);
+            const bool better = ((p.sm_mask >> s) & 1u) && l <= lim.key_cap && (e < be || (e == be && l < bl));
+            be = better ? e : be;
+            bl = better ? l : bl;
+        }
+        if (valid && triple_less(be, bl, id, ek, el, ei)) { ek = be; el = bl; ei = id; }
     };
 
     // The same for every array shape, one after the other: key_of_terms(terms) is the item's least key.
@@ -783,7 +847,12 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 if (any(some)) {
                     const int64_t y = some ? x : 0, rho = oi.recompute[c] != 0 ? (int64_t)tb.b[LOOP_J] : 1;
                     auto key = [&](const StatTerms& t) { return fused_least_key<OBJ>(t, y, rho, p.sm_mask, p.c_dram_gb, lim.key_cap); };
+                    auto pair = [&](int s, int64_t& e, int64_t& l) {
+                        e = p.c_dram_gb * y + tb.st.P1[s / 3] * rho + tb.st.P2[s % 3];
+                        l = max64(y, tb.st.Q1[s / 3] * rho + tb.st.Q2[s % 3]);
+                    };
                     if (ARRAYS) offer_arrays(key, slot, id, some);
+                    else if (FRONT) offer_front(pair, id, some);
                     else offer(key(tb.st), id, some);
                 }
             } else {
@@ -805,7 +874,12 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                     if (some) my_rows += rows;
                     const int64_t pass = phi == 2 ? 2 * dw.il : 0;
                     auto key = [&](const StatTerms& t) { return unfused_least_key<OBJ>(t, y1, y2, pass, p.sm_mask, p.c_dram_gb, lim.key_cap); };
+                    auto pair = [&](int s, int64_t& e, int64_t& l) {
+                        e = p.c_dram_gb * (y1 + y2 + pass) + tb.st.P1[s / 3] + tb.st.P2[s % 3];
+                        l = max64(y1, tb.st.Q1[s / 3]) + pass + max64(y2, tb.st.Q2[s % 3]);
+                    };
                     if (ARRAYS) offer_arrays(key, slot, id + block, some);
+                    else if (FRONT) offer_front(pair, id + block, some);
                     else offer(key(tb.st), id + block, some);
                     block += n_orders;
                 }
@@ -819,6 +893,13 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     if (lane == 0) sh.feasible_rows[warp] = my_rows;
     if (MULTI) {
         merge_warps(sh, k, lane, warp, ek, ei);
+    } else if (FRONT) {
+        warp_min_triple(ek, el, ei);
+        if (lane == 0) {
+            sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
+            sh.tops[warp][1] = make_longlong2((long long)ei, 0);
+        }
+        __syncthreads();
     } else if (!ARRAYS) {
         warp_min_pair(ek, ei);
         if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)ek, (long long)ei);
@@ -852,6 +933,13 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             g_end = __shfl_sync(kFull, g_end, 0);
             count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey && ek <= g_end));
             if (lane < (int)max(count, 1u)) out->e[lane] = make_longlong2((long long)ek, (long long)ei);
+        } else if (FRONT) {
+            ek = sh.tops[lane & (kWarps - 1)][0].x;
+            el = sh.tops[lane & (kWarps - 1)][0].y;
+            ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
+            warp_min_triple(ek, el, ei);
+            count = 2;
+            if (lane < 2) out->e[lane] = lane ? make_longlong2((long long)ei, 0) : make_longlong2((long long)ek, (long long)el);
         } else {
             const longlong2 v = sh.tops[lane & (kWarps - 1)][0];
             ek = v.x;
@@ -880,7 +968,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             release_next_kernel();
         }
         __threadfence();
-        finalize_step<OBJ, MODE>(p, lim, sh, shape.chain_to, head, partials, (int)grid, out_best, out_topk);
+        if (FRONT) finalize_front(p, sh, shape.chain_to, head, partials, (int)grid);
+        else finalize_step<OBJ, MODE>(p, lim, sh, shape.chain_to, head, partials, (int)grid, out_best, out_topk);
     }
 }
 
@@ -939,17 +1028,9 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
 
 template <int OBJ>
 __global__ void __launch_bounds__(kSearchThreads, 2)
-resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* __restrict__ chain, uint32_t first_step, bool odd_only,
-               mmee_result_t* __restrict__ out) {
+resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* __restrict__ chain, mmee_result_t* __restrict__ out) {
     __shared__ Shared sh;
     const ChainRecord c = chain[blockIdx.x];
-    if (c.key != kInfKey && odd_only && !((first_step + blockIdx.x) & 1u)) {
-        if (threadIdx.x == 0) {         // (the host asks of this one only whether something was found)
-            out[blockIdx.x].idx = 0;
-            out[blockIdx.x].status = MMEE_OK;
-        }
-        return;
-    }
     const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
     resolve_record<OBJ, OBJ != MMEE_OBJ_ENERGY>(p, lim, p.pe_rows, p.pe_cols, sh, c.key, c.where, c.n_feasible, out + blockIdx.x);
 }
@@ -979,15 +1060,15 @@ resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, c
                               rows * p.n_sm, out + blockIdx.x);
 }
 
-// (only the objectives of the Pareto fronts are chained)
+// (only the searches of the Pareto fronts are chained)
 template <int OBJ>
-constexpr int chain_mode() { return OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? kModeSingle : kModeChain; }
+constexpr int chain_mode() { return OBJ == MMEE_OBJ_ENERGY || OBJ == MMEE_OBJ_ENERGY_LCAP ? kModeChain : kModeSingle; }
 
 template <int OBJ>
 cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials,
                             mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
     auto* kernel = shape.n_arrays ? search_kernel<OBJ, kModeArrays>
-                   : shape.chain ? (OBJ == MMEE_OBJ_LATENCY || OBJ == MMEE_OBJ_EDP ? nullptr : search_kernel<OBJ, chain_mode<OBJ>()>)
+                   : shape.chain ? (chain_mode<OBJ>() == kModeChain ? search_kernel<OBJ, chain_mode<OBJ>()> : nullptr)
                    : p.row_pruning ? search_kernel<OBJ, kModePrune>
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
     if (!kernel) return cudaErrorInvalidValue;
@@ -1018,11 +1099,10 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
     }
 }
 
-cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, uint32_t first_step, bool odd_only,
-                           mmee_result_t* out, cudaStream_t st) {
+cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, mmee_result_t* out, cudaStream_t st) {
     switch (p.objective) {
-        case MMEE_OBJ_ENERGY: resolve_kernel<MMEE_OBJ_ENERGY><<<n, kSearchThreads, 0, st>>>(p, chain, first_step, odd_only, out); break;
-        case MMEE_OBJ_LATENCY_ECAP: resolve_kernel<MMEE_OBJ_LATENCY_ECAP><<<n, kSearchThreads, 0, st>>>(p, chain, first_step, odd_only, out); break;
+        case MMEE_OBJ_ENERGY: resolve_kernel<MMEE_OBJ_ENERGY><<<n, kSearchThreads, 0, st>>>(p, chain, out); break;
+        case MMEE_OBJ_LATENCY_ECAP: resolve_kernel<MMEE_OBJ_LATENCY_ECAP><<<n, kSearchThreads, 0, st>>>(p, chain, out); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -39,8 +39,8 @@ struct Scratch {
 
 constexpr uint32_t kMaxArrays = MMEE_MAX_TOPK;      // one entry of a partial list each
 
-// What a chained search leaves of its optimum: the key (kInfKey: nothing fits), the mapping's index (energy) or the block
-// that holds it (capped objectives), the mappings that fit, and the bound it was found under.
+// What a chained search leaves of its optimum: key kInfKey if nothing fits; an energy search its key, the mapping's index
+// and the buffer words it was found under; a search of the energy-latency front the latency, the block and the energy.
 struct ChainRecord {
     long long key;
     unsigned long long where;
@@ -61,8 +61,8 @@ struct LaunchShape {
 };
 // Chained searches (k = 1, no row pruning; the Pareto fronts): each takes a bound from what the one before it on the
 // stream found, on the device, so that the host waits once for several: the buffer words (energy) or the bound on the
-// other key (capped objectives) come from the scratch instead of the plan (and are not above the plan's), and the bound
-// for the next search is left there.  After a search that found nothing the others end at once.  A chained search writes
+// latency (energy under a latency bound: then the least latency at the least energy) come from the scratch instead of the
+// plan (and are not above the plan's), and the bound for the next search is left there.  After a search that found nothing the others end at once.  A chained search writes
 // no record but a ChainRecord: the next one has to wait for its end, and the records of all can be made side by side
 // afterwards (launch_resolve).
 
@@ -77,10 +77,9 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
                           mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st);
 // The same search (k = 1) on each of shape.n_arrays logical arrays, one record each in `out`: two launches.
 cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partial* partials, mmee_result_t* out, cudaStream_t st);
-// Full records of the optima that n chained searches left, one CTA each; those with an odd number only (`odd_only`; the
-// others' records say no more than whether something was found).
-cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, uint32_t first_step, bool odd_only,
-                           mmee_result_t* out, cudaStream_t st);
+// Full records of the optima that n chained searches left, one CTA each: of the energy searches themselves (`p` their
+// plan), or of the searches of the energy-latency front (`p` with the objective MMEE_OBJ_LATENCY_ECAP).
+cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, mmee_result_t* out, cudaStream_t st);
 cudaError_t launch_reset(SearchHeader* head, cudaStream_t st);
 
 // Every key of the plan's tiling range (kInfKey where a mapping does not fit or its stationary pair is not offered).
