@@ -785,7 +785,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         }
         if (CHAIN && shape.chain_read && m0 == 0) {
             wait_previous_kernel();
-            const int64_t bound = __ldcg(&head->chain_bound);
+            const int64_t bound = *reinterpret_cast<volatile long long*>(&head->chain_bound);
             if (OBJ == MMEE_OBJ_ENERGY) {
                 lim.cap_words = bound;
                 capc = (int)bound;
@@ -978,16 +978,14 @@ __global__ void reset_kernel(SearchHeader* head) {
     head->done_ctas = 0;
 }
 
-// The full record of an optimum, by one CTA: mapping `where`, or (IN_BLOCK) the first mapping with key `key` of block
-// `where`.  key kInfKey: nothing fits.
+// The full record of an optimum, by one CTA after load_shared: mapping `where`, or (IN_BLOCK) the first mapping with key
+// `key` of block `where`.  key kInfKey: nothing fits.
 template <int OBJ, bool IN_BLOCK>
-__device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim, uint32_t pe_rows, uint32_t pe_cols, Shared& sh,
+__device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim, Shared& sh,
                                                int64_t key, uint64_t where, unsigned long long n_feasible, mmee_result_t* out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     mmee_result_t& r = sh.record[0];
     if (key != kInfKey) {
-        load_shared<false>(p, pe_rows, pe_cols, sh);
-        __syncthreads();
         int64_t ek = key;
         uint64_t ei = where;
         if (IN_BLOCK) {
@@ -1028,27 +1026,36 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
 
 template <int OBJ>
 __global__ void __launch_bounds__(kSearchThreads, 2)
-resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* __restrict__ chain, mmee_result_t* __restrict__ out) {
+resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* chain, mmee_result_t* out) {
     __shared__ Shared sh;
-    const ChainRecord c = chain[blockIdx.x];
+    load_shared<false>(p, p.pe_rows, p.pe_cols, sh);
+    __syncthreads();
+    wait_previous_kernel();
+    // (volatile: read after the wait, not as data that no kernel writes meanwhile)
+    const volatile ChainRecord* from = chain + blockIdx.x;
+    const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound};
     const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
-    resolve_record<OBJ, OBJ != MMEE_OBJ_ENERGY>(p, lim, p.pe_rows, p.pe_cols, sh, c.key, c.where, c.n_feasible, out + blockIdx.x);
+    resolve_record<OBJ, OBJ != MMEE_OBJ_ENERGY>(p, lim, sh, c.key, c.where, c.n_feasible, out + blockIdx.x);
 }
 
 // Merge of the CTAs' best items of array shape blockIdx.x, and the record of the optimum.
 template <int OBJ>
 __global__ void __launch_bounds__(kSearchThreads, 2)
-resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, const Partial* __restrict__ partials,
-                      mmee_result_t* __restrict__ out) {
+resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, const Partial* partials, mmee_result_t* out) {
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    load_shared<false>(p, shape.array[blockIdx.x][0], shape.array[blockIdx.x][1], sh);
+    __syncthreads();
+    wait_previous_kernel();
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
     unsigned long long rows = 0;
     for (uint32_t c = tid; c < shape.grid; c += kSearchThreads) {
-        const longlong2 v = partials[c].e[blockIdx.x];
-        rows += partials[c].feasible_rows;
-        if (pair_less(v.x, (uint64_t)v.y, ek, ei)) { ek = v.x; ei = (uint64_t)v.y; }
+        const volatile Partial* from = partials + c;        // (volatile: read after the wait)
+        const int64_t key = from->e[blockIdx.x].x;
+        const uint64_t num = (uint64_t)from->e[blockIdx.x].y;
+        rows += from->feasible_rows;
+        if (pair_less(key, num, ek, ei)) { ek = key; ei = num; }
     }
     for (int off = 16; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
     if (lane == 0) sh.feasible_rows[warp] = rows;
@@ -1056,8 +1063,23 @@ resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, c
     min_over_warps(sh, lane, warp, ek, ei);
     rows = 0;
     for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
-    resolve_record<OBJ, true>(p, Limits{p.cap_words, p.key_cap}, shape.array[blockIdx.x][0], shape.array[blockIdx.x][1], sh, ek, ei,
+    resolve_record<OBJ, true>(p, Limits{p.cap_words, p.key_cap}, sh, ek, ei,
                               rows * p.n_sm, out + blockIdx.x);
+}
+
+// A launch that may start before the kernel before it on the stream has ended (`overlap`): the kernel waits itself.
+template <class... Args>
+cudaError_t launch_overlapped(bool overlap, unsigned grid, cudaStream_t st, void (*kernel)(Args...), Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kSearchThreads);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // (only the searches of the Pareto fronts are chained)
@@ -1072,16 +1094,7 @@ cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeade
                    : p.row_pruning ? search_kernel<OBJ, kModePrune>
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
     if (!kernel) return cudaErrorInvalidValue;
-    cudaLaunchAttribute overlap;
-    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    overlap.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(shape.grid);
-    cfg.blockDim = dim3(kSearchThreads);
-    cfg.stream = st;
-    cfg.attrs = &overlap;
-    cfg.numAttrs = shape.overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, p, shape, head, partials, out_best, out_topk);
+    return launch_overlapped(shape.overlap, shape.grid, st, kernel, p, shape, head, partials, out_best, out_topk);
 }
 
 }  // namespace
@@ -1101,11 +1114,10 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
 
 cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, mmee_result_t* out, cudaStream_t st) {
     switch (p.objective) {
-        case MMEE_OBJ_ENERGY: resolve_kernel<MMEE_OBJ_ENERGY><<<n, kSearchThreads, 0, st>>>(p, chain, out); break;
-        case MMEE_OBJ_LATENCY_ECAP: resolve_kernel<MMEE_OBJ_LATENCY_ECAP><<<n, kSearchThreads, 0, st>>>(p, chain, out); break;
+        case MMEE_OBJ_ENERGY: return launch_overlapped(true, n, st, resolve_kernel<MMEE_OBJ_ENERGY>, p, chain, out);
+        case MMEE_OBJ_LATENCY_ECAP: return launch_overlapped(true, n, st, resolve_kernel<MMEE_OBJ_LATENCY_ECAP>, p, chain, out);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 uint32_t search_chunk(uint32_t n_arrays) {
@@ -1116,14 +1128,14 @@ cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partia
     const cudaError_t e = launch_search(p, shape, nullptr, partials, nullptr, nullptr, st);
     if (e != cudaSuccess) return e;
     const unsigned n = shape.n_arrays;
+    const Partial* from = partials;
     switch (p.objective) {
-        case MMEE_OBJ_ENERGY: resolve_arrays_kernel<MMEE_OBJ_ENERGY><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
-        case MMEE_OBJ_LATENCY: resolve_arrays_kernel<MMEE_OBJ_LATENCY><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
-        case MMEE_OBJ_EDP: resolve_arrays_kernel<MMEE_OBJ_EDP><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
-        case MMEE_OBJ_ENERGY_LCAP: resolve_arrays_kernel<MMEE_OBJ_ENERGY_LCAP><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
-        default: resolve_arrays_kernel<MMEE_OBJ_LATENCY_ECAP><<<n, kSearchThreads, 0, st>>>(p, shape, partials, out); break;
+        case MMEE_OBJ_ENERGY: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_ENERGY>, p, shape, from, out);
+        case MMEE_OBJ_LATENCY: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_LATENCY>, p, shape, from, out);
+        case MMEE_OBJ_EDP: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_EDP>, p, shape, from, out);
+        case MMEE_OBJ_ENERGY_LCAP: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_ENERGY_LCAP>, p, shape, from, out);
+        default: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_LATENCY_ECAP>, p, shape, from, out);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_reset(SearchHeader* head, cudaStream_t st) {
