@@ -342,22 +342,34 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
     mmee_result_t held = {};
     bool have = false;
     uint32_t n = 0;
-    // Searches with a shrinking buffer: each returns the least DRAM traffic that fits, with the buffer words its
-    // mapping needs; the next one allows one word less than that.  While the traffic stays the same the mapping
-    // found needs less buffer for the same traffic; when it rises, the mapping held is a point of the front.
+    // Searches with a shrinking buffer: each returns the least DRAM traffic that fits, with the least buffer words that a
+    // mapping of the first block with that traffic needs; the next one allows one word less than that.  While the traffic
+    // stays the same the mapping found needs less buffer for the same traffic; when it rises, the mapping held is a point
+    // of the front.
+    auto emit = [&]() {
+        if (n < capacity) out_points[n] = held;
+        ++n;
+    };
     rc = run_chain(plan, plan, 8, [&](const mmee_result_t& r) {
-        if (have && r.e_key != held.e_key) {
-            if (n < capacity) out_points[n] = held;
-            ++n;
-        }
+        if (have && r.e_key != held.e_key) emit();
         held = r;
         have = true;
         plan.cap_words = r.bs - 1;      // (for the tables of the next batch: tilings that cannot fit are left out)
         return plan.cap_words >= 0;
     });
-    if (rc == MMEE_OK && have) {
-        if (n < capacity) out_points[n] = held;
-        ++n;
+    if (rc == MMEE_OK && have) emit();
+    // (points whose count of fitting mappings belongs to another bound: see resolve_record)
+    mmee_handle_t* h = nullptr;
+    for (uint32_t i = 0; i < n && i < capacity && rc == MMEE_OK; ++i) {
+        const uint32_t before = out_points[i].reserved2[0];
+        if (!before) continue;
+        if (!h && (rc = mmee_create(workload, &a, &o, &h))) break;
+        h->plan.cap_words = (int64_t)before - 1;
+        rc = mmee_search_host(h, &out_points[i], nullptr);
+    }
+    if (h) {
+        const int rc2 = mmee_destroy(h);
+        if (rc == MMEE_OK) rc = rc2;
     }
     *n_points = n;
     if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;

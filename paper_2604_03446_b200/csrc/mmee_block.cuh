@@ -84,6 +84,7 @@ __device__ __forceinline__ void block_item(const Plan& p, const Divisors& dv, ui
 // One row of the block: levels (beta - 3) of A, B, C, D, E (C's is 0 when unfused).
 struct RowTerms {
     bool fits;
+    int64_t need;               // buffer words (Eq. 4)
     int64_t x1, x2;             // DRAM words of A and B, of D and E (unfused: C's write-back and read-back included)
     int64_t rho;                // recomputation factor of C
 };
@@ -97,7 +98,8 @@ __device__ __forceinline__ RowTerms row_terms(const Plan& p, const Limits& lim, 
         need2 += (a ? A : 0) + (b ? B : 0);
         rc = p.q.recompute[p.order_id[bt.slot]][c];
     }
-    r.fits = max64(need1, need2) <= lim.cap_words;
+    r.need = max64(need1, need2);
+    r.fits = r.need <= lim.cap_words;
     r.rho = rc ? (int64_t)bt.jD : 1;
     r.x1 = bt.g[0][a][rc] + bt.g[1][b][rc];
     r.x2 = bt.g[3][d][0] + bt.g[4][e][0];
@@ -117,15 +119,6 @@ __device__ __forceinline__ RowTerms block_row(const Plan& p, const Limits& lim, 
     const int e = (int)(row % 5u), d = (int)(row / 5u % 5u);
     if (bt.phi == 0) return row_terms(p, lim, bt, (int)(row / 625u), (int)(row / 125u % 5u), (int)(row / 25u % 5u), d, e);
     return row_terms(p, lim, bt, (int)(row / 125u), (int)(row / 25u % 5u), 0, d, e);
-}
-// Buffer words that row `row` of the block needs (Eq. 4).  Exact for a row that fits.
-__device__ __forceinline__ int64_t block_need(const BlockTab& bt, uint32_t row) {
-    const int e = (int)(row % 5u), d = (int)(row / 5u % 5u);
-    const bool fused = bt.phi == 0;
-    const int c = fused ? (int)(row / 25u % 5u) : 0, a = (int)(fused ? row / 625u : row / 125u), b = (int)(fused ? row / 125u % 5u : row / 25u % 5u);
-    const int64_t A = bt.size[0][a], B = bt.size[1][b], C = bt.size[2][c], D = bt.size[3][d], E = bt.size[4][e];
-    if (!fused) return max64(A + B + C, C + D + E);
-    return max64(A + B + C + (d ? D : 0) + (e ? E : 0), C + D + E + (a ? A : 0) + (b ? B : 0));
 }
 __device__ __forceinline__ uint32_t block_rows(const BlockTab& bt) { return bt.phi == 0 ? 3125u : 625u; }
 

@@ -68,9 +68,10 @@ MMEE_HD uint64_t size_words(const uint32_t dim[4], const uint32_t g[4], int slot
 // changes nothing: a dropped row's keys are never below those of a kept one.
 // ANY(x): true if x holds for some lane of the warp (device), for this call (host); a choice of A and B that leaves no
 // lane any room is skipped.
-template <bool PRUNE, class Any>
+// NEED: also the least buffer need (Eq. 4) of a row that fits with the least DRAM words.
+template <bool PRUNE, bool NEED, class Any>
 MMEE_HD void fused_class(const TileTab& tb, const OrderInfo& oi, const DimWords& dw, int c, int capc,
-                         const uint16_t* kept, Any any, uint32_t& rows, int64_t& words) {
+                         const uint16_t* kept, Any any, uint32_t& rows, int64_t& words, int& need) {
     const int C = tb.size[oi.size_c[c]];
     const int A[3] = {tb.size[S_ik], tb.size[S_iK], tb.size[S_IK]};
     const int B[3] = {tb.size[S_kl], tb.size[S_Kl], tb.size[S_KL]};
@@ -97,6 +98,7 @@ MMEE_HD void fused_class(const TileTab& tb, const OrderInfo& oi, const DimWords&
         for (int y = 0; y < 3; ++y) V[x][y] = D[x] + E[y];          // at most 2^31 - 2
     uint32_t total = 0;
     int64_t best = kNoRow;
+    int best_need = kSizeCap;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
 #pragma unroll
@@ -146,6 +148,23 @@ MMEE_HD void fused_class(const TileTab& tb, const OrderInfo& oi, const DimWords&
                 total += n * (uint32_t)(oi.width[OP_A][a] * oi.width[OP_B][b]);
             }
             const bool f_d = Dr <= s1 && Dr + E[0] <= s2, f_e = Er <= s1 && D[0] + Er <= s2;
+            if (NEED) {
+                // every choice of D and E by (words, need): where a loop bound is 1 several fetch the same words
+                // (unsigned: the sums of a choice that does not fit may exceed 2^31)
+                auto offer = [&](bool ok, int64_t y, uint32_t d, uint32_t e, uint32_t held) {
+                    const uint32_t n1 = (uint32_t)A[a] + (uint32_t)B[b] + (uint32_t)C + held;
+                    const uint32_t n2 = (uint32_t)C + d + e + (a ? (uint32_t)A[a] : 0u) + (b ? (uint32_t)B[b] : 0u);
+                    const int n = (int)(n1 > n2 ? n1 : n2);
+                    const int64_t w = gA[a] + gB[b] + y;
+                    if (ok && (w < best || (w == best && n < best_need))) { best = w; best_need = n; }
+                };
+                const uint32_t dr = (uint32_t)Dr, er = (uint32_t)Er;
+                offer(s1 >= 0 && V[0][0] <= s2, y_none, (uint32_t)D[0], (uint32_t)E[0], 0u);
+                offer(f_d, y_d, dr, (uint32_t)E[0], dr);
+                offer(f_e, y_e, (uint32_t)D[0], er, er);
+                offer(Dr + Er <= s1, y_held, dr, er, dr + er);
+                continue;
+            }
             int64_t y = (s1 >= 0 && V[0][0] <= s2) ? y_none : kNoRow;
             y = (d_first ? f_e : f_d) ? y_next : y;
             y = (d_first ? f_d : f_e) ? y_best : y;
@@ -155,13 +174,14 @@ MMEE_HD void fused_class(const TileTab& tb, const OrderInfo& oi, const DimWords&
     }
     rows = total * (PRUNE ? 1u : (uint32_t)oi.width[OP_C][c]);
     words = best < kNoRow ? best : kNoRow;
+    need = best_need;
 }
 
 // Both nests of an unfused block (any mode): feasible rows (of 625, or kept ones) and the least DRAM words of each nest,
-// C's write-back in the first and its read-back in the second included.
-template <bool PRUNE>
+// C's write-back in the first and its read-back in the second included.  NEED: as above.
+template <bool PRUNE, bool NEED>
 MMEE_HD void unfused_nests(const TileTab& tb, const OrderInfo& oi, const DimWords& dw, int capc,
-                           uint32_t& fit1, uint32_t& fit2, uint32_t& rows, int64_t& words1, int64_t& words2) {
+                           uint32_t& fit1, uint32_t& fit2, uint32_t& rows, int64_t& words1, int64_t& words2, int& need) {
     const uint32_t f = oi.flags;
     const int s = capc - tb.size[S_il];
     const int A[3] = {tb.size[S_ik], tb.size[S_iK], tb.size[S_IK]};
@@ -174,6 +194,7 @@ MMEE_HD void unfused_nests(const TileTab& tb, const OrderInfo& oi, const DimWord
     const int64_t gE[3] = {dw.ij * ((f & kLaboveE1) ? tb.b[LOOP_L] : 1u), dw.ij * ((f & kLaboveE2) ? tb.b[LOOP_L] : 1u), dw.ij};
     uint32_t n1 = 0, n2 = 0, m1 = 0, m2 = 0;
     int64_t x1 = kNoRow, x2 = kNoRow;
+    int u1 = kSizeCap, u2 = kSizeCap;       // least sizes of the two operands at those words
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -186,12 +207,19 @@ MMEE_HD void unfused_nests(const TileTab& tb, const OrderInfo& oi, const DimWord
                 n1 += o1 ? (uint32_t)(oi.width[OP_A][a] * oi.width[OP_B][b]) : 0u;
                 n2 += o2 ? (oi.width[OP_D][a + 1] + (a ? 0u : 1u)) * (oi.width[OP_E][b + 1] + (b ? 0u : 1u)) : 0u;
             }
-            x1 = o1 ? min64(x1, gA[a] + gB[b]) : x1;
-            x2 = o2 ? min64(x2, gD[a] + gE[b]) : x2;
+            if (NEED) {
+                const int64_t w1 = gA[a] + gB[b], w2 = gD[a] + gE[b];
+                if (o1 && (w1 < x1 || (w1 == x1 && A[a] + B[b] < u1))) { x1 = w1; u1 = A[a] + B[b]; }
+                if (o2 && (w2 < x2 || (w2 == x2 && D[a] + E[b] < u2))) { x2 = w2; u2 = D[a] + E[b]; }
+            } else {
+                x1 = o1 ? min64(x1, gA[a] + gB[b]) : x1;
+                x2 = o2 ? min64(x2, gD[a] + gE[b]) : x2;
+            }
         }
     fit1 = m1;
     fit2 = m2;
     rows = n1 * n2;
+    need = tb.size[S_il] + (u1 > u2 ? u1 : u2);
     const bool some = x1 < kNoRow && x2 < kNoRow;
     words1 = some ? x1 + dw.il : kNoRow;
     words2 = some ? x2 + dw.il * ((f & kJaboveC) ? tb.b[LOOP_J] : 1u) : kNoRow;

@@ -197,8 +197,9 @@ __device__ __forceinline__ uint32_t row_of(bool fused, int a, int b, int c, int 
 // The best mapping of one block whose least key is `key`: the lowest index with that key (the first row of a class
 // combination precedes its other rows, so only those are looked at).  All threads of the CTA; the pair ends up in every
 // lane of every warp's own share, to be reduced over the warps.
-template <int OBJ>
-__device__ __forceinline__ void best_of_block(const Plan& p, const Limits& lim, const Shared& sh, int64_t key, int64_t& ek, uint64_t& ei) {
+template <int OBJ, bool NEED>
+__device__ __forceinline__ void best_of_block(const Plan& p, const Limits& lim, const Shared& sh, int64_t key, int64_t need,
+                                              int64_t& ek, uint64_t& ei) {
     const BlockTab& bt = sh.block[0];
     const OrderInfo& o = sh.order[bt.slot];
     const bool fused = bt.phi == 0;
@@ -213,9 +214,31 @@ __device__ __forceinline__ void best_of_block(const Plan& p, const Limits& lim, 
         for (int s = 8; s >= 0; --s)
             if (((p.sm_mask >> s) & 1u) && mapping_key<OBJ>(p, lim, bt, t, s) == key) at = (uint32_t)s;
         const uint64_t idx = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u + at;
-        if (at < 9u && idx < ei) { ek = key; ei = idx; }
+        if (at < 9u && idx < ei && (!NEED || t.need == need)) { ek = key; ei = idx; }
     }
     warp_min_pair(ek, ei);
+}
+
+// The least buffer need among the mappings of the block with that key and an index below `idx` (UINT64_MAX: none); each
+// warp's in all its lanes.
+template <int OBJ>
+__device__ __forceinline__ uint64_t least_need_before(const Plan& p, const Limits& lim, const Shared& sh, int64_t key, uint64_t idx) {
+    const BlockTab& bt = sh.block[0];
+    const OrderInfo& o = sh.order[bt.slot];
+    const bool fused = bt.phi == 0;
+    uint64_t least = UINT64_MAX;
+    for (uint32_t r = threadIdx.x; r < (fused ? kFusedReps : kUnfusedReps); r += kSearchThreads) {
+        const Rep q = decode_rep(o, fused, r);
+        const RowTerms t = row_terms(p, lim, bt, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]);
+        if (!t.fits || (uint64_t)t.need >= least) continue;
+        bool has = false;
+        const uint64_t first = bt.first_idx + row_of(fused, q.lv[0], q.lv[1], q.lv[2], q.lv[3], q.lv[4]) * 9u;
+        for (int s = 0; s < 9; ++s)
+            has |= ((p.sm_mask >> s) & 1u) && first + (uint32_t)s < idx && mapping_key<OBJ>(p, lim, bt, t, s) == key;
+        if (has) least = (uint64_t)t.need;
+    }
+    bool in = true;
+    return warp_min_u64(least, in);
 }
 
 __device__ __forceinline__ longlong2 ld_volatile(const longlong2* a) {
@@ -379,11 +402,13 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
     return warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (warp == 2 && lane == 0 ? 31 : -1));
 }
 
-// The end of one search of the energy-latency front, by all threads of the last CTA: the least (energy, latency, block) of
-// all CTAs is the next point of the front.  It is left as a latency optimum under that energy, which is what
-// launch_resolve looks for in the block; the next search allows one word less of latency.
-__device__ __noinline__ void finalize_front(const Plan& p, Shared& sh, ChainRecord* chain_to, SearchHeader* __restrict__ head,
-                                            const Partial* __restrict__ partials, int n_partials) {
+// The end of a chained search, by all threads of the last CTA; its record is made later (launch_resolve).
+// FRONT: the least (energy, latency, block) of all CTAs is the next point of the energy-latency front.  It is left as a
+// latency optimum under that energy; the next search allows one word less of latency.
+// Else: the least (energy, block, buffer need); the next search allows one word of buffer less than that need.
+template <bool FRONT>
+__device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to,
+                                            SearchHeader* __restrict__ head, const Partial* __restrict__ partials, int n_partials) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int64_t ek = kInfKey, el = kInfKey;
     uint64_t ei = UINT64_MAX;
@@ -410,15 +435,17 @@ __device__ __noinline__ void finalize_front(const Plan& p, Shared& sh, ChainReco
     warp_min_triple(ek, el, ei);
     if (lane == 0) {
         const bool found = ek != kInfKey;
-        *chain_to = {(long long)(found ? el : kInfKey), (unsigned long long)ei, rows * p.n_sm, (long long)ek};
-        head->chain_bound = found ? el - 1 : -1;
+        const unsigned long long fit = rows * p.n_sm;
+        if (FRONT) *chain_to = {(long long)(found ? el : kInfKey), (unsigned long long)ei, fit, (long long)ek, 0, 0};
+        else *chain_to = {(long long)ek, (unsigned long long)el, fit, (long long)lim.cap_words, (long long)ei, 0};
+        head->chain_bound = !found ? -1 : (FRONT ? el : (int64_t)ei) - 1;
         head->done_ctas = 0;
     }
 }
 
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
 template <int OBJ, int MODE>
-__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to, SearchHeader* __restrict__ head,
+__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, SearchHeader* __restrict__ head,
                                            const Partial* __restrict__ partials, int n_partials,
                                            mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -476,30 +503,15 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         min_over_warps(sh, lane, warp, ek, ei);
         found = ek != kInfKey ? 1 : 0;
         bound = ek;
-        if (MODE == kModeChain && tid == 0) {
-            unsigned long long fit = 0;
-            for (int w = 0; w < kWarps; ++w) fit += sh.feasible_rows[w];
-            *chain_to = {(long long)ek, (unsigned long long)ei, fit * p.n_sm, (long long)lim.cap_words};
-            if (!found) head->chain_bound = -1;
-            head->done_ctas = 0;
-        }
         // ---- the winning block, mapping by mapping
         const int item = split_item(warp, lane);
         if (found && item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)ei, item, &sh.block[0]);
         __syncthreads();
         if (found) {
             n_groups = block_rows(sh.block[0]) / 5u;
-            best_of_block<OBJ>(p, lim, sh, bound, ek, ei);
+            best_of_block<OBJ, false>(p, lim, sh, bound, 0, ek, ei);
         }
         min_over_warps(sh, lane, warp, ek, ei);
-        if (MODE == kModeChain) {
-            // energy: the mapping itself, and one word of buffer less than it needs for the next search
-            if (tid == 0 && found) {
-                chain_to->where = ei;
-                head->chain_bound = block_need(sh.block[0], (uint32_t)((ei - sh.block[0].first_idx) / 9u)) - 1;
-            }
-            return;
-        }
     } else {
         merge_warps(sh, k, lane, warp, ek, ei);
         const longlong2 e = lane < kTopK ? sh.tops[0][lane] : make_longlong2(kInfKey, -1ll);
@@ -664,6 +676,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
     constexpr bool ARRAYS = MODE == kModeArrays;
     constexpr bool FRONT = CHAIN && OBJ == MMEE_OBJ_ENERGY_LCAP;      // least (energy, latency) under a bound on the latency
+    constexpr bool STAIRS = CHAIN && OBJ == MMEE_OBJ_ENERGY;          // least (energy, block, buffer need) under a capacity
+    static_assert(FRONT || STAIRS || !CHAIN, "only the searches of the Pareto fronts are chained");
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool late = shape.late;
@@ -693,7 +707,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
-    int64_t el = kInfKey;           // FRONT: its latency
+    int64_t el = kInfKey;           // FRONT: its latency.  STAIRS: (el, ei) are the block and its need
     unsigned long long my_rows = 0;
     uint32_t my_live = 0;
 
@@ -726,6 +740,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             bl = better ? l : bl;
         }
         if (valid && triple_less(be, bl, id, ek, el, ei)) { ek = be; el = bl; ei = id; }
+    };
+
+    auto offer_stairs = [&](int64_t key, uint32_t id, int need, bool valid) {
+        if (valid && triple_less(key, (int64_t)id, (uint64_t)need, ek, el, ei)) { ek = key; el = id; ei = (uint64_t)need; }
     };
 
     // The same for every array shape, one after the other: key_of_terms(terms) is the item's least key.
@@ -793,7 +811,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 lim.key_cap = bound;
             }
             if (bound < 0) {            // the search before found nothing: neither does this one, nor the next
-                if (blockIdx.x == 0 && tid == 0) *shape.chain_to = {kInfKey, 0, 0, -1};
+                if (blockIdx.x == 0 && tid == 0) *shape.chain_to = {kInfKey, 0, 0, -1, 0, 0};
                 return;
             }
         }
@@ -841,7 +859,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             if (fused) {
                 uint32_t rows;
                 int64_t x;
-                fused_class<PRUNE>(tb, oi, dw, (int)c, capc, PRUNE ? sh.kept.fused[os][c] : nullptr, any, rows, x);
+                int need;
+                fused_class<PRUNE, STAIRS>(tb, oi, dw, (int)c, capc, PRUNE ? sh.kept.fused[os][c] : nullptr, any, rows, x, need);
                 if (valid) my_rows += rows;
                 const bool some = valid && x < kNoRow;
                 if (any(some)) {
@@ -853,12 +872,14 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                     };
                     if (ARRAYS) offer_arrays(key, slot, id, some);
                     else if (FRONT) offer_front(pair, id, some);
+                    else if (STAIRS) offer_stairs(key(tb.st), id, need, some);
                     else offer(key(tb.st), id, some);
                 }
             } else {
                 uint32_t fit1, fit2, rows;
                 int64_t x1, x2;
-                unfused_nests<PRUNE>(tb, oi, dw, capc, fit1, fit2, rows, x1, x2);
+                int need;
+                unfused_nests<PRUNE, STAIRS>(tb, oi, dw, capc, fit1, fit2, rows, x1, x2, need);
                 const bool some = valid && x1 < kNoRow;
                 if (!any(some)) continue;
                 const int64_t y1 = some ? x1 : 0, y2 = some ? x2 : 0;
@@ -880,6 +901,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                     };
                     if (ARRAYS) offer_arrays(key, slot, id + block, some);
                     else if (FRONT) offer_front(pair, id + block, some);
+                    else if (STAIRS) offer_stairs(key(tb.st), id + block, need, some);
                     else offer(key(tb.st), id + block, some);
                     block += n_orders;
                 }
@@ -893,7 +915,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     if (lane == 0) sh.feasible_rows[warp] = my_rows;
     if (MULTI) {
         merge_warps(sh, k, lane, warp, ek, ei);
-    } else if (FRONT) {
+    } else if (CHAIN) {
         warp_min_triple(ek, el, ei);
         if (lane == 0) {
             sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
@@ -933,7 +955,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             g_end = __shfl_sync(kFull, g_end, 0);
             count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey && ek <= g_end));
             if (lane < (int)max(count, 1u)) out->e[lane] = make_longlong2((long long)ek, (long long)ei);
-        } else if (FRONT) {
+        } else if (CHAIN) {
             ek = sh.tops[lane & (kWarps - 1)][0].x;
             el = sh.tops[lane & (kWarps - 1)][0].y;
             ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
@@ -968,8 +990,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             release_next_kernel();
         }
         __threadfence();
-        if (FRONT) finalize_front(p, sh, shape.chain_to, head, partials, (int)grid);
-        else finalize_step<OBJ, MODE>(p, lim, sh, shape.chain_to, head, partials, (int)grid, out_best, out_topk);
+        if (CHAIN) finalize_chain<FRONT>(p, lim, sh, shape.chain_to, head, partials, (int)grid);
+        else finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
     }
 }
 
@@ -978,23 +1000,38 @@ __global__ void reset_kernel(SearchHeader* head) {
     head->done_ctas = 0;
 }
 
-// The full record of an optimum, by one CTA after load_shared: mapping `where`, or (IN_BLOCK) the first mapping with key
-// `key` of block `where`.  key kInfKey: nothing fits.
-template <int OBJ, bool IN_BLOCK>
+// The full record of an optimum, by one CTA after load_shared: the first mapping with key `key` of block `where`.  key
+// kInfKey: nothing fits.
+// STAIRS: the first one that also has the buffer need `need`, the least of them.  A search that returns the first mapping
+// with the least key and then searches on with one word less than that mapping's need would meet those with larger needs
+// before it: the record's n_feasible is the number of mappings that fit under the last bound of such a sequence.  Where
+// that is not the bound this one was found under, reserved2[0] says what it is, plus one (a rare case: index order
+// raises needs), and the caller searches there.
+template <int OBJ, bool STAIRS>
 __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim, Shared& sh,
-                                               int64_t key, uint64_t where, unsigned long long n_feasible, mmee_result_t* out) {
+                                               int64_t key, uint64_t where, unsigned long long n_feasible, int64_t need,
+                                               mmee_result_t* out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     mmee_result_t& r = sh.record[0];
+    uint32_t before_need = 0;
     if (key != kInfKey) {
-        int64_t ek = key;
-        uint64_t ei = where;
-        if (IN_BLOCK) {
-            const int item = split_item(warp, lane);
-            if (item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)where, item, &sh.block[0]);
-            __syncthreads();
-            best_of_block<OBJ>(p, lim, sh, key, ek, ei);
+        int64_t ek = kInfKey;
+        uint64_t ei = UINT64_MAX;
+        uint64_t before = UINT64_MAX;           // STAIRS: least need of a mapping with that key before the one found
+        const int item = split_item(warp, lane);
+        if (item >= 0) block_item(p, SharedDivisors{sh}, (uint32_t)where, item, &sh.block[0]);
+        __syncthreads();
+        if (STAIRS) {
+            best_of_block<OBJ, true>(p, lim, sh, key, need, ek, ei);
+            min_over_warps(sh, lane, warp, ek, ei);
+            before = least_need_before<OBJ>(p, lim, sh, key, ei);
+            int64_t zero = 0;
+            min_over_warps(sh, lane, warp, zero, before);
+        } else {
+            best_of_block<OBJ, false>(p, lim, sh, key, 0, ek, ei);
             min_over_warps(sh, lane, warp, ek, ei);
         }
+        if (before != UINT64_MAX) before_need = (uint32_t)before;
         if (warp == 0) {
             const bool have = ek == key;
             evaluate_candidate_lanes<32>(p, SharedDivisors{sh}, have ? ei : 0, lim.cap_words, lane, lane == 0, r);
@@ -1016,6 +1053,7 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
         if (lane == 0) {
             r.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
             r.n_feasible = n_feasible;
+            if (STAIRS) r.reserved2[0] = before_need;
         }
         __syncwarp();
         const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
@@ -1033,9 +1071,9 @@ resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* chain, mmee_re
     wait_previous_kernel();
     // (volatile: read after the wait, not as data that no kernel writes meanwhile)
     const volatile ChainRecord* from = chain + blockIdx.x;
-    const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound};
+    const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound, from->need, 0};
     const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
-    resolve_record<OBJ, OBJ != MMEE_OBJ_ENERGY>(p, lim, sh, c.key, c.where, c.n_feasible, out + blockIdx.x);
+    resolve_record<OBJ, OBJ == MMEE_OBJ_ENERGY>(p, lim, sh, c.key, c.where, c.n_feasible, c.need, out + blockIdx.x);
 }
 
 // Merge of the CTAs' best items of array shape blockIdx.x, and the record of the optimum.
@@ -1063,8 +1101,7 @@ resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, c
     min_over_warps(sh, lane, warp, ek, ei);
     rows = 0;
     for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
-    resolve_record<OBJ, true>(p, Limits{p.cap_words, p.key_cap}, sh, ek, ei,
-                              rows * p.n_sm, out + blockIdx.x);
+    resolve_record<OBJ, false>(p, Limits{p.cap_words, p.key_cap}, sh, ek, ei, rows * p.n_sm, 0, out + blockIdx.x);
 }
 
 // A launch that may start before the kernel before it on the stream has ended (`overlap`): the kernel waits itself.

@@ -39,13 +39,15 @@ struct Scratch {
 
 constexpr uint32_t kMaxArrays = MMEE_MAX_TOPK;      // one entry of a partial list each
 
-// What a chained search leaves of its optimum: key kInfKey if nothing fits; an energy search its key, the mapping's index
-// and the buffer words it was found under; a search of the energy-latency front the latency, the block and the energy.
+// What a chained search leaves of its optimum: key kInfKey if nothing fits; an energy search its key, the block, the buffer
+// words it was found under and the least need of a mapping of the block with that key; a search of the energy-latency
+// front the latency, the block and the energy.
 struct ChainRecord {
     long long key;
     unsigned long long where;
     unsigned long long n_feasible;
     long long bound;
+    long long need, pad;
 };
 
 struct LaunchShape {

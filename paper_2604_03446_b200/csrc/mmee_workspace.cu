@@ -37,7 +37,7 @@ int make_workspace(int device, Workspace** out) {
     int rc = max_search_ctas(device, &ws->max_ctas);
     if (rc) { delete ws; return rc; }
     // one allocation: the chained searches' optima, then the two scratches
-    static_assert(sizeof(ChainRecord) == 32, "a multiple of 16 bytes keeps the scratches aligned");
+    static_assert(sizeof(ChainRecord) == 48, "a multiple of 16 bytes keeps the scratches aligned");
     const size_t chain = kHostRecords * sizeof(ChainRecord), bytes = scratch_bytes(ws->max_ctas);
     unsigned char* mem = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), chain + 2 * bytes);

@@ -137,6 +137,27 @@ def test_buffer_size_dram_traffic_pareto_front(seed):
         assert r.e_key == r.n[0]                # the search's key was the DRAM word count
 
 
+@pytest.mark.parametrize("seed", [1, 4, 5, 7, 9, 10, 13, 21])
+def test_chained_front_equals_one_search_after_the_other(seed):
+    """The buffer-size / DRAM-traffic front takes its searches' bounds from the device, block by block; its records are
+    those of plain searches, each allowed one word of buffer less than the mapping before it needs, byte for byte (the
+    count of fitting mappings included, which depends on the bound a point was found under)."""
+    cfg = mi.random_tiny_problem(seed)
+    obj = shrink_to(cfg, dict(cfg["searches"][0], objective=mi.OBJ_ENERGY, topk=1), 1_000_000)
+    wb = cfg["workload"]["word_bytes"]
+    arch = dict(cfg["arch"], e_dram_pj=1.0, e_gb_pj=0.0, e_rf_pj=0.0, e_mac_pj=0.0, c_softmax=0.0, energy_quantum_pj=1.0)
+    want, held, cap = [], None, arch["gb_bytes"] // wb
+    while cap > 0:
+        r = mm.mmee_solve_host(cfg["workload"], dict(arch, gb_bytes=cap * wb), obj)[0]
+        if held is not None and (r.idx == mm.NO_INDEX or r.e_key != held.e_key):
+            want.append(bytes(held))
+        if r.idx == mm.NO_INDEX:
+            break
+        held, cap = r, r.bs - 1
+    got = mm.mmee_pareto_front_bs_da(cfg["workload"], cfg["arch"], obj)
+    assert [bytes(r) for r in got] == want and len(want) >= 2
+
+
 def test_buffer_size_dram_traffic_front_of_the_ffn_task():
     """On the fused feed-forward GEMMs of the paper's buffer-size study the front is a staircase: strictly less
     buffer and strictly more traffic from point to point, no point above the buffer, the last one at the
