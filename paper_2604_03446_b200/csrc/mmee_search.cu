@@ -144,6 +144,7 @@ struct Shared {
     unsigned long long feasible_rows[kWarps];
     uint32_t live_tilings[kWarps];
     uint32_t n_live;                // tilings of the current pass that can fit
+    uint32_t n_fit;                 // STAIRS: those of them that fit under the bound of the search before
     uint32_t cursor;                // next group of 32 items
     uint32_t last_cta, check_failed;
     union {
@@ -687,8 +688,11 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     // the warps' best items of shape y in sh.tops[.][y].
     StatTerms* terms = reinterpret_cast<StatTerms*>(&sh.tile[shape.chunk]);
     if (ARRAYS && tid < kWarps * (int)MMEE_MAX_TOPK) sh.tops[tid / (int)MMEE_MAX_TOPK][tid % (int)MMEE_MAX_TOPK] = make_longlong2(kInfKey, -1ll);
+    // STAIRS: the table slots of the tilings that fit under the bound, where the kept rows of the other modes lie.
+    uint8_t* fit_slots = reinterpret_cast<uint8_t*>(&sh.kept);
+    static_assert(kMaxChunk <= 256 && kMaxChunk <= sizeof(KeptMasks), "one byte per table");
     if (tid == 0) {
-        sh.n_live = 0;
+        sh.n_live = sh.n_fit = 0;
         sh.cursor = 0;
         sh.check_failed = 0;
     }
@@ -766,7 +770,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     for (uint32_t m0 = 0; (uint64_t)m0 * grid < n_tilings; m0 += shape.chunk) {
         if (m0) {
             __syncthreads();                // the previous pass's tables are no longer in use
-            if (tid == 0) { sh.n_live = 0; sh.cursor = 0; }
+            if (tid == 0) { sh.n_live = sh.n_fit = 0; sh.cursor = 0; }
             __syncthreads();
         }
         for (uint32_t j0 = 0; j0 < shape.chunk; j0 += kSearchThreads / 8) {
@@ -830,8 +834,19 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             __syncthreads();
         }
 
-        const uint32_t per_class = sh.n_live * n_orders;
-        if (tid == 0) my_live += sh.n_live;
+        if (STAIRS) {
+            // The tables were made while the search before was still under way, for the bound the plan has.  (Front of
+            // the GPT-3 FFN, twenty searches: 281 us with items for every table, 263 with this.)
+            if ((uint32_t)tid < sh.n_live) {
+                const uint32_t* b = sh.tile[tid].b;
+                const uint64_t tc = (uint64_t)b[4] * b[6];
+                const uint64_t first = (uint64_t)b[4] * b[5] + (uint64_t)b[5] * b[6], second = (uint64_t)b[6] * b[7] + (uint64_t)b[4] * b[7];
+                if (tc + max(first, second) <= (uint64_t)capc) fit_slots[atomicAdd(&sh.n_fit, 1u)] = (uint8_t)tid;
+            }
+            __syncthreads();
+        }
+        const uint32_t n_tiles = STAIRS ? sh.n_fit : sh.n_live, per_class = n_tiles * n_orders;
+        if (tid == 0) my_live += n_tiles;
         const uint32_t fused_items = (p.fuse_mask & 1u) ? 3u * per_class : 0u;
         const uint32_t fused_groups = (fused_items + 31u) / 32u;
         const uint32_t groups = fused_groups + ((p.fuse_mask & 6u) ? (per_class + 31u) / 32u : 0u);
@@ -852,7 +867,9 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 c = i >= 2u * per_class ? 2u : (i >= per_class ? 1u : 0u);
                 i -= c * per_class;
             }
-            const uint32_t slot = n_orders == 6u ? i / 6u : i / 2u, os = i - slot * n_orders;
+            uint32_t slot = n_orders == 6u ? i / 6u : i / 2u;
+            const uint32_t os = i - slot * n_orders;
+            if (STAIRS) slot = fit_slots[slot];
             const TileTab& tb = sh.tile[slot];
             const OrderInfo& oi = sh.order[os];
             const uint32_t id = tb.t * p.n_blocks + os;
