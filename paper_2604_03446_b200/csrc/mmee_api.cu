@@ -62,10 +62,11 @@ int max_search_ctas(int device, uint32_t* out) {
     return MMEE_OK;
 }
 
-int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape) {
+int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape, uint32_t spare) {
     uint32_t most = 0;
     const int rc = max_search_ctas(device, &most);
     if (rc) return rc;
+    most = most > spare ? most - spare : 1;
     // Small problems take fewer CTAs, with at least eight tilings each.
     const uint64_t tilings = p.t_end - p.t_begin;
     constexpr uint64_t kMinTilings = 8;
@@ -82,7 +83,8 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
     shape->n_arrays = n_arrays;
     shape->overlap = true;
     shape->late = n_arrays == 0 && (p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling));
-    shape->chain = shape->chain_read = false;
+    shape->chain_steps = shape->chain_epoch = 0;
+    shape->chain_read = false;
     shape->chain_to = nullptr;
     shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
     return MMEE_OK;
@@ -92,43 +94,34 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
 
 namespace {
 
-// Searches chained on the device (see LaunchShape::chain) until one finds nothing: their optima in order, through `take`
-// (which returns false to stop).  The host waits for a batch of them at a time, first `first_batch`, then twice as many as
-// before; what is launched beyond the last one ends at once.  The records are made with the plan `records`.
+// Searches chained on the device (see LaunchShape::chain_steps) until one finds nothing: their optima in order, through
+// `take` (which returns false to stop).  The host waits for kHostRecords of them at a time.
 template <class Take>
-int run_chain(const Plan& plan, const Plan& records, uint32_t first_batch, Take take) {
+int run_chain(const Plan& plan, Take take) {
     int device = 0;
     int rc = cuda_status(cudaGetDevice(&device));
     if (rc) return rc;
     LaunchShape shape;
-    if ((rc = choose_launch_shape(plan, device, 0, 0, &shape))) return rc;
+    if ((rc = choose_launch_shape(plan, device, 0, 0, &shape, kRecordCtas - 1))) return rc;
     Workspace* ws = nullptr;
     if ((rc = workspace_acquire(device, &ws))) return rc;
-    bool clean = true, more = true;
-    uint32_t step = 0;
-    for (uint32_t batch = first_batch; more && rc == MMEE_OK; batch = 2 * batch < kHostRecords ? 2 * batch : kHostRecords) {
-        uint32_t n = 0;
-        for (; n < batch && rc == MMEE_OK; ++n) {
-            shape.chain = true;
-            shape.late = false;
-            shape.chain_read = step + n > 0;
-            shape.chain_to = ws->chain + n;
-            rc = cuda_status(launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial,
-                                           nullptr, nullptr, nullptr));
-        }
-        if (rc == MMEE_OK) rc = cuda_status(launch_resolve(records, ws->chain, n, ws->host_dev, nullptr));
-        if (rc) clean = false;
+    shape.late = false;
+    shape.chain_steps = kHostRecords;
+    shape.chain_to = ws->chain;
+    bool more = true;
+    while (more && rc == MMEE_OK) {
+        shape.chain_epoch = ++ws->chains * kHostRecords;
+        rc = cuda_status(launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial, nullptr, ws->host_dev, nullptr));
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
-        if (rc2) clean = false;
         if (rc == MMEE_OK) rc = rc2;
-        for (uint32_t i = 0; i < n && more && rc == MMEE_OK; ++i) {
+        for (uint32_t i = 0; i < kHostRecords && more && rc == MMEE_OK; ++i) {
             const mmee_result_t& r = ws->host[i];
             if (r.status == MMEE_ERR_CHECK) { rc = MMEE_ERR_CHECK; break; }
             more = r.idx != MMEE_NO_INDEX && take(r);
         }
-        step += n;
+        shape.chain_read = true;
     }
-    const int rc2 = workspace_release(ws, clean);
+    const int rc2 = workspace_release(ws, rc == MMEE_OK);
     return rc ? rc : rc2;
 }
 
@@ -308,16 +301,14 @@ int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch, 
     *n_points = 0;
     mmee_objective_t o = *objective;
     o.topk = 1; o.row_pruning = 0; o.key_cap = INT64_MAX - 1;
-    Plan plan, records;
-    int rc;
     o.objective = MMEE_OBJ_ENERGY_LCAP;
-    if ((rc = build_plan(workload, arch, &o, &plan))) return rc;
-    o.objective = MMEE_OBJ_LATENCY_ECAP;
-    if ((rc = build_plan(workload, arch, &o, &records))) return rc;
+    Plan plan;
+    int rc = build_plan(workload, arch, &o, &plan);
+    if (rc) return rc;
     uint32_t n = 0;
     // Each search finds the least energy among the mappings that are still faster than the previous point, and the least
     // latency at that energy: the next point of the front, with its lowest index.  None: the front is complete.
-    rc = run_chain(plan, records, 3, [&](const mmee_result_t& r) {
+    rc = run_chain(plan, [&](const mmee_result_t& r) {
         if (n < capacity) out_points[n] = r;
         ++n;
         return true;
@@ -350,11 +341,11 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
         if (n < capacity) out_points[n] = held;
         ++n;
     };
-    rc = run_chain(plan, plan, 8, [&](const mmee_result_t& r) {
+    rc = run_chain(plan, [&](const mmee_result_t& r) {
         if (have && r.e_key != held.e_key) emit();
         held = r;
         have = true;
-        plan.cap_words = r.bs - 1;      // (for the tables of the next batch: tilings that cannot fit are left out)
+        plan.cap_words = r.bs - 1;      // (for the tables of the next chain: tilings that cannot fit are left out)
         return plan.cap_words >= 0;
     });
     if (rc == MMEE_OK && have) emit();

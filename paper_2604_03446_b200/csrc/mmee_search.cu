@@ -145,6 +145,7 @@ struct Shared {
     uint32_t live_tilings[kWarps];
     uint32_t n_live;                // tilings of the current pass that can fit
     uint32_t n_fit;                 // STAIRS: those of them that fit under the bound of the search before
+    long long bound;                // chained searches: that bound
     uint32_t cursor;                // next group of 32 items
     uint32_t last_cta, check_failed;
     union {
@@ -403,12 +404,31 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
     return warp == 0 ? (lane < 25 ? lane : -1) : (warp == 1 ? (lane < 6 ? 25 + lane : -1) : (warp == 2 && lane == 0 ? 31 : -1));
 }
 
-// The end of a chained search, by all threads of the last CTA; its record is made later (launch_resolve).
+// Chained searches run one after the other in one kernel, whose CTAs are all resident (a cooperative launch): a CTA that
+// has published its part of one waits for the CTA that merges the parts, which sets the header's epoch to that search's
+// when it has left the bound for the next.  kRecordCtas more make the records meanwhile.  The wait is limited, at a few
+// seconds; true: the search is over.
+// Steps of about 8 us are bound by publish, ticket, merge and this wait, the first of a large front by their items.  Front of
+// the GPT-3 FFN (20 searches), a launch per search that waited for the one before 264 us, steps of one kernel 202;
+// 99 random fronts 241 and 198 us; the energy-latency front of 10 816 tilings 56.5 and 55.3.
+constexpr uint32_t kMaxPolls = 1u << 22;
+constexpr int64_t kNoBound = INT64_MIN;         // what a search leaves that found nothing
+
+__device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t epoch) {
+    for (uint32_t i = 0; i < kMaxPolls; ++i) {
+        uint32_t now;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&head->chain_epoch) : "memory");
+        if ((int32_t)(now - epoch) >= 0) return true;
+    }
+    return false;
+}
+
+// The end of a chained search, by all threads of the last CTA; its record is made after the chain.
 // FRONT: the least (energy, latency, block) of all CTAs is the next point of the energy-latency front.  It is left as a
 // latency optimum under that energy; the next search allows one word less of latency.
 // Else: the least (energy, block, buffer need); the next search allows one word of buffer less than that need.
 template <bool FRONT>
-__device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to,
+__device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to, uint32_t epoch,
                                             SearchHeader* __restrict__ head, const Partial* __restrict__ partials, int n_partials) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int64_t ek = kInfKey, el = kInfKey;
@@ -434,13 +454,14 @@ __device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Sh
     el = sh.tops[lane & (kWarps - 1)][0].y;
     ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
     warp_min_triple(ek, el, ei);
+    const bool found = ek != kInfKey;
     if (lane == 0) {
-        const bool found = ek != kInfKey;
         const unsigned long long fit = rows * p.n_sm;
         if (FRONT) *chain_to = {(long long)(found ? el : kInfKey), (unsigned long long)ei, fit, (long long)ek, 0, 0};
         else *chain_to = {(long long)ek, (unsigned long long)el, fit, (long long)lim.cap_words, (long long)ei, 0};
-        head->chain_bound = !found ? -1 : (FRONT ? el : (int64_t)ei) - 1;
+        head->chain_bound = !found ? kNoBound : (FRONT ? el : (int64_t)ei) - 1;
         head->done_ctas = 0;
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&head->chain_epoch), "r"(epoch) : "memory");
     }
 }
 
@@ -639,384 +660,6 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
     }
 }
 
-// ------------------------------------------------------------------------------------------------
-// the search kernel
-// ------------------------------------------------------------------------------------------------
-
-// Searches launched one after the other overlap (programmatic dependent launch), in one of two ways.
-//   early: a search lets the next one start at once; that one's CTAs move in as this one's leave, and wait for its end
-//          before they publish (k > 1, chained: before their items), since it may still use their scratch;
-//   late:  only the CTA that finalizes waits for the kernel before, and lets the next search start after that wait.  The
-//          CTAs then publish while the search before finalizes, into the other one of the handle's two scratches: the
-//          search that used theirs last had ended before the one before them let them start.
-// A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  Searches one after
-// the other, without and with this (us each): smallest configuration 20.5 and 8.9, BERT energy 22.9 and 10.4, GQA latency
-// 28.7 and 13.7, convolution chain top-16 133 and 58 (other changes between them included).
-__device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
-// and the sizes between them.
-template <bool TERMS>
-__device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
-    if (TERMS && sub < 6) {
-        const int op = sub >= 3 ? 1 : 0, sm = sub - 3 * op;
-        int64_t P, Q;
-        stationary_terms(p, SharedDivisors{sh}, b, op, sm, P, Q);
-        (op ? tb->st.P2 : tb->st.P1)[sm] = P;
-        (op ? tb->st.Q2 : tb->st.Q1)[sm] = Q;
-    }
-    for (int i = sub; i < kSizeSlots; i += 8) tb->size[i] = sat_size(size_words(p.dim, tb->b + 4, i));
-    if (sub == 7) tb->t = t;
-}
-
-template <int OBJ, int MODE>
-__global__ void __launch_bounds__(kSearchThreads, 2)
-search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ head, Partial* __restrict__ partials,
-              mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
-    constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
-    constexpr bool ARRAYS = MODE == kModeArrays;
-    constexpr bool FRONT = CHAIN && OBJ == MMEE_OBJ_ENERGY_LCAP;      // least (energy, latency) under a bound on the latency
-    constexpr bool STAIRS = CHAIN && OBJ == MMEE_OBJ_ENERGY;          // least (energy, block, buffer need) under a capacity
-    static_assert(FRONT || STAIRS || !CHAIN, "only the searches of the Pareto fronts are chained");
-    __shared__ Shared sh;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool late = shape.late;
-    if (!late) release_next_kernel();
-    load_shared<PRUNE>(p, p.pe_rows, p.pe_cols, sh);
-    // Array shapes: the stationary-pair terms of shape y and tiling slot i at [y * chunk + i], behind the tilings' tables;
-    // the warps' best items of shape y in sh.tops[.][y].
-    StatTerms* terms = reinterpret_cast<StatTerms*>(&sh.tile[shape.chunk]);
-    if (ARRAYS && tid < kWarps * (int)MMEE_MAX_TOPK) sh.tops[tid / (int)MMEE_MAX_TOPK][tid % (int)MMEE_MAX_TOPK] = make_longlong2(kInfKey, -1ll);
-    // STAIRS: the table slots of the tilings that fit under the bound, where the kept rows of the other modes lie.
-    uint8_t* fit_slots = reinterpret_cast<uint8_t*>(&sh.kept);
-    static_assert(kMaxChunk <= 256 && kMaxChunk <= sizeof(KeptMasks), "one byte per table");
-    if (tid == 0) {
-        sh.n_live = sh.n_fit = 0;
-        sh.cursor = 0;
-        sh.check_failed = 0;
-    }
-    __syncthreads();
-
-    const int k = MULTI ? (int)p.topk : 1;
-    const int64_t I = p.dim[0], K = p.dim[1], L = p.dim[2], J = p.dim[3];
-    const DimWords dw = {I * K, K * L, L * J, I * J, I * L};
-    // (a chained search: the bound that the search before it left, read before the items)
-    Limits lim = {p.cap_words, p.key_cap};
-    int capc = (int)p.cap_words;
-    const uint32_t grid = gridDim.x, n_tilings = (uint32_t)(p.t_end - p.t_begin);
-    const uint32_t n_orders = p.n_orders;
-    auto any = [](bool v) { return __any_sync(kFull, v) != 0; };
-
-    // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
-    int64_t ek = kInfKey;
-    uint64_t ei = UINT64_MAX;
-    int64_t el = kInfKey;           // FRONT: its latency.  STAIRS: (el, ei) are the block and its need
-    unsigned long long my_rows = 0;
-    uint32_t my_live = 0;
-
-    auto offer = [&](int64_t key, uint32_t id, bool valid) {
-        if (!MULTI) {
-            if (valid && pair_less(key, id, ek, ei)) { ek = key; ei = id; }
-            return;
-        }
-        const int64_t lk = __shfl_sync(kFull, ek, k - 1);
-        const uint64_t li = __shfl_sync(kFull, ei, k - 1);
-        const bool pend = valid && key != kInfKey && key <= *reinterpret_cast<volatile long long*>(&sh.G) && pair_less(key, id, lk, li);
-        if (!__any_sync(kFull, pend)) return;
-        warp_offer(ek, ei, k, key, id, pend, lane);
-        // a full list bounds the k-th smallest key for everybody
-        if (lane == k - 1 && ek < *reinterpret_cast<volatile long long*>(&sh.G)) {
-            atomicMin(&sh.G, (long long)ek);
-            atomicMin(&head->G, (long long)ek);
-        }
-    };
-
-    // FRONT: the item's least (energy, latency) over the stationary pairs; pair(s, e, l) forms those of pair s.
-    auto offer_front = [&](auto pair, uint32_t id, bool valid) {
-        int64_t be = kInfKey, bl = kInfKey;
-#pragma unroll
-        for (int s = 0; s < 9; ++s) {
-            int64_t e, l;
-            pair(s, e, l);
-            const bool better = ((p.sm_mask >> s) & 1u) && l <= lim.key_cap && (e < be || (e == be && l < bl));
-            be = better ? e : be;
-            bl = better ? l : bl;
-        }
-        if (valid && triple_less(be, bl, id, ek, el, ei)) { ek = be; el = bl; ei = id; }
-    };
-
-    auto offer_stairs = [&](int64_t key, uint32_t id, int need, bool valid) {
-        if (valid && triple_less(key, (int64_t)id, (uint64_t)need, ek, el, ei)) { ek = key; el = id; ei = (uint64_t)need; }
-    };
-
-    // The same for every array shape, one after the other: key_of_terms(terms) is the item's least key.
-    auto offer_arrays = [&](auto key_of_terms, uint32_t slot, uint32_t id, bool valid) {
-        for (uint32_t y = 0; y < shape.n_arrays; ++y) {
-            const int64_t key = key_of_terms(terms[y * shape.chunk + slot]);
-            const longlong2 own = sh.tops[warp][y];
-            const bool better = valid && pair_less(key, id, own.x, (uint64_t)own.y);
-            if (!any(better)) continue;
-            int64_t nk = better ? key : kInfKey;
-            uint64_t ni = better ? id : UINT64_MAX;
-            warp_min_pair(nk, ni);
-            if (lane == 0) sh.tops[warp][y] = make_longlong2((long long)nk, (long long)ni);
-            __syncwarp();
-        }
-    };
-
-    // Tiling number m of this CTA is one of the m-th `grid` consecutive ones, a different one in every round (a fixed
-    // one would be the same divisor of the last dimension again and again).
-    for (uint32_t m0 = 0; (uint64_t)m0 * grid < n_tilings; m0 += shape.chunk) {
-        if (m0) {
-            __syncthreads();                // the previous pass's tables are no longer in use
-            if (tid == 0) { sh.n_live = sh.n_fit = 0; sh.cursor = 0; }
-            __syncthreads();
-        }
-        for (uint32_t j0 = 0; j0 < shape.chunk; j0 += kSearchThreads / 8) {
-            const uint32_t j = j0 + (uint32_t)tid / 8u, m = m0 + j;
-            uint64_t rel = (uint64_t)m * grid;
-            const bool mine = j < shape.chunk && rel < n_tilings;
-            rel += (blockIdx.x + m) % grid;
-            uint32_t b[8], t = 0;
-            bool live = mine && rel < n_tilings;
-            if (live) {
-                t = (uint32_t)(p.t_begin + rel);
-                tiling_bounds(p, SharedDivisors{sh}, t, b);
-                // With every operand at L3 the buffer need is smallest: max(A+B+C, C+D+E) tiles (Eq. 1-4).
-                const uint64_t ta = (uint64_t)b[4] * b[5], tbb = (uint64_t)b[5] * b[6], tc = (uint64_t)b[4] * b[6];
-                const uint64_t td = (uint64_t)b[6] * b[7], te = (uint64_t)b[4] * b[7];
-                live = ta + tbb + tc <= (uint64_t)capc && tc + td + te <= (uint64_t)capc;
-            }
-            uint32_t slot = 0;
-            if (live && (tid & 7) == 0) slot = atomicAdd(&sh.n_live, 1u);
-            slot = __shfl_sync(kFull, slot, lane & ~7);
-            if (live) {
-                uint32_t own = b[0];
-#pragma unroll
-                for (int d = 1; d < 8; ++d) own = (tid & 7) == d ? b[d] : own;
-                sh.tile[slot].b[tid & 7] = own;
-            }
-            __syncwarp();
-            if (live) build_tile<!ARRAYS>(p, sh, b, t, tid & 7, &sh.tile[slot]);
-        }
-        if (MULTI && m0 == 0) {
-            // (k > 1 shares a bound through the scratch while it works on the items)
-            if (!late) wait_previous_kernel();
-            if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
-        }
-        if (CHAIN && shape.chain_read && m0 == 0) {
-            wait_previous_kernel();
-            const int64_t bound = *reinterpret_cast<volatile long long*>(&head->chain_bound);
-            if (OBJ == MMEE_OBJ_ENERGY) {
-                lim.cap_words = bound;
-                capc = (int)bound;
-            } else {
-                lim.key_cap = bound;
-            }
-            if (bound < 0) {            // the search before found nothing: neither does this one, nor the next
-                if (blockIdx.x == 0 && tid == 0) *shape.chain_to = {kInfKey, 0, 0, -1, 0, 0};
-                return;
-            }
-        }
-        __syncthreads();
-        if (ARRAYS) {
-            const uint32_t n_live = sh.n_live;
-            for (uint32_t i = tid; i < n_live * 6u * shape.n_arrays; i += kSearchThreads) {
-                const uint32_t y = i / (n_live * 6u), u = i - y * n_live * 6u, slot = u / 6u;
-                const int op = u - slot * 6u >= 3u ? 1 : 0, sm = (int)(u - slot * 6u) - 3 * op;
-                StatTerms& st = terms[y * shape.chunk + slot];
-                int64_t P, Q;
-                stationary_terms(p, ArrayDivisors{sh, shape.array[y][0], shape.array[y][1]}, sh.tile[slot].b, op, sm, P, Q);
-                (op ? st.P2 : st.P1)[sm] = P;
-                (op ? st.Q2 : st.Q1)[sm] = Q;
-            }
-            __syncthreads();
-        }
-
-        if (STAIRS) {
-            // The tables were made while the search before was still under way, for the bound the plan has.  (Front of
-            // the GPT-3 FFN, twenty searches: 281 us with items for every table, 263 with this.)
-            if ((uint32_t)tid < sh.n_live) {
-                const uint32_t* b = sh.tile[tid].b;
-                const uint64_t tc = (uint64_t)b[4] * b[6];
-                const uint64_t first = (uint64_t)b[4] * b[5] + (uint64_t)b[5] * b[6], second = (uint64_t)b[6] * b[7] + (uint64_t)b[4] * b[7];
-                if (tc + max(first, second) <= (uint64_t)capc) fit_slots[atomicAdd(&sh.n_fit, 1u)] = (uint8_t)tid;
-            }
-            __syncthreads();
-        }
-        const uint32_t n_tiles = STAIRS ? sh.n_fit : sh.n_live, per_class = n_tiles * n_orders;
-        if (tid == 0) my_live += n_tiles;
-        const uint32_t fused_items = (p.fuse_mask & 1u) ? 3u * per_class : 0u;
-        const uint32_t fused_groups = (fused_items + 31u) / 32u;
-        const uint32_t groups = fused_groups + ((p.fuse_mask & 6u) ? (per_class + 31u) / 32u : 0u);
-        while (true) {
-            uint32_t g = 0;
-            if (lane == 0) g = atomicAdd(&sh.cursor, 1u);
-            g = __shfl_sync(kFull, g, 0);
-            if (g >= groups) break;
-            long long g_seen = 0;       // k > 1: the other CTAs' bound, used after this item
-            if (MULTI && lane == 0) g_seen = *reinterpret_cast<volatile long long*>(&head->G);
-            const bool fused = g < fused_groups;
-            uint32_t i = (fused ? g : g - fused_groups) * 32u + (uint32_t)lane;
-            const uint32_t n_items = fused ? fused_items : per_class;
-            const bool valid = i < n_items;
-            i = valid ? i : n_items - 1;
-            uint32_t c = 0;
-            if (fused) {
-                c = i >= 2u * per_class ? 2u : (i >= per_class ? 1u : 0u);
-                i -= c * per_class;
-            }
-            uint32_t slot = n_orders == 6u ? i / 6u : i / 2u;
-            const uint32_t os = i - slot * n_orders;
-            if (STAIRS) slot = fit_slots[slot];
-            const TileTab& tb = sh.tile[slot];
-            const OrderInfo& oi = sh.order[os];
-            const uint32_t id = tb.t * p.n_blocks + os;
-            if (fused) {
-                uint32_t rows;
-                int64_t x;
-                int need;
-                fused_class<PRUNE, STAIRS>(tb, oi, dw, (int)c, capc, PRUNE ? sh.kept.fused[os][c] : nullptr, any, rows, x, need);
-                if (valid) my_rows += rows;
-                const bool some = valid && x < kNoRow;
-                if (any(some)) {
-                    const int64_t y = some ? x : 0, rho = oi.recompute[c] != 0 ? (int64_t)tb.b[LOOP_J] : 1;
-                    auto key = [&](const StatTerms& t) { return fused_least_key<OBJ>(t, y, rho, p.sm_mask, p.c_dram_gb, lim.key_cap); };
-                    auto pair = [&](int s, int64_t& e, int64_t& l) {
-                        e = p.c_dram_gb * y + tb.st.P1[s / 3] * rho + tb.st.P2[s % 3];
-                        l = max64(y, tb.st.Q1[s / 3] * rho + tb.st.Q2[s % 3]);
-                    };
-                    if (ARRAYS) offer_arrays(key, slot, id, some);
-                    else if (FRONT) offer_front(pair, id, some);
-                    else if (STAIRS) offer_stairs(key(tb.st), id, need, some);
-                    else offer(key(tb.st), id, some);
-                }
-            } else {
-                uint32_t fit1, fit2, rows;
-                int64_t x1, x2;
-                int need;
-                unfused_nests<PRUNE, STAIRS>(tb, oi, dw, capc, fit1, fit2, rows, x1, x2, need);
-                const bool some = valid && x1 < kNoRow;
-                if (!any(some)) continue;
-                const int64_t y1 = some ? x1 : 0, y2 = some ? x2 : 0;
-                uint32_t block = p.n_fused_blocks;
-#pragma unroll
-                for (int phi = 1; phi <= 2; ++phi) {
-                    if (!((p.fuse_mask >> phi) & 1u)) continue;
-                    if (PRUNE) {
-                        rows = 0;
-                        for (int ab = 0; ab < 9; ++ab)
-                            if ((fit1 >> ab) & 1u) rows += (uint32_t)__popc(fit2 & sh.kept.unfused[phi - 1][os][ab]);
-                    }
-                    if (some) my_rows += rows;
-                    const int64_t pass = phi == 2 ? 2 * dw.il : 0;
-                    auto key = [&](const StatTerms& t) { return unfused_least_key<OBJ>(t, y1, y2, pass, p.sm_mask, p.c_dram_gb, lim.key_cap); };
-                    auto pair = [&](int s, int64_t& e, int64_t& l) {
-                        e = p.c_dram_gb * (y1 + y2 + pass) + tb.st.P1[s / 3] + tb.st.P2[s % 3];
-                        l = max64(y1, tb.st.Q1[s / 3]) + pass + max64(y2, tb.st.Q2[s % 3]);
-                    };
-                    if (ARRAYS) offer_arrays(key, slot, id + block, some);
-                    else if (FRONT) offer_front(pair, id + block, some);
-                    else if (STAIRS) offer_stairs(key(tb.st), id + block, need, some);
-                    else offer(key(tb.st), id + block, some);
-                    block += n_orders;
-                }
-            }
-            if (MULTI && lane == 0 && g_seen < sh.G) atomicMin(&sh.G, g_seen);
-        }
-    }
-
-    // ---- this CTA's result
-    for (int off = 16; off; off >>= 1) my_rows += __shfl_down_sync(kFull, my_rows, off);
-    if (lane == 0) sh.feasible_rows[warp] = my_rows;
-    if (MULTI) {
-        merge_warps(sh, k, lane, warp, ek, ei);
-    } else if (CHAIN) {
-        warp_min_triple(ek, el, ei);
-        if (lane == 0) {
-            sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
-            sh.tops[warp][1] = make_longlong2((long long)ei, 0);
-        }
-        __syncthreads();
-    } else if (!ARRAYS) {
-        warp_min_pair(ek, ei);
-        if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)ek, (long long)ei);
-        __syncthreads();
-    }
-    if (!late) wait_previous_kernel();      // from here on the scratch is touched
-    if (ARRAYS) {
-        // the best item of every shape; the kernel that follows merges them (resolve_arrays_kernel)
-        __syncthreads();
-        Partial* out = &partials[blockIdx.x];
-        for (uint32_t y = warp; y < shape.n_arrays; y += kWarps) {
-            const longlong2 v = sh.tops[lane & (kWarps - 1)][y];
-            int64_t nk = v.x;
-            uint64_t ni = (uint64_t)v.y;
-            warp_min_pair(nk, ni);
-            if (lane == 0) out->e[y] = make_longlong2((long long)nk, (long long)ni);
-        }
-        if (tid == 0) {
-            unsigned long long rows = 0;
-            for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
-            out->feasible_rows = rows;
-        }
-        return;
-    }
-    if (warp == 0) {
-        Partial* out = &partials[blockIdx.x];
-        uint32_t count;
-        if (MULTI) {
-            // an entry above the bound (some full list's last key) is not among the k best
-            long long g_end = lane == 0 ? *reinterpret_cast<volatile long long*>(&head->G) : 0;
-            g_end = __shfl_sync(kFull, g_end, 0);
-            count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey && ek <= g_end));
-            if (lane < (int)max(count, 1u)) out->e[lane] = make_longlong2((long long)ek, (long long)ei);
-        } else if (CHAIN) {
-            ek = sh.tops[lane & (kWarps - 1)][0].x;
-            el = sh.tops[lane & (kWarps - 1)][0].y;
-            ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
-            warp_min_triple(ek, el, ei);
-            count = 2;
-            if (lane < 2) out->e[lane] = lane ? make_longlong2((long long)ei, 0) : make_longlong2((long long)ek, (long long)el);
-        } else {
-            const longlong2 v = sh.tops[lane & (kWarps - 1)][0];
-            ek = v.x;
-            ei = (uint64_t)v.y;
-            warp_min_pair(ek, ei);
-            count = ek != kInfKey ? 1u : 0u;
-            if (lane == 0) out->e[0] = make_longlong2((long long)ek, (long long)ei);
-        }
-        unsigned long long rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
-        for (int off = kWarps / 2; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
-        if (lane == 0) {
-            out->count = count;
-            out->live_tilings = my_live;
-            out->feasible_rows = rows;
-        }
-        // Grid reduction without a wait: every CTA makes its partial list visible, then draws a ticket; the CTA that
-        // draws the last one knows that all lists are there and runs the finalize step.
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) sh.last_cta = atomicAdd(&head->done_ctas, 1u) == grid - 1 ? 1u : 0u;
-    }
-    __syncthreads();
-    if (sh.last_cta) {
-        if (late) {
-            wait_previous_kernel();         // from here on the result records are touched
-            release_next_kernel();
-        }
-        __threadfence();
-        if (CHAIN) finalize_chain<FRONT>(p, lim, sh, shape.chain_to, head, partials, (int)grid);
-        else finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
-    }
-}
-
-__global__ void reset_kernel(SearchHeader* head) {
-    head->G = kInfKey - 1;
-    head->done_ctas = 0;
-}
-
 // The full record of an optimum, by one CTA after load_shared: the first mapping with key `key` of block `where`.  key
 // kInfKey: nothing fits.
 // STAIRS: the first one that also has the buffer need `need`, the least of them.  A search that returns the first mapping
@@ -1079,18 +722,421 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
     }
 }
 
-template <int OBJ>
+// The records of chained searches as they end, by kRecordCtas CTAs, this one number `which`: the first search has the epoch
+// shape.chain_epoch, the last one finds nothing.
+template <bool FRONT>
+__device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& shape, Shared& sh, const SearchHeader* head, uint32_t which,
+                                           mmee_result_t* out) {
+    for (uint32_t i = 0; i < shape.chain_steps; ++i) {
+        __syncthreads();
+        if (threadIdx.x == 0 && !await_epoch(head, shape.chain_epoch + i)) sh.check_failed = 1;
+        __syncthreads();
+        if (sh.check_failed) {
+            if (threadIdx.x == 0) out[i].status = MMEE_ERR_CHECK;
+            return;
+        }
+        const volatile ChainRecord* from = shape.chain_to + i;
+        const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound, from->need, 0};
+        if (i % kRecordCtas == which) {
+            if (FRONT) resolve_record<MMEE_OBJ_LATENCY_ECAP, false>(p, Limits{p.cap_words, c.bound}, sh, c.key, c.where, c.n_feasible, 0, out + i);
+            else resolve_record<MMEE_OBJ_ENERGY, true>(p, Limits{c.bound, 0}, sh, c.key, c.where, c.n_feasible, c.need, out + i);
+        }
+        if (c.key == kInfKey) return;
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// the search kernel
+// ------------------------------------------------------------------------------------------------
+
+// Searches launched one after the other overlap (programmatic dependent launch), in one of two ways.
+//   early: a search lets the next one start at once; that one's CTAs move in as this one's leave, and wait for its end
+//          before they publish (k > 1: before their items), since it may still use their scratch;
+//   late:  only the CTA that finalizes waits for the kernel before, and lets the next search start after that wait.  The
+//          CTAs then publish while the search before finalizes, into the other one of the handle's two scratches: the
+//          search that used theirs last had ended before the one before them let them start.
+// A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  Searches one after
+// the other, without and with this (us each): smallest configuration 20.5 and 8.9, BERT energy 22.9 and 10.4, GQA latency
+// 28.7 and 13.7, convolution chain top-16 133 and 58 (other changes between them included).
+__device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
+// and the sizes between them.
+template <bool TERMS>
+__device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
+    if (TERMS && sub < 6) {
+        const int op = sub >= 3 ? 1 : 0, sm = sub - 3 * op;
+        int64_t P, Q;
+        stationary_terms(p, SharedDivisors{sh}, b, op, sm, P, Q);
+        (op ? tb->st.P2 : tb->st.P1)[sm] = P;
+        (op ? tb->st.Q2 : tb->st.Q1)[sm] = Q;
+    }
+    for (int i = sub; i < kSizeSlots; i += 8) tb->size[i] = sat_size(size_words(p.dim, tb->b + 4, i));
+    if (sub == 7) tb->t = t;
+}
+
+template <int OBJ, int MODE>
 __global__ void __launch_bounds__(kSearchThreads, 2)
-resolve_kernel(const __grid_constant__ Plan p, const ChainRecord* chain, mmee_result_t* out) {
+search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ head, Partial* __restrict__ partials,
+              mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
+    constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
+    constexpr bool ARRAYS = MODE == kModeArrays;
+    constexpr bool FRONT = CHAIN && OBJ == MMEE_OBJ_ENERGY_LCAP;      // least (energy, latency) under a bound on the latency
+    constexpr bool STAIRS = CHAIN && OBJ == MMEE_OBJ_ENERGY;          // least (energy, block, buffer need) under a capacity
+    static_assert(FRONT || STAIRS || !CHAIN, "only the searches of the Pareto fronts are chained");
     __shared__ Shared sh;
-    load_shared<false>(p, p.pe_rows, p.pe_cols, sh);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool late = shape.late;
+    if (!late) release_next_kernel();
+    load_shared<PRUNE>(p, p.pe_rows, p.pe_cols, sh);
+    // Array shapes: the stationary-pair terms of shape y and tiling slot i at [y * chunk + i], behind the tilings' tables;
+    // the warps' best items of shape y in sh.tops[.][y].
+    StatTerms* terms = reinterpret_cast<StatTerms*>(&sh.tile[shape.chunk]);
+    if (ARRAYS && tid < kWarps * (int)MMEE_MAX_TOPK) sh.tops[tid / (int)MMEE_MAX_TOPK][tid % (int)MMEE_MAX_TOPK] = make_longlong2(kInfKey, -1ll);
+    // STAIRS: the table slots of the tilings that fit under the bound, where the kept rows of the other modes lie.
+    uint8_t* fit_slots = reinterpret_cast<uint8_t*>(&sh.kept);
+    static_assert(kMaxChunk <= 256 && kMaxChunk <= sizeof(KeptMasks), "one byte per table");
+    if (tid == 0) {
+        sh.n_live = sh.n_fit = 0;
+        sh.cursor = 0;
+        sh.check_failed = 0;
+    }
     __syncthreads();
-    wait_previous_kernel();
-    // (volatile: read after the wait, not as data that no kernel writes meanwhile)
-    const volatile ChainRecord* from = chain + blockIdx.x;
-    const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound, from->need, 0};
-    const Limits lim = {OBJ == MMEE_OBJ_ENERGY ? c.bound : p.cap_words, c.bound};
-    resolve_record<OBJ, OBJ == MMEE_OBJ_ENERGY>(p, lim, sh, c.key, c.where, c.n_feasible, c.need, out + blockIdx.x);
+
+    if (CHAIN && blockIdx.x >= shape.grid) {
+        resolve_chain<FRONT>(p, shape, sh, head, blockIdx.x - shape.grid, out_topk);
+        return;
+    }
+
+    const int k = MULTI ? (int)p.topk : 1;
+    const int64_t I = p.dim[0], K = p.dim[1], L = p.dim[2], J = p.dim[3];
+    const DimWords dw = {I * K, K * L, L * J, I * J, I * L};
+    Limits lim = {p.cap_words, p.key_cap};
+    int capc = (int)p.cap_words;
+    const uint32_t grid = CHAIN ? shape.grid : gridDim.x, n_tilings = (uint32_t)(p.t_end - p.t_begin);
+    const uint32_t n_orders = p.n_orders;
+    auto any = [](bool v) { return __any_sync(kFull, v) != 0; };
+
+    // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
+    int64_t ek = kInfKey;
+    uint64_t ei = UINT64_MAX;
+    int64_t el = kInfKey;           // FRONT: its latency.  STAIRS: (el, ei) are the block and its need
+    unsigned long long my_rows = 0;
+    uint32_t my_live = 0;
+
+    auto offer = [&](int64_t key, uint32_t id, bool valid) {
+        if (!MULTI) {
+            if (valid && pair_less(key, id, ek, ei)) { ek = key; ei = id; }
+            return;
+        }
+        const int64_t lk = __shfl_sync(kFull, ek, k - 1);
+        const uint64_t li = __shfl_sync(kFull, ei, k - 1);
+        const bool pend = valid && key != kInfKey && key <= *reinterpret_cast<volatile long long*>(&sh.G) && pair_less(key, id, lk, li);
+        if (!__any_sync(kFull, pend)) return;
+        warp_offer(ek, ei, k, key, id, pend, lane);
+        // a full list bounds the k-th smallest key for everybody
+        if (lane == k - 1 && ek < *reinterpret_cast<volatile long long*>(&sh.G)) {
+            atomicMin(&sh.G, (long long)ek);
+            atomicMin(&head->G, (long long)ek);
+        }
+    };
+
+    // FRONT: the item's least (energy, latency) over the stationary pairs; pair(s, e, l) forms those of pair s.
+    auto offer_front = [&](auto pair, uint32_t id, bool valid) {
+        int64_t be = kInfKey, bl = kInfKey;
+#pragma unroll
+        for (int s = 0; s < 9; ++s) {
+            int64_t e, l;
+            pair(s, e, l);
+            const bool better = ((p.sm_mask >> s) & 1u) && l <= lim.key_cap && (e < be || (e == be && l < bl));
+            be = better ? e : be;
+            bl = better ? l : bl;
+        }
+        if (valid && triple_less(be, bl, id, ek, el, ei)) { ek = be; el = bl; ei = id; }
+    };
+
+    auto offer_stairs = [&](int64_t key, uint32_t id, int need, bool valid) {
+        if (valid && triple_less(key, (int64_t)id, (uint64_t)need, ek, el, ei)) { ek = key; el = id; ei = (uint64_t)need; }
+    };
+
+    // The same for every array shape, one after the other: key_of_terms(terms) is the item's least key.
+    auto offer_arrays = [&](auto key_of_terms, uint32_t slot, uint32_t id, bool valid) {
+        for (uint32_t y = 0; y < shape.n_arrays; ++y) {
+            const int64_t key = key_of_terms(terms[y * shape.chunk + slot]);
+            const longlong2 own = sh.tops[warp][y];
+            const bool better = valid && pair_less(key, id, own.x, (uint64_t)own.y);
+            if (!any(better)) continue;
+            int64_t nk = better ? key : kInfKey;
+            uint64_t ni = better ? id : UINT64_MAX;
+            warp_min_pair(nk, ni);
+            if (lane == 0) sh.tops[warp][y] = make_longlong2((long long)nk, (long long)ni);
+            __syncwarp();
+        }
+    };
+
+    const bool one_pass = (uint64_t)shape.chunk * grid >= n_tilings;        // chained: the tables stay
+    for (uint32_t step = 0;; ++step) {
+        if (CHAIN && (step || shape.chain_read)) {
+            __syncthreads();                // the counters of the search before are no longer in use
+            if (tid == 0) {
+                const bool over = !step || await_epoch(head, shape.chain_epoch + step - 1);
+                sh.bound = over ? *reinterpret_cast<volatile long long*>(&head->chain_bound) : kNoBound;
+                sh.n_fit = sh.cursor = 0;
+                if (!one_pass) sh.n_live = 0;
+            }
+            __syncthreads();
+            const int64_t bound = sh.bound;
+            if (bound == kNoBound) return;
+            if (OBJ == MMEE_OBJ_ENERGY) {
+                lim.cap_words = bound;
+                capc = (int)bound;
+            } else {
+                lim.key_cap = bound;
+            }
+            ek = el = kInfKey;
+            ei = UINT64_MAX;
+            my_rows = 0;
+        }
+        // Tiling number m of this CTA is one of the m-th `grid` consecutive ones, a different one in every round (a fixed
+        // one would be the same divisor of the last dimension again and again).
+        for (uint32_t m0 = 0; (uint64_t)m0 * grid < n_tilings; m0 += shape.chunk) {
+            if (m0) {
+                __syncthreads();                // the previous pass's tables are no longer in use
+                if (tid == 0) { sh.n_live = sh.n_fit = 0; sh.cursor = 0; }
+                __syncthreads();
+            }
+            for (uint32_t j0 = 0; j0 < (step && one_pass ? 0 : shape.chunk); j0 += kSearchThreads / 8) {
+                const uint32_t j = j0 + (uint32_t)tid / 8u, m = m0 + j;
+                uint64_t rel = (uint64_t)m * grid;
+                const bool mine = j < shape.chunk && rel < n_tilings;
+                rel += (blockIdx.x + m) % grid;
+                uint32_t b[8], t = 0;
+                bool live = mine && rel < n_tilings;
+                if (live) {
+                    t = (uint32_t)(p.t_begin + rel);
+                    tiling_bounds(p, SharedDivisors{sh}, t, b);
+                    // With every operand at L3 the buffer need is smallest: max(A+B+C, C+D+E) tiles (Eq. 1-4).
+                    const uint64_t ta = (uint64_t)b[4] * b[5], tbb = (uint64_t)b[5] * b[6], tc = (uint64_t)b[4] * b[6];
+                    const uint64_t td = (uint64_t)b[6] * b[7], te = (uint64_t)b[4] * b[7];
+                    live = ta + tbb + tc <= (uint64_t)capc && tc + td + te <= (uint64_t)capc;
+                }
+                uint32_t slot = 0;
+                if (live && (tid & 7) == 0) slot = atomicAdd(&sh.n_live, 1u);
+                slot = __shfl_sync(kFull, slot, lane & ~7);
+                if (live) {
+                    uint32_t own = b[0];
+    #pragma unroll
+                    for (int d = 1; d < 8; ++d) own = (tid & 7) == d ? b[d] : own;
+                    sh.tile[slot].b[tid & 7] = own;
+                }
+                __syncwarp();
+                if (live) build_tile<!ARRAYS>(p, sh, b, t, tid & 7, &sh.tile[slot]);
+            }
+            if (MULTI && m0 == 0) {
+                // (k > 1 shares a bound through the scratch while it works on the items)
+                if (!late) wait_previous_kernel();
+                if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
+            }
+            __syncthreads();
+            if (ARRAYS) {
+                const uint32_t n_live = sh.n_live;
+                for (uint32_t i = tid; i < n_live * 6u * shape.n_arrays; i += kSearchThreads) {
+                    const uint32_t y = i / (n_live * 6u), u = i - y * n_live * 6u, slot = u / 6u;
+                    const int op = u - slot * 6u >= 3u ? 1 : 0, sm = (int)(u - slot * 6u) - 3 * op;
+                    StatTerms& st = terms[y * shape.chunk + slot];
+                    int64_t P, Q;
+                    stationary_terms(p, ArrayDivisors{sh, shape.array[y][0], shape.array[y][1]}, sh.tile[slot].b, op, sm, P, Q);
+                    (op ? st.P2 : st.P1)[sm] = P;
+                    (op ? st.Q2 : st.Q1)[sm] = Q;
+                }
+                __syncthreads();
+            }
+
+            if (STAIRS) {
+                // The tables are those of the bound the plan has.  (Front of the GPT-3 FFN, twenty searches: 281 us with
+                // items for every table, 263 with this.)
+                if ((uint32_t)tid < sh.n_live) {
+                    const uint32_t* b = sh.tile[tid].b;
+                    const uint64_t tc = (uint64_t)b[4] * b[6];
+                    const uint64_t first = (uint64_t)b[4] * b[5] + (uint64_t)b[5] * b[6], second = (uint64_t)b[6] * b[7] + (uint64_t)b[4] * b[7];
+                    if (tc + max(first, second) <= (uint64_t)capc) fit_slots[atomicAdd(&sh.n_fit, 1u)] = (uint8_t)tid;
+                }
+                __syncthreads();
+            }
+            const uint32_t n_tiles = STAIRS ? sh.n_fit : sh.n_live, per_class = n_tiles * n_orders;
+            if (tid == 0) my_live += n_tiles;
+            const uint32_t fused_items = (p.fuse_mask & 1u) ? 3u * per_class : 0u;
+            const uint32_t fused_groups = (fused_items + 31u) / 32u;
+            const uint32_t groups = fused_groups + ((p.fuse_mask & 6u) ? (per_class + 31u) / 32u : 0u);
+            while (true) {
+                uint32_t g = 0;
+                if (lane == 0) g = atomicAdd(&sh.cursor, 1u);
+                g = __shfl_sync(kFull, g, 0);
+                if (g >= groups) break;
+                long long g_seen = 0;       // k > 1: the other CTAs' bound, used after this item
+                if (MULTI && lane == 0) g_seen = *reinterpret_cast<volatile long long*>(&head->G);
+                const bool fused = g < fused_groups;
+                uint32_t i = (fused ? g : g - fused_groups) * 32u + (uint32_t)lane;
+                const uint32_t n_items = fused ? fused_items : per_class;
+                const bool valid = i < n_items;
+                i = valid ? i : n_items - 1;
+                uint32_t c = 0;
+                if (fused) {
+                    c = i >= 2u * per_class ? 2u : (i >= per_class ? 1u : 0u);
+                    i -= c * per_class;
+                }
+                uint32_t slot = n_orders == 6u ? i / 6u : i / 2u;
+                const uint32_t os = i - slot * n_orders;
+                if (STAIRS) slot = fit_slots[slot];
+                const TileTab& tb = sh.tile[slot];
+                const OrderInfo& oi = sh.order[os];
+                const uint32_t id = tb.t * p.n_blocks + os;
+                if (fused) {
+                    uint32_t rows;
+                    int64_t x;
+                    int need;
+                    fused_class<PRUNE, STAIRS>(tb, oi, dw, (int)c, capc, PRUNE ? sh.kept.fused[os][c] : nullptr, any, rows, x, need);
+                    if (valid) my_rows += rows;
+                    const bool some = valid && x < kNoRow;
+                    if (any(some)) {
+                        const int64_t y = some ? x : 0, rho = oi.recompute[c] != 0 ? (int64_t)tb.b[LOOP_J] : 1;
+                        auto key = [&](const StatTerms& t) { return fused_least_key<OBJ>(t, y, rho, p.sm_mask, p.c_dram_gb, lim.key_cap); };
+                        auto pair = [&](int s, int64_t& e, int64_t& l) {
+                            e = p.c_dram_gb * y + tb.st.P1[s / 3] * rho + tb.st.P2[s % 3];
+                            l = max64(y, tb.st.Q1[s / 3] * rho + tb.st.Q2[s % 3]);
+                        };
+                        if (ARRAYS) offer_arrays(key, slot, id, some);
+                        else if (FRONT) offer_front(pair, id, some);
+                        else if (STAIRS) offer_stairs(key(tb.st), id, need, some);
+                        else offer(key(tb.st), id, some);
+                    }
+                } else {
+                    uint32_t fit1, fit2, rows;
+                    int64_t x1, x2;
+                    int need;
+                    unfused_nests<PRUNE, STAIRS>(tb, oi, dw, capc, fit1, fit2, rows, x1, x2, need);
+                    const bool some = valid && x1 < kNoRow;
+                    if (!any(some)) continue;
+                    const int64_t y1 = some ? x1 : 0, y2 = some ? x2 : 0;
+                    uint32_t block = p.n_fused_blocks;
+    #pragma unroll
+                    for (int phi = 1; phi <= 2; ++phi) {
+                        if (!((p.fuse_mask >> phi) & 1u)) continue;
+                        if (PRUNE) {
+                            rows = 0;
+                            for (int ab = 0; ab < 9; ++ab)
+                                if ((fit1 >> ab) & 1u) rows += (uint32_t)__popc(fit2 & sh.kept.unfused[phi - 1][os][ab]);
+                        }
+                        if (some) my_rows += rows;
+                        const int64_t pass = phi == 2 ? 2 * dw.il : 0;
+                        auto key = [&](const StatTerms& t) { return unfused_least_key<OBJ>(t, y1, y2, pass, p.sm_mask, p.c_dram_gb, lim.key_cap); };
+                        auto pair = [&](int s, int64_t& e, int64_t& l) {
+                            e = p.c_dram_gb * (y1 + y2 + pass) + tb.st.P1[s / 3] + tb.st.P2[s % 3];
+                            l = max64(y1, tb.st.Q1[s / 3]) + pass + max64(y2, tb.st.Q2[s % 3]);
+                        };
+                        if (ARRAYS) offer_arrays(key, slot, id + block, some);
+                        else if (FRONT) offer_front(pair, id + block, some);
+                        else if (STAIRS) offer_stairs(key(tb.st), id + block, need, some);
+                        else offer(key(tb.st), id + block, some);
+                        block += n_orders;
+                    }
+                }
+                if (MULTI && lane == 0 && g_seen < sh.G) atomicMin(&sh.G, g_seen);
+            }
+        }
+
+        // ---- this CTA's result
+        for (int off = 16; off; off >>= 1) my_rows += __shfl_down_sync(kFull, my_rows, off);
+        if (lane == 0) sh.feasible_rows[warp] = my_rows;
+        if (MULTI) {
+            merge_warps(sh, k, lane, warp, ek, ei);
+        } else if (CHAIN) {
+            warp_min_triple(ek, el, ei);
+            if (lane == 0) {
+                sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
+                sh.tops[warp][1] = make_longlong2((long long)ei, 0);
+            }
+            __syncthreads();
+        } else if (!ARRAYS) {
+            warp_min_pair(ek, ei);
+            if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)ek, (long long)ei);
+            __syncthreads();
+        }
+        if (!late && !CHAIN) wait_previous_kernel();        // from here on the scratch is touched
+        if (ARRAYS) {
+            // the best item of every shape; the kernel that follows merges them (resolve_arrays_kernel)
+            __syncthreads();
+            Partial* out = &partials[blockIdx.x];
+            for (uint32_t y = warp; y < shape.n_arrays; y += kWarps) {
+                const longlong2 v = sh.tops[lane & (kWarps - 1)][y];
+                int64_t nk = v.x;
+                uint64_t ni = (uint64_t)v.y;
+                warp_min_pair(nk, ni);
+                if (lane == 0) out->e[y] = make_longlong2((long long)nk, (long long)ni);
+            }
+            if (tid == 0) {
+                unsigned long long rows = 0;
+                for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
+                out->feasible_rows = rows;
+            }
+            return;
+        }
+        if (warp == 0) {
+            Partial* out = &partials[blockIdx.x];
+            uint32_t count;
+            if (MULTI) {
+                // an entry above the bound (some full list's last key) is not among the k best
+                long long g_end = lane == 0 ? *reinterpret_cast<volatile long long*>(&head->G) : 0;
+                g_end = __shfl_sync(kFull, g_end, 0);
+                count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey && ek <= g_end));
+                if (lane < (int)max(count, 1u)) out->e[lane] = make_longlong2((long long)ek, (long long)ei);
+            } else if (CHAIN) {
+                ek = sh.tops[lane & (kWarps - 1)][0].x;
+                el = sh.tops[lane & (kWarps - 1)][0].y;
+                ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
+                warp_min_triple(ek, el, ei);
+                count = 2;
+                if (lane < 2) out->e[lane] = lane ? make_longlong2((long long)ei, 0) : make_longlong2((long long)ek, (long long)el);
+            } else {
+                const longlong2 v = sh.tops[lane & (kWarps - 1)][0];
+                ek = v.x;
+                ei = (uint64_t)v.y;
+                warp_min_pair(ek, ei);
+                count = ek != kInfKey ? 1u : 0u;
+                if (lane == 0) out->e[0] = make_longlong2((long long)ek, (long long)ei);
+            }
+            unsigned long long rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
+            for (int off = kWarps / 2; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+            if (lane == 0) {
+                out->count = count;
+                out->live_tilings = my_live;
+                out->feasible_rows = rows;
+            }
+            // Grid reduction without a wait: every CTA makes its partial list visible, then draws a ticket; the CTA that
+            // draws the last one knows that all lists are there and runs the finalize step.
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) sh.last_cta = atomicAdd(&head->done_ctas, 1u) == grid - 1 ? 1u : 0u;
+        }
+        __syncthreads();
+        if (sh.last_cta) {
+            if (late) {
+                wait_previous_kernel();         // from here on the result records are touched
+                release_next_kernel();
+            }
+            __threadfence();
+            if (CHAIN) finalize_chain<FRONT>(p, lim, sh, shape.chain_to + step, shape.chain_epoch + step, head, partials, (int)grid);
+            else finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
+        }
+        if (!CHAIN || step + 1 == shape.chain_steps) return;
+    }
+}
+
+__global__ void reset_kernel(SearchHeader* head) {
+    head->G = kInfKey - 1;
+    head->done_ctas = 0;
+    head->chain_epoch = 0;
 }
 
 // Merge of the CTAs' best items of array shape blockIdx.x, and the record of the optimum.
@@ -1122,17 +1168,23 @@ resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, c
 }
 
 // A launch that may start before the kernel before it on the stream has ended (`overlap`): the kernel waits itself.
+// `together`: a cooperative one instead, whose CTAs are resident at the same time.
 template <class... Args>
-cudaError_t launch_overlapped(bool overlap, unsigned grid, cudaStream_t st, void (*kernel)(Args...), Args... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_overlapped(bool overlap, bool together, unsigned grid, cudaStream_t st, void (*kernel)(Args...), Args... args) {
+    cudaLaunchAttribute attr = {};
+    if (together) {
+        attr.id = cudaLaunchAttributeCooperative;
+        attr.val.cooperative = 1;
+    } else {
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kSearchThreads);
     cfg.stream = st;
     cfg.attrs = &attr;
-    cfg.numAttrs = overlap ? 1 : 0;
+    cfg.numAttrs = overlap || together ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -1144,11 +1196,12 @@ template <int OBJ>
 cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials,
                             mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
     auto* kernel = shape.n_arrays ? search_kernel<OBJ, kModeArrays>
-                   : shape.chain ? (chain_mode<OBJ>() == kModeChain ? search_kernel<OBJ, chain_mode<OBJ>()> : nullptr)
+                   : shape.chain_steps ? (chain_mode<OBJ>() == kModeChain ? search_kernel<OBJ, chain_mode<OBJ>()> : nullptr)
                    : p.row_pruning ? search_kernel<OBJ, kModePrune>
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
     if (!kernel) return cudaErrorInvalidValue;
-    return launch_overlapped(shape.overlap, shape.grid, st, kernel, p, shape, head, partials, out_best, out_topk);
+    const uint32_t grid = shape.chain_steps ? shape.grid + kRecordCtas : shape.grid;
+    return launch_overlapped(shape.overlap, shape.chain_steps != 0, grid, st, kernel, p, shape, head, partials, out_best, out_topk);
 }
 
 }  // namespace
@@ -1166,14 +1219,6 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
     }
 }
 
-cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, mmee_result_t* out, cudaStream_t st) {
-    switch (p.objective) {
-        case MMEE_OBJ_ENERGY: return launch_overlapped(true, n, st, resolve_kernel<MMEE_OBJ_ENERGY>, p, chain, out);
-        case MMEE_OBJ_LATENCY_ECAP: return launch_overlapped(true, n, st, resolve_kernel<MMEE_OBJ_LATENCY_ECAP>, p, chain, out);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
 uint32_t search_chunk(uint32_t n_arrays) {
     return (uint32_t)(kMaxChunk * sizeof(TileTab) / (sizeof(TileTab) + n_arrays * sizeof(StatTerms)));
 }
@@ -1184,11 +1229,11 @@ cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partia
     const unsigned n = shape.n_arrays;
     const Partial* from = partials;
     switch (p.objective) {
-        case MMEE_OBJ_ENERGY: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_ENERGY>, p, shape, from, out);
-        case MMEE_OBJ_LATENCY: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_LATENCY>, p, shape, from, out);
-        case MMEE_OBJ_EDP: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_EDP>, p, shape, from, out);
-        case MMEE_OBJ_ENERGY_LCAP: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_ENERGY_LCAP>, p, shape, from, out);
-        default: return launch_overlapped(true, n, st, resolve_arrays_kernel<MMEE_OBJ_LATENCY_ECAP>, p, shape, from, out);
+        case MMEE_OBJ_ENERGY: return launch_overlapped(true, false, n, st, resolve_arrays_kernel<MMEE_OBJ_ENERGY>, p, shape, from, out);
+        case MMEE_OBJ_LATENCY: return launch_overlapped(true, false, n, st, resolve_arrays_kernel<MMEE_OBJ_LATENCY>, p, shape, from, out);
+        case MMEE_OBJ_EDP: return launch_overlapped(true, false, n, st, resolve_arrays_kernel<MMEE_OBJ_EDP>, p, shape, from, out);
+        case MMEE_OBJ_ENERGY_LCAP: return launch_overlapped(true, false, n, st, resolve_arrays_kernel<MMEE_OBJ_ENERGY_LCAP>, p, shape, from, out);
+        default: return launch_overlapped(true, false, n, st, resolve_arrays_kernel<MMEE_OBJ_LATENCY_ECAP>, p, shape, from, out);
     }
 }
 

@@ -27,7 +27,8 @@ struct SearchHeader {
     unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
     long long chain_bound;                  // what a chained search leaves to the next one; -1: it found nothing
     unsigned int done_ctas;                 // ticket counter: the CTA that draws the last ticket runs the finalize step
-    unsigned int pad[7];
+    unsigned int chain_epoch;               // the last chained search that has ended on this scratch
+    unsigned int pad[6];
 };
 static_assert(sizeof(SearchHeader) == 64, "the header is 64 bytes");
 
@@ -57,16 +58,20 @@ struct LaunchShape {
     uint32_t array[kMaxArrays][2];      // their PE rows and columns
     bool overlap;           // may start before the kernel before it on the stream has ended (see mmee_search.cu)
     bool late;              // ... and its CTAs wait for that end in the finalize step only
-    bool chain;             // one of a chain of searches:
-    bool chain_read;        // ... not the first
-    ChainRecord* chain_to;  // device: where it leaves its optimum
+    uint32_t chain_steps;   // a chain of this many searches in one launch, 0: one search
+    uint32_t chain_epoch;   // ... their numbers on this scratch, ascending and greater than any before: the first one's
+    bool chain_read;        // ... that goes on from the launch before
+    ChainRecord* chain_to;  // device: where they leave their optima
 };
-// Chained searches (k = 1, no row pruning; the Pareto fronts): each takes a bound from what the one before it on the
-// stream found, on the device, so that the host waits once for several: the buffer words (energy) or the bound on the
-// latency (energy under a latency bound: then the least latency at the least energy) come from the scratch instead of the
-// plan (and are not above the plan's), and the bound for the next search is left there.  After a search that found nothing the others end at once.  A chained search writes
-// no record but a ChainRecord: the next one has to wait for its end, and the records of all can be made side by side
-// afterwards (launch_resolve).
+// Chained searches (k = 1, no row pruning; the Pareto fronts): each takes a bound from what the one before it found: the
+// buffer words (energy) or the bound on the latency (energy under a latency bound: then the least latency at the least
+// energy), not above the plan's.  They are the steps of one kernel, so that the host waits once for all and the tilings'
+// tables stay in shared memory; after one that found nothing the chain ends.  A chained search leaves no record but a
+// ChainRecord: the next one has to wait for it, and the records are made by
+// kRecordCtas more while the searches go on (in out_topk).  (A record takes longer than a short search.  Front of the GPT-3 FFN:
+// one 217 us, two 202, four 205 because the searches have fewer CTAs; records after the chain 204, where a front of one point
+// takes 59 instead of 55.)
+constexpr uint32_t kRecordCtas = 2;
 
 inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 
@@ -79,9 +84,6 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
                           mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st);
 // The same search (k = 1) on each of shape.n_arrays logical arrays, one record each in `out`: two launches.
 cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partial* partials, mmee_result_t* out, cudaStream_t st);
-// Full records of the optima that n chained searches left, one CTA each: of the energy searches themselves (`p` their
-// plan), or of the searches of the energy-latency front (`p` with the objective MMEE_OBJ_LATENCY_ECAP).
-cudaError_t launch_resolve(const Plan& p, const ChainRecord* chain, uint32_t n, mmee_result_t* out, cudaStream_t st);
 cudaError_t launch_reset(SearchHeader* head, cudaStream_t st);
 
 // Every key of the plan's tiling range (kInfKey where a mapping does not fit or its stationary pair is not offered).
@@ -94,8 +96,8 @@ cudaError_t measure_alu_peak(double* giops);
 // Most CTAs that a search on `device` takes.
 int max_search_ctas(int device, uint32_t* out);
 // Launch shape of a search of n_arrays array shapes (0: the plan's own) on `device` (at most max_ctas CTAs when that is not
-// 0: MMEE_ERR_RANGE if it would take more).
-int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape);
+// 0: MMEE_ERR_RANGE if it would take more).  `spare` CTAs fewer where it takes the most.
+int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape, uint32_t spare = 0);
 
 // MMEE_OK, or MMEE_ERR_CUDA with the error kept for mmee_last_cuda_error (per host thread).
 int cuda_status(cudaError_t e);

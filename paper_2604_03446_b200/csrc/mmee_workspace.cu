@@ -3,7 +3,7 @@
 // A one-shot search takes 20 to 30 us on the device, but cudaMalloc and cudaFree of its scratch took about 700 us of
 // host time around it: with no other allocation of the library alive the driver maps and unmaps a 2 MB slab each time
 // (a search of 768 tilings through mmee_solve_host: 730 us).  So a workspace that is no longer in use stays in a list,
-// at most kMaxIdle of them (0.16 MB of device and 6 KB of pinned host memory each), for the next handle on its device.
+// at most kMaxIdle of them (0.16 MB of device and 11 KB of pinned host memory each), for the next handle on its device.
 // A workspace belongs to one handle or call at a time, whatever thread or stream uses it; mmee_trim frees the idle ones.
 #include "mmee_workspace.h"
 

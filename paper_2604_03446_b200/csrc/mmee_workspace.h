@@ -12,12 +12,13 @@ struct Workspace {
                                     // publishes while the one before it on the handle still finalizes
     uint32_t max_ctas;              // partial lists a scratch has room for
     ChainRecord* chain;             // device, kHostRecords: what chained searches left
-    mmee_result_t* host;            // pinned host memory: 1 + MMEE_MAX_TOPK records that kernels write into
+    uint32_t chains;                // launches of them
+    mmee_result_t* host;            // pinned host memory: kHostRecords records that kernels write into
     mmee_result_t* host_dev;        // the same memory as the device addresses it
     Workspace* next;
 };
 
-constexpr uint32_t kHostRecords = 1 + MMEE_MAX_TOPK;
+constexpr uint32_t kHostRecords = 2 * MMEE_MAX_TOPK;
 static_assert(kMaxArrays <= kHostRecords, "one record per array shape");
 
 // A workspace on the current device (`device`), for the caller alone until it is given back.

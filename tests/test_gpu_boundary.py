@@ -158,6 +158,29 @@ def test_chained_front_equals_one_search_after_the_other(seed):
     assert [bytes(r) for r in got] == want and len(want) >= 2
 
 
+@pytest.mark.parametrize("shape,gb_bytes,tilings,least_searches", [
+    ((12544, 576, 192, 128), 1 << 20, None, 2),     # 63 504 tilings: several passes of tables in every search
+    ((5040, 360, 1680, 96), 8 << 20, 42000, 33),    # more searches than one chain has
+    ((64, 64, 64, 64), 1 << 18, 3, 2),              # one block of threads
+], ids=["passes", "chains", "few"])
+def test_chains_of_searches_equal_plain_searches(shape, gb_bytes, tilings, least_searches):
+    """The searches of a front as steps of one kernel, at the edges of its shapes: tables that do not stay between steps,
+    a front that needs a second chain, a handful of tilings; byte for byte the records of plain searches."""
+    w, arch = mi.two_gemm(*shape), mi.arch_dram_only(gb_bytes)
+    obj = mi.objective(mi.OBJ_ENERGY, 1, t_end=tilings or 0)
+    want, held, cap, searches = [], None, gb_bytes // 2, 0
+    while True:
+        r = mm.mmee_solve_host(w, dict(arch, gb_bytes=cap * 2), obj)[0]
+        searches += 1
+        if held is not None and (r.idx == mm.NO_INDEX or r.e_key != held.e_key):
+            want.append(bytes(held))
+        if r.idx == mm.NO_INDEX:
+            break
+        held, cap = r, r.bs - 1
+    assert [bytes(r) for r in mm.mmee_pareto_front_bs_da(w, arch, obj)] == want
+    assert min(searches, len(want) + 1) >= least_searches
+
+
 def test_buffer_size_dram_traffic_front_of_the_ffn_task():
     """On the fused feed-forward GEMMs of the paper's buffer-size study the front is a staircase: strictly less
     buffer and strictly more traffic from point to point, no point above the buffer, the last one at the
