@@ -761,6 +761,14 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
 __device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The number of CTAs that drew a ticket before; what they wrote before that is visible from here on, and what the calling
+// warp has written is to those that draw one later.
+__device__ __forceinline__ uint32_t draw_ticket(unsigned int* count) {
+    uint32_t n;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(n) : "l"(count) : "memory");
+    return n;
+}
+
 // The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
 // and the sizes between them.
 template <bool TERMS>
@@ -1115,9 +1123,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             }
             // Grid reduction without a wait: every CTA makes its partial list visible, then draws a ticket; the CTA that
             // draws the last one knows that all lists are there and runs the finalize step.
-            __threadfence();
             __syncwarp();
-            if (lane == 0) sh.last_cta = atomicAdd(&head->done_ctas, 1u) == grid - 1 ? 1u : 0u;
+            if (lane == 0) sh.last_cta = draw_ticket(&head->done_ctas) == grid - 1 ? 1u : 0u;
         }
         __syncthreads();
         if (sh.last_cta) {
@@ -1125,7 +1132,6 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 wait_previous_kernel();         // from here on the result records are touched
                 release_next_kernel();
             }
-            __threadfence();
             if (CHAIN) finalize_chain<FRONT>(p, lim, sh, shape.chain_to + step, shape.chain_epoch + step, head, partials, (int)grid);
             else finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
         }
