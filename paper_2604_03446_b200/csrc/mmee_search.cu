@@ -414,11 +414,13 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
 constexpr uint32_t kMaxPolls = 1u << 22;
 constexpr int64_t kNoBound = INT64_MIN;         // what a search leaves that found nothing
 
-__device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t epoch) {
+// The low half of the header's word is the bound where it has 32 bits (a capacity).
+__device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t epoch, uint32_t& low) {
     for (uint32_t i = 0; i < kMaxPolls; ++i) {
-        uint32_t now;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&head->chain_epoch) : "memory");
-        if ((int32_t)(now - epoch) >= 0) return true;
+        unsigned long long now;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(&head->chain_epoch) : "memory");
+        low = (uint32_t)now;
+        if ((int32_t)((uint32_t)(now >> 32) - epoch) >= 0) return true;
     }
     return false;
 }
@@ -470,9 +472,11 @@ __device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Sh
         const unsigned long long fit = rows * p.n_sm;
         if (FRONT) *chain_to = {(long long)(found ? el : kInfKey), (unsigned long long)ei, fit, (long long)ek, 0, 0};
         else *chain_to = {(long long)ek, (unsigned long long)el, fit, (long long)lim.cap_words, (long long)ei, 0};
-        head->chain_bound = !found ? kNoBound : (FRONT ? el : (int64_t)ei) - 1;
+        const int64_t bound = !found ? kNoBound : (FRONT ? el : (int64_t)ei) - 1;
+        const unsigned long long word = (unsigned long long)epoch << 32 | (found ? (uint32_t)bound : 0xffffffffu);
+        head->chain_bound = bound;
         head->done_ctas = 0;
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&head->chain_epoch), "r"(epoch) : "memory");
+        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&head->chain_epoch), "l"(word) : "memory");
     }
 }
 
@@ -750,7 +754,8 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
                                            mmee_result_t* out) {
     for (uint32_t i = 0; i < shape.chain_steps; ++i) {
         __syncthreads();
-        if (threadIdx.x == 0 && !await_epoch(head, shape.chain_epoch + i)) sh.check_failed = 1;
+        uint32_t low;
+        if (threadIdx.x == 0 && !await_epoch(head, shape.chain_epoch + i, low)) sh.check_failed = 1;
         __syncthreads();
         if (sh.check_failed) {
             if (threadIdx.x == 0) out[i].status = MMEE_ERR_CHECK;
@@ -909,8 +914,11 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         if (CHAIN && (step || shape.chain_read)) {
             __syncthreads();                // the counters of the search before are no longer in use
             if (tid == 0) {
-                const bool over = !step || await_epoch(head, shape.chain_epoch + step - 1);
-                sh.bound = over ? *reinterpret_cast<volatile long long*>(&head->chain_bound) : kNoBound;
+                uint32_t low = 0;
+                const bool over = !step || await_epoch(head, shape.chain_epoch + step - 1, low);
+                if (!over) sh.bound = kNoBound;
+                else if (step && STAIRS) sh.bound = low == 0xffffffffu ? kNoBound : (int64_t)low;
+                else sh.bound = *reinterpret_cast<volatile long long*>(&head->chain_bound);
                 sh.n_fit = sh.cursor = 0;
                 if (!one_pass) sh.n_live = 0;
             }

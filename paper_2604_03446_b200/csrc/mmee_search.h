@@ -26,9 +26,9 @@ struct SearchHeader {
     unsigned long long last_exact_groups;   // groups of 45 mappings of the winning blocks, evaluated one by one
     unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
     long long chain_bound;                  // what a chained search leaves to the next one; -1: it found nothing
+    unsigned long long chain_epoch;         // the last chained search that has ended on this scratch (high half)
     unsigned int done_ctas;                 // ticket counter: the CTA that draws the last ticket runs the finalize step
-    unsigned int chain_epoch;               // the last chained search that has ended on this scratch
-    unsigned int pad[6];
+    unsigned int pad[5];
 };
 static_assert(sizeof(SearchHeader) == 64, "the header is 64 bytes");
 
