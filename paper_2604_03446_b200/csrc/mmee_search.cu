@@ -409,7 +409,7 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
 // when it has left the bound for the next.  kRecordCtas more make the records meanwhile.  The wait is limited, at a few
 // seconds; true: the search is over.
 // Steps of about 8 us are bound by publish, ticket, merge and this wait, the first of a large front by their items.  Front of
-// the GPT-3 FFN (20 searches), a launch per search that waited for the one before 264 us, steps of one kernel 202;
+// the GPT-3 FFN (20 searches), a launch per search that waited for the one before 264 us, steps of one kernel 202 (now 187);
 // 99 random fronts 241 and 198 us; the energy-latency front of 10 816 tilings 56.5 and 55.3.
 constexpr uint32_t kMaxPolls = 1u << 22;
 constexpr int64_t kNoBound = INT64_MIN;         // what a search leaves that found nothing
@@ -425,7 +425,7 @@ __device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t e
     return false;
 }
 
-// The end of a chained search, by all threads of the last CTA; its record is made after the chain.
+// The end of a chained search, by all threads of the last CTA; its record is made by another (resolve_chain).
 // FRONT: the least (energy, latency, block) of all CTAs is the next point of the energy-latency front.  It is left as a
 // latency optimum under that energy; the next search allows one word less of latency.
 // Else: the least (energy, block, buffer need); the next search allows one word of buffer less than that need.
