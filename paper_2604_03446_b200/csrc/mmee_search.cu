@@ -122,6 +122,11 @@ __device__ __forceinline__ void warp_min_triple(int64_t& k, int64_t& k2, uint64_
     k2 = (int64_t)warp_min_u64((uint64_t)k2, in);
     i = warp_min_u64(i, in);
 }
+__device__ __forceinline__ int64_t min3(const int64_t (&v)[3]) {
+    const int64_t m = v[0] < v[1] ? v[0] : v[1];
+    return m < v[2] ? m : v[2];
+}
+
 __device__ __forceinline__ bool triple_less(int64_t ka, int64_t la, uint64_t ia, int64_t kb, int64_t lb, uint64_t ib) {
     return ka < kb || (ka == kb && (la < lb || (la == lb && ia < ib)));
 }
@@ -1044,7 +1049,12 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                             l = max64(y, tb.st.Q1[s / 3] * rho + tb.st.Q2[s % 3]);
                         };
                         if (ARRAYS) offer_arrays(key, slot, id, some);
-                        else if (FRONT) offer_front(pair, id, some);
+                        else if (FRONT) {
+                            // No mapping of the item is faster than this; after the first search few are fast enough
+                            // (front of 10 816 tilings, one point: 53.9 us without this test, 52.5 with it).
+                            const bool can = some && max64(y, min3(tb.st.Q1) * rho + min3(tb.st.Q2)) <= lim.key_cap;
+                            if (any(can)) offer_front(pair, id, can);
+                        }
                         else if (STAIRS) offer_stairs(key(tb.st), id, need, some);
                         else offer(key(tb.st), id, some);
                     }
@@ -1073,7 +1083,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                             l = max64(y1, tb.st.Q1[s / 3]) + pass + max64(y2, tb.st.Q2[s % 3]);
                         };
                         if (ARRAYS) offer_arrays(key, slot, id + block, some);
-                        else if (FRONT) offer_front(pair, id + block, some);
+                        else if (FRONT) {
+                            const bool can = some && max64(y1, min3(tb.st.Q1)) + pass + max64(y2, min3(tb.st.Q2)) <= lim.key_cap;
+                            if (any(can)) offer_front(pair, id + block, can);
+                        }
                         else if (STAIRS) offer_stairs(key(tb.st), id + block, need, some);
                         else offer(key(tb.st), id + block, some);
                         block += n_orders;
