@@ -20,8 +20,6 @@
 
 namespace mmee {
 
-#define MMEE_HD __host__ __device__ __forceinline__
-
 constexpr int kSizeCap = (1 << 30) - 1;        // buffer sizes saturate here, above every admissible capacity
 constexpr int64_t kNoRow = INT64_C(1) << 62;   // DRAM words of "no row fits"; sums of words stay below 2^62
 

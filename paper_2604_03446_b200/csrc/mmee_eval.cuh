@@ -28,7 +28,7 @@ struct TileForm {
     uint32_t ea, eb;            // extents of the stationary operand
     int64_t c0, ca, cb, third;
 };
-__device__ __forceinline__ TileForm tile_form(int sm, uint32_t m, uint32_t r, uint32_t n) {
+MMEE_HD TileForm tile_form(int sm, uint32_t m, uint32_t r, uint32_t n) {
     const int64_t mr = (int64_t)m * r, rn = (int64_t)r * n, mn = (int64_t)m * n;
     TileForm f;
     f.ea = sm == 0 ? r : m;
@@ -40,16 +40,19 @@ __device__ __forceinline__ TileForm tile_form(int sm, uint32_t m, uint32_t r, ui
     return f;
 }
 
-// The array's rows and columns, the divisors of dimension d in ascending order, and how often one has to be folded onto the array's rows / columns: read from
-// the plan (here) or from a CTA's shared copy.
+// ceil(x / n), x >= 1: how often x elements are folded onto n rows or columns (x + n may exceed 32 bits).
+MMEE_HD uint32_t folds(uint32_t x, uint32_t n) { return (x - 1u) / n + 1u; }
+
+// The array's rows and columns, the divisors of dimension d in ascending order, and how often one has to be folded onto the
+// array's rows / columns: read from the plan (here) or from a CTA's shared copy.
 struct PlanDivisors {
     const Plan& p;
-    __device__ __forceinline__ uint32_t rows() const { return p.pe_rows; }
-    __device__ __forceinline__ uint32_t cols() const { return p.pe_cols; }
-    __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return p.divs[d][i]; }
-    __device__ __forceinline__ uint32_t cofactor(int d, uint32_t i) const { return p.dim[d] / p.divs[d][i]; }
-    __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_rows - 1) / p.pe_rows; }
-    __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return (p.divs[d][i] + p.pe_cols - 1) / p.pe_cols; }
+    MMEE_HD uint32_t rows() const { return p.pe_rows; }
+    MMEE_HD uint32_t cols() const { return p.pe_cols; }
+    MMEE_HD uint32_t div(int d, uint32_t i) const { return p.divs[d][i]; }
+    MMEE_HD uint32_t cofactor(int d, uint32_t i) const { return p.dim[d] / p.divs[d][i]; }
+    MMEE_HD uint32_t row_folds(int d, uint32_t i) const { return folds(p.divs[d][i], p.pe_rows); }
+    MMEE_HD uint32_t col_folds(int d, uint32_t i) const { return folds(p.divs[d][i], p.pe_cols); }
 };
 
 // Register-file-level tiling (objective.rf_tiling): the stationary operand is processed in blocks of a x b elements, a
@@ -63,8 +66,8 @@ struct PlanDivisors {
 // na * nb (a BERT-base latency search 97 -> 50 us; as one loop whose lanes stay together 23.0 -> 20.6 us).
 // blk receives the block as (m, r, n) extents, 1 for the streamed extent.
 template <class Divisors>
-__device__ __forceinline__ void rf_block_terms(const Plan& p, const Divisors& dv, int sm, const TileForm& f, int da, int db,
-                                               int64_t& words, int64_t& cycles, uint32_t blk[3]) {
+MMEE_HD void rf_block_terms(const Plan& p, const Divisors& dv, int sm, const TileForm& f, int da, int db,
+                            int64_t& words, int64_t& cycles, uint32_t blk[3]) {
     const bool latency = p.objective == MMEE_OBJ_LATENCY;
     const uint32_t most = p.rf_words - 2;
     const uint32_t na = p.ndiv[da];
@@ -121,8 +124,8 @@ __device__ __forceinline__ void rf_block_terms(const Plan& p, const Divisors& dv
 // Words and cycles of one tile of operator `op` (0: (i_G x k_G)(k_G x l_G), 1: (i_G x l_G)(l_G x j_G)) under
 // stationary mode sm: one array fold per pass, or the register-file block search.
 template <class Divisors>
-__device__ __forceinline__ void tile_array_terms(const Plan& p, const Divisors& dv, const uint32_t b[8], int op, int sm, int64_t& words,
-                                                 int64_t& cycles, uint32_t blk[3]) {
+MMEE_HD void tile_array_terms(const Plan& p, const Divisors& dv, const uint32_t b[8], int op, int sm, int64_t& words,
+                              int64_t& cycles, uint32_t blk[3]) {
     const uint32_t m = b[4], r = op == 0 ? b[5] : b[6], n = op == 0 ? b[6] : b[7];
     const TileForm f = tile_form(sm, m, r, n);
     if (p.rf_tiling) {
@@ -130,7 +133,7 @@ __device__ __forceinline__ void tile_array_terms(const Plan& p, const Divisors& 
         const int dm = LOOP_I, dr = op == 0 ? LOOP_K : LOOP_L, dn = op == 0 ? LOOP_L : LOOP_J;
         rf_block_terms(p, dv, sm, f, sm == 0 ? dr : dm, sm == 0 ? dn : (sm == 1 ? dr : dn), words, cycles, blk);
     } else {
-        const int64_t qa = (f.ea + dv.rows() - 1) / dv.rows(), qb = (f.eb + dv.cols() - 1) / dv.cols();
+        const int64_t qa = folds(f.ea, dv.rows()), qb = folds(f.eb, dv.cols());
         words = f.c0 + f.ca * qa + f.cb * qb;
         cycles = f.third * qa * qb;
         blk[0] = blk[1] = blk[2] = 0;
@@ -319,7 +322,7 @@ __device__ __forceinline__ void assemble_record(const Plan& p, uint64_t idx, con
     o.feasible = (uint8_t)(o.bs <= cap_words && ((p.sm_mask >> d.s) & 1u));
     o.edp_key = __dmul_rn((double)e_key, (double)l_key);
     o.energy_pj = __dmul_rn(__dmul_rn((double)e_key, p.quantum_pj), (double)p.instances);
-    const uint32_t waves = (p.instances + p.n_arrays - 1) / p.n_arrays;
+    const uint32_t waves = folds(p.instances, p.n_arrays);
     o.latency_cycles = __dmul_rn(__ddiv_rn((double)l_key, (double)p.bw), (double)waves);
     o.n_total = 0; o.n_feasible = 0;
     for (int i = 0; i < 3; ++i) { o.rf_block[i] = blk1[i]; o.rf_block[3 + i] = blk2[i]; }

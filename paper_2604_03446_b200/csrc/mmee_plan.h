@@ -12,6 +12,9 @@ constexpr int kRowsPerTask = 125;   // one middle level (C when fused, B when un
 constexpr int kCandPerTask = 1125;  // rows x 9 stationary pairs
 constexpr int64_t kInfKey = INT64_MAX;
 
+// Model arithmetic that the host can run as well as the kernels.
+#define MMEE_HD __host__ __device__ __forceinline__
+
 // Operand / loop numbering shared by host planner and kernels.
 enum { OP_A = 0, OP_B = 1, OP_C = 2, OP_D = 3, OP_E = 4 };
 enum { LOOP_I = 0, LOOP_K = 1, LOOP_L = 2, LOOP_J = 3 };

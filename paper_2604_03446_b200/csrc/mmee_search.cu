@@ -162,12 +162,12 @@ struct Shared {
 
 struct SharedDivisors {       // see PlanDivisors
     const Shared& sh;
-    __device__ __forceinline__ uint32_t rows() const { return sh.pe_rows; }
-    __device__ __forceinline__ uint32_t cols() const { return sh.pe_cols; }
-    __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
-    __device__ __forceinline__ uint32_t cofactor(int d, uint32_t i) const { return sh.cofactors[d][i]; }
-    __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return sh.row_folds[d][i]; }
-    __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return sh.col_folds[d][i]; }
+    MMEE_HD uint32_t rows() const { return sh.pe_rows; }
+    MMEE_HD uint32_t cols() const { return sh.pe_cols; }
+    MMEE_HD uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
+    MMEE_HD uint32_t cofactor(int d, uint32_t i) const { return sh.cofactors[d][i]; }
+    MMEE_HD uint32_t row_folds(int d, uint32_t i) const { return sh.row_folds[d][i]; }
+    MMEE_HD uint32_t col_folds(int d, uint32_t i) const { return sh.col_folds[d][i]; }
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -372,11 +372,11 @@ __device__ __forceinline__ void min_over_warps(Shared& sh, int lane, int warp, i
 struct ArrayDivisors {        // the same with another array's rows and columns
     const Shared& sh;
     uint32_t pe_rows, pe_cols;
-    __device__ __forceinline__ uint32_t rows() const { return pe_rows; }
-    __device__ __forceinline__ uint32_t cols() const { return pe_cols; }
-    __device__ __forceinline__ uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
-    __device__ __forceinline__ uint32_t row_folds(int d, uint32_t i) const { return (sh.divs[d][i] + pe_rows - 1) / pe_rows; }
-    __device__ __forceinline__ uint32_t col_folds(int d, uint32_t i) const { return (sh.divs[d][i] + pe_cols - 1) / pe_cols; }
+    MMEE_HD uint32_t rows() const { return pe_rows; }
+    MMEE_HD uint32_t cols() const { return pe_cols; }
+    MMEE_HD uint32_t div(int d, uint32_t i) const { return sh.divs[d][i]; }
+    MMEE_HD uint32_t row_folds(int d, uint32_t i) const { return folds(sh.divs[d][i], pe_rows); }
+    MMEE_HD uint32_t col_folds(int d, uint32_t i) const { return folds(sh.divs[d][i], pe_cols); }
 };
 
 // What the kernels look up in shared memory, by all threads of a CTA (the caller synchronises).
@@ -394,8 +394,8 @@ __device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uin
         sh.divs[d][i] = p.divs[d][i];
         sh.cofactors[d][i] = (p.mirrored >> d) & 1u ? p.divs[d][p.ndiv[d] - 1 - i] : p.dim[d] / p.divs[d][i];
         if (p.rf_tiling) {
-            sh.row_folds[d][i] = (p.divs[d][i] + pe_rows - 1) / pe_rows;
-            sh.col_folds[d][i] = (p.divs[d][i] + pe_cols - 1) / pe_cols;
+            sh.row_folds[d][i] = folds(p.divs[d][i], pe_rows);
+            sh.col_folds[d][i] = folds(p.divs[d][i], pe_cols);
         }
     }
     if (tid == 0) {

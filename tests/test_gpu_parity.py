@@ -641,3 +641,19 @@ def test_top16_over_several_passes_equals_the_merge_of_its_parts():
     assert best.n_feasible == feasible
     for r in whole:
         assert_same_record(r, oracle.evaluate(p, r.idx))
+
+
+@pytest.mark.parametrize("dims,pe", [((2, 4294967294, 3, 4), (4, 7)), ((24, 30, 20, 6), (2 ** 32 - 1, 2 ** 32 - 8))])
+def test_records_whose_folds_come_near_the_32_bit_limit(dims, pe):
+    """Extent + rows - 1 above 2^32, and more instances than 2^32 less the arrays: sampled records against the oracle."""
+    cfg = dict(workload=mi.workload(2 ** 32 - 1, 1, 1, dims[0], dims[2], dims[1], dims[3], 2),
+               arch=mi.arch(pe[0], pe[1], 3, 1 << 20, 0, 1, 1.0, 1.0, 1.0, 1.0))
+    obj = mi.objective(mi.OBJ_ENERGY, 1)
+    p = oracle.make_problem(cfg["workload"], cfg["arch"], obj)
+    buf = mm.result_buffer(9)
+    with Handle(cfg, obj) as h:
+        for t in range(p.T):
+            start = (t * p.R + 131 * t % p.R) * 9
+            mm.mmee_eval(h, start, 9, buf)
+            for g, o in zip(mm.read_results(buf, 9), oracle.evaluate_range(p, start, 9)):
+                assert_same_record(g, o, "idx %d" % o.idx)

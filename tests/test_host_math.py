@@ -1,0 +1,88 @@
+"""The kernels' arithmetic that the host can run as well, compiled for the CPU and checked there: no GPU is used."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+import mmee_inputs as mi
+import paper_2604_03446_b200.binding as mm
+from paper_2604_03446_b200 import build as lib_build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="session")
+def host(tmp_path_factory):
+    """host_math.cu and the planner as a shared object."""
+    out = str(tmp_path_factory.mktemp("host_math") / "host_math.so")
+    flags = [f for f in lib_build.NVCC_FLAGS if f not in ("-lineinfo", "-O3")]
+    subprocess.check_call([lib_build._nvcc()] + flags + ["-O1", "-o", out, os.path.join(HERE, "host_math.cu"),
+                                                         os.path.join(lib_build.CSRC, "mmee_plan.cu")])
+    return C.CDLL(out)
+
+
+def tile_terms(lib, dims, pe, tile, op, sm, objective=mi.OBJ_ENERGY, rf_words=0):
+    """(words, cycles, block) of one tile with extents (i, k, l, j)."""
+    w = mm._fill(mm.Workload(), mi.workload(1, 1, 1, dims[0], dims[2], dims[1], dims[3], 2))
+    a = mm._fill(mm.Arch(), dict(mi.arch(pe[0], pe[1], 1, 1 << 20, 2 * rf_words, 1, 1.0, 1.0, 1.0, 1.0)))
+    o = mm._fill(mm.Objective(), mi.objective(objective, 1, rf_tiling=1 if rf_words else 0))
+    b = (C.c_uint32 * 8)(*([d // t for d, t in zip(dims, tile)] + list(tile)))
+    out, blk = (C.c_int64 * 2)(), (C.c_uint32 * 3)()
+    assert lib.host_tile_terms(C.byref(w), C.byref(a), C.byref(o), b, op, sm, out, blk) == mm.OK
+    return out[0], out[1], list(blk)
+
+
+def ceil_div(a, b):
+    return -(-a // b)
+
+
+def divisors(n):
+    ds = [d for d in range(1, int(n ** 0.5) + 2) if n % d == 0 and d * d <= n]
+    return sorted(set(ds + [n // d for d in ds]))
+
+
+def expected_terms(pe, tile, op, sm, objective, rf_words):
+    """The definition, in Python integers: the stationary operand's extents cut into parts of the array (or, with a
+    register file, of the best admissible block), operands and partial sums moved once per part."""
+    m, r, n = (tile[0], tile[1], tile[2]) if op == 0 else (tile[0], tile[2], tile[3])
+    ea, eb = {0: (r, n), 1: (m, r), 2: (m, n)}[sm]
+
+    def terms(qa, qb, held):
+        words = {0: r * n + m * r * qb + m * n * (2 * qa - 1), 1: m * r + r * n * qa + m * n * (2 * qb - 1),
+                 2: m * r * qb + r * n * qa + m * n}[sm]
+        return words, {0: m, 1: n, 2: r}[sm] * qa * qb * held
+
+    if not rf_words:
+        return terms(ceil_div(ea, pe[0]), ceil_div(eb, pe[1]), 1) + ([0, 0, 0],)
+    best = None
+    for a in divisors(ea):
+        for b in divisors(eb):
+            held = ceil_div(a, pe[0]) * ceil_div(b, pe[1])
+            if held + 2 > rf_words:
+                continue
+            w, c = terms(ea // a, eb // b, held)
+            key = (w, c) if objective == mi.OBJ_ENERGY else (c, w)
+            if best is None or key < best[0]:
+                best = (key, w, c, [1, a, b] if sm == 0 else ([a, b, 1] if sm == 1 else [a, 1, b]))
+    return best[1:]
+
+
+HUGE = 2 ** 32 - 1
+
+
+@pytest.mark.parametrize("dims,pe,rf_words", [
+    ((2, 4294967294, 3, 4), (4, 7), 0),              # extents within one fold of 2^32
+    ((4294967294, 2, 3, 4), (2147483648, 5), 0),
+    ((48, 30, 20, 6), (HUGE, HUGE - 7), 0),          # arrays that hold any tile
+    ((2, 4294967294, 3, 4), (4, 7), 12),
+    ((4294967294, 2, 3, 4), (65536, 65536), 70000),
+    ((48, 30, 20, 6), (HUGE, HUGE - 7), 6),
+], ids=["k", "i", "array", "k_rf", "i_rf", "array_rf"])
+def test_folds_near_the_32_bit_limit(host, dims, pe, rf_words):
+    """ceil(extent / rows) where extent + rows - 1 exceeds 32 bits."""
+    for op in (0, 1):
+        for sm in (0, 1, 2):
+            for objective in (mi.OBJ_ENERGY, mi.OBJ_LATENCY):
+                want = expected_terms(pe, dims, op, sm, objective, rf_words)
+                assert tile_terms(host, dims, pe, dims, op, sm, objective, rf_words) == want, (op, sm, objective)
