@@ -92,9 +92,10 @@ MMEE_HD void rf_block_terms(const Plan& p, const Divisors& dv, int sm, const Til
             qb = q;
             hb = dv.col_folds(db, ib);
         }
-        const uint32_t a = ia < na ? dv.div(da, ia) : 0xffffffffu;
-        const uint32_t ha = ia < na ? dv.row_folds(da, ia) : 0u;
-        if (a <= f.ea && (uint64_t)ha * hb <= most) {
+        const bool left = ia < na;              // (an extent of 2^32 - 1 leaves no value of a to mark the end with)
+        const uint32_t a = left ? dv.div(da, ia) : 0u;
+        const uint32_t ha = left ? dv.row_folds(da, ia) : 0u;
+        if (left && a <= f.ea && (uint64_t)ha * hb <= most) {
             ++ia;
             const uint32_t qa = f.ea / a;
             const uint64_t fa = (uint64_t)qa * ha;

@@ -1,5 +1,6 @@
 """The kernels' arithmetic that the host can run as well, compiled for the CPU and checked there: no GPU is used."""
 import ctypes as C
+import multiprocessing
 import os
 import subprocess
 
@@ -19,7 +20,9 @@ def host(tmp_path_factory):
     flags = [f for f in lib_build.NVCC_FLAGS if f not in ("-lineinfo", "-O3")]
     subprocess.check_call([lib_build._nvcc()] + flags + ["-O1", "-o", out, os.path.join(HERE, "host_math.cu"),
                                                          os.path.join(lib_build.CSRC, "mmee_plan.cu")])
-    return C.CDLL(out)
+    lib = C.CDLL(out)
+    lib.path = out
+    return lib
 
 
 def tile_terms(lib, dims, pe, tile, op, sm, objective=mi.OBJ_ENERGY, rf_words=0):
@@ -31,6 +34,10 @@ def tile_terms(lib, dims, pe, tile, op, sm, objective=mi.OBJ_ENERGY, rf_words=0)
     out, blk = (C.c_int64 * 2)(), (C.c_uint32 * 3)()
     assert lib.host_tile_terms(C.byref(w), C.byref(a), C.byref(o), b, op, sm, out, blk) == mm.OK
     return out[0], out[1], list(blk)
+
+
+def _tile_terms_at(path, *args):
+    return tile_terms(C.CDLL(path), *args)
 
 
 def ceil_div(a, b):
@@ -86,3 +93,23 @@ def test_folds_near_the_32_bit_limit(host, dims, pe, rf_words):
             for objective in (mi.OBJ_ENERGY, mi.OBJ_LATENCY):
                 want = expected_terms(pe, dims, op, sm, objective, rf_words)
                 assert tile_terms(host, dims, pe, dims, op, sm, objective, rf_words) == want, (op, sm, objective)
+
+
+@pytest.mark.parametrize("dims,pe,rf_words", [
+    ((HUGE, 3, 5, 1), (65536, 65536), 2 ** 31 - 1),      # every divisor of 2^32 - 1 is admissible
+    ((3, HUGE, 1, 1), (2, 3), 2 ** 32 - 1),
+    ((HUGE, 1, 3, 2), (HUGE, 1), 7),
+])
+def test_register_file_walk_ends_at_an_extent_of_all_ones(host, dims, pe, rf_words):
+    """The walk over the two divisor lists, with an extent equal to its mark for "no divisor left"; in a process of its own
+    with a time limit, since a walk that mistakes one for the other does not end."""
+    pool = multiprocessing.get_context("spawn").Pool(1)
+    try:
+        for op in (0, 1):
+            for sm in (0, 1, 2):
+                for objective in (mi.OBJ_ENERGY, mi.OBJ_LATENCY):
+                    args = (dims, pe, dims, op, sm, objective, rf_words)
+                    got = pool.apply_async(_tile_terms_at, (host.path,) + args).get(timeout=60)
+                    assert got == expected_terms(pe, dims, op, sm, objective, rf_words), args
+    finally:
+        pool.terminate()
