@@ -202,7 +202,9 @@ int mmee_destroy(mmee_handle_t* handle);
 /*
  * mmee_trim -- free the idle workspaces.  Device scratch and pinned host memory of released handles and one-shot calls
  * stay with the library for the next handle on the same device, at most eight of them (0.16 MB of device memory and
- * 11 KB of pinned host memory each); no two handles or calls share one.  Handles in use are not affected.
+ * 11 KB of pinned host memory each); no two handles or calls share one.  Handles in use are not affected.  A kept workspace
+ * belongs to the CUDA context it was made in and is dropped when that has ended (cudaDeviceReset): no call is needed before
+ * a reset, but handles must not be used after it, only destroyed.
  */
 int mmee_trim(void);
 

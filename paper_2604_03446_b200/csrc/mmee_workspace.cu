@@ -5,7 +5,11 @@
 // (a search of 768 tilings through mmee_solve_host: 730 us).  So a workspace that is no longer in use stays in a list,
 // at most kMaxIdle of them (0.16 MB of device and 11 KB of pinned host memory each), for the next handle on its device.
 // A workspace belongs to one handle or call at a time, whatever thread or stream uses it; mmee_trim frees the idle ones.
+// Its memory belongs to the context it was allocated in and ends with it (cudaDeviceReset, a destroyed driver context), so a
+// kept one is taken, or freed, only after the driver has confirmed that its allocation is still that one.
 #include "mmee_workspace.h"
+
+#include <cuda.h>
 
 #include <mutex>
 #include <new>
@@ -20,7 +24,61 @@ std::mutex g_mutex;
 Workspace* g_idle = nullptr;
 int g_n_idle = 0;
 
+// Driver calls, looked up through the runtime so that the library links no driver library; null where there is none.
+struct Driver {
+    CUresult (*pointer_attribute)(void*, CUpointer_attribute, CUdeviceptr) = nullptr;
+    CUresult (*current_context)(CUcontext*) = nullptr;
+
+    Driver() {
+        cudaDriverEntryPointQueryResult found;
+        void *a = nullptr, *b = nullptr;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &a, cudaEnableDefault, &found) != cudaSuccess ||
+            cudaGetDriverEntryPoint("cuCtxGetCurrent", &b, cudaEnableDefault, &found) != cudaSuccess || !a || !b) {
+            cudaGetLastError();
+            return;
+        }
+        pointer_attribute = reinterpret_cast<decltype(pointer_attribute)>(a);
+        current_context = reinterpret_cast<decltype(current_context)>(b);
+    }
+};
+
+const Driver& driver() {
+    static const Driver d;
+    return d;
+}
+
+// The driver's number of a device allocation, 0 if it is none (any more).
+unsigned long long allocation_id(const void* mem) {
+    unsigned long long id = 0;
+    const Driver& d = driver();
+    if (!d.pointer_attribute || d.pointer_attribute(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, (CUdeviceptr)mem) != CUDA_SUCCESS) return 0;
+    return id;
+}
+
+// Whether the workspace's memory still exists; without the driver calls nothing is kept, so that it does.
+bool alive(const Workspace* ws) { return !ws->id || allocation_id(ws->chain) == ws->id; }
+
+// The calling thread's context on `device`, its current device.
+CUcontext context_on(int device) {
+    CUcontext c = nullptr;
+    const Driver& d = driver();
+    if (!d.current_context) return nullptr;
+    if (d.current_context(&c) == CUDA_SUCCESS && c) return c;
+    // (a thread that has not called the runtime yet, or a context that was reset: the device's primary one)
+    if (cudaSetDevice(device) != cudaSuccess || d.current_context(&c) != CUDA_SUCCESS) return nullptr;
+    return c;
+}
+
+bool in_context(const Workspace* ws, CUcontext c) {
+    CUcontext own = nullptr;
+    return c && driver().pointer_attribute(&own, CU_POINTER_ATTRIBUTE_CONTEXT, (CUdeviceptr)ws->chain) == CUDA_SUCCESS && own == c;
+}
+
 int free_workspace(Workspace* ws) {
+    if (ws->chain && !alive(ws)) {      // gone with its context, the pinned memory as well
+        delete ws;
+        return MMEE_OK;
+    }
     cudaError_t e = ws->chain ? cudaFree(ws->chain) : cudaSuccess;
     if (ws->host) {
         const cudaError_t e2 = cudaFreeHost(ws->host);
@@ -42,6 +100,7 @@ int make_workspace(int device, Workspace** out) {
     unsigned char* mem = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), chain + 2 * bytes);
     ws->chain = reinterpret_cast<ChainRecord*>(mem);
+    if (e == cudaSuccess) ws->id = allocation_id(mem);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + chain + i * bytes);
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation
@@ -64,12 +123,21 @@ int make_workspace(int device, Workspace** out) {
 int workspace_acquire(int device, Workspace** out) {
     {
         std::lock_guard<std::mutex> lock(g_mutex);
-        for (Workspace** at = &g_idle; *at; at = &(*at)->next) {
-            if ((*at)->device != device) continue;
-            *out = *at;
-            *at = (*at)->next;
-            --g_n_idle;
-            return MMEE_OK;
+        const CUcontext context = g_idle ? context_on(device) : nullptr;
+        for (Workspace** at = &g_idle; *at;) {
+            Workspace* ws = *at;
+            const bool gone = !alive(ws);
+            if (gone || (ws->device == device && in_context(ws, context))) {
+                *at = ws->next;
+                --g_n_idle;
+                if (!gone) {
+                    *out = ws;
+                    return MMEE_OK;
+                }
+                delete ws;
+            } else {
+                at = &ws->next;
+            }
         }
     }
     const int rc = make_workspace(device, out);
@@ -79,7 +147,7 @@ int workspace_acquire(int device, Workspace** out) {
 }
 
 int workspace_release(Workspace* ws, bool clean) {
-    if (clean) {
+    if (clean && ws->id) {
         std::lock_guard<std::mutex> lock(g_mutex);
         if (g_n_idle < kMaxIdle) {
             ws->next = g_idle;

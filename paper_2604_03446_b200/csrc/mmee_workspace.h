@@ -8,6 +8,7 @@ namespace mmee {
 // One search's workspace.  Everything a search on the device needs fits it, whatever the problem.
 struct Workspace {
     int device;
+    unsigned long long id;          // the device allocation's number: the driver gives no other allocation the same one
     Scratch* scratch[2];            // device; headers are clean while the workspace is not in use.  Two, for a search that
                                     // publishes while the one before it on the handle still finalizes
     uint32_t max_ctas;              // partial lists a scratch has room for

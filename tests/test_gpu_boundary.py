@@ -1,5 +1,6 @@
 """GPU tests of the C-ABI boundary's helpers: decoding one index, launch counters, device checks."""
 import ctypes as C
+import os
 
 import numpy as np
 import pytest
@@ -480,3 +481,41 @@ def test_register_file_blocks_with_many_divisors(pe, rf_words, objective):
             mm.mmee_eval(h, int(start) * 9, 9, buf)          # one row: the nine stationary pairs
             for g, o in zip(mm.read_results(buf, 9), oracle.evaluate_range(p, int(start) * 9, 9)):
                 assert_same_record(g, o, "idx %d" % o.idx)
+
+
+RESET_SCRIPT = """
+import ctypes, glob, os, sys
+import mmee_inputs as mi
+import paper_2604_03446_b200.binding as mm
+cfg = mi.random_tiny_problem(3)
+obj = dict(cfg["searches"][0], topk=2)
+args = (cfg["workload"], cfg["arch"], obj)
+solve = lambda: [bytes(r) for r in mm.mmee_solve_host(*args)[1]]
+front = lambda: [bytes(r) for r in mm.mmee_pareto_front_bs_da(cfg["workload"], cfg["arch"], obj)]
+runtime = ctypes.CDLL(glob.glob(sys.argv[1])[0])
+want = solve(), front()
+held = mm.mmee_create(*args)
+for _ in range(2):
+    assert runtime.cudaDeviceReset() == 0
+    assert (solve(), front()) == want
+    mm.mmee_destroy(held)                       # its workspace went with the first context
+    held = mm.mmee_create(*args)
+    assert bytes(mm.mmee_search_host(held, True, 2)[1][0]) == want[0][0]
+assert runtime.cudaDeviceReset() == 0
+mm.mmee_trim()
+assert (solve(), front()) == want
+print("same records")
+"""
+
+
+def test_one_shot_calls_after_a_device_reset():
+    """cudaDeviceReset (between calls, nothing in flight) takes the kept workspaces with it: what follows gets memory of its
+    own.  In a process of its own, since a reset ends torch's context as well."""
+    import glob
+    import subprocess
+    import sys
+    libs = [p for d in sys.path for p in glob.glob(os.path.join(d, "nvidia", "cuda_runtime", "lib", "libcudart.so.*"))]
+    libs += glob.glob("/usr/local/cuda/lib64/libcudart.so.1*")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET_SCRIPT, libs[0]], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "same records" in r.stdout, r.stdout + r.stderr

@@ -1,0 +1,72 @@
+"""The library's host side against a stand-in for the CUDA runtime (fake_cuda.cpp), on the CPU: what it does when calls
+fail, when a wait runs out, and when memory it has kept is gone.  No GPU is used and none of the kernels."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+import mmee_inputs as mi
+import paper_2604_03446_b200.binding as mm
+from paper_2604_03446_b200 import build as lib_build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(lib_build._nvcc()))), "include")
+
+
+@pytest.fixture(scope="session")
+def fake_path(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("fake_runtime") / "host_side.so")
+    sources = [os.path.join(lib_build.CSRC, s) for s in ("mmee_api.cu", "mmee_workspace.cu", "mmee_plan.cu", "mmee_prune.cu")]
+    subprocess.check_call(["g++", "-x", "c++", "-std=c++17", "-O1", "-shared", "-fPIC", "-pthread", "-Wl,-Bsymbolic", "-I", CUDA_INCLUDE,
+                           "-o", out] + sources + [os.path.join(HERE, "fake_cuda.cpp")])
+    return out
+
+
+@pytest.fixture
+def fake(fake_path, tmp_path):
+    """A copy of its own for each test: the library's and the stand-in's state start fresh."""
+    import shutil
+    lib = C.CDLL(shutil.copy(fake_path, str(tmp_path / "host_side.so")))
+    lib.mmee_destroy.argtypes = [C.c_void_p]
+    return lib
+
+
+def problem(topk=2):
+    cfg = mi.config1()
+    return (C.byref(mm._fill(mm.Workload(), cfg["workload"])), C.byref(mm._fill(mm.Arch(), cfg["arch"])),
+            C.byref(mm._fill(mm.Objective(), mi.objective(mi.OBJ_ENERGY, topk))))
+
+
+def solve(lib):
+    best, topk = mm.Result(), (mm.Result * 2)()
+    return lib.mmee_solve_host(*problem(), C.byref(best), topk, None, None), best.idx
+
+
+def test_a_kept_workspace_does_not_outlive_its_context(fake):
+    """A device reset takes kept device and pinned memory with it: the next call gets memory of its own, and nothing that is
+    gone is used or freed again, whether it was idle at the reset or came back with its handle afterwards."""
+    assert solve(fake) == (mm.OK, 7) and fake.fake_live() == 2
+    fake.fake_device_reset()
+    assert solve(fake) == (mm.OK, 7) and fake.fake_bad_pointers() == 0 and fake.fake_live() == 2
+    fake.fake_device_reset()
+    assert fake.mmee_trim() == mm.OK and fake.fake_bad_pointers() == 0 and fake.fake_live() == 0
+
+    handles = []
+    for _ in range(10):                              # more than are kept
+        h = C.c_void_p()
+        assert fake.mmee_create(*problem(), C.byref(h)) == mm.OK
+        handles.append(h)
+    fake.fake_device_reset()
+    for h in handles:
+        assert fake.mmee_destroy(h) == mm.OK
+    assert solve(fake) == (mm.OK, 7) and fake.fake_bad_pointers() == 0 and fake.fake_live() == 2
+
+
+def test_a_kept_workspace_stays_in_its_context(fake):
+    """Several contexts on one device: each gets memory of its own, and keeps it."""
+    for c in (1, 2, 1, 2):
+        fake.fake_set_context(c)
+        assert solve(fake) == (mm.OK, 7)
+    assert fake.fake_bad_pointers() == 0 and fake.fake_live() == 4
+    assert fake.mmee_trim() == mm.OK and fake.fake_live() == 0
