@@ -65,7 +65,8 @@ extern "C" {
 #define MMEE_ERR_QUANTUM      3   /* an energy is not an integer multiple of energy_quantum_pj     */
 #define MMEE_ERR_NO_FEASIBLE  4   /* no mapping fits the buffer (reported in mmee_result_t.status) */
 #define MMEE_ERR_CUDA         5   /* a CUDA runtime call failed (no device, launch error, ...)     */
-#define MMEE_ERR_TIMEOUT      6   /* reserved: the kernels contain no device-side wait             */
+#define MMEE_ERR_TIMEOUT      6   /* a Pareto front's searches, steps of one kernel, waited for one another longer than a few
+                                     seconds (the only device-side wait, a limited one): the points are not a result      */
 #define MMEE_ERR_RANGE        7   /* request exceeds a documented maximum                          */
 #define MMEE_ERR_CHECK        8   /* a winner's ranking key is not the key of its full evaluation (internal
                                      consistency check of the finalize step): the records are not a result.

@@ -85,6 +85,7 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
     shape->late = n_arrays == 0 && (p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling));
     shape->chain_steps = shape->chain_epoch = 0;
     shape->chain_read = false;
+    shape->chain_polls = 0;
     shape->chain_to = nullptr;
     shape->chunk = (uint32_t)(passes ? (per_cta + passes - 1) / passes : 1);
     return MMEE_OK;
@@ -95,9 +96,10 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
 namespace {
 
 // Searches chained on the device (see LaunchShape::chain_steps) until one finds nothing: their optima in order, through
-// `take` (which returns false to stop).  The host waits for kHostRecords of them at a time.
+// `take` (which returns false to stop).  The host waits for kHostRecords of them at a time.  Every record a chain may write
+// is marked before its launch as one that did not come: whatever its CTAs did not get to shows, MMEE_ERR_TIMEOUT.
 template <class Take>
-int run_chain(const Plan& plan, Take take) {
+int run_chain(const Plan& plan, uint32_t polls, Take take) {
     int device = 0;
     int rc = cuda_status(cudaGetDevice(&device));
     if (rc) return rc;
@@ -108,21 +110,95 @@ int run_chain(const Plan& plan, Take take) {
     shape.late = false;
     shape.chain_steps = kHostRecords;
     shape.chain_to = ws->chain;
+    shape.chain_polls = polls;
     bool more = true;
     while (more && rc == MMEE_OK) {
         shape.chain_epoch = ++ws->chains * kHostRecords;
+        for (uint32_t i = 0; i < kHostRecords; ++i) ws->host[i].status = MMEE_ERR_TIMEOUT;
         rc = cuda_status(launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial, nullptr, ws->host_dev, nullptr));
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc == MMEE_OK) rc = rc2;
         for (uint32_t i = 0; i < kHostRecords && more && rc == MMEE_OK; ++i) {
             const mmee_result_t& r = ws->host[i];
-            if (r.status == MMEE_ERR_CHECK) { rc = MMEE_ERR_CHECK; break; }
+            if (r.status == MMEE_ERR_CHECK || r.status == MMEE_ERR_TIMEOUT) { rc = r.status; break; }
             more = r.idx != MMEE_NO_INDEX && take(r);
         }
         shape.chain_read = true;
     }
     const int rc2 = workspace_release(ws, rc == MMEE_OK);
     return rc ? rc : rc2;
+}
+
+int front_energy_latency(const mmee_workload_t* workload, const mmee_arch_t* arch, const mmee_objective_t* objective,
+                         uint32_t polls, mmee_result_t* out_points, uint32_t capacity, uint32_t* n_points) {
+    if (!objective || !n_points || (!out_points && capacity)) return MMEE_ERR_ARG;
+    *n_points = 0;
+    mmee_objective_t o = *objective;
+    o.topk = 1; o.row_pruning = 0; o.key_cap = INT64_MAX - 1;
+    o.objective = MMEE_OBJ_ENERGY_LCAP;
+    Plan plan;
+    int rc = build_plan(workload, arch, &o, &plan);
+    if (rc) return rc;
+    uint32_t n = 0;
+    // Each search finds the least energy among the mappings that are still faster than the previous point, and the least
+    // latency at that energy: the next point of the front, with its lowest index.  None: the front is complete.
+    rc = run_chain(plan, polls, [&](const mmee_result_t& r) {
+        if (n < capacity) out_points[n] = r;
+        ++n;
+        return true;
+    });
+    *n_points = n;
+    if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
+    return rc;
+}
+
+int front_buffer_dram(const mmee_workload_t* workload, const mmee_arch_t* arch, const mmee_objective_t* objective,
+                      uint32_t polls, mmee_result_t* out_points, uint32_t capacity, uint32_t* n_points) {
+    if (!arch || !objective || !n_points || (!out_points && capacity)) return MMEE_ERR_ARG;
+    *n_points = 0;
+    // DRAM words as the key: one quantum per DRAM word, nothing else costs anything
+    mmee_arch_t a = *arch;
+    a.e_dram_pj = 1.0; a.e_gb_pj = a.e_rf_pj = a.e_mac_pj = 0.0; a.c_softmax = 0.0; a.energy_quantum_pj = 1.0;
+    mmee_objective_t o = *objective;
+    o.objective = MMEE_OBJ_ENERGY; o.topk = 1; o.row_pruning = 0; o.key_cap = 0;
+    Plan plan;
+    int rc = build_plan(workload, &a, &o, &plan);
+    if (rc) return rc;
+    mmee_result_t held = {};
+    bool have = false;
+    uint32_t n = 0;
+    // Searches with a shrinking buffer: each returns the least DRAM traffic that fits, with the least buffer words that a
+    // mapping of the first block with that traffic needs; the next one allows one word less than that.  While the traffic
+    // stays the same the mapping found needs less buffer for the same traffic; when it rises, the mapping held is a point
+    // of the front.
+    auto emit = [&]() {
+        if (n < capacity) out_points[n] = held;
+        ++n;
+    };
+    rc = run_chain(plan, polls, [&](const mmee_result_t& r) {
+        if (have && r.e_key != held.e_key) emit();
+        held = r;
+        have = true;
+        plan.cap_words = r.bs - 1;      // (for the tables of the next chain: tilings that cannot fit are left out)
+        return plan.cap_words >= 0;
+    });
+    if (rc == MMEE_OK && have) emit();
+    // (points whose count of fitting mappings belongs to another bound: see resolve_record)
+    mmee_handle_t* h = nullptr;
+    for (uint32_t i = 0; i < n && i < capacity && rc == MMEE_OK; ++i) {
+        const uint32_t before = out_points[i].reserved2[0];
+        if (!before) continue;
+        if (!h && (rc = mmee_create(workload, &a, &o, &h))) break;
+        h->plan.cap_words = (int64_t)before - 1;
+        rc = mmee_search_host(h, &out_points[i], nullptr);
+    }
+    if (h) {
+        const int rc2 = mmee_destroy(h);
+        if (rc == MMEE_OK) rc = rc2;
+    }
+    *n_points = n;
+    if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
+    return rc;
 }
 
 }  // namespace
@@ -297,74 +373,18 @@ int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch, co
 
 int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch, const mmee_objective_t* objective,
                       mmee_result_t* out_points, uint32_t capacity, uint32_t* n_points) {
-    if (!objective || !n_points || (!out_points && capacity)) return MMEE_ERR_ARG;
-    *n_points = 0;
-    mmee_objective_t o = *objective;
-    o.topk = 1; o.row_pruning = 0; o.key_cap = INT64_MAX - 1;
-    o.objective = MMEE_OBJ_ENERGY_LCAP;
-    Plan plan;
-    int rc = build_plan(workload, arch, &o, &plan);
-    if (rc) return rc;
-    uint32_t n = 0;
-    // Each search finds the least energy among the mappings that are still faster than the previous point, and the least
-    // latency at that energy: the next point of the front, with its lowest index.  None: the front is complete.
-    rc = run_chain(plan, [&](const mmee_result_t& r) {
-        if (n < capacity) out_points[n] = r;
-        ++n;
-        return true;
-    });
-    *n_points = n;
-    if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
-    return rc;
+    return front_energy_latency(workload, arch, objective, kChainPolls, out_points, capacity, n_points);
 }
 
 int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* arch, const mmee_objective_t* objective,
                             mmee_result_t* out_points, uint32_t capacity, uint32_t* n_points) {
-    if (!arch || !objective || !n_points || (!out_points && capacity)) return MMEE_ERR_ARG;
-    *n_points = 0;
-    // DRAM words as the key: one quantum per DRAM word, nothing else costs anything
-    mmee_arch_t a = *arch;
-    a.e_dram_pj = 1.0; a.e_gb_pj = a.e_rf_pj = a.e_mac_pj = 0.0; a.c_softmax = 0.0; a.energy_quantum_pj = 1.0;
-    mmee_objective_t o = *objective;
-    o.objective = MMEE_OBJ_ENERGY; o.topk = 1; o.row_pruning = 0; o.key_cap = 0;
-    Plan plan;
-    int rc = build_plan(workload, &a, &o, &plan);
-    if (rc) return rc;
-    mmee_result_t held = {};
-    bool have = false;
-    uint32_t n = 0;
-    // Searches with a shrinking buffer: each returns the least DRAM traffic that fits, with the least buffer words that a
-    // mapping of the first block with that traffic needs; the next one allows one word less than that.  While the traffic
-    // stays the same the mapping found needs less buffer for the same traffic; when it rises, the mapping held is a point
-    // of the front.
-    auto emit = [&]() {
-        if (n < capacity) out_points[n] = held;
-        ++n;
-    };
-    rc = run_chain(plan, [&](const mmee_result_t& r) {
-        if (have && r.e_key != held.e_key) emit();
-        held = r;
-        have = true;
-        plan.cap_words = r.bs - 1;      // (for the tables of the next chain: tilings that cannot fit are left out)
-        return plan.cap_words >= 0;
-    });
-    if (rc == MMEE_OK && have) emit();
-    // (points whose count of fitting mappings belongs to another bound: see resolve_record)
-    mmee_handle_t* h = nullptr;
-    for (uint32_t i = 0; i < n && i < capacity && rc == MMEE_OK; ++i) {
-        const uint32_t before = out_points[i].reserved2[0];
-        if (!before) continue;
-        if (!h && (rc = mmee_create(workload, &a, &o, &h))) break;
-        h->plan.cap_words = (int64_t)before - 1;
-        rc = mmee_search_host(h, &out_points[i], nullptr);
-    }
-    if (h) {
-        const int rc2 = mmee_destroy(h);
-        if (rc == MMEE_OK) rc = rc2;
-    }
-    *n_points = n;
-    if (rc == MMEE_OK && n > capacity) rc = MMEE_ERR_RANGE;
-    return rc;
+    return front_buffer_dram(workload, arch, objective, kChainPolls, out_points, capacity, n_points);
+}
+
+int mmee_front_with_polls(int buffer_dram, const mmee_workload_t* workload, const mmee_arch_t* arch,
+                          const mmee_objective_t* objective, uint32_t polls, mmee_result_t* out_points, uint32_t capacity,
+                          uint32_t* n_points) {
+    return (buffer_dram ? front_buffer_dram : front_energy_latency)(workload, arch, objective, polls, out_points, capacity, n_points);
 }
 
 int mmee_search_shapes(const mmee_workload_t* workload, const mmee_arch_t* arch, const mmee_objective_t* objective,

@@ -153,6 +153,7 @@ struct Shared {
     long long bound;                // chained searches: that bound
     uint32_t cursor;                // next group of 32 items
     uint32_t last_cta, check_failed;
+    uint32_t waited;                // chained searches: the one waited for is over
     union {
         TileTab tile[kMaxChunk];
         BlockTab block[kWarps];
@@ -411,17 +412,16 @@ __device__ __forceinline__ int split_item(int warp, int lane) {
 
 // Chained searches run one after the other in one kernel, whose CTAs are all resident (a cooperative launch): a CTA that
 // has published its part of one waits for the CTA that merges the parts, which sets the header's epoch to that search's
-// when it has left the bound for the next.  kRecordCtas more make the records meanwhile.  The wait is limited, at a few
-// seconds; true: the search is over.
+// when it has left the bound for the next.  kRecordCtas more make the records meanwhile.  The wait is limited (`polls`);
+// true: the search is over.
 // Steps of about 8 us are bound by publish, ticket, merge and this wait, the first of a large front by their items.  Front of
 // the GPT-3 FFN (20 searches), a launch per search that waited for the one before 264 us, steps of one kernel 202 (now 187);
 // 99 random fronts 241 and 198 us; the energy-latency front of 10 816 tilings 56.5 and 55.3.
-constexpr uint32_t kMaxPolls = 1u << 22;
 constexpr int64_t kNoBound = INT64_MIN;         // what a search leaves that found nothing
 
 // The low half of the header's word is the bound where it has 32 bits (a capacity).
-__device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t epoch, uint32_t& low) {
-    for (uint32_t i = 0; i < kMaxPolls; ++i) {
+__device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t epoch, uint32_t polls, uint32_t& low) {
+    for (uint32_t i = 0; i < polls; ++i) {
         unsigned long long now;
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(now) : "l"(&head->chain_epoch) : "memory");
         low = (uint32_t)now;
@@ -753,19 +753,16 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
 }
 
 // The records of chained searches as they end, by kRecordCtas CTAs, this one number `which`: the first search has the epoch
-// shape.chain_epoch, the last one finds nothing.
+// shape.chain_epoch, the last one finds nothing.  A record is written as a whole or not at all.
 template <bool FRONT>
 __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& shape, Shared& sh, const SearchHeader* head, uint32_t which,
                                            mmee_result_t* out) {
     for (uint32_t i = 0; i < shape.chain_steps; ++i) {
         __syncthreads();
         uint32_t low;
-        if (threadIdx.x == 0 && !await_epoch(head, shape.chain_epoch + i, low)) sh.check_failed = 1;
+        if (threadIdx.x == 0) sh.waited = await_epoch(head, shape.chain_epoch + i, shape.chain_polls, low) ? 1u : 0u;
         __syncthreads();
-        if (sh.check_failed) {
-            if (threadIdx.x == 0) out[i].status = MMEE_ERR_CHECK;
-            return;
-        }
+        if (!sh.waited) return;
         const volatile ChainRecord* from = shape.chain_to + i;
         const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound, from->need, 0};
         if (i % kRecordCtas == which) {
@@ -920,7 +917,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             __syncthreads();                // the counters of the search before are no longer in use
             if (tid == 0) {
                 uint32_t low = 0;
-                const bool over = !step || await_epoch(head, shape.chain_epoch + step - 1, low);
+                const bool over = !step || await_epoch(head, shape.chain_epoch + step - 1, shape.chain_polls, low);
                 if (!over) sh.bound = kNoBound;
                 else if (step && STAIRS) sh.bound = low == 0xffffffffu ? kNoBound : (int64_t)low;
                 else sh.bound = *reinterpret_cast<volatile long long*>(&head->chain_bound);

@@ -61,6 +61,7 @@ struct LaunchShape {
     uint32_t chain_steps;   // a chain of this many searches in one launch, 0: one search
     uint32_t chain_epoch;   // ... their numbers on this scratch, ascending and greater than any before: the first one's
     bool chain_read;        // ... that goes on from the launch before
+    uint32_t chain_polls;   // ... how often a CTA looks for the end of a search before it gives up (see kChainPolls)
     ChainRecord* chain_to;  // device: where they leave their optima
 };
 // Chained searches (k = 1, no row pruning; the Pareto fronts): each takes a bound from what the one before it found: the
@@ -72,6 +73,9 @@ struct LaunchShape {
 // one 217 us, two 202, four 205 because the searches have fewer CTAs; records after the chain 204, where a front of one point
 // takes 59 instead of 55.)
 constexpr uint32_t kRecordCtas = 2;
+// The wait for a chained search is limited, at a few seconds.  A CTA whose wait runs out leaves without a trace: it takes no
+// part in later searches, which then do not end, and makes no more records, so that the caller finds one that was not made.
+constexpr uint32_t kChainPolls = 1u << 22;
 
 inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 

@@ -31,3 +31,9 @@ int workspace_release(Workspace* ws, bool clean);
 int workspace_trim();
 
 }  // namespace mmee
+
+// The Pareto fronts (0: energy-latency, 1: buffer size / DRAM traffic) with a limit of their own on the waits between their
+// searches, LaunchShape::chain_polls: 0 lets every wait run out.  For tests; not part of the ABI.
+extern "C" int mmee_front_with_polls(int buffer_dram, const mmee_workload_t* workload, const mmee_arch_t* arch,
+                                     const mmee_objective_t* objective, uint32_t polls, mmee_result_t* out_points,
+                                     uint32_t capacity, uint32_t* n_points);

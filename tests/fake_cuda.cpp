@@ -19,6 +19,8 @@ int g_context = 1;                              // current context
 cudaError_t g_last = cudaSuccess;               // the runtime's last error: kept until it is read
 int g_fail_malloc = 0, g_fail_host = 0;         // fail that many calls
 int g_bad_pointers = 0;                         // launches and frees that were given memory that is not there
+int g_points = 0;                               // optima a chain of searches finds
+unsigned g_missing = 0;                         // bit i: the record of its search i is not made
 
 cudaError_t failed(cudaError_t e) { return g_last = e; }
 
@@ -75,6 +77,7 @@ void fake_device_reset() {
 }
 void fake_set_context(int c) { g_context = c; }
 void fake_fail(int mallocs, int host_allocs) { g_fail_malloc = mallocs; g_fail_host = host_allocs; }
+void fake_chain(int points, unsigned missing) { g_points = points; g_missing = missing; }
 int fake_live() { return (int)g_live.size(); }
 int fake_bad_pointers() { return g_bad_pointers; }
 int fake_last_error() { return (int)g_last; }
@@ -119,10 +122,18 @@ static mmee_result_t found() {
     return r;
 }
 
-cudaError_t launch_search(const Plan& p, const LaunchShape&, SearchHeader* head, Partial* partials, mmee_result_t* best,
+cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials, mmee_result_t* best,
                           mmee_result_t* topk, cudaStream_t) {
     touch(head);
     touch(partials);
+    for (int i = 0; i < (int)shape.chain_steps; ++i) {
+        mmee_result_t r = found();
+        r.e_key = i;
+        r.bs = 1000 - i;
+        if (i >= g_points) { r.idx = MMEE_NO_INDEX; r.status = MMEE_ERR_NO_FEASIBLE; }
+        if (!(g_missing >> i & 1u)) topk[i] = r;
+        if (i >= g_points) return cudaSuccess;
+    }
     if (find(best)) *best = found();
     for (uint32_t i = 0; topk && find(topk) && i < p.topk; ++i) topk[i] = found();
     return cudaSuccess;

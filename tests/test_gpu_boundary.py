@@ -519,3 +519,29 @@ def test_one_shot_calls_after_a_device_reset():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", RESET_SCRIPT, libs[0]], cwd=root, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and "same records" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("buffer_dram", [0, 1])
+def test_fronts_whose_waits_run_out(buffer_dram):
+    """The searches of a front wait for one another on the device, a limited number of looks: with a limit that is too low
+    the call ends with a status of its own and leaves nothing behind that a later call would see.  (A limit in between may
+    suffice or not; what is returned then is the whole front.)"""
+    cfg = mi.random_tiny_problem(9)
+    obj = shrink_to(cfg, dict(cfg["searches"][0], objective=mi.OBJ_ENERGY, topk=1), 1_000_000)
+    args = [C.byref(mm._fill(s(), d)) for s, d in ((mm.Workload, cfg["workload"]), (mm.Arch, cfg["arch"]), (mm.Objective, obj))]
+    public = (mm.mmee_pareto_front, mm.mmee_pareto_front_bs_da)[buffer_dram]
+    want = [bytes(r) for r in public(cfg["workload"], cfg["arch"], obj)]
+    assert want
+
+    def limited(polls):
+        pts, n = (mm.Result * 256)(), C.c_uint32()
+        status = mm.library().mmee_front_with_polls(buffer_dram, *args, C.c_uint32(polls), pts, 256, C.byref(n))
+        return status, [bytes(r) for r in pts[:n.value]]
+
+    assert limited(1 << 22) == (mm.OK, want)
+    for polls in (0, 0, 1, 10, 30, 100, 300, 1000):
+        status, got = limited(polls)
+        assert status == mm.ERR_TIMEOUT if polls == 0 else (status == mm.ERR_TIMEOUT or (status, got) == (mm.OK, want))
+        if polls in (0, 100):
+            assert [bytes(r) for r in public(cfg["workload"], cfg["arch"], obj)] == want
+    assert limited(1 << 22) == (mm.OK, want)

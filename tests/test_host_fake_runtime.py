@@ -70,3 +70,20 @@ def test_a_kept_workspace_stays_in_its_context(fake):
         assert solve(fake) == (mm.OK, 7)
     assert fake.fake_bad_pointers() == 0 and fake.fake_live() == 4
     assert fake.mmee_trim() == mm.OK and fake.fake_live() == 0
+
+
+@pytest.mark.parametrize("front", ["mmee_pareto_front", "mmee_pareto_front_bs_da"])
+@pytest.mark.parametrize("missing", [1, 2, 4, 8, 0b1010])
+def test_a_front_whose_wait_ran_out_returns_no_older_record(fake, front, missing):
+    """Records that a front's kernel did not get to make are not read from what an earlier call left in the same memory: the
+    status says that the wait ran out.  The next call starts clean."""
+    def call():
+        pts, n = (mm.Result * 8)(), C.c_uint32()
+        return getattr(fake, front)(*problem(), pts, 8, C.byref(n)), n.value, [r.e_key for r in pts[:n.value]]
+
+    fake.fake_chain(3, 0)
+    assert call() == (mm.OK, 3, [0, 1, 2])
+    fake.fake_chain(3, missing)
+    assert call()[0] == mm.ERR_TIMEOUT
+    fake.fake_chain(2, 0)
+    assert call() == (mm.OK, 2, [0, 1]) and fake.fake_bad_pointers() == 0
