@@ -62,11 +62,11 @@ int max_search_ctas(int device, uint32_t* out) {
     return MMEE_OK;
 }
 
-int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape, uint32_t spare) {
-    uint32_t most = 0;
-    const int rc = max_search_ctas(device, &most);
-    if (rc) return rc;
-    most = most > spare ? most - spare : 1;
+int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape, uint32_t most) {
+    if (!most) {
+        const int rc = max_search_ctas(device, &most);
+        if (rc) return rc;
+    }
     // Small problems take fewer CTAs, with at least eight tilings each.
     const uint64_t tilings = p.t_end - p.t_begin;
     constexpr uint64_t kMinTilings = 8;
@@ -103,19 +103,30 @@ int run_chain(const Plan& plan, uint32_t polls, Take take) {
     int device = 0;
     int rc = cuda_status(cudaGetDevice(&device));
     if (rc) return rc;
+    uint32_t most = 0;
+    if ((rc = max_search_ctas(device, &most))) return rc;
+    most -= kRecordCtas - 1;
     LaunchShape shape;
-    if ((rc = choose_launch_shape(plan, device, 0, 0, &shape, kRecordCtas - 1))) return rc;
+    if ((rc = choose_launch_shape(plan, device, 0, 0, &shape, most))) return rc;
     Workspace* ws = nullptr;
     if ((rc = workspace_acquire(device, &ws))) return rc;
-    shape.late = false;
-    shape.chain_steps = kHostRecords;
-    shape.chain_to = ws->chain;
-    shape.chain_polls = polls;
-    bool more = true;
+    bool more = true, read = false;
     while (more && rc == MMEE_OK) {
+        shape.late = false;
+        shape.chain_steps = kHostRecords;
+        shape.chain_to = ws->chain;
+        shape.chain_polls = polls;
+        shape.chain_read = read;
         shape.chain_epoch = ++ws->chains * kHostRecords;
         for (uint32_t i = 0; i < kHostRecords; ++i) ws->host[i].status = MMEE_ERR_TIMEOUT;
-        rc = cuda_status(launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial, nullptr, ws->host_dev, nullptr));
+        const cudaError_t e = launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial, nullptr, ws->host_dev, nullptr);
+        if (e == cudaErrorCooperativeLaunchTooLarge && shape.grid > 1) {
+            // the calling context has a part of the device's SMs: half the CTAs, until they are resident together
+            cudaGetLastError();
+            rc = choose_launch_shape(plan, device, 0, 0, &shape, shape.grid / 2);
+            continue;
+        }
+        rc = cuda_status(e);
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc == MMEE_OK) rc = rc2;
         for (uint32_t i = 0; i < kHostRecords && more && rc == MMEE_OK; ++i) {
@@ -123,7 +134,7 @@ int run_chain(const Plan& plan, uint32_t polls, Take take) {
             if (r.status == MMEE_ERR_CHECK || r.status == MMEE_ERR_TIMEOUT) { rc = r.status; break; }
             more = r.idx != MMEE_NO_INDEX && take(r);
         }
-        shape.chain_read = true;
+        read = true;
     }
     const int rc2 = workspace_release(ws, rc == MMEE_OK);
     return rc ? rc : rc2;

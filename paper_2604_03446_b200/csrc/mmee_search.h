@@ -99,9 +99,9 @@ cudaError_t measure_alu_peak(double* giops);
 
 // Most CTAs that a search on `device` takes.
 int max_search_ctas(int device, uint32_t* out);
-// Launch shape of a search of n_arrays array shapes (0: the plan's own) on `device` (at most max_ctas CTAs when that is not
-// 0: MMEE_ERR_RANGE if it would take more).  `spare` CTAs fewer where it takes the most.
-int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape, uint32_t spare = 0);
+// Launch shape of a search of n_arrays array shapes (0: the plan's own) on `device` (for a scratch of max_ctas CTAs when that
+// is not 0: MMEE_ERR_RANGE if it would take more).  `most`: CTAs it takes at most, when that is not 0.
+int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t max_ctas, LaunchShape* shape, uint32_t most = 0);
 
 // MMEE_OK, or MMEE_ERR_CUDA with the error kept for mmee_last_cuda_error (per host thread).
 int cuda_status(cudaError_t e);

@@ -545,3 +545,38 @@ def test_fronts_whose_waits_run_out(buffer_dram):
         if polls in (0, 100):
             assert [bytes(r) for r in public(cfg["workload"], cfg["arch"], obj)] == want
     assert limited(1 << 22) == (mm.OK, want)
+
+
+PART_SCRIPT = """
+import ctypes as C
+import mmee_inputs as mi
+import paper_2604_03446_b200.binding as mm
+w, a, o = mi.workload(1, 1, 1, 4096, 4096, 128, 128), mi.arch_edge(), mi.objective(mi.OBJ_ENERGY, 1)
+fronts = lambda: [[bytes(r) for r in f(w, a, o)] for f in (mm.mmee_pareto_front, mm.mmee_pareto_front_bs_da)]
+want = fronts()
+driver = C.CDLL("libcuda.so.1")
+def call(name, *args):
+    status = getattr(driver, name)(*args)
+    assert status == 0, (name, status)
+dev, whole, rest, part = C.c_int(), (C.c_ubyte * 256)(), (C.c_ubyte * 256)(), (C.c_ubyte * 256)()
+call("cuDeviceGet", C.byref(dev), 0)
+call("cuDeviceGetDevResource", dev, whole, 1)
+n, desc, green, context = C.c_uint(1), C.c_void_p(), C.c_void_p(), C.c_void_p()
+call("cuDevSmResourceSplitByCount", part, C.byref(n), whole, rest, 0, 32)
+call("cuDevResourceGenerateDesc", C.byref(desc), part, 1)
+call("cuGreenCtxCreate", C.byref(green), desc, dev, 1)
+call("cuCtxFromGreenCtx", C.byref(context), green)
+call("cuCtxSetCurrent", context)
+assert fronts() == want
+print("same records")
+"""
+
+
+def test_fronts_in_a_context_with_a_part_of_the_sms():
+    """In a context that owns 32 SMs the steps of a front cannot have as many CTAs as the device holds: the fronts' points are
+    those found with all SMs.  In a process of its own, which ends with that context."""
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", PART_SCRIPT], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "same records" in r.stdout, r.stdout + r.stderr

@@ -87,3 +87,15 @@ def test_a_front_whose_wait_ran_out_returns_no_older_record(fake, front, missing
     assert call()[0] == mm.ERR_TIMEOUT
     fake.fake_chain(2, 0)
     assert call() == (mm.OK, 2, [0, 1]) and fake.fake_bad_pointers() == 0
+
+
+@pytest.mark.parametrize("front", ["mmee_pareto_front", "mmee_pareto_front_bs_da"])
+def test_fronts_take_the_ctas_that_can_be_resident_together(fake, front):
+    """A context with a part of the SMs holds fewer CTAs at once than the device: the front runs on those."""
+    for resident, status in ((296, mm.OK), (295, mm.OK), (64, mm.OK), (3, mm.OK), (2, mm.ERR_CUDA), (1000, mm.OK)):
+        fake.fake_resident(resident)
+        fake.fake_chain(3, 0)
+        pts, n = (mm.Result * 8)(), C.c_uint32()
+        assert getattr(fake, front)(*problem(), pts, 8, C.byref(n)) == status and n.value == (3 if status == mm.OK else 0)
+        assert fake.fake_last_error() == 0 or status != mm.OK
+    assert fake.fake_bad_pointers() == 0
