@@ -36,9 +36,12 @@ thread_local cudaError_t g_last_cuda_error = cudaSuccess;
 
 namespace mmee {
 
+// (An error that is reported here is taken off the runtime, which would otherwise give it to the next launch that asks for
+// its last error.)
 int cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return MMEE_OK;
     g_last_cuda_error = e;
+    cudaGetLastError();
     return MMEE_ERR_CUDA;
 }
 

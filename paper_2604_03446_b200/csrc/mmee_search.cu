@@ -1283,8 +1283,10 @@ cudaError_t launch_search_arrays(const Plan& p, const LaunchShape& shape, Partia
 }
 
 cudaError_t launch_reset(SearchHeader* head, cudaStream_t st) {
-    reset_kernel<<<1, 1, 0, st>>>(head);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = cfg.blockDim = dim3(1);
+    cfg.stream = st;
+    return cudaLaunchKernelEx(&cfg, reset_kernel, head);        // this launch's error, not the runtime's last one
 }
 
 }  // namespace mmee

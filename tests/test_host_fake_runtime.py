@@ -99,3 +99,28 @@ def test_fronts_take_the_ctas_that_can_be_resident_together(fake, front):
         assert getattr(fake, front)(*problem(), pts, 8, C.byref(n)) == status and n.value == (3 if status == mm.OK else 0)
         assert fake.fake_last_error() == 0 or status != mm.OK
     assert fake.fake_bad_pointers() == 0
+
+
+@pytest.mark.parametrize("mallocs,host_allocs", [(1, 0), (0, 1)])
+def test_a_failed_allocation_is_tried_again_without_the_idle_workspaces(fake, mallocs, host_allocs):
+    """An allocation that fails once succeeds after the idle workspaces are freed; its error does not come back as the
+    status of a later launch."""
+    fake.fake_set_context(1)
+    assert solve(fake) == (mm.OK, 7)                 # leaves an idle workspace of another context
+    fake.fake_set_context(2)
+    fake.fake_fail(mallocs, host_allocs)
+    assert solve(fake) == (mm.OK, 7)
+    assert fake.fake_live() == 2 and fake.fake_last_error() == 0 and fake.fake_bad_pointers() == 0
+
+
+def test_an_allocation_that_keeps_failing_is_reported_once(fake):
+    fake.fake_fail(2, 0)
+    assert solve(fake)[0] == mm.ERR_CUDA and fake.fake_live() == 0 and fake.fake_last_error() == 0
+    assert solve(fake) == (mm.OK, 7)
+    h = C.c_void_p()
+    assert fake.mmee_create(*problem(), C.byref(h)) == mm.OK
+    fake.fake_fail(2, 0)
+    other = C.c_void_p()
+    assert fake.mmee_create(*problem(), C.byref(other)) == mm.ERR_CUDA and not other.value
+    assert fake.mmee_decode(h, C.c_uint64(0), C.byref(mm.Result())) == mm.OK       # not that call's error
+    assert fake.mmee_destroy(h) == mm.OK
