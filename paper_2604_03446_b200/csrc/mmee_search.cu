@@ -144,7 +144,7 @@ struct Shared {
     uint32_t pe_rows, pe_cols;      // the array's logical shape
     uint32_t row_folds[4][MMEE_MAX_DIVISORS], col_folds[4][MMEE_MAX_DIVISORS];      // register-file tiling only
     alignas(16) longlong2 tops[kWarps][MMEE_MAX_TOPK];
-    longlong2 kth[kWarps];          // finalize, k > 1: the k-th pair of each warp's list (kInfKey: not full)
+    long long kth[kWarps];          // finalize, k > 1: the k-th key of each warp's list (kInfKey: not full)
     long long G;                    // k > 1: upper bound on the k-th smallest key
     unsigned long long feasible_rows[kWarps];
     uint32_t live_tilings[kWarps];
@@ -249,12 +249,6 @@ __device__ __forceinline__ uint64_t least_need_before(const Plan& p, const Limit
     return warp_min_u64(least, in);
 }
 
-__device__ __forceinline__ longlong2 ld_volatile(const longlong2* a) {
-    longlong2 v;
-    asm volatile("ld.volatile.shared.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"((uint32_t)__cvta_generic_to_shared(a)));
-    return v;
-}
-
 // The mappings of block `j` of sh.block that precede the running k-th pair (lk, li), none above `bound`, into the warps'
 // lists.  A lane holds one class combination and walks its mappings in (key, index) order: the stationary pairs of its
 // least key over its rows, then those of the next larger key; the warp takes the smallest of its lanes' next mappings
@@ -278,12 +272,17 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits&
         uint32_t pairs = 0, left = 0;           // stationary pairs with that key, those left of the row
         uint32_t row = 0;                       // the row, and where its levels stand within their classes
         int at[5] = {0, 0, 0, 0, 0};
-        // (every warp's k-th pair bounds the block's: a torn view is impossible, a pair is one 16-byte word)
-        const longlong2 other = ld_volatile(&sh.kth[lane & (kWarps - 1)]);
-        int64_t ok = other.x, nk = kInfKey;
-        uint64_t oi = (uint64_t)other.y, ni = UINT64_MAX;
-        warp_min_pair(ok, oi);
-        if (pair_less(ok, oi, lk, li)) { lk = ok; li = oi; }
+        int64_t nk = kInfKey;
+        uint64_t ni = UINT64_MAX;
+        // This warp's k-th pair bounds the block's; of the other warps' the key alone does, with any index, since they may be
+        // writing it: one 64-bit access each.
+        static_assert(sizeof(sh.kth[0]) == 8, "read without a barrier: a word that cannot be seen half written");
+        const int64_t own_k = __shfl_sync(kFull, ek, k - 1);
+        const uint64_t own_i = __shfl_sync(kFull, ei, k - 1);
+        if (pair_less(own_k, own_i, lk, li)) { lk = own_k; li = own_i; }
+        bool in = true;
+        const int64_t other = (int64_t)warp_min_u64((uint64_t)*const_cast<volatile long long*>(&sh.kth[lane & (kWarps - 1)]), in);
+        if (other < lk) { lk = other; li = UINT64_MAX; }
         bool advance = r < n_reps && t.fits;
         if (!advance) hk = kInfKey;
         int64_t level = -1;                     // the key whose mappings are being taken
@@ -340,7 +339,7 @@ __device__ __forceinline__ void best_of_block_multi(const Plan& p, const Limits&
             ++i;
         }
         reg_merge(ek, ei, k, nk, ni, lane);
-        if (lane == k - 1) sh.kth[threadIdx.x >> 5] = make_longlong2((long long)ek, (long long)ei);
+        if (lane == k - 1) *const_cast<volatile long long*>(&sh.kth[threadIdx.x >> 5]) = ek;
         __syncwarp();
     }
 }
@@ -599,7 +598,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
                 const int item = j0 ? (j == warp ? lane : -1) : split_item(warp, lane);
                 if (item >= 0) block_item(p, SharedDivisors{sh}, id, item, &sh.block[j]);
             }
-            if (lane == 0) sh.kth[warp] = make_longlong2(kInfKey, -1ll);
+            if (lane == 0) sh.kth[warp] = kInfKey;
             __syncthreads();
 #pragma unroll 1
             for (int j = 0; j < n_batch; ++j) {

@@ -657,3 +657,18 @@ def test_records_whose_folds_come_near_the_32_bit_limit(dims, pe):
             mm.mmee_eval(h, start, 9, buf)
             for g, o in zip(mm.read_results(buf, 9), oracle.evaluate_range(p, start, 9)):
                 assert_same_record(g, o, "idx %d" % o.idx)
+
+
+@pytest.mark.parametrize("topk", [2, 7, 16])
+@pytest.mark.parametrize("fuse_mask", [7, 1, 6])
+def test_lists_of_mappings_that_all_tie(fuse_mask, topk):
+    """No access costs anything, so that every mapping that fits has the key zero: the list holds the lowest indices, which
+    the warps that walk the winning block find at the same time, each bounded by what the others have; three capacities."""
+    for kb in (1, 3, 32):
+        cfg = dict(name="ties", workload=mi.workload(1, 1, 1, 48, 40, 24, 12, 2),
+                   arch=mi.arch(4, 4, 1, kb * 1024, 0, 2, 0.0, 0.0, 0.0, 0.0, c_softmax=0.0))
+        obj = mi.objective(mi.OBJ_ENERGY, topk, fuse_mask=fuse_mask, t_begin=1500, t_end=1512)
+        check_search(cfg, obj)
+        want = [r.idx for r in gpu_search(cfg, obj)[1]]
+        for _ in range(30):
+            assert [r.idx for r in gpu_search(cfg, obj)[1]] == want
