@@ -377,9 +377,9 @@ int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch, co
     if (rc) return rc;
     const uint32_t k = h->plan.topk;
     rc = mmee_search_host(h, out_best, out_topk);
-    // The plan (divisor lists, query vectors, coefficients) travels to the device as the kernels'
-    // parameter block: once per launch.
-    if (h2d_bytes) *h2d_bytes = 2ull * sizeof(mmee::Plan);
+    // The plan (divisor lists, query vectors, coefficients) travels to the device as the search kernel's parameter block,
+    // with the launch shape and four pointers: one launch.
+    if (h2d_bytes) *h2d_bytes = sizeof(mmee::Plan) + sizeof(mmee::LaunchShape) + 4 * sizeof(void*);
     if (d2h_bytes) *d2h_bytes = sizeof(mmee_result_t) * (uint64_t)(1 + (out_topk ? k : 0));
     const int rc2 = mmee_destroy(h);
     return rc ? rc : rc2;

@@ -21,6 +21,7 @@ int g_fail_malloc = 0, g_fail_host = 0;         // fail that many calls
 int g_bad_pointers = 0;                         // launches and frees that were given memory that is not there
 int g_points = 0;                               // optima a chain of searches finds
 unsigned g_resident = 1000;                     // CTAs of a chain that can be resident at once
+int g_searches = 0;                             // search launches
 unsigned g_missing = 0;                         // bit i: the record of its search i is not made
 
 cudaError_t failed(cudaError_t e) { return g_last = e; }
@@ -80,6 +81,8 @@ void fake_set_context(int c) { g_context = c; }
 void fake_fail(int mallocs, int host_allocs) { g_fail_malloc = mallocs; g_fail_host = host_allocs; }
 void fake_chain(int points, unsigned missing) { g_points = points; g_missing = missing; }
 void fake_resident(unsigned ctas) { g_resident = ctas; }
+int fake_searches() { return g_searches; }
+int fake_plan_bytes() { return (int)sizeof(mmee::Plan); }
 int fake_live() { return (int)g_live.size(); }
 int fake_bad_pointers() { return g_bad_pointers; }
 int fake_last_error() { return (int)g_last; }
@@ -126,6 +129,7 @@ static mmee_result_t found() {
 
 cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials, mmee_result_t* best,
                           mmee_result_t* topk, cudaStream_t) {
+    ++g_searches;
     touch(head);
     touch(partials);
     if (shape.chain_steps && shape.grid + kRecordCtas > g_resident) return failed(cudaErrorCooperativeLaunchTooLarge);

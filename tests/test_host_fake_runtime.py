@@ -124,3 +124,11 @@ def test_an_allocation_that_keeps_failing_is_reported_once(fake):
     assert fake.mmee_create(*problem(), C.byref(other)) == mm.ERR_CUDA and not other.value
     assert fake.mmee_decode(h, C.c_uint64(0), C.byref(mm.Result())) == mm.OK       # not that call's error
     assert fake.mmee_destroy(h) == mm.OK
+
+
+def test_bytes_that_a_one_shot_call_says_it_moved(fake):
+    """To the device the parameters of the launches it makes: one plan for one search; back the records."""
+    best, topk, h2d, d2h = mm.Result(), (mm.Result * 2)(), C.c_uint64(), C.c_uint64()
+    assert fake.mmee_solve_host(*problem(), C.byref(best), topk, C.byref(h2d), C.byref(d2h)) == mm.OK
+    assert fake.fake_searches() == 1 and d2h.value == 3 * mm.RESULT_BYTES
+    assert fake.fake_plan_bytes() <= h2d.value < fake.fake_plan_bytes() + 512
