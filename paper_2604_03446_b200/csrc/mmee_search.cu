@@ -778,10 +778,11 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
 
 // Searches launched one after the other overlap (programmatic dependent launch), in one of two ways.
 //   early: a search lets the next one start at once; that one's CTAs move in as this one's leave, and wait for its end
-//          before they publish (k > 1: before their items), since it may still use their scratch;
+//          before they publish, since it may still use their scratch;
 //   late:  only the CTA that finalizes waits for the kernel before, and lets the next search start after that wait.  The
 //          CTAs then publish while the search before finalizes, into the other one of the handle's two scratches: the
-//          search that used theirs last had ended before the one before them let them start.
+//          search that used theirs last had ended before the one before them let them start.  (Always for k > 1, whose CTAs
+//          share a bound through the scratch while they work on their items.)
 // A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  Searches one after
 // the other, without and with this (us each): smallest configuration 20.5 and 8.9, BERT energy 22.9 and 10.4, GQA latency
 // 28.7 and 13.7, convolution chain top-16 133 and 58 (other changes between them included).
@@ -822,7 +823,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     static_assert(FRONT || STAIRS || !CHAIN, "only the searches of the Pareto fronts are chained");
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool late = shape.late;
+    const bool late = MULTI || shape.late;
     if (!late) release_next_kernel();
     load_shared<PRUNE>(p, p.pe_rows, p.pe_cols, sh);
     // Array shapes: the stationary-pair terms of shape y and tiling slot i at [y * chunk + i], behind the tilings' tables;
@@ -971,11 +972,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 __syncwarp();
                 if (live) build_tile<!ARRAYS>(p, sh, b, t, tid & 7, &sh.tile[slot]);
             }
-            if (MULTI && m0 == 0) {
-                // (k > 1 shares a bound through the scratch while it works on the items)
-                if (!late) wait_previous_kernel();
-                if (tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
-            }
+            if (MULTI && m0 == 0 && tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
             __syncthreads();
             if (ARRAYS) {
                 const uint32_t n_live = sh.n_live;
