@@ -4,9 +4,11 @@ import multiprocessing
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 import mmee_inputs as mi
+import oracle
 import paper_2604_03446_b200.binding as mm
 from paper_2604_03446_b200 import build as lib_build
 
@@ -18,8 +20,8 @@ def host(tmp_path_factory):
     """host_math.cu and the planner as a shared object."""
     out = str(tmp_path_factory.mktemp("host_math") / "host_math.so")
     flags = [f for f in lib_build.NVCC_FLAGS if f not in ("-lineinfo", "-O3")]
-    subprocess.check_call([lib_build._nvcc()] + flags + ["-O1", "-o", out, os.path.join(HERE, "host_math.cu"),
-                                                         os.path.join(lib_build.CSRC, "mmee_plan.cu")])
+    subprocess.check_call([lib_build._nvcc()] + flags + ["-O1", "-o", out, os.path.join(HERE, "host_math.cu")] +
+                          [os.path.join(lib_build.CSRC, f) for f in ("mmee_plan.cu", "mmee_prune.cu")])
     lib = C.CDLL(out)
     lib.path = out
     return lib
@@ -113,3 +115,53 @@ def test_register_file_walk_ends_at_an_extent_of_all_ones(host, dims, pe, rf_wor
                     assert got == expected_terms(pe, dims, op, sm, objective, rf_words), args
     finally:
         pool.terminate()
+
+
+NO_ROW = 2 ** 62
+
+
+@pytest.mark.parametrize("dims", [(12, 4, 20, 6), (30, 12, 8, 18), (7, 5, 1, 3), (16, 16, 16, 16)])
+@pytest.mark.parametrize("order_set", [mi.ORD_ALL6, mi.ORD_NORECOMP2])
+def test_classes_of_levels_against_the_rows_of_the_oracle(host, dims, order_set):
+    """The search's closed forms -- how many rows of a block fit, the least DRAM words of one that does, the least buffer
+    need at those words, with and without row pruning -- against every row of the block as the oracle evaluates it, for
+    tilings all over the space and capacities from one at which nothing fits to one at which everything does."""
+    w = mi.workload(1, 1, 1, dims[0], dims[2], dims[1], dims[3], 1)
+    base = mi.objective(mi.OBJ_ENERGY, 1, order_set=order_set, fuse_mask=mi.FUSE_FUSED | mi.FUSE_SOFTMAX_IN_OP1, row_pruning=1)
+    arch = mi.arch(2, 3, 1, 1 << 20, 0, 1, 1.0, 0.0, 0.0, 0.0)
+    p = oracle.make_problem(w, arch, base)
+    keep = np.array(mm.mmee_row_pruning_keep(base), dtype=bool)
+    rng = np.random.default_rng(sum(dims))
+    n_orders = p.n_orders
+    for t in sorted({0, p.T - 1} | set(int(v) for v in rng.integers(0, p.T, size=6))):
+        raw = np.frombuffer(oracle.evaluate_range(p, t * p.R * 9, p.R * 9), dtype=np.dtype(oracle.Record))[::9]
+        words, need, lc, da1, da2 = (np.ascontiguousarray(v, dtype=np.int64) for v in
+                                     (raw["n"][:, 0], raw["bs"], raw["beta"][:, 2] - 3, raw["da1"], raw["da2"]))
+        split = n_orders * 3125
+        caps = np.unique(np.concatenate([[need.min() - 1, need.max()], rng.choice(need, size=4)]))
+        for cap in (int(v) for v in caps if v > 0):
+            fits = need <= cap
+            for slot in range(n_orders):
+                out = ((C.c_int64 * 8) * 4)()
+                args = [C.byref(mm._fill(s(), d)) for s, d in ((mm.Workload, w), (mm.Arch, dict(arch, gb_bytes=cap)), (mm.Objective, base))]
+                assert host.host_classes(*args, C.c_uint32(t), slot, out) == mm.OK
+                for c in range(3):
+                    first, width, rows, x, least_need, rows2, x2, kept = out[c]
+                    here = np.zeros(p.R, dtype=bool)
+                    here[slot * 3125:(slot + 1) * 3125] = True
+                    here &= fits & (lc >= first) & (lc < first + width)
+                    assert rows == rows2 == here.sum() and kept == (here & keep).sum()
+                    want = words[here].min() if here.any() else NO_ROW
+                    assert x == x2 == want
+                    if here.any():
+                        assert least_need == need[here & (words == want)].min()
+                _, _, rows, x1, least_need, rows2, x2, kept = out[3]
+                here = np.zeros(p.R, dtype=bool)
+                here[split + slot * 625:split + (slot + 1) * 625] = True
+                here &= fits
+                assert rows == rows2 == here.sum() and kept == (here & keep).sum()
+                if here.any():
+                    assert (x1, x2) == (da1[here].min(), da2[here].min())
+                    assert least_need == need[here & (da1 == x1) & (da2 == x2)].min()
+                else:
+                    assert x1 == NO_ROW
