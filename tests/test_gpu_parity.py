@@ -672,3 +672,30 @@ def test_lists_of_mappings_that_all_tie(fuse_mask, topk):
         want = [r.idx for r in gpu_search(cfg, obj)[1]]
         for _ in range(30):
             assert [r.idx for r in gpu_search(cfg, obj)[1]] == want
+
+
+@pytest.mark.parametrize("dims,pe,gb_bytes,bw,energies,obj,points", [
+    ((360, 240, 2520, 5040), (3, 38), 1600, 64, (1.0, 0.0), dict(fuse_mask=1, stationary_mask=0x100), 34),
+    ((720, 240, 2520, 360), (2, 41), 1600, 16, (200.0, 1.0), dict(fuse_mask=1, stationary_mask=0x1), 32),
+    ((1680, 840, 5040, 60), (22, 16), 40000, 2, (0.0, 7.0), dict(fuse_mask=4, order_set=0), 21),
+    ((360, 720, 5040, 840), (11, 32), 1600, 64, (200.0, 1.0), dict(order_set=0, stationary_mask=0x11), 21),
+    ((240, 120, 240, 60), (5, 9), 6000, 16, (20.0, 7.0), dict(stationary_mask=0x54), 5),
+    ((64, 64, 64, 64), (16, 16), 4096, 4, (20.0, 7.0), dict(t_begin=60, t_end=63), 1),
+], ids=["two_chains", "one_full_chain", "unfused_passes", "mask_passes", "mask", "few"])
+def test_energy_latency_front_equals_alternating_capped_searches(dims, pe, gb_bytes, bw, energies, obj, points):
+    """The front's searches as steps of one kernel, at the edges of its shapes: more points than one launch has steps, just
+    as many, tables that do not stay between steps, a few tilings only, restricted stationary pairs.  Byte for byte the
+    records of one-shot searches: least energy under a bound on the latency, then least latency at that energy."""
+    w = mi.workload(1, 1, 1, dims[0], dims[2], dims[1], dims[3], 2)
+    arch = mi.arch(pe[0], pe[1], 1, gb_bytes, 0, bw, energies[0], energies[1], 0.0, 0.0, c_softmax=1.0)
+    base = mi.objective(mi.OBJ_ENERGY, 1, **obj)
+    want, cap = [], 2 ** 63 - 2
+    while True:
+        e = mm.mmee_solve_host(w, arch, dict(base, objective=mi.OBJ_ENERGY_LCAP, key_cap=cap))[0]
+        if e.idx == mm.NO_INDEX:
+            break
+        r = mm.mmee_solve_host(w, arch, dict(base, objective=mi.OBJ_LATENCY_ECAP, key_cap=e.e_key))[0]
+        want.append(bytes(r))
+        cap = r.l_key - 1
+    got = [bytes(r) for r in mm.mmee_pareto_front(w, arch, base, 4096)]
+    assert got == want and len(want) == points
