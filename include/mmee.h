@@ -196,7 +196,7 @@ int mmee_search_host(mmee_handle_t* handle, mmee_result_t* out_best, mmee_result
 
 /*
  * mmee_destroy -- release the handle; its workspace goes to the idle ones.  Waits for the handle's device when
- * mmee_search was called on the handle.
+ * mmee_search was called on the handle.  A CUDA graph that holds a search of the handle must not be launched afterwards.
  */
 int mmee_destroy(mmee_handle_t* handle);
 
@@ -293,7 +293,8 @@ int mmee_filter_flags(mmee_handle_t* handle, void* cuda_stream, int64_t threshol
 /*
  * mmee_solve_host -- whole path with HOST buffers: plan, upload, search, copy the results back,
  * release.  Synchronous.  out_best: HOST, one record; out_topk: HOST, objective.topk records or
- * NULL.  h2d_bytes / d2h_bytes (HOST, may be NULL) receive the bytes copied in each direction.
+ * NULL.  h2d_bytes / d2h_bytes (HOST, may be NULL) receive the bytes that travel in each direction: the parameters of the
+ * one search launch, the records.
  */
 int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch,
                     const mmee_objective_t* objective, mmee_result_t* out_best,
@@ -310,6 +311,8 @@ int mmee_solve_host(const mmee_workload_t* workload, const mmee_arch_t* arch,
  *   out_points : HOST, `capacity` records; *n_points receives the number of points of the front, also
  *                when it exceeds capacity (then MMEE_ERR_RANGE is returned and the first `capacity`
  *                points are valid).
+ * The searches are steps of one kernel, whose CTAs wait for one another: MMEE_ERR_TIMEOUT if that takes longer than a few
+ * seconds, for instance because other work keeps some of them off the device for that long.
  */
 int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch,
                       const mmee_objective_t* objective, mmee_result_t* out_points, uint32_t capacity,
@@ -325,6 +328,7 @@ int mmee_pareto_front(const mmee_workload_t* workload, const mmee_arch_t* arch,
  * of the returned records (e_key) is the DRAM word count n[0].  Synchronous.
  *   out_points : HOST, `capacity` records; *n_points receives the number of points of the front, also when it
  *                exceeds capacity (then MMEE_ERR_RANGE is returned and the first `capacity` points are valid).
+ * MMEE_ERR_TIMEOUT as mmee_pareto_front.
  */
 int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* arch,
                             const mmee_objective_t* objective, mmee_result_t* out_points, uint32_t capacity,
@@ -332,9 +336,9 @@ int mmee_pareto_front_bs_da(const mmee_workload_t* workload, const mmee_arch_t* 
 
 /*
  * mmee_search_shapes -- reconfigurable PE arrays (Section VII-K): the same search on each of several logical
- * array shapes (the stationary modes the array can switch between are objective.stationary_mask), one device
- * search per shape, and the shape whose optimum has the least key.  arch.pe_rows / pe_cols are replaced by each
- * shape in turn; everything else is as given.  Synchronous.
+ * array shapes (the stationary modes the array can switch between are objective.stationary_mask), and the shape whose
+ * optimum has the least key.  arch.pe_rows / pe_cols are replaced by each shape's; everything else is as given.  Which
+ * rows fit and what they fetch is found once for up to sixteen shapes, the keys for each shape.  Synchronous.
  *   shapes      : HOST, n_shapes pairs (rows, cols), each >= 1.
  *   out_per_shape : HOST, n_shapes records: the optimum on that shape (idx = MMEE_NO_INDEX, status
  *                   MMEE_ERR_NO_FEASIBLE when nothing fits; n_total / n_feasible of that search).

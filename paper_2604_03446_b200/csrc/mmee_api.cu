@@ -50,7 +50,9 @@ int cuda_status(cudaError_t e) {
 // finalizes, not earlier: better while the finalize step is the longer part, worse once the items are.  One energy search
 // after the other, early / late start (us): 4 900 tilings 9.7 / 8.8, 5 929 9.6 / 8.9, 7 056 9.3 / 8.5 (edge accelerator,
 // S = 2048) and 10.6 / 11.4 (ragged S = 96), 8 064 10.4 / 10.9, 10 816 12.0 / 13.4, 18 496 9.9 / 10.5.  With register-file
-// tiling the tables take longest: 23.5 / 26.5 at 4 900.
+// tiling the tables take longest: 23.5 / 26.5 at 4 900.  What decides is the number of tilings that can fit, which the host
+// does not know (the two searches of 7 056 differ in it); the line lies below the first size at which a late start lost, and
+// costs a search above it in which few tilings fit up to 0.8 us.
 constexpr uint64_t kLateTilings = 6000;
 
 // Two CTAs per SM (118 registers a thread, no spills) beat three (80, spilled) and four (64): GQA latency 13.0, 13.7 and
