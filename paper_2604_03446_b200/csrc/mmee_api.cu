@@ -22,7 +22,7 @@ struct mmee_handle {
     bool dirty;                  // a launch failed half-way: the scratch header is reset before the next search
     bool in_flight;              // a search was launched whose end this handle has not waited for
     bool timing;
-    int flip;                    // the scratch of the last search
+    uint32_t turn;               // searches so far: the last one's scratch is number turn % kScratches
     cudaEvent_t ev[2];           // before and after the search kernel
 };
 
@@ -44,16 +44,6 @@ int cuda_status(cudaError_t e) {
     cudaGetLastError();
     return MMEE_ERR_CUDA;
 }
-
-// Searches of at most this many tilings (and those for the k best, which would otherwise wait before their items) wait for
-// the kernel before them in their finalize step only (see mmee_search.cu).  The next search then starts while this one
-// finalizes, not earlier: better while the finalize step is the longer part, worse once the items are.  One energy search
-// after the other, early / late start (us): 4 900 tilings 9.7 / 8.8, 5 929 9.6 / 8.9, 7 056 9.3 / 8.5 (edge accelerator,
-// S = 2048) and 10.6 / 11.4 (ragged S = 96), 8 064 10.4 / 10.9, 10 816 12.0 / 13.4, 18 496 9.9 / 10.5.  With register-file
-// tiling the tables take longest: 23.5 / 26.5 at 4 900.  What decides is the number of tilings that can fit, which the host
-// does not know (the two searches of 7 056 differ in it); the line lies below the first size at which a late start lost, and
-// costs a search above it in which few tilings fit up to 0.8 us.
-constexpr uint64_t kLateTilings = 6000;
 
 // Two CTAs per SM (118 registers a thread, no spills) beat three (80, spilled) and four (64): GQA latency 13.0, 13.7 and
 // 15.1 us, BERT energy 9.4, 10.4 and 12.6, convolution chain top-16 52, 58 and 65.  One slot is left free: a search that follows another starts while that one's
@@ -87,7 +77,7 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
     shape->grid = (uint32_t)grid;
     shape->n_arrays = n_arrays;
     shape->overlap = true;
-    shape->late = n_arrays == 0 && (p.topk > 1 || (tilings <= kLateTilings && !p.rf_tiling));
+    shape->hold = false;
     shape->chain_steps = shape->chain_epoch = 0;
     shape->chain_read = false;
     shape->chain_polls = 0;
@@ -110,14 +100,13 @@ int run_chain(const Plan& plan, uint32_t polls, Take take) {
     if (rc) return rc;
     uint32_t most = 0;
     if ((rc = max_search_ctas(device, &most))) return rc;
-    most -= kRecordCtas - 1;
+    most -= kRecordCtas;        // (and one that merges, in the slot that a single search leaves free)
     LaunchShape shape;
     if ((rc = choose_launch_shape(plan, device, 0, 0, &shape, most))) return rc;
     Workspace* ws = nullptr;
     if ((rc = workspace_acquire(device, &ws))) return rc;
     bool more = true, read = false;
     while (more && rc == MMEE_OK) {
-        shape.late = false;
         shape.chain_steps = kHostRecords;
         shape.chain_to = ws->chain;
         shape.chain_polls = polls;
@@ -256,13 +245,14 @@ static int search_on(mmee_handle* h, cudaStream_t st, mmee_result_t* out_best, m
     if (rc) return rc;
     LaunchShape shape = h->shape;
     if (h->dirty) {        // an earlier launch on this handle failed: a header may hold a used ticket counter
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < kScratches; ++i)
             if ((rc = cuda_status(launch_reset(&h->ws->scratch[i]->head, st)))) return rc;
         h->dirty = false;
         shape.overlap = false;          // (its CTAs touch the headers: not before the resets have ended)
     }
-    h->flip ^= 1;
-    Scratch* scratch = h->ws->scratch[h->flip];
+    ++h->turn;
+    shape.hold = h->turn % (kScratches - 1) == 0;
+    Scratch* scratch = h->ws->scratch[h->turn % kScratches];
     if (h->timing) cudaEventRecord(h->ev[0], st);
     const cudaError_t e = launch_search(h->plan, shape, &scratch->head, scratch->partial, out_best, out_topk, st);
     if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
@@ -519,7 +509,7 @@ int mmee_last_search_stats(const mmee_handle_t* h, mmee_launch_stats_t* out) {
     out->rows_tested = 0;
     if (h->last.kernels_launched) {
         unsigned long long counters[2] = {0, 0};      // last_exact_groups, last_tested_rows
-        const int rc = cuda_status(cudaMemcpy(counters, &h->ws->scratch[h->flip]->head.last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
+        const int rc = cuda_status(cudaMemcpy(counters, &h->ws->scratch[h->turn % kScratches]->head.last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
         if (rc) return rc;
         out->exact_path_visits = counters[0];
         out->rows_tested = counters[1];

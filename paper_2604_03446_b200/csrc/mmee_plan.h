@@ -13,7 +13,11 @@ constexpr int kCandPerTask = 1125;  // rows x 9 stationary pairs
 constexpr int64_t kInfKey = INT64_MAX;
 
 // Model arithmetic that the host can run as well as the kernels.
+#ifdef __CUDACC__
 #define MMEE_HD __host__ __device__ __forceinline__
+#else
+#define MMEE_HD inline
+#endif
 
 // Operand / loop numbering shared by host planner and kernels.
 enum { OP_A = 0, OP_B = 1, OP_C = 2, OP_D = 3, OP_E = 4 };
@@ -56,7 +60,17 @@ enum OrderFlag {
 struct alignas(4) KeptMasks {
     uint16_t fused[kMaxOrders][3][9];         // [order slot][class of C][3 * class of A + class of B]: bit 4 * d + e
     uint16_t unfused[2][kMaxOrders][9];       // [unfused mode][order slot][3 * a + b]: bit 3 * d + e (L3, L4 merged)
+    uint32_t weights[158];                    // the same as CountWeights, four bits each (at most two modes of six orders)
 };
+
+// Where a tiling's count keeps rows with D and E of classes d, e (0: L3, 1..3), by their size slots (CountWeights): 4 * x + y both
+// retained, 16 + x D retained and E at L3, 20 + y the other way round, 24 both at L3.  `lo`: the size slot of class 2 behind that
+// of class 1, 1 or 2.
+MMEE_HD constexpr int de_choice(int d, int e, int d_lo, int e_lo) {
+    return d && e ? 4 * (d == 3 ? 3 : (d == 2 ? d_lo : 0)) + (e == 3 ? 3 : (e == 2 ? e_lo : 0))
+                  : (d ? 16 + (d == 3 ? 3 : (d == 2 ? d_lo : 0)) : (e ? 20 + (e == 3 ? 3 : (e == 2 ? e_lo : 0)) : 24));
+}
+constexpr int kCountChoices = 28;           // with padding
 
 struct Plan {
     uint32_t dim[4];              // I, K, L, J of one instance

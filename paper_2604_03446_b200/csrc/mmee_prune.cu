@@ -184,6 +184,24 @@ static int find_kept_masks(Plan* p, uint32_t* kept_rows) {
             p->kept.unfused[p->block_phi[block] - 1][slot][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (3 * d + e));
         }
     }
+    // the kept rows as weights of a tiling's count: [3 * a + b][size slot of C, or 4 for an unfused mode][choice of D and E]
+    static_assert(9 * 5 * kCountChoices <= 8 * sizeof(p->kept.weights) / 4, "four bits each");
+    for (uint32_t slot = 0; slot < p->n_orders; ++slot) {
+        const OrderInfo& o = p->order[slot];
+        const int d_lo = o.size_d_lo - S_lj, e_lo = o.size_e_lo - S_ij;
+        auto add = [&](int ab, int c, int de) {
+            const int at = (ab * 5 + c) * kCountChoices + de;
+            p->kept.weights[at / 8] += 1u << (4 * (at % 8));
+        };
+        for (int ab = 0; ab < 9; ++ab) {
+            for (int c = 0; c < 3; ++c)
+                for (int de = 0; de < 16; ++de)
+                    if (p->kept.fused[slot][c][ab] >> de & 1) add(ab, o.size_c[c] - S_il, de_choice(de / 4, de % 4, d_lo, e_lo));
+            for (int mode = 0; mode < 2; ++mode)
+                for (int de = 0; de < 9; ++de)
+                    if (p->kept.unfused[mode][slot][ab] >> de & 1) add(ab, 4, de_choice(de / 3 + 1, de % 3 + 1, d_lo, e_lo));
+        }
+    }
     return MMEE_OK;
 }
 

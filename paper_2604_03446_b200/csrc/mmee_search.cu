@@ -28,9 +28,11 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = kSearchThreads / 32;
 constexpr int kTopK = (int)MMEE_MAX_TOPK;
-// One optimum; one optimum over the rows kept by symbolic pruning; the k best; one optimum of a chain of searches;
-// one optimum for each of several array shapes.
-constexpr int kModeSingle = 0, kModePrune = 1, kModeMulti = 2, kModeChain = 3, kModeArrays = 4;
+// One optimum; the k best; one optimum of a chain of searches; one optimum for each of several array shapes.
+constexpr int kModeSingle = 0, kModeMulti = 1, kModeChain = 2, kModeArrays = 3;
+
+// Weights of the rows of two and of six orders (see count_rows).
+__device__ const CountWeights kCountWeights[2] = {count_weights(2), count_weights(6)};
 
 // ------------------------------------------------------------------------------------------------
 // (key, number) pairs
@@ -131,6 +133,9 @@ __device__ __forceinline__ bool triple_less(int64_t ka, int64_t la, uint64_t ia,
     return ka < kb || (ka == kb && (la < lb || (la == lb && ia < ib)));
 }
 
+__device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------------------------
 // shared memory
 // ------------------------------------------------------------------------------------------------
@@ -138,20 +143,23 @@ __device__ __forceinline__ bool triple_less(int64_t ka, int64_t la, uint64_t ia,
 struct Shared {
     // What lanes index with different indices (the constant bank would serialise them), copied from the plan.
     OrderInfo order[kMaxOrders];
-    KeptMasks kept;
+    CountWeights weights;
+    uint8_t done[kMaxChunk];        // tilings of the current pass that were evaluated first
+    uint8_t list[kMaxChunk];        // ... that are evaluated after them
     uint32_t divs[4][MMEE_MAX_DIVISORS];
     uint32_t cofactors[4][MMEE_MAX_DIVISORS];       // dimension / divisor
     uint32_t pe_rows, pe_cols;      // the array's logical shape
     uint32_t row_folds[4][MMEE_MAX_DIVISORS], col_folds[4][MMEE_MAX_DIVISORS];      // register-file tiling only
     alignas(16) longlong2 tops[kWarps][MMEE_MAX_TOPK];
+    longlong2 up;                   // k > 1: nothing that follows this pair is among the k best
     long long kth[kWarps];          // finalize, k > 1: the k-th key of each warp's list (kInfKey: not full)
-    long long G;                    // k > 1: upper bound on the k-th smallest key
     unsigned long long feasible_rows[kWarps];
     uint32_t live_tilings[kWarps];
     uint32_t n_live;                // tilings of the current pass that can fit
-    uint32_t n_fit;                 // STAIRS: those of them that fit under the bound of the search before
-    long long bound;                // chained searches: that bound
-    uint32_t cursor;                // next group of 32 items
+    long long bound;                // chained searches: the bound that the search before left
+    long long best;                 // ... the least key of a warp so far
+    uint32_t n_list, cursor;        // entries of `list`, next one to be taken
+    uint32_t count_cursor;          // next 32 units of the count
     uint32_t last_cta, check_failed;
     uint32_t waited;                // chained searches: the one waited for is over
     union {
@@ -358,6 +366,25 @@ __device__ __forceinline__ void merge_warps(Shared& sh, int k, int lane, int war
     __syncthreads();
 }
 
+// k > 1: a pair that at least k of the entries of the warps' lists (sh.tops) do not follow; in all lanes.  If q warps hold r
+// entries up to a pair each and q * r >= k, that is one: the least over four ways to cut k.
+__device__ __forceinline__ void bound_of_lists(const Shared& sh, int k, int lane, int64_t& uk, uint64_t& ui) {
+    static_assert(kWarps == 8, "eight lists, four cuts");
+    const int most = kWarps >> (lane >> 3);                 // warps: 8, 4, 2, 1
+    const int r = (k + most - 1) / most, q = (k + r - 1) / r;
+    const longlong2 v = sh.tops[lane & 7][r - 1];
+    int rank = 0;                                           // of this warp's r-th entry among those
+#pragma unroll
+    for (int j = 0; j < kWarps; ++j) {
+        const int64_t ok = __shfl_sync(kFull, (int64_t)v.x, (lane & 24) + j);
+        const uint64_t oi = __shfl_sync(kFull, (uint64_t)v.y, (lane & 24) + j);
+        rank += pair_less(ok, oi, v.x, (uint64_t)v.y) || (ok == v.x && oi == (uint64_t)v.y && j < (lane & 7)) ? 1 : 0;
+    }
+    uk = rank == q - 1 ? v.x : kInfKey;
+    ui = rank == q - 1 ? (uint64_t)v.y : UINT64_MAX;
+    warp_min_pair(uk, ui);
+}
+
 // The smallest of the warps' pairs (k = 1; each warp's in all its lanes), in every thread of the CTA.
 __device__ __forceinline__ void min_over_warps(Shared& sh, int lane, int warp, int64_t& ek, uint64_t& ei) {
     __syncthreads();
@@ -380,14 +407,10 @@ struct ArrayDivisors {        // the same with another array's rows and columns
 };
 
 // What the kernels look up in shared memory, by all threads of a CTA (the caller synchronises).
-template <bool PRUNE>
 __device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uint32_t pe_cols, Shared& sh) {
     const int tid = threadIdx.x;
     for (int i = tid; i < (int)(sizeof(sh.order) / 4); i += kSearchThreads)
         reinterpret_cast<uint32_t*>(sh.order)[i] = reinterpret_cast<const uint32_t*>(p.order)[i];
-    if (PRUNE)
-        for (int i = tid; i < (int)(sizeof(KeptMasks) / 4); i += kSearchThreads)
-            reinterpret_cast<uint32_t*>(&sh.kept)[i] = reinterpret_cast<const uint32_t*>(&p.kept)[i];
     static_assert(kSearchThreads == 4 * MMEE_MAX_DIVISORS, "one thread per divisor");
     if ((uint32_t)(tid & 63) < p.ndiv[tid >> 6]) {
         const int d = tid >> 6, i = tid & 63;
@@ -403,6 +426,21 @@ __device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uin
         sh.pe_cols = pe_cols;
     }
 }
+
+// The weights of the rows, by all threads of a CTA: those of the orders, on their way when this returns (await_weights), or one for
+// every row that pruning keeps.
+__device__ __forceinline__ void start_weights(const Plan& p, Shared& sh) {
+    constexpr int kWords = sizeof(CountWeights) / 4;
+    if (p.row_pruning) {
+        for (int i = threadIdx.x; i < kWords; i += kSearchThreads) (&sh.weights.w[0][0][0])[i] = p.kept.weights[i / 8] >> (4 * (i % 8)) & 15u;
+        return;
+    }
+    const int4* from = reinterpret_cast<const int4*>(&kCountWeights[p.n_orders == kMaxOrders ? 1 : 0]);
+    int4* to = reinterpret_cast<int4*>(&sh.weights);
+    for (int i = threadIdx.x; i < kWords / 4; i += kSearchThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(to + i)), "l"(from + i) : "memory");
+}
+__device__ __forceinline__ void await_weights() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // The items of a block's tables (block_item), their three kinds on three warps.
 __device__ __forceinline__ int split_item(int warp, int lane) {
@@ -431,13 +469,34 @@ __device__ __forceinline__ bool await_epoch(const SearchHeader* head, uint32_t e
     return false;
 }
 
-// The end of a chained search, by all threads of the last CTA; its record is made by another (resolve_chain).
+// Waits for `n` CTAs to have published their parts, limited as above.
+__device__ __forceinline__ bool await_parts(const SearchHeader* head, uint32_t n, uint32_t polls) {
+#pragma unroll 4
+    for (uint32_t i = 0; i < polls; ++i) {
+        uint32_t now;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&head->done_ctas) : "memory");
+        if (now >= n) return true;
+    }
+    return false;
+}
+__device__ __forceinline__ void add_part(SearchHeader* head) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&head->done_ctas) : "memory");
+}
+
+// Whether a chain's CTAs keep their tables from search to search.  They then count the rows that fit under a search's bound while
+// they wait for its end, and add the count to its record before they publish their part of the next one.  Else, and in the
+// launch's last search, the count is a part of what they publish.
+__device__ __forceinline__ bool tables_stay(const Plan& p, const LaunchShape& shape) {
+    return (uint64_t)shape.chunk * shape.grid >= p.t_end - p.t_begin;
+}
+
+// The end of a chained search, by all threads of one CTA; its record is made by another (resolve_chain).  True in warp 0: found.
 // FRONT: the least (energy, latency, block) of all CTAs is the next point of the energy-latency front.  It is left as a
 // latency optimum under that energy; the next search allows one word less of latency.
 // Else: the least (energy, block, buffer need); the next search allows one word of buffer less than that need.
 template <bool FRONT>
-__device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Shared& sh, ChainRecord* chain_to, uint32_t epoch,
-                                            SearchHeader* __restrict__ head, const Partial* __restrict__ partials, int n_partials) {
+__device__ __forceinline__ bool finalize_chain(const Plan& p, int64_t cap_words, Shared& sh, ChainRecord* chain_to, uint32_t epoch, bool last,
+                                               bool own_counts, SearchHeader* __restrict__ head, const Partial* __restrict__ partials, int n_partials) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int64_t ek = kInfKey, el = kInfKey;
     uint64_t ei = UINT64_MAX;
@@ -447,42 +506,65 @@ __device__ __noinline__ void finalize_chain(const Plan& p, const Limits& lim, Sh
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int c = c0 + u * kSearchThreads;
-            v[u] = w[u] = make_longlong2(kInfKey, -1ll);
+            v[u] = make_longlong2(kInfKey, -1ll);
+            w[u] = make_longlong2(-1ll, 0);
             if (c < n_partials) {
                 v[u] = __ldcg(&partials[c].e[0]);
                 w[u] = __ldcg(&partials[c].e[1]);
-                rows += __ldcg(&partials[c].feasible_rows);
             }
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+        for (int u = 0; u < 2; ++u) {
+            rows += (unsigned long long)w[u].y;
             if (triple_less(v[u].x, v[u].y, (uint64_t)w[u].x, ek, el, ei)) { ek = v[u].x; el = v[u].y; ei = (uint64_t)w[u].x; }
+        }
     }
-    for (int off = 16; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+    if (own_counts) {
+        for (int off = 16; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+        if (lane == 0) sh.feasible_rows[warp] = rows;
+    }
     warp_min_triple(ek, el, ei);
     if (lane == 0) {
-        sh.feasible_rows[warp] = rows;
         sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
         sh.tops[warp][1] = make_longlong2((long long)ei, 0);
     }
     __syncthreads();
-    if (warp) return;
-    rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
-    for (int off = kWarps / 2; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+    if (warp) return false;
     ek = sh.tops[lane & (kWarps - 1)][0].x;
     el = sh.tops[lane & (kWarps - 1)][0].y;
     ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
     warp_min_triple(ek, el, ei);
     const bool found = ek != kInfKey;
     if (lane == 0) {
-        const unsigned long long fit = rows * p.n_sm;
+        unsigned long long fit = 0;         // (the CTAs add theirs, else)
+        if (own_counts)
+            for (int w = 0; w < kWarps; ++w) fit += sh.feasible_rows[w];
         if (FRONT) *chain_to = {(long long)(found ? el : kInfKey), (unsigned long long)ei, fit, (long long)ek, 0, 0};
-        else *chain_to = {(long long)ek, (unsigned long long)el, fit, (long long)lim.cap_words, (long long)ei, 0};
+        else *chain_to = {(long long)ek, (unsigned long long)el, fit, (long long)cap_words, (long long)ei, 0};
         const int64_t bound = !found ? kNoBound : (FRONT ? el : (int64_t)ei) - 1;
         const unsigned long long word = (unsigned long long)epoch << 32 | (found ? (uint32_t)bound : 0xffffffffu);
         head->chain_bound = bound;
-        head->done_ctas = 0;
+        if (!found || last) head->done_ctas = 0;
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&head->chain_epoch), "l"(word) : "memory");
+    }
+    return found;
+}
+
+// A CTA of its own merges the parts of a chain's searches: it does not have to count rows before it takes up the next one.
+template <bool FRONT>
+__device__ __noinline__ void merge_chain(const Plan& p, const LaunchShape& shape, Shared& sh, SearchHeader* head, const Partial* partials) {
+    int64_t cap = shape.chain_read && !FRONT ? *reinterpret_cast<volatile long long*>(&head->chain_bound) : p.cap_words;
+    const bool stay = tables_stay(p, shape);
+    for (uint32_t step = 0; step < shape.chain_steps; ++step) {
+        if (threadIdx.x == 0) sh.waited = await_parts(head, (step + 1) * shape.grid, shape.chain_polls) ? 1u : 0u;
+        __syncthreads();
+        if (!sh.waited) return;
+        const bool found = finalize_chain<FRONT>(p, cap, sh, shape.chain_to + step, shape.chain_epoch + step, step + 1 == shape.chain_steps,
+                                                 !stay || step + 1 == shape.chain_steps, head, partials, (int)shape.grid);
+        if (threadIdx.x == 0) sh.n_list = found ? 1u : 0u;
+        __syncthreads();
+        if (!sh.n_list) return;
+        if (!FRONT) cap = *reinterpret_cast<volatile long long*>(&head->chain_bound);
     }
 }
 
@@ -658,6 +740,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
             }
         }
         __syncwarp();
+        wait_previous_kernel();                     // from here on the result records are touched
         if (out_topk && rec < k) {
             const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
             unsigned long long* to = reinterpret_cast<unsigned long long*>(&out_topk[rec]);
@@ -676,6 +759,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
             if (sh.check_failed) best.status = MMEE_ERR_CHECK;
         }
         __syncwarp();
+        wait_previous_kernel();
         const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&best);
         unsigned long long* to = reinterpret_cast<unsigned long long*>(out_best);
         for (int i = lane; i < kWords; i += 32) to[i] = from[i];
@@ -683,7 +767,7 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         // ready for the next search on this scratch
         unsigned long long all_live = 0;
         for (int w = 0; w < kWarps; ++w) all_live += sh.live_tilings[w];
-        head->G = kInfKey - 1;
+        head->bound = kInfKey;
         head->last_exact_groups = n_groups;
         const uint32_t unfused_modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
         head->last_tested_rows = all_live * p.n_orders * ((p.fuse_mask & 1u ? kFusedReps : 0u) + (unfused_modes ? 18u : 0u));
@@ -698,10 +782,10 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
 // before it: the record's n_feasible is the number of mappings that fit under the last bound of such a sequence.  Where
 // that is not the bound this one was found under, reserved2[0] says what it is, plus one (a rare case: index order
 // raises needs), and the caller searches there.
-template <int OBJ, bool STAIRS>
+// fitting(n): sets n to the number of mappings that fit (one thread); false: it did not come, and no record is written.
+template <int OBJ, bool STAIRS, class Fitting>
 __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim, Shared& sh,
-                                               int64_t key, uint64_t where, unsigned long long n_feasible, int64_t need,
-                                               mmee_result_t* out) {
+                                               int64_t key, uint64_t where, Fitting fitting, int64_t need, mmee_result_t* out) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     mmee_result_t& r = sh.record[0];
     uint32_t before_need = 0;
@@ -741,11 +825,15 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
         }
     }
     if (warp == 0) {
+        bool came = true;
         if (lane == 0) {
             r.n_total = (p.t_end - p.t_begin) * (uint64_t)p.rows_per_tiling * 9u;
-            r.n_feasible = n_feasible;
+            unsigned long long n = 0;
+            came = fitting(n);
+            r.n_feasible = n;
             if (STAIRS) r.reserved2[0] = before_need;
         }
+        if (!__shfl_sync(kFull, came ? 1 : 0, 0)) return;
         __syncwarp();
         const unsigned long long* from = reinterpret_cast<const unsigned long long*>(&r);
         unsigned long long* to = reinterpret_cast<unsigned long long*>(out);
@@ -758,6 +846,7 @@ __device__ __forceinline__ void resolve_record(const Plan& p, const Limits& lim,
 template <bool FRONT>
 __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& shape, Shared& sh, const SearchHeader* head, uint32_t which,
                                            mmee_result_t* out) {
+    const bool stay = tables_stay(p, shape);
     for (uint32_t i = 0; i < shape.chain_steps; ++i) {
         __syncthreads();
         uint32_t low;
@@ -765,10 +854,17 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
         __syncthreads();
         if (!sh.waited) return;
         const volatile ChainRecord* from = shape.chain_to + i;
-        const ChainRecord c = {from->key, from->where, from->n_feasible, from->bound, from->need, 0};
+        const ChainRecord c = {from->key, from->where, 0, from->bound, from->need, 0};
+        const bool later = stay && c.key != kInfKey && i + 1 < shape.chain_steps;        // the count comes with the next search
+        auto fitting = [&](unsigned long long& n) {
+            uint32_t unused;
+            if (later && !await_epoch(head, shape.chain_epoch + i + 1, shape.chain_polls, unused)) return false;
+            n = from->n_feasible * p.n_sm;
+            return true;
+        };
         if (i % kRecordCtas == which) {
-            if (FRONT) resolve_record<MMEE_OBJ_LATENCY_ECAP, false>(p, Limits{p.cap_words, c.bound}, sh, c.key, c.where, c.n_feasible, 0, out + i);
-            else resolve_record<MMEE_OBJ_ENERGY, true>(p, Limits{c.bound, 0}, sh, c.key, c.where, c.n_feasible, c.need, out + i);
+            if (FRONT) resolve_record<MMEE_OBJ_LATENCY_ECAP, false>(p, Limits{p.cap_words, c.bound}, sh, c.key, c.where, fitting, 0, out + i);
+            else resolve_record<MMEE_OBJ_ENERGY, true>(p, Limits{c.bound, 0}, sh, c.key, c.where, fitting, c.need, out + i);
         }
         if (c.key == kInfKey) return;
     }
@@ -778,18 +874,13 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
 // the search kernel
 // ------------------------------------------------------------------------------------------------
 
-// Searches launched one after the other overlap (programmatic dependent launch), in one of two ways.
-//   early: a search lets the next one start at once; that one's CTAs move in as this one's leave, and wait for its end
-//          before they publish, since it may still use their scratch;
-//   late:  only the CTA that finalizes waits for the kernel before, and lets the next search start after that wait.  The
-//          CTAs then publish while the search before finalizes, into the other one of the handle's two scratches: the
-//          search that used theirs last had ended before the one before them let them start.  (Always for k > 1, whose CTAs
-//          share a bound through the scratch while they work on their items.)
-// A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  Searches one after
-// the other, without and with this (us each): smallest configuration 20.5 and 8.9, BERT energy 22.9 and 10.4, GQA latency
-// 28.7 and 13.7, convolution chain top-16 133 and 58 (other changes between them included).
-__device__ __forceinline__ void release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Searches launched one after the other overlap (programmatic dependent launch): the next one's CTAs move in as this one's
+// leave, publish into a scratch of their own and merge, and only the records wait for the end of the search before, right before
+// they are written, so that searches end in order.  A handle has kScratches scratches in turn.  Every (kScratches - 1)-th of its
+// searches (`hold`) lets the next kernel start only after the kernel before it has ended (CTA 0 waits for that; the others need
+// not): of two searches with the same scratch the second then starts after a search between them has seen the first one's end.
+// A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  The waits are the
+// hardware's grid dependency; a CTA waits for none that could start after it.
 
 // The number of CTAs that drew a ticket before; what they wrote before that is visible from here on, and what the calling
 // warp has written is to those that draw one later.
@@ -802,7 +893,10 @@ __device__ __forceinline__ uint32_t draw_ticket(unsigned int* count) {
 // The tables of one tiling, by eight threads (sub = 0..7) once tb->b is there: one stationary mode of one operator each,
 // and the sizes between them.
 template <bool TERMS>
-__device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, const uint32_t b[8], uint32_t t, int sub, TileTab* tb) {
+__device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, int sub, TileTab* tb) {
+    uint32_t b[8];
+#pragma unroll
+    for (int d = 0; d < 8; ++d) b[d] = tb->b[d];
     if (TERMS && sub < 6) {
         const int op = sub >= 3 ? 1 : 0, sm = sub - 3 * op;
         int64_t P, Q;
@@ -811,39 +905,38 @@ __device__ __forceinline__ void build_tile(const Plan& p, const Shared& sh, cons
         (op ? tb->st.Q2 : tb->st.Q1)[sm] = Q;
     }
     for (int i = sub; i < kSizeSlots; i += 8) tb->size[i] = sat_size(size_words(p.dim, tb->b + 4, i));
-    if (sub == 7) tb->t = t;
 }
 
 template <int OBJ, int MODE>
 __global__ void __launch_bounds__(kSearchThreads, 2)
 search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ head, Partial* __restrict__ partials,
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
-    constexpr bool PRUNE = MODE == kModePrune, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain;
-    constexpr bool ARRAYS = MODE == kModeArrays;
+    constexpr bool MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain, ARRAYS = MODE == kModeArrays;
     constexpr bool FRONT = CHAIN && OBJ == MMEE_OBJ_ENERGY_LCAP;      // least (energy, latency) under a bound on the latency
     constexpr bool STAIRS = CHAIN && OBJ == MMEE_OBJ_ENERGY;          // least (energy, block, buffer need) under a capacity
     static_assert(FRONT || STAIRS || !CHAIN, "only the searches of the Pareto fronts are chained");
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool late = MULTI || shape.late;
-    if (!late) release_next_kernel();
-    load_shared<PRUNE>(p, p.pe_rows, p.pe_cols, sh);
+    if (!shape.hold) release_next_kernel();
+    if (!CHAIN || blockIdx.x < shape.grid) start_weights(p, sh);
+    load_shared(p, p.pe_rows, p.pe_cols, sh);
     // Array shapes: the stationary-pair terms of shape y and tiling slot i at [y * chunk + i], behind the tilings' tables;
     // the warps' best items of shape y in sh.tops[.][y].
     StatTerms* terms = reinterpret_cast<StatTerms*>(&sh.tile[shape.chunk]);
     if (ARRAYS && tid < kWarps * (int)MMEE_MAX_TOPK) sh.tops[tid / (int)MMEE_MAX_TOPK][tid % (int)MMEE_MAX_TOPK] = make_longlong2(kInfKey, -1ll);
-    // STAIRS: the table slots of the tilings that fit under the bound, where the kept rows of the other modes lie.
-    uint8_t* fit_slots = reinterpret_cast<uint8_t*>(&sh.kept);
-    static_assert(kMaxChunk <= 256 && kMaxChunk <= sizeof(KeptMasks), "one byte per table");
+    static_assert(kMaxChunk <= 256 && kMaxChunk <= 32 * kWarps, "one byte per table, one lane per table");
+
+    if (tid < (int)kMaxChunk) sh.done[tid] = 0;
     if (tid == 0) {
-        sh.n_live = sh.n_fit = 0;
-        sh.cursor = 0;
+        sh.n_live = sh.n_list = sh.cursor = sh.count_cursor = 0;
         sh.check_failed = 0;
+        sh.best = kInfKey;
     }
     __syncthreads();
 
     if (CHAIN && blockIdx.x >= shape.grid) {
-        resolve_chain<FRONT>(p, shape, sh, head, blockIdx.x - shape.grid, out_topk);
+        if (blockIdx.x < shape.grid + kRecordCtas) resolve_chain<FRONT>(p, shape, sh, head, blockIdx.x - shape.grid, out_topk);
+        else merge_chain<FRONT>(p, shape, sh, head, partials);
         return;
     }
 
@@ -856,6 +949,17 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     const uint32_t n_orders = p.n_orders;
     auto any = [](bool v) { return __any_sync(kFull, v) != 0; };
 
+    // A warp evaluates `per` tilings at a time, `n_items` lanes each: this lane the tiling `sub`, its fused block of order `os` with
+    // C at class c, or its block of that order and unfused mode phi.
+    const uint32_t fused_items = (p.fuse_mask & 1u) ? 3u * n_orders : 0u, unfused_modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
+    const uint32_t n_items = fused_items + unfused_modes * n_orders;
+    const uint32_t per = 32u / n_items, sub = (uint32_t)lane / n_items, item = (uint32_t)lane - sub * n_items;
+    const bool fused = item < fused_items;
+    const uint32_t mode = (fused ? item : item - fused_items) / n_orders, os = item % n_orders;     // class of C, or how many modes before phi
+    const int c = fused ? (int)mode : 0, phi = fused ? 0 : (mode || !(p.fuse_mask & 2u) ? 2 : 1);
+    const uint32_t block = os + (fused ? 0u : p.n_fused_blocks + mode * n_orders);
+    const OrderInfo& oi = sh.order[os];
+
     // the best item so far: k = 1 of this thread, else the warp's list (lane j holds entry j)
     int64_t ek = kInfKey;
     uint64_t ei = UINT64_MAX;
@@ -863,6 +967,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     unsigned long long my_rows = 0;
     uint32_t my_live = 0;
 
+    int64_t uk = kInfKey;           // nothing that follows this pair is among the k best
+    uint64_t ui = UINT64_MAX;
     auto offer = [&](int64_t key, uint32_t id, bool valid) {
         if (!MULTI) {
             if (valid && pair_less(key, id, ek, ei)) { ek = key; ei = id; }
@@ -870,14 +976,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         }
         const int64_t lk = __shfl_sync(kFull, ek, k - 1);
         const uint64_t li = __shfl_sync(kFull, ei, k - 1);
-        const bool pend = valid && key != kInfKey && key <= *reinterpret_cast<volatile long long*>(&sh.G) && pair_less(key, id, lk, li);
-        if (!__any_sync(kFull, pend)) return;
-        warp_offer(ek, ei, k, key, id, pend, lane);
-        // a full list bounds the k-th smallest key for everybody
-        if (lane == k - 1 && ek < *reinterpret_cast<volatile long long*>(&sh.G)) {
-            atomicMin(&sh.G, (long long)ek);
-            atomicMin(&head->G, (long long)ek);
-        }
+        const bool pend = valid && key != kInfKey && pair_less(key, id, lk, li) && !pair_less(uk, ui, key, id);
+        if (__any_sync(kFull, pend)) warp_offer(ek, ei, k, key, id, pend, lane);
     };
 
     // FRONT: the item's least (energy, latency) over the stationary pairs; pair(s, e, l) forms those of pair s.
@@ -898,23 +998,84 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
         if (valid && triple_less(key, (int64_t)id, (uint64_t)need, ek, el, ei)) { ek = key; el = id; ei = (uint64_t)need; }
     };
 
-    // The same for every array shape, one after the other: key_of_terms(terms) is the item's least key.
-    auto offer_arrays = [&](auto key_of_terms, uint32_t slot, uint32_t id, bool valid) {
-        for (uint32_t y = 0; y < shape.n_arrays; ++y) {
-            const int64_t key = key_of_terms(terms[y * shape.chunk + slot]);
-            const longlong2 own = sh.tops[warp][y];
-            const bool better = valid && pair_less(key, id, own.x, (uint64_t)own.y);
-            if (!any(better)) continue;
-            int64_t nk = better ? key : kInfKey;
-            uint64_t ni = better ? id : UINT64_MAX;
-            warp_min_pair(nk, ni);
-            if (lane == 0) sh.tops[warp][y] = make_longlong2((long long)nk, (long long)ni);
-            __syncwarp();
+    // The items of up to `per` tilings, this lane's of the one in table `slot` (`valid`: there is one; else any table) with the
+    // stationary-pair terms `st`.
+    auto evaluate_with = [&](uint32_t slot, bool valid, const StatTerms& st) {
+        const TileTab& tb = sh.tile[slot];
+        const uint32_t id = tb.t * p.n_blocks + block;
+        int64_t x = kNoRow, x1 = 0, x2 = 0;
+        int need = 0;
+        if (fused_items) {
+            const bool mine = valid && fused;
+            fused_words<STAIRS>(tb, oi, dw, c, capc, [&](bool v) { return any(v && mine); }, x, need);
+        }
+        if (unfused_modes) {
+            int need2;
+            unfused_words<STAIRS>(tb, oi, dw, capc, x1, x2, need2);
+            if (!fused) { x = x1; need = need2; }
+        }
+        const bool some = valid && x < kNoRow;
+        if (!any(some)) return;
+        const int64_t y = some ? x : 0, y1 = some ? x1 : 0, y2 = some ? x2 : 0, pass = phi == 2 ? 2 * dw.il : 0;
+        const int64_t rho = fused && oi.recompute[c] != 0 ? (int64_t)tb.b[LOOP_J] : 1;
+        auto key = [&]() {
+            if (OBJ == MMEE_OBJ_ENERGY)         // (one form for both kinds)
+                return fused_least_key<OBJ>(st, fused ? y : y1 + y2 + pass, rho, p.sm_mask, p.c_dram_gb, lim.key_cap);
+            return fused ? fused_least_key<OBJ>(st, y, rho, p.sm_mask, p.c_dram_gb, lim.key_cap)
+                         : unfused_least_key<OBJ>(st, y1, y2, pass, p.sm_mask, p.c_dram_gb, lim.key_cap);
+        };
+        if (FRONT) {
+            // No mapping of the item is faster than this; after the first search few are fast enough (front of 10 816
+            // tilings, one point: 53.9 us without this test, 52.5 with it).
+            const int64_t q1 = min3(st.Q1), q2 = min3(st.Q2);
+            const int64_t least = fused ? max64(y, q1 * rho + q2) : max64(y1, q1) + pass + max64(y2, q2);
+            const bool can = some && least <= lim.key_cap;
+            auto pair = [&](int s, int64_t& e, int64_t& l) {
+                e = p.c_dram_gb * (fused ? y : y1 + y2 + pass) + st.P1[s / 3] * rho + st.P2[s % 3];
+                l = fused ? max64(y, st.Q1[s / 3] * rho + st.Q2[s % 3]) : max64(y1, st.Q1[s / 3]) + pass + max64(y2, st.Q2[s % 3]);
+            };
+            if (any(can)) offer_front(pair, id, can);
+        } else if (STAIRS) {
+            offer_stairs(key(), id, need, some);
+        } else {
+            offer(key(), id, some);
+        }
+    };
+    auto evaluate = [&](uint32_t slot, bool valid) { evaluate_with(slot, valid, sh.tile[slot].st); };
+
+    // How many rows fit: units of one (A, B) of a tiling, or of one (A, B, C) if there are few.
+    auto count_fitting = [&](uint32_t n_tiles) {
+        const uint32_t c0 = fused_items ? 0u : 4u, n_c = (unfused_modes ? 5u : 4u) - c0;
+        const uint32_t split = n_tiles <= 14u ? n_c : 1u, units = 9u * split * n_tiles;
+        while (true) {
+            uint32_t i = 0;
+            if (lane == 0) i = atomicAdd(&sh.count_cursor, 32u);
+            i = __shfl_sync(kFull, i, 0);
+            if (i >= units) break;
+            i += (uint32_t)lane;
+            const bool valid = i < units;
+            const uint32_t u = valid ? i / n_tiles : 0u, ab = split > 1u ? u / split : u, c = split > 1u ? c0 + u - ab * split : c0;
+            const uint32_t n = count_rows(sh.tile[valid ? i - u * n_tiles : 0u].size, (int)ab, (int)c, (int)(split > 1u ? c + 1u : c0 + n_c),
+                                          p.row_pruning ? 1u : unfused_modes, capc, sh.weights, [&](bool v) { return any(v && valid); });
+            if (valid) my_rows += n;
         }
     };
 
-    const bool one_pass = (uint64_t)shape.chunk * grid >= n_tilings;        // chained: the tables stay
+    const bool one_pass = CHAIN && tables_stay(p, shape);
+    // chained: the best triple of this lane's tiling (see below), the tiling's first block and the least that it has of what is
+    // bounded (latency, buffer need)
+    int64_t ck = kInfKey, cl = 0;
+    uint64_t ci = 0, first = 0;
+    int64_t limited = 0;
+    bool valid = false;
     for (uint32_t step = 0;; ++step) {
+        // chained: the rows that fit under the bound before; whether those of this one are counted before it is published, or the
+        // count of the launch's first search stands (the bound is on the latency)
+        const bool last = CHAIN && step + 1 == shape.chain_steps, counted = FRONT && one_pass && step;
+        const bool count_now = !counted && (!one_pass || last);
+        if (CHAIN && !counted) my_rows = 0;
+        int64_t bk = kInfKey, bl = kInfKey;       // chained: the warp's best triple
+        uint64_t bi = UINT64_MAX;
         if (CHAIN && (step || shape.chain_read)) {
             __syncthreads();                // the counters of the search before are no longer in use
             if (tid == 0) {
@@ -923,58 +1084,71 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 if (!over) sh.bound = kNoBound;
                 else if (step && STAIRS) sh.bound = low == 0xffffffffu ? kNoBound : (int64_t)low;
                 else sh.bound = *reinterpret_cast<volatile long long*>(&head->chain_bound);
-                sh.n_fit = sh.cursor = 0;
+                sh.n_list = sh.cursor = sh.count_cursor = 0;
+                sh.best = kInfKey;
                 if (!one_pass) sh.n_live = 0;
             }
             __syncthreads();
             const int64_t bound = sh.bound;
             if (bound == kNoBound) return;
-            if (OBJ == MMEE_OBJ_ENERGY) {
+            if (tid == 0 && step && one_pass) {     // (before this thread says that the CTA's next part is there)
+                unsigned long long rows = 0;
+                for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
+                atomicAdd(&shape.chain_to[step - 1].n_feasible, rows);
+            }
+            if (STAIRS) {
                 lim.cap_words = bound;
                 capc = (int)bound;
             } else {
                 lim.key_cap = bound;
             }
-            ek = el = kInfKey;
-            ei = UINT64_MAX;
-            my_rows = 0;
         }
         // Tiling number m of this CTA is one of the m-th `grid` consecutive ones, a different one in every round (a fixed
         // one would be the same divisor of the last dimension again and again).
         for (uint32_t m0 = 0; (uint64_t)m0 * grid < n_tilings; m0 += shape.chunk) {
             if (m0) {
                 __syncthreads();                // the previous pass's tables are no longer in use
-                if (tid == 0) { sh.n_live = sh.n_fit = 0; sh.cursor = 0; }
+                if (tid == 0) sh.n_live = sh.n_list = sh.cursor = sh.count_cursor = 0;
                 __syncthreads();
             }
-            for (uint32_t j0 = 0; j0 < (step && one_pass ? 0 : shape.chunk); j0 += kSearchThreads / 8) {
-                const uint32_t j = j0 + (uint32_t)tid / 8u, m = m0 + j;
-                uint64_t rel = (uint64_t)m * grid;
-                const bool mine = j < shape.chunk && rel < n_tilings;
-                rel += (blockIdx.x + m) % grid;
+            if (!step || !one_pass) {
+                // the tilings that can fit, one per thread: with every operand at L3 the buffer need is smallest,
+                // max(A+B+C, C+D+E) tiles (Eq. 1-4)
+                const uint32_t m = m0 + (uint32_t)tid;
+                uint64_t rel = (uint64_t)m * grid + (blockIdx.x + m) % grid;
                 uint32_t b[8], t = 0;
-                bool live = mine && rel < n_tilings;
+                bool live = (uint32_t)tid < shape.chunk && (uint64_t)m * grid < n_tilings && rel < n_tilings;
                 if (live) {
                     t = (uint32_t)(p.t_begin + rel);
                     tiling_bounds(p, SharedDivisors{sh}, t, b);
-                    // With every operand at L3 the buffer need is smallest: max(A+B+C, C+D+E) tiles (Eq. 1-4).
                     const uint64_t ta = (uint64_t)b[4] * b[5], tbb = (uint64_t)b[5] * b[6], tc = (uint64_t)b[4] * b[6];
                     const uint64_t td = (uint64_t)b[6] * b[7], te = (uint64_t)b[4] * b[7];
                     live = ta + tbb + tc <= (uint64_t)capc && tc + td + te <= (uint64_t)capc;
                 }
-                uint32_t slot = 0;
-                if (live && (tid & 7) == 0) slot = atomicAdd(&sh.n_live, 1u);
-                slot = __shfl_sync(kFull, slot, lane & ~7);
+                const unsigned who = __ballot_sync(kFull, live);
+                uint32_t at = 0;
+                if (who && lane == 0) at = atomicAdd(&sh.n_live, (uint32_t)__popc(who));
+                at = __shfl_sync(kFull, at, 0) + (uint32_t)__popc(who & ((1u << lane) - 1u));
                 if (live) {
-                    uint32_t own = b[0];
-    #pragma unroll
-                    for (int d = 1; d < 8; ++d) own = (tid & 7) == d ? b[d] : own;
-                    sh.tile[slot].b[tid & 7] = own;
+                    TileTab& tb = sh.tile[at];
+                    tb.t = t;
+#pragma unroll
+                    for (int d = 0; d < 8; ++d) tb.b[d] = b[d];
                 }
-                __syncwarp();
-                if (live) build_tile<!ARRAYS>(p, sh, b, t, tid & 7, &sh.tile[slot]);
+                __syncthreads();
+                // their tables, eight threads each
+                const uint32_t n_live = sh.n_live;
+                for (uint32_t i = (uint32_t)tid; i - (uint32_t)lane < 8u * n_live; i += kSearchThreads) {
+                    const bool valid = i < 8u * n_live;
+                    TileTab& tb = sh.tile[valid ? i / 8u : 0u];
+                    if (valid) build_tile<!ARRAYS>(p, sh, (int)(i & 7u), &tb);
+                    if (!ARRAYS && !CHAIN) {
+                        __syncwarp();
+                        if (valid && (i & 7u) == 7u) tb.least = tile_least_key<OBJ>(tb.st, dw, p.c_dram_gb, lim.key_cap);
+                    }
+                }
             }
-            if (MULTI && m0 == 0 && tid == 0) sh.G = *reinterpret_cast<volatile long long*>(&head->G);
+            if (!step && !m0) await_weights();
             __syncthreads();
             if (ARRAYS) {
                 const uint32_t n_live = sh.n_live;
@@ -990,117 +1164,214 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 __syncthreads();
             }
 
-            if (STAIRS) {
-                // The tables are those of the bound the plan has.  (Front of the GPT-3 FFN, twenty searches: 281 us with
-                // items for every table, 263 with this.)
-                if ((uint32_t)tid < sh.n_live) {
-                    const uint32_t* b = sh.tile[tid].b;
-                    const uint64_t tc = (uint64_t)b[4] * b[6];
-                    const uint64_t first = (uint64_t)b[4] * b[5] + (uint64_t)b[5] * b[6], second = (uint64_t)b[6] * b[7] + (uint64_t)b[4] * b[7];
-                    if (tc + max(first, second) <= (uint64_t)capc) fit_slots[atomicAdd(&sh.n_fit, 1u)] = (uint8_t)tid;
+            const uint32_t n_tiles = sh.n_live;
+            if (tid == 0) my_live += n_tiles;
+
+            // ---- the least keys: first of the tilings whose least_of is smallest among a warp's own, by half of the warps for a single
+            // optimum (the others count meanwhile), by all for the k best
+            const bool all_at_once = ARRAYS || CHAIN || n_tiles <= per * (uint32_t)kWarps;
+            if (CHAIN) {
+                // This lane keeps the best triple of its tiling over the searches: valid while it is within the bound, else a triple
+                // that the tiling's best one does not precede.  The warp evaluates the most promising of those until its best
+                // triple is a valid one, or worse than another warp's.  (Front of the GPT-3 FFN, evaluating every tiling that
+                // fits in each of its twenty searches: 242 us.)
+                const uint32_t own = (uint32_t)(warp + kWarps * lane);
+                if (!step || !one_pass) {
+                    valid = false;
+                    ck = kInfKey;
+                    if (own < n_tiles) {
+                        const TileTab& tb = sh.tile[own];
+                        ck = tile_least_key<OBJ>(tb.st, dw, p.c_dram_gb, INT64_MAX);
+                        first = (uint64_t)tb.t * p.n_blocks;
+                        const int one = sat_add(tb.size[S_ik], tb.size[S_kl]), two = sat_add(tb.size[S_lj], tb.size[S_ij]);
+                        limited = FRONT ? tile_least_key<MMEE_OBJ_LATENCY>(tb.st, dw, 0, 0) : (int64_t)sat_add(tb.size[S_il], one > two ? one : two);
+                    }
+                }
+                if (valid && (FRONT ? cl > lim.key_cap : (int64_t)ci > lim.cap_words)) valid = false;
+                if (limited > (FRONT ? lim.key_cap : lim.cap_words)) ck = kInfKey;
+                while (true) {
+                    int64_t mk = ck, ml = valid ? cl : (STAIRS ? (int64_t)first : 0);
+                    uint64_t mi = valid ? ci : 0;
+                    const int64_t own_l = ml;
+                    const uint64_t own_i = mi;
+                    warp_min_triple(mk, ml, mi);
+                    if (mk == kInfKey || mk > *reinterpret_cast<volatile long long*>(&sh.best)) break;
+                    const unsigned who = __ballot_sync(kFull, ck == mk && own_l == ml && own_i == mi);
+                    if ((__ballot_sync(kFull, valid) >> (__ffs(who) - 1)) & 1u) {
+                        if (lane == 0) atomicMin(&sh.best, (long long)mk);
+                        if (triple_less(mk, ml, mi, bk, bl, bi)) { bk = mk; bl = ml; bi = mi; }
+                        break;
+                    }
+                    // up to `per` tilings
+                    uint32_t slot = 0;
+                    int src = 0;
+                    bool chosen = false;
+                    uint32_t n = 0;
+#pragma unroll 1
+                    for (; n < per; ++n) {
+                        int at = __ffs(who) - 1;
+                        if (n) {
+                            int64_t lk = valid || chosen ? kInfKey : ck;
+                            uint64_t li = valid || chosen ? UINT64_MAX : first;
+                            const uint64_t own_first = li;
+                            warp_min_pair(lk, li);
+                            if (lk == kInfKey) break;
+                            at = __ffs(__ballot_sync(kFull, own_first == li)) - 1;
+                        }
+                        if (lane == at) chosen = true;
+                        if (sub >= n) slot = (uint32_t)(warp + kWarps * at);
+                        if (sub == n) src = at;
+                    }
+                    ek = el = kInfKey;
+                    ei = UINT64_MAX;
+                    evaluate(slot, sub < n);
+#pragma unroll 1
+                    for (uint32_t j = 0; j < n; ++j) {
+                        int64_t tk = sub == j ? ek : kInfKey, tl = sub == j ? el : kInfKey;
+                        uint64_t ti = sub == j ? ei : UINT64_MAX;
+                        warp_min_triple(tk, tl, ti);
+                        const int at = __shfl_sync(kFull, src, (int)(j * n_items));
+                        if (lane == at) { ck = tk; cl = tl; ci = ti; valid = tk != kInfKey; }
+                    }
+                }
+            } else if (ARRAYS) {
+                // One shape and 32 tilings by a warp: those whose least key may still be better, the most promising first.
+                const uint32_t blocks = (n_tiles + 31u) / 32u;
+                for (uint32_t u = (uint32_t)warp; u < shape.n_arrays * blocks; u += kWarps) {
+                    const uint32_t y = u / blocks, mine = (u - y * blocks) * 32u + (uint32_t)lane;
+                    const longlong2 own = sh.tops[warp][y];
+                    ek = own.x;
+                    ei = (uint64_t)own.y;
+                    const StatTerms* st = terms + y * shape.chunk;
+                    const bool have = mine < n_tiles;
+                    const uint64_t first = have ? (uint64_t)sh.tile[mine].t * p.n_blocks : UINT64_MAX;
+                    const int64_t least = have ? tile_least_key<OBJ>(st[mine], dw, p.c_dram_gb, lim.key_cap) : kInfKey;
+                    bool open = have;
+                    while (true) {
+                        int64_t lk = open ? least : kInfKey, bk = ek;
+                        uint64_t li = open ? first : UINT64_MAX, bi = ei;
+                        warp_min_pair(lk, li);
+                        warp_min_pair(bk, bi);
+                        if (!pair_less(lk, li, bk, bi)) break;
+                        const unsigned who = __ballot_sync(kFull, open && least == lk && first == li);
+                        const int src = __ffs(who) - 1;
+                        if (lane == src) open = false;
+                        const uint32_t slot = mine - (uint32_t)lane + (uint32_t)src;
+                        evaluate_with(slot, sub == 0, st[slot]);
+                    }
+                    warp_min_pair(ek, ei);
+                    if (lane == 0) sh.tops[warp][y] = make_longlong2((long long)ek, (long long)ei);
+                }
+            } else if (all_at_once) {
+                for (uint32_t i = (uint32_t)warp * per; i < n_tiles; i += per * (uint32_t)kWarps)
+                    evaluate(i + sub < n_tiles ? i + sub : i, sub < per && i + sub < n_tiles);
+            } else if (!m0 && (MULTI || warp < kWarps / 2)) {
+                const uint32_t first = (uint32_t)warp, every = MULTI ? (uint32_t)kWarps : (uint32_t)kWarps / 2u;
+                uint32_t slot = 0;
+                bool valid = false;
+                for (uint32_t i = 0; i < per; ++i) {
+                    int64_t lk = kInfKey;
+                    uint64_t li = UINT64_MAX;
+                    uint32_t mine = 0;
+                    for (uint32_t at = first + (uint32_t)lane * every; at < n_tiles; at += 32u * every) {
+                        const uint32_t s = at;
+                        const int64_t key = sh.tile[s].least;
+                        if (!sh.done[s] && pair_less(key, sh.tile[s].t, lk, li)) { lk = key; li = sh.tile[s].t; mine = s; }
+                    }
+                    const uint64_t own = li;
+                    warp_min_pair(lk, li);
+                    if (li == UINT64_MAX) break;
+                    const int src = __ffs(__ballot_sync(kFull, own == li)) - 1;
+                    const uint32_t s = __shfl_sync(kFull, mine, src);
+                    if (lane == 0) sh.done[s] = 1;
+                    __syncwarp();
+                    if (sub >= i) slot = s;
+                    if (sub == i) valid = true;
+                }
+                evaluate(slot, valid);
+            }
+
+            if (MULTI && !all_at_once) {
+                // a bound for this CTA from the warps' lists, and for all CTAs
+                if (lane < kTopK) sh.tops[warp][lane] = make_longlong2((long long)ek, (long long)ei);
+                __syncthreads();
+                if (!warp) {
+                    bound_of_lists(sh, k, lane, uk, ui);
+                    if (lane == 0 && uk != kInfKey) atomicMin(&head->bound, (long long)uk);
+                }
+            }
+
+            if (!CHAIN || count_now) count_fitting(n_tiles);
+
+            if (all_at_once) continue;
+            // ---- what those left may be better than: nothing that follows it is among the k best
+            if (MULTI) {
+                if (tid == 0) {
+                    const long long g = *reinterpret_cast<volatile long long*>(&head->bound);
+                    sh.up = g < uk ? make_longlong2(g, -1ll) : make_longlong2((long long)uk, (long long)ui);
                 }
                 __syncthreads();
+                uk = sh.up.x;
+                ui = (uint64_t)sh.up.y;
+            } else {
+                int64_t lk = ek;
+                uint64_t li = ei;
+                warp_min_pair(lk, li);
+                if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)lk, (long long)li);
+                __syncthreads();
+                const longlong2 v = sh.tops[lane & (kWarps - 1)][0];
+                uk = v.x;
+                ui = (uint64_t)v.y;
+                warp_min_pair(uk, ui);
             }
-            const uint32_t n_tiles = STAIRS ? sh.n_fit : sh.n_live, per_class = n_tiles * n_orders;
-            if (tid == 0) my_live += n_tiles;
-            const uint32_t fused_items = (p.fuse_mask & 1u) ? 3u * per_class : 0u;
-            const uint32_t fused_groups = (fused_items + 31u) / 32u;
-            const uint32_t groups = fused_groups + ((p.fuse_mask & 6u) ? (per_class + 31u) / 32u : 0u);
+            const uint32_t own = (uint32_t)(warp + kWarps * lane);
+            bool open = own < n_tiles;
+            const uint32_t own_slot = open ? own : 0u;
+            if (open) {
+                const TileTab& tb = sh.tile[own_slot];
+                const int64_t key = tb.least;
+                open = !sh.done[own_slot] && key != kInfKey && !pair_less(uk, ui, key, (uint64_t)tb.t * p.n_blocks);
+                sh.done[own_slot] = 0;
+            }
+            {
+                const unsigned m = __ballot_sync(kFull, open);
+                uint32_t at = 0;
+                if (m && lane == 0) at = atomicAdd(&sh.n_list, (uint32_t)__popc(m));
+                at = __shfl_sync(kFull, at, 0) + (uint32_t)__popc(m & ((1u << lane) - 1u));
+                if (open) sh.list[at] = (uint8_t)own_slot;
+            }
+            __syncthreads();
+            const uint32_t n_list = sh.n_list;
             while (true) {
-                uint32_t g = 0;
-                if (lane == 0) g = atomicAdd(&sh.cursor, 1u);
-                g = __shfl_sync(kFull, g, 0);
-                if (g >= groups) break;
-                long long g_seen = 0;       // k > 1: the other CTAs' bound, used after this item
-                if (MULTI && lane == 0) g_seen = *reinterpret_cast<volatile long long*>(&head->G);
-                const bool fused = g < fused_groups;
-                uint32_t i = (fused ? g : g - fused_groups) * 32u + (uint32_t)lane;
-                const uint32_t n_items = fused ? fused_items : per_class;
-                const bool valid = i < n_items;
-                i = valid ? i : n_items - 1;
-                uint32_t c = 0;
-                if (fused) {
-                    c = i >= 2u * per_class ? 2u : (i >= per_class ? 1u : 0u);
-                    i -= c * per_class;
+                uint32_t i = 0;
+                if (lane == 0) i = atomicAdd(&sh.cursor, per);
+                i = __shfl_sync(kFull, i, 0);
+                if (i >= n_list) break;
+                const uint32_t slot = sh.list[i + sub < n_list ? i + sub : i];
+                bool valid = sub < per && i + sub < n_list;
+                if (MULTI) {                    // (the warp's own list may have got better)
+                    const int64_t lk = __shfl_sync(kFull, ek, k - 1);
+                    const uint64_t li = __shfl_sync(kFull, ei, k - 1);
+                    valid = valid && pair_less(sh.tile[slot].least, (uint64_t)sh.tile[slot].t * p.n_blocks, lk, li);
+                    if (!any(valid)) continue;
                 }
-                uint32_t slot = n_orders == 6u ? i / 6u : i / 2u;
-                const uint32_t os = i - slot * n_orders;
-                if (STAIRS) slot = fit_slots[slot];
-                const TileTab& tb = sh.tile[slot];
-                const OrderInfo& oi = sh.order[os];
-                const uint32_t id = tb.t * p.n_blocks + os;
-                if (fused) {
-                    uint32_t rows;
-                    int64_t x;
-                    int need;
-                    fused_class<PRUNE, STAIRS>(tb, oi, dw, (int)c, capc, PRUNE ? sh.kept.fused[os][c] : nullptr, any, rows, x, need);
-                    if (valid) my_rows += rows;
-                    const bool some = valid && x < kNoRow;
-                    if (any(some)) {
-                        const int64_t y = some ? x : 0, rho = oi.recompute[c] != 0 ? (int64_t)tb.b[LOOP_J] : 1;
-                        auto key = [&](const StatTerms& t) { return fused_least_key<OBJ>(t, y, rho, p.sm_mask, p.c_dram_gb, lim.key_cap); };
-                        auto pair = [&](int s, int64_t& e, int64_t& l) {
-                            e = p.c_dram_gb * y + tb.st.P1[s / 3] * rho + tb.st.P2[s % 3];
-                            l = max64(y, tb.st.Q1[s / 3] * rho + tb.st.Q2[s % 3]);
-                        };
-                        if (ARRAYS) offer_arrays(key, slot, id, some);
-                        else if (FRONT) {
-                            // No mapping of the item is faster than this; after the first search few are fast enough
-                            // (front of 10 816 tilings, one point: 53.9 us without this test, 52.5 with it).
-                            const bool can = some && max64(y, min3(tb.st.Q1) * rho + min3(tb.st.Q2)) <= lim.key_cap;
-                            if (any(can)) offer_front(pair, id, can);
-                        }
-                        else if (STAIRS) offer_stairs(key(tb.st), id, need, some);
-                        else offer(key(tb.st), id, some);
-                    }
-                } else {
-                    uint32_t fit1, fit2, rows;
-                    int64_t x1, x2;
-                    int need;
-                    unfused_nests<PRUNE, STAIRS>(tb, oi, dw, capc, fit1, fit2, rows, x1, x2, need);
-                    const bool some = valid && x1 < kNoRow;
-                    if (!any(some)) continue;
-                    const int64_t y1 = some ? x1 : 0, y2 = some ? x2 : 0;
-                    uint32_t block = p.n_fused_blocks;
-    #pragma unroll
-                    for (int phi = 1; phi <= 2; ++phi) {
-                        if (!((p.fuse_mask >> phi) & 1u)) continue;
-                        if (PRUNE) {
-                            rows = 0;
-                            for (int ab = 0; ab < 9; ++ab)
-                                if ((fit1 >> ab) & 1u) rows += (uint32_t)__popc(fit2 & sh.kept.unfused[phi - 1][os][ab]);
-                        }
-                        if (some) my_rows += rows;
-                        const int64_t pass = phi == 2 ? 2 * dw.il : 0;
-                        auto key = [&](const StatTerms& t) { return unfused_least_key<OBJ>(t, y1, y2, pass, p.sm_mask, p.c_dram_gb, lim.key_cap); };
-                        auto pair = [&](int s, int64_t& e, int64_t& l) {
-                            e = p.c_dram_gb * (y1 + y2 + pass) + tb.st.P1[s / 3] + tb.st.P2[s % 3];
-                            l = max64(y1, tb.st.Q1[s / 3]) + pass + max64(y2, tb.st.Q2[s % 3]);
-                        };
-                        if (ARRAYS) offer_arrays(key, slot, id + block, some);
-                        else if (FRONT) {
-                            const bool can = some && max64(y1, min3(tb.st.Q1)) + pass + max64(y2, min3(tb.st.Q2)) <= lim.key_cap;
-                            if (any(can)) offer_front(pair, id + block, can);
-                        }
-                        else if (STAIRS) offer_stairs(key(tb.st), id + block, need, some);
-                        else offer(key(tb.st), id + block, some);
-                        block += n_orders;
-                    }
-                }
-                if (MULTI && lane == 0 && g_seen < sh.G) atomicMin(&sh.G, g_seen);
+                evaluate(slot, valid);
             }
         }
 
         // ---- this CTA's result
-        for (int off = 16; off; off >>= 1) my_rows += __shfl_down_sync(kFull, my_rows, off);
-        if (lane == 0) sh.feasible_rows[warp] = my_rows;
+        unsigned long long rows_here = 0;
+        if (!CHAIN || count_now || (counted && last)) {
+            rows_here = my_rows;
+            for (int off = 16; off; off >>= 1) rows_here += __shfl_down_sync(kFull, rows_here, off);
+        }
+        if (!CHAIN && lane == 0) sh.feasible_rows[warp] = rows_here;
         if (MULTI) {
             merge_warps(sh, k, lane, warp, ek, ei);
         } else if (CHAIN) {
-            warp_min_triple(ek, el, ei);
             if (lane == 0) {
-                sh.tops[warp][0] = make_longlong2((long long)ek, (long long)el);
-                sh.tops[warp][1] = make_longlong2((long long)ei, 0);
+                sh.tops[warp][0] = make_longlong2((long long)bk, (long long)bl);
+                sh.tops[warp][1] = make_longlong2((long long)bi, (long long)rows_here);
             }
             __syncthreads();
         } else if (!ARRAYS) {
@@ -1108,8 +1379,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             if (lane == 0) sh.tops[warp][0] = make_longlong2((long long)ek, (long long)ei);
             __syncthreads();
         }
-        if (!late && !CHAIN) wait_previous_kernel();        // from here on the scratch is touched
         if (ARRAYS) {
+            wait_previous_kernel();             // from here on the scratch is touched
             // the best item of every shape; the kernel that follows merges them (resolve_arrays_kernel)
             __syncthreads();
             Partial* out = &partials[blockIdx.x];
@@ -1131,18 +1402,18 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             Partial* out = &partials[blockIdx.x];
             uint32_t count;
             if (MULTI) {
-                // an entry above the bound (some full list's last key) is not among the k best
-                long long g_end = lane == 0 ? *reinterpret_cast<volatile long long*>(&head->G) : 0;
-                g_end = __shfl_sync(kFull, g_end, 0);
-                count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey && ek <= g_end));
+                count = (uint32_t)__popc(__ballot_sync(kFull, ek != kInfKey));
                 if (lane < (int)max(count, 1u)) out->e[lane] = make_longlong2((long long)ek, (long long)ei);
             } else if (CHAIN) {
                 ek = sh.tops[lane & (kWarps - 1)][0].x;
                 el = sh.tops[lane & (kWarps - 1)][0].y;
                 ei = (uint64_t)sh.tops[lane & (kWarps - 1)][1].x;
                 warp_min_triple(ek, el, ei);
+                unsigned long long own = lane < kWarps ? (unsigned long long)sh.tops[lane][1].y : 0;
+                for (int off = kWarps / 2; off; off >>= 1) own += __shfl_xor_sync(kFull, own, off);
+                own = __shfl_sync(kFull, own, 0);
                 count = 2;
-                if (lane < 2) out->e[lane] = lane ? make_longlong2((long long)ei, 0) : make_longlong2((long long)ek, (long long)el);
+                if (lane < 2) out->e[lane] = lane ? make_longlong2((long long)ei, (long long)own) : make_longlong2((long long)ek, (long long)el);
             } else {
                 const longlong2 v = sh.tops[lane & (kWarps - 1)][0];
                 ek = v.x;
@@ -1151,9 +1422,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 count = ek != kInfKey ? 1u : 0u;
                 if (lane == 0) out->e[0] = make_longlong2((long long)ek, (long long)ei);
             }
-            unsigned long long rows = lane < kWarps ? sh.feasible_rows[lane] : 0;
-            for (int off = kWarps / 2; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
-            if (lane == 0) {
+            unsigned long long rows = !CHAIN && lane < kWarps ? sh.feasible_rows[lane] : 0;
+            if (!CHAIN)
+                for (int off = kWarps / 2; off; off >>= 1) rows += __shfl_down_sync(kFull, rows, off);
+            if (!CHAIN && lane == 0) {
                 out->count = count;
                 out->live_tilings = my_live;
                 out->feasible_rows = rows;
@@ -1161,23 +1433,33 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             // Grid reduction without a wait: every CTA makes its partial list visible, then draws a ticket; the CTA that
             // draws the last one knows that all lists are there and runs the finalize step.
             __syncwarp();
-            if (lane == 0) sh.last_cta = draw_ticket(&head->done_ctas) == grid - 1 ? 1u : 0u;
+            if (lane == 0) {
+                if (CHAIN) add_part(head);
+                else sh.last_cta = draw_ticket(&head->done_ctas) == grid - 1 ? 1u : 0u;
+            }
+        }
+        if (CHAIN) {
+            if (last) return;
+            if (one_pass && !counted) count_fitting(sh.n_live);
+            if (one_pass) {
+                rows_here = my_rows;
+                for (int off = 16; off; off >>= 1) rows_here += __shfl_down_sync(kFull, rows_here, off);
+                if (lane == 0) sh.feasible_rows[warp] = rows_here;
+            }
+            continue;
         }
         __syncthreads();
-        if (sh.last_cta) {
-            if (late) {
-                wait_previous_kernel();         // from here on the result records are touched
-                release_next_kernel();
-            }
-            if (CHAIN) finalize_chain<FRONT>(p, lim, sh, shape.chain_to + step, shape.chain_epoch + step, head, partials, (int)grid);
-            else finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
+        if (shape.hold && (sh.last_cta || !blockIdx.x)) {
+            if (!blockIdx.x) wait_previous_kernel();
+            release_next_kernel();              // (takes effect once every CTA has said so or ended)
         }
-        if (!CHAIN || step + 1 == shape.chain_steps) return;
+        if (sh.last_cta) finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
+        return;
     }
 }
 
 __global__ void reset_kernel(SearchHeader* head) {
-    head->G = kInfKey - 1;
+    head->bound = kInfKey;
     head->done_ctas = 0;
     head->chain_epoch = 0;
 }
@@ -1188,7 +1470,7 @@ __global__ void __launch_bounds__(kSearchThreads, 2)
 resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, const Partial* partials, mmee_result_t* out) {
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    load_shared<false>(p, shape.array[blockIdx.x][0], shape.array[blockIdx.x][1], sh);
+    load_shared(p, shape.array[blockIdx.x][0], shape.array[blockIdx.x][1], sh);
     __syncthreads();
     wait_previous_kernel();
     int64_t ek = kInfKey;
@@ -1207,7 +1489,11 @@ resolve_arrays_kernel(const __grid_constant__ Plan p, const LaunchShape shape, c
     min_over_warps(sh, lane, warp, ek, ei);
     rows = 0;
     for (int w = 0; w < kWarps; ++w) rows += sh.feasible_rows[w];
-    resolve_record<OBJ, false>(p, Limits{p.cap_words, p.key_cap}, sh, ek, ei, rows * p.n_sm, 0, out + blockIdx.x);
+    auto fitting = [&](unsigned long long& n) {
+        n = rows * p.n_sm;
+        return true;
+    };
+    resolve_record<OBJ, false>(p, Limits{p.cap_words, p.key_cap}, sh, ek, ei, fitting, 0, out + blockIdx.x);
 }
 
 // A launch that may start before the kernel before it on the stream has ended (`overlap`): the kernel waits itself.
@@ -1240,10 +1526,9 @@ cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeade
                             mmee_result_t* out_best, mmee_result_t* out_topk, cudaStream_t st) {
     auto* kernel = shape.n_arrays ? search_kernel<OBJ, kModeArrays>
                    : shape.chain_steps ? (chain_mode<OBJ>() == kModeChain ? search_kernel<OBJ, chain_mode<OBJ>()> : nullptr)
-                   : p.row_pruning ? search_kernel<OBJ, kModePrune>
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
     if (!kernel) return cudaErrorInvalidValue;
-    const uint32_t grid = shape.chain_steps ? shape.grid + kRecordCtas : shape.grid;
+    const uint32_t grid = shape.chain_steps ? shape.grid + kRecordCtas + 1 : shape.grid;
     return launch_overlapped(shape.overlap, shape.chain_steps != 0, grid, st, kernel, p, shape, head, partials, out_best, out_topk);
 }
 

@@ -22,7 +22,7 @@ struct alignas(16) Partial {
 // What one search's CTAs share: the bound (k > 1) and the ticket counter, reset by the finalize step, which also keeps the
 // finished search's counters.
 struct SearchHeader {
-    long long G;                            // upper bound on the k-th smallest key
+    long long bound;                        // k > 1: upper bound on the k-th smallest key
     unsigned long long last_exact_groups;   // groups of 45 mappings of the winning blocks, evaluated one by one
     unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
     long long chain_bound;                  // what a chained search leaves to the next one; -1: it found nothing
@@ -32,7 +32,10 @@ struct SearchHeader {
 };
 static_assert(sizeof(SearchHeader) == 64, "the header is 64 bytes");
 
-// Global scratch of one handle: a header and one partial list per CTA.
+// Scratches of a handle, taken in turn (see mmee_search.cu): searches under way at the same time.
+constexpr int kScratches = 4;
+
+// Global scratch of one search: a header and one partial list per CTA.
 struct Scratch {
     SearchHeader head;
     Partial partial[1];     // grid entries follow
@@ -57,7 +60,7 @@ struct LaunchShape {
     uint32_t n_arrays;      // logical array shapes searched by one launch, 0: the plan's own
     uint32_t array[kMaxArrays][2];      // their PE rows and columns
     bool overlap;           // may start before the kernel before it on the stream has ended (see mmee_search.cu)
-    bool late;              // ... and its CTAs wait for that end in the finalize step only
+    bool hold;              // ... and lets the one after it start only then
     uint32_t chain_steps;   // a chain of this many searches in one launch, 0: one search
     uint32_t chain_epoch;   // ... their numbers on this scratch, ascending and greater than any before: the first one's
     bool chain_read;        // ... that goes on from the launch before

@@ -3,7 +3,7 @@
 // A one-shot search takes 20 to 30 us on the device, but cudaMalloc and cudaFree of its scratch took about 700 us of
 // host time around it: with no other allocation of the library alive the driver maps and unmaps a 2 MB slab each time
 // (a search of 768 tilings through mmee_solve_host: 730 us).  So a workspace that is no longer in use stays in a list,
-// at most kMaxIdle of them (0.16 MB of device and 11 KB of pinned host memory each), for the next handle on its device.
+// at most kMaxIdle of them (0.32 MB of device and 11 KB of pinned host memory each), for the next handle on its device.
 // A workspace belongs to one handle or call at a time, whatever thread or stream uses it; mmee_trim frees the idle ones.
 // Its memory belongs to the context it was allocated in and ends with it (cudaDeviceReset, a destroyed driver context), so a
 // kept one is taken, or freed, only after the driver has confirmed that its allocation is still that one.
@@ -94,21 +94,21 @@ int make_workspace(int device, Workspace** out) {
     ws->device = device;
     int rc = max_search_ctas(device, &ws->max_ctas);
     if (rc) { delete ws; return rc; }
-    // one allocation: the chained searches' optima, then the two scratches
+    // one allocation: the chained searches' optima, then the scratches
     static_assert(sizeof(ChainRecord) == 48, "a multiple of 16 bytes keeps the scratches aligned");
     const size_t chain = kHostRecords * sizeof(ChainRecord), bytes = scratch_bytes(ws->max_ctas);
     unsigned char* mem = nullptr;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), chain + 2 * bytes);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), chain + kScratches * bytes);
     ws->chain = reinterpret_cast<ChainRecord*>(mem);
     if (e == cudaSuccess) ws->id = allocation_id(mem);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + chain + i * bytes);
+    for (int i = 0; i < kScratches && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + chain + i * bytes);
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t),
                           cudaHostAllocMapped | cudaHostAllocPortable);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ws->host_dev), ws->host, 0);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = launch_reset(&ws->scratch[i]->head, 0);
+    for (int i = 0; i < kScratches && e == cudaSuccess; ++i) e = launch_reset(&ws->scratch[i]->head, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         free_workspace(ws);

@@ -9,8 +9,7 @@ namespace mmee {
 struct Workspace {
     int device;
     unsigned long long id;          // the device allocation's number: the driver gives no other allocation the same one
-    Scratch* scratch[2];            // device; headers are clean while the workspace is not in use.  Two, for a search that
-                                    // publishes while the one before it on the handle still finalizes
+    Scratch* scratch[kScratches];   // device; headers are clean while the workspace is not in use
     uint32_t max_ctas;              // partial lists a scratch has room for
     ChainRecord* chain;             // device, kHostRecords: what chained searches left
     uint32_t chains;                // launches of them

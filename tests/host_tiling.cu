@@ -1,0 +1,66 @@
+// The search's counts and least words of whole tilings beside the same by blocks and classes, for a check on the CPU
+// (tests/test_host_tiling.py).
+#include "../paper_2604_03446_b200/csrc/mmee_classes.cuh"
+
+// Every `stride`-th tiling of a problem: the rows of all its blocks that fit, all of them and (with `pruned`) the kept ones, and every
+// block's least words and needs.  Returns MMEE_OK, or MMEE_ERR_CHECK with the tiling in *at where the two differ.
+extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_objective_t* o, uint32_t stride, uint64_t* at) {
+    using namespace mmee;
+    Plan p;
+    uint32_t n_kept;
+    int rc = build_plan(w, a, o, &p);
+    if (rc || (rc = set_kept_masks(&p, &n_kept))) return rc;
+    const CountWeights all = count_weights((int)p.n_orders);
+    CountWeights kept = {};
+    for (int i = 0; i < (int)(sizeof(kept) / 4); ++i) (&kept.w[0][0][0])[i] = p.kept.weights[i / 8] >> (4 * (i % 8)) & 15u;
+    const int64_t I = p.dim[0], K = p.dim[1], L = p.dim[2], J = p.dim[3];
+    const DimWords dw = {I * K, K * L, L * J, I * J, I * L};
+    const int cap = (int)p.cap_words;
+    const uint32_t modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
+    auto any = [](bool v) { return v; };
+    for (uint64_t tiling = 0; tiling < p.n_tilings; tiling += stride) {
+        *at = tiling;
+        TileTab tb = {};
+        uint64_t t = tiling;
+        for (int d = 3; d >= 0; --d) {
+            tb.b[4 + d] = p.divs[d][t % p.ndiv[d]];
+            tb.b[d] = p.dim[d] / tb.b[4 + d];
+            t /= p.ndiv[d];
+        }
+        for (int i = 0; i < kSizeSlots; ++i) tb.size[i] = sat_size(size_words(p.dim, tb.b + 4, i));
+        uint64_t rows = 0, rows_kept = 0, want = 0, want_kept = 0;
+        const int c0 = (p.fuse_mask & 1u) ? 0 : 4, c1 = modes ? 5 : 4;
+        for (int ab = 0; ab < 9; ++ab) {
+            rows += count_rows(tb.size, ab, c0, c1, modes, cap, all, any);
+            for (int c = c0; c < c1; ++c) rows_kept += count_rows(tb.size, ab, c, c + 1, 1u, cap, kept, any);
+        }
+        for (uint32_t s = 0; s < p.n_orders; ++s) {
+            uint32_t n, fit1, fit2;
+            int64_t x, x2, y, y2;
+            int need, need2;
+            for (int c = 0; c < 3 && (p.fuse_mask & 1u); ++c) {
+                fused_class<false, true>(tb, p.order[s], dw, c, cap, nullptr, any, n, x, need);
+                want += n;
+                fused_words<true>(tb, p.order[s], dw, c, cap, any, y, need2);
+                if (x != y || (x < kNoRow && need != need2)) return MMEE_ERR_CHECK;
+                fused_words<false>(tb, p.order[s], dw, c, cap, any, y, need2);
+                if (x != y) return MMEE_ERR_CHECK;
+                fused_class<true, false>(tb, p.order[s], dw, c, cap, p.kept.fused[s][c], any, n, x, need);
+                want_kept += n;
+            }
+            if (!modes) continue;
+            unfused_nests<false, true>(tb, p.order[s], dw, cap, fit1, fit2, n, x, x2, need);
+            want += (uint64_t)n * modes;
+            unfused_words<true>(tb, p.order[s], dw, cap, y, y2, need2);
+            if (x != y || x2 != y2 || (x < kNoRow && need != need2)) return MMEE_ERR_CHECK;
+            unfused_words<false>(tb, p.order[s], dw, cap, y, y2, need2);
+            if (x != y || x2 != y2) return MMEE_ERR_CHECK;
+            unfused_nests<true, false>(tb, p.order[s], dw, cap, fit1, fit2, n, x, x2, need);
+            for (uint32_t phi = 1; phi <= 2; ++phi)
+                for (int ab = 0; ab < 9 && ((p.fuse_mask >> phi) & 1u); ++ab)
+                    if ((fit1 >> ab) & 1u) want_kept += (uint64_t)__builtin_popcount(fit2 & p.kept.unfused[phi - 1][s][ab]);
+        }
+        if (rows != want || rows_kept != want_kept) return MMEE_ERR_CHECK;
+    }
+    return MMEE_OK;
+}
