@@ -78,6 +78,8 @@ int choose_launch_shape(const Plan& p, int device, uint32_t n_arrays, uint32_t m
     shape->n_arrays = n_arrays;
     shape->overlap = true;
     shape->hold = false;
+    shape->turn = 0;
+    shape->stats = nullptr;
     shape->chain_steps = shape->chain_epoch = 0;
     shape->chain_read = false;
     shape->chain_polls = 0;
@@ -113,7 +115,7 @@ int run_chain(const Plan& plan, uint32_t polls, Take take) {
         shape.chain_read = read;
         shape.chain_epoch = ++ws->chains * kHostRecords;
         for (uint32_t i = 0; i < kHostRecords; ++i) ws->host[i].status = MMEE_ERR_TIMEOUT;
-        const cudaError_t e = launch_search(plan, shape, &ws->scratch[0]->head, ws->scratch[0]->partial, nullptr, ws->host_dev, nullptr);
+        const cudaError_t e = launch_search(plan, shape, ws->head, ws->partial[0], nullptr, ws->host_dev, nullptr);
         if (e == cudaErrorCooperativeLaunchTooLarge && shape.grid > 1) {
             // the calling context has a part of the device's SMs: half the CTAs, until they are resident together
             cudaGetLastError();
@@ -245,16 +247,16 @@ static int search_on(mmee_handle* h, cudaStream_t st, mmee_result_t* out_best, m
     if (rc) return rc;
     LaunchShape shape = h->shape;
     if (h->dirty) {        // an earlier launch on this handle failed: a header may hold a used ticket counter
-        for (int i = 0; i < kScratches; ++i)
-            if ((rc = cuda_status(launch_reset(&h->ws->scratch[i]->head, st)))) return rc;
+        if ((rc = cuda_status(launch_reset(h->ws->head, st)))) return rc;
         h->dirty = false;
-        shape.overlap = false;          // (its CTAs touch the headers: not before the resets have ended)
+        shape.overlap = false;          // (its CTAs touch the header: not before the reset has ended)
     }
     ++h->turn;
     shape.hold = h->turn % (kScratches - 1) == 0;
-    Scratch* scratch = h->ws->scratch[h->turn % kScratches];
+    shape.turn = h->turn % kScratches;
+    shape.stats = h->ws->stats;
     if (h->timing) cudaEventRecord(h->ev[0], st);
-    const cudaError_t e = launch_search(h->plan, shape, &scratch->head, scratch->partial, out_best, out_topk, st);
+    const cudaError_t e = launch_search(h->plan, shape, h->ws->head, h->ws->partial[shape.turn], out_best, out_topk, st);
     if (e != cudaSuccess) { h->dirty = true; return cuda_status(e); }
     if (h->timing) cudaEventRecord(h->ev[1], st);
     h->last.kernels_launched = 1;
@@ -424,7 +426,7 @@ int mmee_search_shapes(const mmee_workload_t* workload, const mmee_arch_t* arch,
         LaunchShape shape;
         if ((rc = choose_launch_shape(plan, device, n, 0, &shape))) break;
         std::memcpy(shape.array, shapes + 2 * i0, n * sizeof(shape.array[0]));
-        if ((rc = cuda_status(launch_search_arrays(plan, shape, ws->scratch[0]->partial, ws->host_dev, nullptr)))) clean = false;
+        if ((rc = cuda_status(launch_search_arrays(plan, shape, ws->partial[0], ws->host_dev, nullptr)))) clean = false;
         const int rc2 = cuda_status(cudaStreamSynchronize(nullptr));
         if (rc2) clean = false;
         if (rc == MMEE_OK) rc = rc2;
@@ -508,8 +510,8 @@ int mmee_last_search_stats(const mmee_handle_t* h, mmee_launch_stats_t* out) {
     out->exact_path_visits = 0;
     out->rows_tested = 0;
     if (h->last.kernels_launched) {
-        unsigned long long counters[2] = {0, 0};      // last_exact_groups, last_tested_rows
-        const int rc = cuda_status(cudaMemcpy(counters, &h->ws->scratch[h->turn % kScratches]->head.last_exact_groups, sizeof(counters), cudaMemcpyDeviceToHost));
+        unsigned long long counters[2] = {0, 0};      // (LaunchShape::stats)
+        const int rc = cuda_status(cudaMemcpy(counters, h->ws->stats, sizeof(counters), cudaMemcpyDeviceToHost));
         if (rc) return rc;
         out->exact_path_visits = counters[0];
         out->rows_tested = counters[1];

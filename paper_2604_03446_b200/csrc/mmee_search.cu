@@ -474,13 +474,13 @@ __device__ __forceinline__ bool await_parts(const SearchHeader* head, uint32_t n
 #pragma unroll 4
     for (uint32_t i = 0; i < polls; ++i) {
         uint32_t now;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&head->done_ctas) : "memory");
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&head->done_ctas[0]) : "memory");
         if (now >= n) return true;
     }
     return false;
 }
 __device__ __forceinline__ void add_part(SearchHeader* head) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&head->done_ctas) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&head->done_ctas[0]) : "memory");
 }
 
 // Whether a chain's CTAs keep their tables from search to search.  They then count the rows that fit under a search's bound while
@@ -544,7 +544,7 @@ __device__ __forceinline__ bool finalize_chain(const Plan& p, int64_t cap_words,
         const int64_t bound = !found ? kNoBound : (FRONT ? el : (int64_t)ei) - 1;
         const unsigned long long word = (unsigned long long)epoch << 32 | (found ? (uint32_t)bound : 0xffffffffu);
         head->chain_bound = bound;
-        if (!found || last) head->done_ctas = 0;
+        if (!found || last) head->done_ctas[0] = 0;
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&head->chain_epoch), "l"(word) : "memory");
     }
     return found;
@@ -570,7 +570,7 @@ __device__ __noinline__ void merge_chain(const Plan& p, const LaunchShape& shape
 
 // Run by every thread of ONE CTA (the last one to finish) after all CTAs have published their partial lists.
 template <int OBJ, int MODE>
-__device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Shared& sh, SearchHeader* __restrict__ head,
+__device__ __noinline__ void finalize_step(const Plan& p, const LaunchShape& shape, const Limits& lim, Shared& sh, SearchHeader* __restrict__ head,
                                            const Partial* __restrict__ partials, int n_partials,
                                            mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -767,11 +767,14 @@ __device__ __noinline__ void finalize_step(const Plan& p, const Limits& lim, Sha
         // ready for the next search on this scratch
         unsigned long long all_live = 0;
         for (int w = 0; w < kWarps; ++w) all_live += sh.live_tilings[w];
-        head->bound = kInfKey;
-        head->last_exact_groups = n_groups;
+        head->bound[shape.turn] = kInfKey;
         const uint32_t unfused_modes = (p.fuse_mask >> 1 & 1u) + (p.fuse_mask >> 2 & 1u);
-        head->last_tested_rows = all_live * p.n_orders * ((p.fuse_mask & 1u ? kFusedReps : 0u) + (unfused_modes ? 18u : 0u));
-        head->done_ctas = 0;
+        head->done_ctas[shape.turn] = 0;
+        if (shape.stats) {
+            wait_previous_kernel();         // (the searches before write them as well)
+            shape.stats[0] = n_groups;
+            shape.stats[1] = all_live * p.n_orders * ((p.fuse_mask & 1u ? kFusedReps : 0u) + (unfused_modes ? 18u : 0u));
+        }
     }
 }
 
@@ -1297,7 +1300,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 __syncthreads();
                 if (!warp) {
                     bound_of_lists(sh, k, lane, uk, ui);
-                    if (lane == 0 && uk != kInfKey) atomicMin(&head->bound, (long long)uk);
+                    if (lane == 0 && uk != kInfKey) atomicMin(&head->bound[shape.turn], (long long)uk);
                 }
             }
 
@@ -1307,7 +1310,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             // ---- what those left may be better than: nothing that follows it is among the k best
             if (MULTI) {
                 if (tid == 0) {
-                    const long long g = *reinterpret_cast<volatile long long*>(&head->bound);
+                    const long long g = *reinterpret_cast<volatile long long*>(&head->bound[shape.turn]);
                     sh.up = g < uk ? make_longlong2(g, -1ll) : make_longlong2((long long)uk, (long long)ui);
                 }
                 __syncthreads();
@@ -1435,7 +1438,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             __syncwarp();
             if (lane == 0) {
                 if (CHAIN) add_part(head);
-                else sh.last_cta = draw_ticket(&head->done_ctas) == grid - 1 ? 1u : 0u;
+                else sh.last_cta = draw_ticket(&head->done_ctas[shape.turn]) == grid - 1 ? 1u : 0u;
             }
         }
         if (CHAIN) {
@@ -1453,14 +1456,16 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             if (!blockIdx.x) wait_previous_kernel();
             release_next_kernel();              // (takes effect once every CTA has said so or ended)
         }
-        if (sh.last_cta) finalize_step<OBJ, MODE>(p, lim, sh, head, partials, (int)grid, out_best, out_topk);
+        if (sh.last_cta) finalize_step<OBJ, MODE>(p, shape, lim, sh, head, partials, (int)grid, out_best, out_topk);
         return;
     }
 }
 
 __global__ void reset_kernel(SearchHeader* head) {
-    head->bound = kInfKey;
-    head->done_ctas = 0;
+    for (int i = 0; i < kScratches; ++i) {
+        head->bound[i] = kInfKey;
+        head->done_ctas[i] = 0;
+    }
     head->chain_epoch = 0;
 }
 

@@ -19,23 +19,19 @@ struct alignas(16) Partial {
     uint64_t feasible_rows;
 };
 
-// What one search's CTAs share: the bound (k > 1) and the ticket counter, reset by the finalize step, which also keeps the
-// finished search's counters.
-struct SearchHeader {
-    long long bound;                        // k > 1: upper bound on the k-th smallest key
-    unsigned long long last_exact_groups;   // groups of 45 mappings of the winning blocks, evaluated one by one
-    unsigned long long last_tested_rows;    // different rows of the tilings that were evaluated
-    long long chain_bound;                  // what a chained search leaves to the next one; -1: it found nothing
-    unsigned long long chain_epoch;         // the last chained search that has ended on this scratch (high half)
-    unsigned int done_ctas;                 // ticket counter: the CTA that draws the last ticket runs the finalize step
-    unsigned int pad[5];
-};
-static_assert(sizeof(SearchHeader) == 64, "the header is 64 bytes");
-
 // Scratches of a handle, taken in turn (see mmee_search.cu): searches under way at the same time.
 constexpr int kScratches = 4;
 
-// Global scratch of one search: a header and one partial list per CTA.
+// What the CTAs of one search share, for every scratch: the bound (k > 1) and the ticket counter, reset by the finalize step.
+struct SearchHeader {
+    long long bound[kScratches];            // k > 1: upper bound on the k-th smallest key
+    unsigned int done_ctas[kScratches];     // ticket counter: the CTA that draws the last ticket runs the finalize step
+    long long chain_bound;                  // what a chained search leaves to the next one
+    unsigned long long chain_epoch;         // the last chained search that has ended on this header (high half)
+};
+static_assert(sizeof(SearchHeader) == 64, "the header is 64 bytes");
+
+// Global scratch of one search after the other: a header and one partial list per CTA.
 struct Scratch {
     SearchHeader head;
     Partial partial[1];     // grid entries follow
@@ -59,6 +55,9 @@ struct LaunchShape {
     uint32_t chunk;         // tilings a CTA evaluates per pass, at most kMaxChunk
     uint32_t n_arrays;      // logical array shapes searched by one launch, 0: the plan's own
     uint32_t array[kMaxArrays][2];      // their PE rows and columns
+    uint32_t turn;          // the scratch: which entries of the header
+    unsigned long long* stats;          // device, 2: groups of 45 mappings of the winning blocks, evaluated one by one; different
+                                        // rows of the tilings that were evaluated (null: not wanted)
     bool overlap;           // may start before the kernel before it on the stream has ended (see mmee_search.cu)
     bool hold;              // ... and lets the one after it start only then
     uint32_t chain_steps;   // a chain of this many searches in one launch, 0: one search
@@ -79,8 +78,6 @@ constexpr uint32_t kRecordCtas = 2;
 // The wait for a chained search is limited, at a few seconds.  A CTA whose wait runs out leaves without a trace: it takes no
 // part in later searches, which then do not end, and makes no more records, so that the caller finds one that was not made.
 constexpr uint32_t kChainPolls = 1u << 22;
-
-inline size_t scratch_bytes(uint32_t grid) { return sizeof(Scratch) + (size_t)(grid ? grid - 1 : 0) * sizeof(Partial); }
 
 size_t search_smem_bytes();
 // Tilings whose tables a CTA holds at once, with the stationary-pair terms of n_arrays array shapes.

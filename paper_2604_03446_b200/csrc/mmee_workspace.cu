@@ -94,21 +94,25 @@ int make_workspace(int device, Workspace** out) {
     ws->device = device;
     int rc = max_search_ctas(device, &ws->max_ctas);
     if (rc) { delete ws; return rc; }
-    // one allocation: the chained searches' optima, then the scratches
-    static_assert(sizeof(ChainRecord) == 48, "a multiple of 16 bytes keeps the scratches aligned");
-    const size_t chain = kHostRecords * sizeof(ChainRecord), bytes = scratch_bytes(ws->max_ctas);
+    // one allocation: the chained searches' optima, the header, the counters, then the partial lists
+    static_assert(sizeof(ChainRecord) == 48, "a multiple of 16 bytes keeps the rest aligned");
+    const size_t chain = kHostRecords * sizeof(ChainRecord), bytes = ws->max_ctas * sizeof(Partial), before = chain + sizeof(SearchHeader) + 16;
     unsigned char* mem = nullptr;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), chain + kScratches * bytes);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&mem), before + kScratches * bytes);
     ws->chain = reinterpret_cast<ChainRecord*>(mem);
     if (e == cudaSuccess) ws->id = allocation_id(mem);
-    for (int i = 0; i < kScratches && e == cudaSuccess; ++i) ws->scratch[i] = reinterpret_cast<Scratch*>(mem + chain + i * bytes);
+    if (e == cudaSuccess) {
+        ws->head = reinterpret_cast<SearchHeader*>(mem + chain);
+        ws->stats = reinterpret_cast<unsigned long long*>(mem + chain + sizeof(SearchHeader));
+        for (int i = 0; i < kScratches; ++i) ws->partial[i] = reinterpret_cast<Partial*>(mem + before + i * bytes);
+    }
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation
     if (e == cudaSuccess)
         e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t),
                           cudaHostAllocMapped | cudaHostAllocPortable);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ws->host_dev), ws->host, 0);
-    for (int i = 0; i < kScratches && e == cudaSuccess; ++i) e = launch_reset(&ws->scratch[i]->head, 0);
+    if (e == cudaSuccess) e = launch_reset(ws->head, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         free_workspace(ws);

@@ -9,7 +9,9 @@ namespace mmee {
 struct Workspace {
     int device;
     unsigned long long id;          // the device allocation's number: the driver gives no other allocation the same one
-    Scratch* scratch[kScratches];   // device; headers are clean while the workspace is not in use
+    SearchHeader* head;             // device; clean while the workspace is not in use
+    Partial* partial[kScratches];   // device: the scratches' partial lists
+    unsigned long long* stats;      // device, LaunchShape::stats
     uint32_t max_ctas;              // partial lists a scratch has room for
     ChainRecord* chain;             // device, kHostRecords: what chained searches left
     uint32_t chains;                // launches of them
