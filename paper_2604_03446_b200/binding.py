@@ -141,6 +141,10 @@ def _fill(struct, values: dict):
     return struct
 
 
+def _inputs(workload: dict, arch: dict, objective: dict):
+    return Workload(**workload), Arch(**arch), Objective(**objective)
+
+
 def _record_space(n: int):
     """Uninitialised host memory for n result records (a ctypes array would be zeroed: 30 us for 4096 records)."""
     import numpy as np
@@ -156,11 +160,20 @@ def _check(code: int, where: str):
         raise MmeeError(code, where)
 
 
-def _stream_ptr(stream):
+def _current_stream():
+    """The current stream of the current device as an address; afterwards without the stream object that torch makes for it
+    (1.5 us a call)."""
+    global _current_stream
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    ptr = torch.cuda.current_stream().cuda_stream
+    device, raw = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device and raw:
+        _current_stream = lambda: raw(device())
+    return ptr
+
+
+def _stream_ptr(stream):
+    return _current_stream() if stream is None else stream.cuda_stream
 
 
 def mmee_create(workload: dict, arch: dict, objective: dict) -> C.c_void_p:
@@ -199,9 +212,10 @@ def result_buffer(n: int, device="cuda"):
 
 def mmee_search(handle, out_best, out_topk=None, stream=None) -> None:
     """Asynchronous: out_best / out_topk are uint8 CUDA tensors from result_buffer()."""
-    _check(library().mmee_search(handle, _stream_ptr(stream), C.c_void_p(out_best.data_ptr()),
-                                 C.c_void_p(out_topk.data_ptr()) if out_topk is not None else None),
-           "mmee_search")
+    code = (_lib or library()).mmee_search(handle, _stream_ptr(stream), out_best.data_ptr(),
+                                           out_topk.data_ptr() if out_topk is not None else None)
+    if code:
+        _check(code, "mmee_search")
 
 
 def mmee_search_host(handle, want_topk: bool = False, topk: int = 0):
@@ -251,9 +265,9 @@ def mmee_solve_host(workload: dict, arch: dict, objective: dict):
     k = objective["topk"]
     best, topk = Result(), (Result * k)()
     h2d, d2h = C.c_uint64(), C.c_uint64()
-    _check(library().mmee_solve_host(_fill(Workload(), workload), _fill(Arch(), arch),
-                                     _fill(Objective(), objective), C.byref(best), topk,
-                                     C.byref(h2d), C.byref(d2h)), "mmee_solve_host")
+    code = (_lib or library()).mmee_solve_host(*_inputs(workload, arch, objective), best, topk, h2d, d2h)
+    if code:
+        _check(code, "mmee_solve_host")
     return best, list(topk), h2d.value, d2h.value
 
 
@@ -261,9 +275,7 @@ def mmee_pareto_front(workload: dict, arch: dict, objective: dict, capacity: int
     """Energy-latency Pareto front of the whole mapping space: list of Result, by increasing energy."""
     pts = _record_space(capacity)
     n = C.c_uint32()
-    _check(library().mmee_pareto_front(_fill(Workload(), workload), _fill(Arch(), arch),
-                                       _fill(Objective(), objective), C.cast(pts.ctypes.data, C.POINTER(Result)),
-                                       capacity, C.byref(n)),
+    _check(library().mmee_pareto_front(*_inputs(workload, arch, objective), C.cast(pts.ctypes.data, C.POINTER(Result)), capacity, n),
            "mmee_pareto_front")
     return _records(pts, n.value)
 
@@ -272,9 +284,8 @@ def mmee_pareto_front_bs_da(workload: dict, arch: dict, objective: dict, capacit
     """Buffer-size / DRAM-traffic Pareto front of the whole mapping space: list of Result, by decreasing buffer size."""
     pts = _record_space(capacity)
     n = C.c_uint32()
-    _check(library().mmee_pareto_front_bs_da(_fill(Workload(), workload), _fill(Arch(), arch),
-                                             _fill(Objective(), objective), C.cast(pts.ctypes.data, C.POINTER(Result)),
-                                             capacity, C.byref(n)),
+    _check(library().mmee_pareto_front_bs_da(*_inputs(workload, arch, objective), C.cast(pts.ctypes.data, C.POINTER(Result)), capacity,
+                                             n),
            "mmee_pareto_front_bs_da")
     return _records(pts, n.value)
 
@@ -285,8 +296,7 @@ def mmee_search_shapes(workload: dict, arch: dict, objective: dict, shapes):
     flat = (C.c_uint32 * (2 * n))(*[v for rc in shapes for v in rc])
     out = (Result * n)()
     best = C.c_uint32()
-    _check(library().mmee_search_shapes(_fill(Workload(), workload), _fill(Arch(), arch), _fill(Objective(), objective),
-                                        flat, n, out, C.byref(best)), "mmee_search_shapes")
+    _check(library().mmee_search_shapes(*_inputs(workload, arch, objective), flat, n, out, best), "mmee_search_shapes")
     return list(out), (None if best.value == 2 ** 32 - 1 else best.value)
 
 

@@ -198,9 +198,10 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
         // divisors in ascending order: small ones up, cofactors down
         uint32_t lo[MMEE_MAX_DIVISORS], hi[MMEE_MAX_DIVISORS];
         uint32_t nlo = 0, nhi = 0;
-        for (uint64_t x = 1; x * x <= dims[d]; ++x) {
-            if (dims[d] % x) continue;
-            const uint64_t y = dims[d] / x;
+        const uint32_t whole = p->dim[d];
+        for (uint32_t x = 1; (uint64_t)x * x <= whole; ++x) {
+            if (whole % x) continue;
+            const uint32_t y = whole / x;
             const bool keep_x = o->tiling_set == MMEE_TILE_ALL_DIVISORS || !(x & (x - 1));
             const bool keep_y = (y != x) && (o->tiling_set == MMEE_TILE_ALL_DIVISORS || !(y & (y - 1)));
             if (keep_x) { if (nlo == MMEE_MAX_DIVISORS) return MMEE_ERR_RANGE; lo[nlo++] = (uint32_t)x; }
@@ -286,7 +287,12 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
     const long double limit = 4611686018427387904.0L;     // 2^62
     if (emax >= limit || lmax >= limit) return MMEE_ERR_OVERFLOW;
 
-    build_query_tables(&p->q);
+    static const QueryTables tables = [] {      // (the same for every plan)
+        QueryTables q;
+        build_query_tables(&q);
+        return q;
+    }();
+    p->q = tables;
     for (uint32_t s = 0; s < p->n_orders; ++s) build_order_info(p->order_id[s], p->q, &p->order[s]);
     return MMEE_OK;
 }

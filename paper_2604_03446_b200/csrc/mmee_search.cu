@@ -885,6 +885,16 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
 // A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  The waits are the
 // hardware's grid dependency; a CTA waits for none that could start after it.
 
+// Tells the host that what the CTA's threads have written is there.  All threads of the CTA.
+__device__ __forceinline__ void signal_host(uint32_t* signal, uint32_t value) {
+    if (!signal) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(signal), "r"(value) : "memory");
+    }
+}
+
 // The number of CTAs that drew a ticket before; what they wrote before that is visible from here on, and what the calling
 // warp has written is to those that draw one later.
 __device__ __forceinline__ uint32_t draw_ticket(unsigned int* count) {
@@ -1456,7 +1466,10 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             if (!blockIdx.x) wait_previous_kernel();
             release_next_kernel();              // (takes effect once every CTA has said so or ended)
         }
-        if (sh.last_cta) finalize_step<OBJ, MODE>(p, shape, lim, sh, head, partials, (int)grid, out_best, out_topk);
+        if (sh.last_cta) {
+            finalize_step<OBJ, MODE>(p, shape, lim, sh, head, partials, (int)grid, out_best, out_topk);
+            signal_host(shape.signal, shape.signal_value);
+        }
         return;
     }
 }

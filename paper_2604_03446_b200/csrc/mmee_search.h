@@ -58,6 +58,8 @@ struct LaunchShape {
     uint32_t turn;          // the scratch: which entries of the header
     unsigned long long* stats;          // device, 2: groups of 45 mappings of the winning blocks, evaluated one by one; different
                                         // rows of the tilings that were evaluated (null: not wanted)
+    uint32_t* signal;       // pinned host memory as the device addresses it: `signal_value` goes there when the records are written (null:
+    uint32_t signal_value;  // nobody waits for it)
     bool overlap;           // may start before the kernel before it on the stream has ended (see mmee_search.cu)
     bool hold;              // ... and lets the one after it start only then
     uint32_t chain_steps;   // a chain of this many searches in one launch, 0: one search

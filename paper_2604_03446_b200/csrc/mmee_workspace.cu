@@ -109,9 +109,14 @@ int make_workspace(int device, Workspace** out) {
     // portable: usable from every device's context, mapped: kernels write their records straight into it, so that the
     // host needs no copy call after a search, only the synchronisation
     if (e == cudaSuccess)
-        e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t),
+        e = cudaHostAlloc(reinterpret_cast<void**>(&ws->host), kHostRecords * sizeof(mmee_result_t) + sizeof(uint32_t),
                           cudaHostAllocMapped | cudaHostAllocPortable);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&ws->host_dev), ws->host, 0);
+    if (e == cudaSuccess) {
+        ws->signal = reinterpret_cast<uint32_t*>(ws->host + kHostRecords);
+        ws->signal_dev = reinterpret_cast<uint32_t*>(ws->host_dev + kHostRecords);
+        *ws->signal = 0;
+    }
     if (e == cudaSuccess) e = launch_reset(ws->head, 0);
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {

@@ -17,6 +17,8 @@ struct Workspace {
     uint32_t chains;                // launches of them
     mmee_result_t* host;            // pinned host memory: kHostRecords records that kernels write into
     mmee_result_t* host_dev;        // the same memory as the device addresses it
+    uint32_t *signal, *signal_dev;  // a word behind the records (LaunchShape::signal)
+    uint32_t signals;               // the last value that was waited for
     Workspace* next;
 };
 
