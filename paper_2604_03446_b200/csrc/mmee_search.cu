@@ -1,11 +1,12 @@
 // The search kernel: every mapping decided, capacity pruning, top-k, in one launch.
 //
 // Work decomposition.  CTA c takes one tiling out of every `grid` consecutive ones, so that tilings that cannot fit at
-// all (large tiles, neighbours in the index order) spread evenly, keeps those that can in a compact list with their
-// size and stationary-pair tables in shared memory, and cuts the list into items: (class of C, tiling, order) of the
-// fused mode, then (tiling, order) of the unfused ones.  A warp takes 32 items at a time; one thread decides one item
-// in closed form over classes of levels (mmee_classes.cuh): how many of its rows fit and its least key, exact in
-// 64 bits.  No candidate, row or threshold is kept per mapping, and nothing but the CTA's result leaves the SM.
+// all (large tiles, neighbours in the index order) spread evenly, and keeps those that can in a compact list with their
+// size and stationary-pair tables in shared memory.  How many of their rows fit is counted per tiling over all orders
+// (count_rows).  A tiling's items, (class of C, order) of the fused mode and (order, mode) of the unfused ones, are evaluated by
+// a warp, one lane each: the least key, exact in 64 bits, in closed form (mmee_classes.cuh).  The tilings with the least
+// bounds come first, and those whose bound cannot enter the result any more are left out.  No candidate, row or threshold is
+// kept per mapping, and nothing but the CTA's result leaves the SM.
 //
 // Selection.  A block (tiling, fusion mode, order) is a contiguous range of mapping indices, so that (least key, block
 // number) orders blocks as their best mappings are ordered.  The k best mappings of the whole space lie in the k best
