@@ -24,6 +24,7 @@ struct mmee_handle {
     bool in_flight;              // a search was launched whose end this handle has not waited for
     bool timing;
     uint32_t turn;               // searches so far: the last one's scratch is number turn % kScratches
+    unsigned long long capture;  // what recorded the last one (capture_of)
     cudaEvent_t ev[2];           // before and after the search kernel
 };
 
@@ -263,15 +264,35 @@ static int check_device(const mmee_handle* h) {
     return cur == h->device ? MMEE_OK : MMEE_ERR_ARG;
 }
 
+// The capture that records what is launched on a stream, 0 if there is none.  (The default stream cannot be captured; of one whose
+// state is not told the launch will say why, and no search is taken for the one before it.)
+static unsigned long long capture_of(cudaStream_t st) {
+    if (!st) return 0;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long number = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &number) != cudaSuccess) {
+        cudaGetLastError();
+        return UINT64_MAX;
+    }
+    return status == cudaStreamCaptureStatusNone ? 0 : number | 1ull << 63;
+}
+
 // `signalled`: the host will wait for the workspace's signal.
 static int search_on(mmee_handle* h, cudaStream_t st, mmee_result_t* out_best, mmee_result_t* out_topk, bool signalled) {
     int rc = check_device(h);
     if (rc) return rc;
     LaunchShape shape = h->shape;
+    const unsigned long long capture = capture_of(st);
     if (h->dirty) {        // an earlier launch on this handle failed: a header may hold a used ticket counter
         if ((rc = cuda_status(launch_reset(h->ws->head, st)))) return rc;
-        h->dirty = false;
+        h->dirty = capture != 0;        // (one that is only recorded has not happened)
         shape.overlap = false;          // (its CTAs touch the header: not before the reset has ended)
+    }
+    // The turns of launched searches and of those that a capture records are one count, but they do not run one after the other:
+    // the first after a change of the two (or of captures) starts after what is before it, whose scratches are free then.
+    if (capture != h->capture) {
+        h->capture = capture;
+        shape.overlap = false;
     }
     ++h->turn;
     shape.hold = h->turn % (kScratches - 1) == 0;

@@ -883,6 +883,7 @@ __device__ __noinline__ void resolve_chain(const Plan& p, const LaunchShape& sha
 // they are written, so that searches end in order.  A handle has kScratches scratches in turn.  Every (kScratches - 1)-th of its
 // searches (`hold`) lets the next kernel start only after the kernel before it has ended (CTA 0 waits for that; the others need
 // not): of two searches with the same scratch the second then starts after a search between them has seen the first one's end.
+// (The turns of searches that a stream capture records count along: see search_on.)
 // A kernel that is not launched this way follows a search as usual, and a search follows one as usual.  The waits are the
 // hardware's grid dependency; a CTA waits for none that could start after it.
 

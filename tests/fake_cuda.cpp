@@ -23,6 +23,15 @@ int g_points = 0;                               // optima a chain of searches fi
 unsigned g_resident = 1000;                     // CTAs of a chain that can be resident at once
 int g_searches = 0;                             // search launches
 unsigned g_missing = 0;                         // bit i: the record of its search i is not made
+std::map<cudaStream_t, unsigned long long> g_captures;      // streams that are capturing: the capture's number
+int g_fail_launch = 0;                          // fail that many search launches
+struct Launch { unsigned long long capture; int turn, overlap, hold; };       // turn -1: a reset of the header
+std::vector<Launch> g_launches;
+
+unsigned long long capture_of(cudaStream_t st) {
+    auto it = g_captures.find(st);
+    return it == g_captures.end() ? 0 : it->second;
+}
 
 cudaError_t failed(cudaError_t e) { return g_last = e; }
 
@@ -81,6 +90,18 @@ void fake_set_context(int c) { g_context = c; }
 void fake_fail(int mallocs, int host_allocs) { g_fail_malloc = mallocs; g_fail_host = host_allocs; }
 void fake_chain(int points, unsigned missing) { g_points = points; g_missing = missing; }
 void fake_resident(unsigned ctas) { g_resident = ctas; }
+void fake_capture(void* stream, unsigned long long number) {         // 0: ends
+    if (number) g_captures[static_cast<cudaStream_t>(stream)] = number;
+    else g_captures.erase(static_cast<cudaStream_t>(stream));
+}
+void fake_fail_launch(int n) { g_fail_launch = n; }
+// Launch number i of searches and resets; false: there are no more.
+int fake_launch(int i, unsigned long long* capture, int* turn, int* overlap, int* hold) {
+    if (i >= (int)g_launches.size()) return 0;
+    const Launch& l = g_launches[i];
+    *capture = l.capture; *turn = l.turn; *overlap = l.overlap; *hold = l.hold;
+    return 1;
+}
 int fake_searches() { return g_searches; }
 int fake_plan_bytes() { return (int)sizeof(mmee::Plan); }
 int fake_live() { return (int)g_live.size(); }
@@ -94,6 +115,13 @@ cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamGetCaptureInfo(cudaStream_t st, cudaStreamCaptureStatus* status, unsigned long long* number, cudaGraph_t*,
+                                     const cudaGraphNode_t**, size_t*) {
+    const unsigned long long n = capture_of(st);
+    *status = n ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    if (n) *number = n;
+    return cudaSuccess;
+}
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
 cudaError_t cudaGetLastError() { const cudaError_t e = g_last; g_last = cudaSuccess; return e; }
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "an error"; }
@@ -128,10 +156,12 @@ static mmee_result_t found() {
 }
 
 cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader* head, Partial* partials, mmee_result_t* best,
-                          mmee_result_t* topk, cudaStream_t) {
+                          mmee_result_t* topk, cudaStream_t st) {
     ++g_searches;
     touch(head);
     touch(partials);
+    if (g_fail_launch > 0) { --g_fail_launch; return failed(cudaErrorLaunchOutOfResources); }
+    g_launches.push_back({capture_of(st), (int)shape.turn, shape.overlap, shape.hold});
     if (shape.chain_steps && shape.grid + kRecordCtas > g_resident) return failed(cudaErrorCooperativeLaunchTooLarge);
     if (shape.chain_steps && (uint64_t)shape.chunk > kMaxChunk) ++g_bad_pointers;
     for (int i = 0; i < (int)shape.chain_steps; ++i) {
@@ -151,8 +181,9 @@ cudaError_t launch_search_arrays(const Plan&, const LaunchShape& shape, Partial*
     for (uint32_t i = 0; i < shape.n_arrays; ++i) out[i] = found();
     return cudaSuccess;
 }
-cudaError_t launch_reset(SearchHeader* head, cudaStream_t) {
+cudaError_t launch_reset(SearchHeader* head, cudaStream_t st) {
     touch(head);
+    g_launches.push_back({capture_of(st), -1, 0, 0});
     return cudaGetLastError();
 }
 cudaError_t launch_dump_keys(const Plan&, int64_t*, cudaStream_t) { return cudaGetLastError(); }

@@ -132,3 +132,77 @@ def test_bytes_that_a_one_shot_call_says_it_moved(fake):
     assert fake.mmee_solve_host(*problem(), C.byref(best), topk, C.byref(h2d), C.byref(d2h)) == mm.OK
     assert fake.fake_searches() == 1 and d2h.value == 3 * mm.RESULT_BYTES
     assert fake.fake_plan_bytes() <= h2d.value < fake.fake_plan_bytes() + 512
+
+
+def launches(lib):
+    """Searches and header resets in order: (capture that records it or 0, scratch or -1 for a reset, overlap, hold)."""
+    out = []
+    v = [C.c_ulonglong()] + [C.c_int() for _ in range(3)]
+    while lib.fake_launch(len(out), *map(C.byref, v)):
+        out.append(tuple(x.value for x in v))
+    return out
+
+
+def assert_scratches_are_free(log):
+    """Among the searches that are launched, and among those that one capture records: of two with the same scratch the second
+    starts after the first has ended, because a search between them lets the next one start only after the kernel before it has
+    ended, or because it or one between them does not overlap with what is before it."""
+    for capture in {c for c, *_ in log}:
+        own = [(t, overlap, hold) for c, t, overlap, hold in log if c == capture]
+        for y, (turn, _, _) in enumerate(own):
+            for x in range(y):
+                if turn >= 0 and own[x][0] == turn:
+                    assert any(h for _, _, h in own[x + 1:y]) or not all(o for _, o, _ in own[x + 1:y + 1]), (capture, x, y)
+
+
+def searching(lib, h):
+    out = mm.Result()
+    lib.mmee_search.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
+    return lambda stream: lib.mmee_search(h, stream, C.addressof(out), None)
+
+
+EAGER, GRAPH, OTHER = 16, 32, 48        # streams
+
+
+@pytest.mark.parametrize("order", [[EAGER] * 40, [GRAPH] * 40, [EAGER, GRAPH, EAGER] * 13, [EAGER, EAGER, GRAPH] * 13,
+                                   [EAGER, GRAPH, OTHER] * 13, [GRAPH, OTHER, GRAPH, GRAPH] * 10, [EAGER, GRAPH, GRAPH, GRAPH] * 10, None])
+def test_a_scratch_is_free_when_its_turn_comes(fake, order):
+    """Searches of one handle take the scratches in turn, whether they are launched or recorded by a stream capture: what is
+    recorded is not part of the sequence of launches around it, and the other way round."""
+    import random
+    h = C.c_void_p()
+    assert fake.mmee_create(*problem(), C.byref(h)) == mm.OK
+    search = searching(fake, h)
+    fake.fake_capture(C.c_void_p(GRAPH), C.c_ulonglong(7))
+    fake.fake_capture(C.c_void_p(OTHER), C.c_ulonglong(9))
+    rng = random.Random(11)
+    for stream in order or [rng.choice((EAGER, EAGER, GRAPH, OTHER)) for _ in range(400)]:
+        assert search(stream) == mm.OK
+    log = launches(fake)
+    assert_scratches_are_free(log)
+    if order and len(set(order)) == 1:
+        assert len({t for _, t, _, _ in log}) == 5 and all(o for _, t, o, _ in log[2:] if t >= 0)      # (the first may be without)
+    fake.fake_capture(C.c_void_p(GRAPH), C.c_ulonglong(0))
+    fake.fake_capture(C.c_void_p(OTHER), C.c_ulonglong(0))
+    assert fake.mmee_destroy(h) == mm.OK and fake.fake_bad_pointers() == 0
+
+
+def test_a_header_is_clean_only_after_a_reset_that_was_launched(fake):
+    """After a launch that failed the header is reset before the next search; a reset that a capture has recorded has not
+    happened when that search is followed by one that is launched."""
+    h = C.c_void_p()
+    assert fake.mmee_create(*problem(), C.byref(h)) == mm.OK
+    search = searching(fake, h)
+    fake.fake_capture(C.c_void_p(GRAPH), C.c_ulonglong(7))
+    fake.fake_fail_launch(1)
+    assert search(EAGER) == mm.ERR_CUDA
+    n = len(launches(fake))
+    for stream in (GRAPH, GRAPH, EAGER, EAGER, GRAPH):
+        assert search(stream) == mm.OK
+    log = launches(fake)[n:]
+    kinds = [(c, t < 0) for c, t, _, _ in log]
+    assert kinds == [(7, True), (7, False), (7, True), (7, False), (0, True), (0, False), (0, False), (7, False)]
+    assert not any(o for (_, t, o, _), before in zip(log[1:], log) if t >= 0 and before[1] < 0)
+    assert_scratches_are_free(log)
+    fake.fake_capture(C.c_void_p(GRAPH), C.c_ulonglong(0))
+    assert fake.mmee_destroy(h) == mm.OK and fake.fake_bad_pointers() == 0
