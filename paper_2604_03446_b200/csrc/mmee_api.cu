@@ -246,7 +246,7 @@ int mmee_create(const mmee_workload_t* workload, const mmee_arch_t* arch, const 
     if (rc) { delete h; return rc; }
     if ((rc = cuda_status(cudaGetDevice(&h->device)))) { delete h; return rc; }
     h->kept_rows = h->plan.rows_per_tiling;
-    if (h->plan.row_pruning && (rc = set_kept_masks(&h->plan, &h->kept_rows))) { delete h; return rc; }
+    if (h->plan.row_pruning && (rc = set_kept_weights(&h->plan, &h->kept_rows))) { delete h; return rc; }
     rc = choose_launch_shape(h->plan, h->device, 0, 0, &h->shape);
     if (rc) { delete h; return rc; }
     if ((rc = workspace_acquire(h->device, &h->ws))) { delete h; return rc; }

@@ -57,10 +57,9 @@ enum OrderFlag {
     kLaboveE1 = 128, kLaboveE2 = 256  // l2 above the lower / upper own loop of E
 };
 // Rows kept by symbolic pruning, by classes (every kept row is the first of its class combination).
-struct alignas(4) KeptMasks {
+struct KeptMasks {
     uint16_t fused[kMaxOrders][3][9];         // [order slot][class of C][3 * class of A + class of B]: bit 4 * d + e
     uint16_t unfused[2][kMaxOrders][9];       // [unfused mode][order slot][3 * a + b]: bit 3 * d + e (L3, L4 merged)
-    uint32_t weights[158];                    // the same as CountWeights, four bits each (at most two modes of six orders)
 };
 
 // Where a tiling's count keeps rows with D and E of classes d, e (0: L3, 1..3), by their size slots (CountWeights): 4 * x + y both
@@ -107,7 +106,7 @@ struct Plan {
     double   quantum_pj;
     QueryTables q;
     OrderInfo order[kMaxOrders];  // by order slot
-    KeptMasks kept;               // row pruning only
+    alignas(16) uint32_t kept_weights[160];   // row pruning only: the kept rows as CountWeights, four bits each
     uint32_t divs[4][MMEE_MAX_DIVISORS];
 };
 
@@ -116,8 +115,9 @@ int build_plan(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_object
 void build_query_tables(QueryTables* q);
 
 // Tie-safe symbolic row pruning (mmee_prune.cu): keep[row] = 1 for the rows of a tiling that are evaluated; the number
-// of them; and their class masks in plan->kept (a plan with row_pruning).
+// of them; the same by classes; and what the search counts with, in plan->kept_weights (a plan with row_pruning).
 void row_pruning_keep(const Plan& plan, uint8_t* keep, uint32_t* kept_rows);
-int set_kept_masks(Plan* plan, uint32_t* kept_rows);
+int find_kept_masks(const Plan& plan, KeptMasks* masks, uint32_t* kept_rows);
+int set_kept_weights(Plan* plan, uint32_t* kept_rows);
 
 }  // namespace mmee

@@ -155,18 +155,18 @@ void row_pruning_keep(const Plan& p, uint8_t* out, uint32_t* kept_rows) {
 
 // The kept rows as masks over classes of levels.  A row that is not the first of its class combination has equal
 // buffer needs and DRAM words as that first row and a higher index, so it is never kept; MMEE_ERR_CHECK if it were.
-static int find_kept_masks(Plan* p, uint32_t* kept_rows) {
-    std::vector<uint8_t> keep(p->rows_per_tiling);
-    row_pruning_keep(*p, keep.data(), kept_rows);
-    std::memset(&p->kept, 0, sizeof(p->kept));
-    for (uint32_t row = 0; row < p->rows_per_tiling; ++row) {
+int find_kept_masks(const Plan& p, KeptMasks* masks, uint32_t* kept_rows) {
+    std::vector<uint8_t> keep(p.rows_per_tiling);
+    row_pruning_keep(p, keep.data(), kept_rows);
+    *masks = {};
+    for (uint32_t row = 0; row < p.rows_per_tiling; ++row) {
         if (!keep[row]) continue;
         const uint32_t task = row / 125u, mid = row % 125u / 25u, de = row % 25u;
-        const bool fused = task < p->fused_tasks;
-        const uint32_t u = fused ? task : task - p->fused_tasks, per = fused ? 25u : 5u;
-        const uint32_t block = fused ? u / per : p->n_fused_blocks + u / per;
-        const uint32_t slot = p->block_order_slot[block];
-        const OrderInfo& o = p->order[slot];
+        const bool fused = task < p.fused_tasks;
+        const uint32_t u = fused ? task : task - p.fused_tasks, per = fused ? 25u : 5u;
+        const uint32_t block = fused ? u / per : p.n_fused_blocks + u / per;
+        const uint32_t slot = p.block_order_slot[block];
+        const OrderInfo& o = p.order[slot];
         const uint32_t lv[5] = {fused ? u % 25u / 5u : u % 5u, fused ? u % 5u : mid, fused ? mid : 0u, de / 5u, de % 5u};
         uint32_t cls[5];
         for (int x = 0; x < 5; ++x) {
@@ -176,51 +176,60 @@ static int find_kept_masks(Plan* p, uint32_t* kept_rows) {
             cls[x] = (uint32_t)c;
         }
         if (fused) {
-            p->kept.fused[slot][cls[OP_C]][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (4 * cls[OP_D] + cls[OP_E]));
+            masks->fused[slot][cls[OP_C]][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (4 * cls[OP_D] + cls[OP_E]));
         } else {
             // an unfused nest knows no retained operands: L3 and the class from L4 on are one class of D and of E
             if (cls[OP_D] == 1 || cls[OP_E] == 1) return MMEE_ERR_CHECK;
             const uint32_t d = cls[OP_D] ? cls[OP_D] - 1 : 0, e = cls[OP_E] ? cls[OP_E] - 1 : 0;
-            p->kept.unfused[p->block_phi[block] - 1][slot][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (3 * d + e));
-        }
-    }
-    // the kept rows as weights of a tiling's count: [3 * a + b][size slot of C, or 4 for an unfused mode][choice of D and E]
-    static_assert(9 * 5 * kCountChoices <= 8 * sizeof(p->kept.weights) / 4, "four bits each");
-    for (uint32_t slot = 0; slot < p->n_orders; ++slot) {
-        const OrderInfo& o = p->order[slot];
-        const int d_lo = o.size_d_lo - S_lj, e_lo = o.size_e_lo - S_ij;
-        auto add = [&](int ab, int c, int de) {
-            const int at = (ab * 5 + c) * kCountChoices + de;
-            p->kept.weights[at / 8] += 1u << (4 * (at % 8));
-        };
-        for (int ab = 0; ab < 9; ++ab) {
-            for (int c = 0; c < 3; ++c)
-                for (int de = 0; de < 16; ++de)
-                    if (p->kept.fused[slot][c][ab] >> de & 1) add(ab, o.size_c[c] - S_il, de_choice(de / 4, de % 4, d_lo, e_lo));
-            for (int mode = 0; mode < 2; ++mode)
-                for (int de = 0; de < 9; ++de)
-                    if (p->kept.unfused[mode][slot][ab] >> de & 1) add(ab, 4, de_choice(de / 3 + 1, de % 3 + 1, d_lo, e_lo));
+            masks->unfused[p.block_phi[block] - 1][slot][3 * cls[OP_A] + cls[OP_B]] |= (uint16_t)(1u << (3 * d + e));
         }
     }
     return MMEE_OK;
 }
 
-// The masks depend on the orders and the fusion modes alone, not on the problem: like the paper's offline pruning they are
+// The same as weights of a tiling's count, [3 * a + b][size slot of C, or 4 for an unfused mode][choice of D and E]: at most twelve
+// rows (two modes of six orders) have one.
+static int find_kept_weights(Plan* p, uint32_t* kept_rows) {
+    KeptMasks masks;
+    const int rc = find_kept_masks(*p, &masks, kept_rows);
+    if (rc) return rc;
+    std::memset(p->kept_weights, 0, sizeof(p->kept_weights));
+    static_assert(9 * 5 * kCountChoices <= 8 * sizeof(p->kept_weights) / 4, "four bits each");
+    for (uint32_t slot = 0; slot < p->n_orders; ++slot) {
+        const OrderInfo& o = p->order[slot];
+        const int d_lo = o.size_d_lo - S_lj, e_lo = o.size_e_lo - S_ij;
+        auto add = [&](int ab, int c, int de) {
+            const int at = (ab * 5 + c) * kCountChoices + de;
+            p->kept_weights[at / 8] += 1u << (4 * (at % 8));
+        };
+        for (int ab = 0; ab < 9; ++ab) {
+            for (int c = 0; c < 3; ++c)
+                for (int de = 0; de < 16; ++de)
+                    if (masks.fused[slot][c][ab] >> de & 1) add(ab, o.size_c[c] - S_il, de_choice(de / 4, de % 4, d_lo, e_lo));
+            for (int mode = 0; mode < 2; ++mode)
+                for (int de = 0; de < 9; ++de)
+                    if (masks.unfused[mode][slot][ab] >> de & 1) add(ab, 4, de_choice(de / 3 + 1, de % 3 + 1, d_lo, e_lo));
+        }
+    }
+    return MMEE_OK;
+}
+
+// They depend on the orders and the fusion modes alone, not on the problem: like the paper's offline pruning they are
 // found once for each of the 14 choices (13 ms of host time) and kept.
-int set_kept_masks(Plan* p, uint32_t* kept_rows) {
+int set_kept_weights(Plan* p, uint32_t* kept_rows) {
     struct Entry {
         std::once_flag once;
         int status = MMEE_OK;
         uint32_t rows = 0;
-        KeptMasks masks = {};
+        uint32_t weights[sizeof(Plan::kept_weights) / 4] = {};
     };
     static Entry entries[2][8];
     Entry& e = entries[p->n_orders == kMaxOrders ? 1 : 0][p->fuse_mask & 7u];
     std::call_once(e.once, [&] {
-        e.status = find_kept_masks(p, &e.rows);
-        e.masks = p->kept;
+        e.status = find_kept_weights(p, &e.rows);
+        std::memcpy(e.weights, p->kept_weights, sizeof(e.weights));
     });
-    p->kept = e.masks;
+    std::memcpy(p->kept_weights, e.weights, sizeof(e.weights));
     *kept_rows = e.rows;
     return e.status;
 }

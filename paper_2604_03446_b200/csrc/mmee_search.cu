@@ -433,7 +433,16 @@ __device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uin
 __device__ __forceinline__ void start_weights(const Plan& p, Shared& sh) {
     constexpr int kWords = sizeof(CountWeights) / 4;
     if (p.row_pruning) {
-        for (int i = threadIdx.x; i < kWords; i += kSearchThreads) (&sh.weights.w[0][0][0])[i] = p.kept.weights[i / 8] >> (4 * (i % 8)) & 15u;
+        // (a warp's 32 weights are one 16-byte word of the parameters: lanes that read different words there wait for one another)
+        const uint4* packed = reinterpret_cast<const uint4*>(p.kept_weights);
+#pragma unroll
+        for (int j = 0; j < (kWords + kSearchThreads - 1) / kSearchThreads; ++j) {
+            const int i = (int)threadIdx.x + j * kSearchThreads;
+            if (i >= kWords) break;
+            const uint4 v = packed[i / 32];
+            const uint32_t lo = i & 8 ? v.y : v.x, hi = i & 8 ? v.w : v.z;
+            (&sh.weights.w[0][0][0])[i] = (i & 16 ? hi : lo) >> (4 * (i & 7)) & 15u;
+        }
         return;
     }
     const int4* from = reinterpret_cast<const int4*>(&kCountWeights[p.n_orders == kMaxOrders ? 1 : 0]);

@@ -22,7 +22,8 @@ extern "C" int host_classes(const mmee_workload_t* w, const mmee_arch_t* a, cons
     Plan p;
     uint32_t kept;
     int rc = build_plan(w, a, o, &p);
-    if (rc || (rc = set_kept_masks(&p, &kept))) return rc;
+    KeptMasks masks;
+    if (rc || (rc = find_kept_masks(p, &masks, &kept))) return rc;
     TileTab tb = {};
     for (int d = 3; d >= 0; --d) {
         const uint32_t g = p.divs[d][t % p.ndiv[d]];
@@ -47,7 +48,7 @@ extern "C" int host_classes(const mmee_workload_t* w, const mmee_arch_t* a, cons
         fused_class<false, false>(tb, oi, dw, c, cap, nullptr, any, rows, out[c][6], unused);
         out[c][5] = rows;
         int64_t x;
-        fused_class<true, false>(tb, oi, dw, c, cap, p.kept.fused[slot][c], any, rows, x, unused);
+        fused_class<true, false>(tb, oi, dw, c, cap, masks.fused[slot][c], any, rows, x, unused);
         out[c][7] = rows;
         if (x != out[c][6]) return MMEE_ERR_CHECK;
     }
@@ -63,6 +64,6 @@ extern "C" int host_classes(const mmee_workload_t* w, const mmee_arch_t* a, cons
     unfused_nests<true, false>(tb, oi, dw, cap, fit1, fit2, rows, x1, x2, unused);
     out[3][7] = 0;
     for (int ab = 0; ab < 9; ++ab)
-        if ((fit1 >> ab) & 1u) out[3][7] += __builtin_popcount(fit2 & p.kept.unfused[0][slot][ab]);
+        if ((fit1 >> ab) & 1u) out[3][7] += __builtin_popcount(fit2 & masks.unfused[0][slot][ab]);
     return x1 == out[3][3] && x2 == out[3][6] ? MMEE_OK : MMEE_ERR_CHECK;
 }

@@ -9,10 +9,11 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
     Plan p;
     uint32_t n_kept;
     int rc = build_plan(w, a, o, &p);
-    if (rc || (rc = set_kept_masks(&p, &n_kept))) return rc;
+    KeptMasks masks;
+    if (rc || (rc = find_kept_masks(p, &masks, &n_kept)) || (rc = set_kept_weights(&p, &n_kept))) return rc;
     const CountWeights all = count_weights((int)p.n_orders);
     CountWeights kept = {};
-    for (int i = 0; i < (int)(sizeof(kept) / 4); ++i) (&kept.w[0][0][0])[i] = p.kept.weights[i / 8] >> (4 * (i % 8)) & 15u;
+    for (int i = 0; i < (int)(sizeof(kept) / 4); ++i) (&kept.w[0][0][0])[i] = p.kept_weights[i / 8] >> (4 * (i % 8)) & 15u;
     const int64_t I = p.dim[0], K = p.dim[1], L = p.dim[2], J = p.dim[3];
     const DimWords dw = {I * K, K * L, L * J, I * J, I * L};
     const int cap = (int)p.cap_words;
@@ -45,7 +46,7 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
                 if (x != y || (x < kNoRow && need != need2)) return MMEE_ERR_CHECK;
                 fused_words<false>(tb, p.order[s], dw, c, cap, any, y, need2);
                 if (x != y) return MMEE_ERR_CHECK;
-                fused_class<true, false>(tb, p.order[s], dw, c, cap, p.kept.fused[s][c], any, n, x, need);
+                fused_class<true, false>(tb, p.order[s], dw, c, cap, masks.fused[s][c], any, n, x, need);
                 want_kept += n;
             }
             if (!modes) continue;
@@ -58,7 +59,7 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
             unfused_nests<true, false>(tb, p.order[s], dw, cap, fit1, fit2, n, x, x2, need);
             for (uint32_t phi = 1; phi <= 2; ++phi)
                 for (int ab = 0; ab < 9 && ((p.fuse_mask >> phi) & 1u); ++ab)
-                    if ((fit1 >> ab) & 1u) want_kept += (uint64_t)__builtin_popcount(fit2 & p.kept.unfused[phi - 1][s][ab]);
+                    if ((fit1 >> ab) & 1u) want_kept += (uint64_t)__builtin_popcount(fit2 & masks.unfused[phi - 1][s][ab]);
         }
         if (rows != want || rows_kept != want_kept) return MMEE_ERR_CHECK;
     }
