@@ -124,7 +124,7 @@ int run_chain(const Plan& plan, uint32_t polls, Take take) {
     if (rc) return rc;
     uint32_t most = 0;
     if ((rc = max_search_ctas(device, &most))) return rc;
-    most -= kRecordCtas;        // (and one that merges, in the slot that a single search leaves free)
+    most = most + 1 - kChainExtraCtas;      // (all slots: one of them a single search leaves free)
     LaunchShape shape;
     if ((rc = choose_launch_shape(plan, device, 0, 0, &shape, most))) return rc;
     Workspace* ws = nullptr;

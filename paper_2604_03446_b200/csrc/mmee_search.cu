@@ -1579,7 +1579,7 @@ cudaError_t launch_search_t(const Plan& p, const LaunchShape& shape, SearchHeade
                    : shape.chain_steps ? (chain_mode<OBJ>() == kModeChain ? search_kernel<OBJ, chain_mode<OBJ>()> : nullptr)
                    : p.topk > 1    ? search_kernel<OBJ, kModeMulti> : search_kernel<OBJ, kModeSingle>;
     if (!kernel) return cudaErrorInvalidValue;
-    const uint32_t grid = shape.chain_steps ? shape.grid + kRecordCtas + 1 : shape.grid;
+    const uint32_t grid = shape.chain_steps ? shape.grid + kChainExtraCtas : shape.grid;
     return launch_overlapped(shape.overlap, shape.chain_steps != 0, grid, st, kernel, p, shape, head, partials, out_best, out_topk);
 }
 

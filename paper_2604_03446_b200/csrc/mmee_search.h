@@ -77,6 +77,8 @@ struct LaunchShape {
 // one 217 us, two 202, four 205 because the searches have fewer CTAs; records after the chain 204, where a front of one point
 // takes 59 instead of 55.)
 constexpr uint32_t kRecordCtas = 2;
+// CTAs of a chain beside those that search: they make the records, and one merges what the others publish.
+constexpr uint32_t kChainExtraCtas = kRecordCtas + 1;
 // The wait for a chained search is limited, at a few seconds.  A CTA whose wait runs out leaves without a trace: it takes no
 // part in later searches, which then do not end, and makes no more records, so that the caller finds one that was not made.
 constexpr uint32_t kChainPolls = 1u << 22;

@@ -5,6 +5,7 @@
 
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <vector>
 
@@ -25,8 +26,12 @@ int g_searches = 0;                             // search launches
 unsigned g_missing = 0;                         // bit i: the record of its search i is not made
 std::map<cudaStream_t, unsigned long long> g_captures;      // streams that are capturing: the capture's number
 int g_fail_launch = 0;                          // fail that many search launches
+int g_late = 0;                                 // that many searches end only when the host waits for their stream
+int g_fail_sync = 0;                            // fail that many waits for a stream
+int g_syncs = 0;                                // waits for a stream
 struct Launch { unsigned long long capture; int turn, overlap, hold; };       // turn -1: a reset of the header
 std::vector<Launch> g_launches;
+std::function<void()> g_pending;                // the end of a search that is late
 
 unsigned long long capture_of(cudaStream_t st) {
     auto it = g_captures.find(st);
@@ -95,6 +100,8 @@ void fake_capture(void* stream, unsigned long long number) {         // 0: ends
     else g_captures.erase(static_cast<cudaStream_t>(stream));
 }
 void fake_fail_launch(int n) { g_fail_launch = n; }
+void fake_late(int searches, int failing_syncs) { g_late = searches; g_fail_sync = failing_syncs; }
+int fake_syncs() { return g_syncs; }
 // Launch number i of searches and resets; false: there are no more.
 int fake_launch(int i, unsigned long long* capture, int* turn, int* overlap, int* hold) {
     if (i >= (int)g_launches.size()) return 0;
@@ -114,7 +121,13 @@ extern "C" {
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+    ++g_syncs;
+    if (g_fail_sync > 0) { --g_fail_sync; return failed(cudaErrorLaunchFailure); }
+    if (g_pending) g_pending();
+    g_pending = nullptr;
+    return cudaSuccess;
+}
 cudaError_t cudaStreamGetCaptureInfo(cudaStream_t st, cudaStreamCaptureStatus* status, unsigned long long* number, cudaGraph_t*,
                                      const cudaGraphNode_t**, size_t*) {
     const unsigned long long n = capture_of(st);
@@ -162,7 +175,7 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
     touch(partials);
     if (g_fail_launch > 0) { --g_fail_launch; return failed(cudaErrorLaunchOutOfResources); }
     g_launches.push_back({capture_of(st), (int)shape.turn, shape.overlap, shape.hold});
-    if (shape.chain_steps && shape.grid + kRecordCtas > g_resident) return failed(cudaErrorCooperativeLaunchTooLarge);
+    if (shape.chain_steps && shape.grid + kChainExtraCtas > g_resident) return failed(cudaErrorCooperativeLaunchTooLarge);
     if (shape.chain_steps && (uint64_t)shape.chunk > kMaxChunk) ++g_bad_pointers;
     for (int i = 0; i < (int)shape.chain_steps; ++i) {
         mmee_result_t r = found();
@@ -172,8 +185,18 @@ cudaError_t launch_search(const Plan& p, const LaunchShape& shape, SearchHeader*
         if (!(g_missing >> i & 1u)) topk[i] = r;
         if (i >= g_points) return cudaSuccess;
     }
-    if (find(best)) *best = found();
-    for (uint32_t i = 0; topk && find(topk) && i < p.topk; ++i) topk[i] = found();
+    auto end = [k = p.topk, shape, best, topk] {
+        if (find(best)) *best = found();
+        for (uint32_t i = 0; topk && find(topk) && i < k; ++i) topk[i] = found();
+        touch(shape.signal);
+        if (shape.signal && find(shape.signal)) *shape.signal = shape.signal_value;
+    };
+    if (g_late > 0) {
+        --g_late;
+        g_pending = end;
+    } else {
+        end();
+    }
     return cudaSuccess;
 }
 cudaError_t launch_search_arrays(const Plan&, const LaunchShape& shape, Partial* partials, mmee_result_t* out, cudaStream_t) {

@@ -91,8 +91,9 @@ def test_a_front_whose_wait_ran_out_returns_no_older_record(fake, front, missing
 
 @pytest.mark.parametrize("front", ["mmee_pareto_front", "mmee_pareto_front_bs_da"])
 def test_fronts_take_the_ctas_that_can_be_resident_together(fake, front):
-    """A context with a part of the SMs holds fewer CTAs at once than the device: the front runs on those."""
-    for resident, status in ((296, mm.OK), (295, mm.OK), (64, mm.OK), (3, mm.OK), (2, mm.ERR_CUDA), (1000, mm.OK)):
+    """A context with a part of the SMs holds fewer CTAs at once than the device: the front runs on those, from four on (one
+    that searches, one that merges, two that make the records)."""
+    for resident, status in ((296, mm.OK), (295, mm.OK), (64, mm.OK), (4, mm.OK), (3, mm.ERR_CUDA), (2, mm.ERR_CUDA), (1000, mm.OK)):
         fake.fake_resident(resident)
         fake.fake_chain(3, 0)
         pts, n = (mm.Result * 8)(), C.c_uint32()
@@ -206,3 +207,28 @@ def test_a_header_is_clean_only_after_a_reset_that_was_launched(fake):
     assert_scratches_are_free(log)
     fake.fake_capture(C.c_void_p(GRAPH), C.c_ulonglong(0))
     assert fake.mmee_destroy(h) == mm.OK and fake.fake_bad_pointers() == 0
+
+
+def test_records_are_taken_when_their_signal_comes_or_the_stream_has_ended(fake):
+    """A call with host records returns when the search's word is in host memory; where that does not come in time it waits for
+    the stream, and a wait that fails is the call's status.  With kernel timing on it waits for the stream at once."""
+    h = C.c_void_p()
+    assert fake.mmee_create(*problem(), C.byref(h)) == mm.OK
+    fake.mmee_search_host.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p]
+    fake.mmee_kernel_timing.argtypes = [C.c_void_p, C.c_int]
+    best = mm.Result()
+
+    def call():
+        before, best.idx = fake.fake_syncs(), 0
+        return fake.mmee_search_host(h, C.addressof(best), None), best.idx, fake.fake_syncs() - before
+
+    for _ in range(3):
+        assert call() == (mm.OK, 7, 0)
+        fake.fake_late(1, 0)
+        assert call() == (mm.OK, 7, 1)
+    fake.fake_late(1, 1)
+    assert call() == (mm.ERR_CUDA, 0, 1)
+    fake.fake_late(0, 0)
+    assert call() == (mm.OK, 7, 0)
+    assert fake.mmee_kernel_timing(h, 1) == mm.OK and call() == (mm.OK, 7, 1)
+    assert fake.mmee_destroy(h) == mm.OK and solve(fake) == (mm.OK, 7) and fake.fake_bad_pointers() == 0
