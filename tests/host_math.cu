@@ -1,5 +1,5 @@
 // The kernels' host/device arithmetic as plain functions, for checks on the CPU (tests/test_host_math.py).
-#include "../paper_2604_03446_b200/csrc/mmee_classes.cuh"
+#include "class_forms.h"
 #include "../paper_2604_03446_b200/csrc/mmee_eval.cuh"
 
 // Words and cycles of one tile of operator `op` under stationary mode `sm`, and its register-file block.

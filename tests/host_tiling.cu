@@ -1,6 +1,6 @@
 // The search's counts and least words of whole tilings beside the same by blocks and classes, for a check on the CPU
 // (tests/test_host_tiling.py).
-#include "../paper_2604_03446_b200/csrc/mmee_classes.cuh"
+#include "class_forms.h"
 
 // Every `stride`-th tiling of a problem: the rows of all its blocks that fit, all of them and (with `pruned`) the kept ones, and every
 // block's least words and needs.  Returns MMEE_OK, or MMEE_ERR_CHECK with the tiling in *at where the two differ.
