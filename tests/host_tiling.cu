@@ -2,8 +2,42 @@
 // (tests/test_host_tiling.py).
 #include "class_forms.h"
 
-// Every `stride`-th tiling of a problem: the rows of all its blocks that fit, all of them and (with `pruned`) the kept ones, and every
-// block's least words and needs.  Returns MMEE_OK, or MMEE_ERR_CHECK with the tiling in *at where the two differ.
+namespace {
+
+using namespace mmee;
+
+// Whether a tiling's bound is not above the least key of one of its items, whatever the accelerator: stationary-pair terms, energy of
+// a DRAM word, bound on the other key and offered pairs drawn from `seed`.  (x1 + x2: an unfused block.)
+template <int OBJ>
+bool bound_holds(const DimWords& dw, int64_t x1, int64_t x2, bool fused, int64_t rho, uint64_t seed) {
+    auto next = [&](uint64_t n) {
+        seed = seed * 6364136223846793005ull + 1442695040888963407ull;
+        return (int64_t)((seed >> 33) % n);
+    };
+    const int64_t scale = (int64_t)1 << next(24);
+    StatTerms st;
+    for (int i = 0; i < 3; ++i) { st.P1[i] = next(scale); st.P2[i] = next(scale); st.Q1[i] = next(scale); st.Q2[i] = next(scale); }
+    const int64_t c_dram = next(4) ? next(300) : 0, pass = fused || next(2) ? 0 : 2 * dw.il;
+    const uint32_t mask = next(2) ? 0x1ffu : (uint32_t)(1 + next(511));
+    // a bound near what the item has of the other key, so that it decides
+    const int64_t other = OBJ == MMEE_OBJ_ENERGY_LCAP ? x1 + x2 + st.Q1[0] : c_dram * (x1 + x2) + st.P1[0];
+    const int64_t cap = next(3) ? other * next(200) / 100 : INT64_MAX - 1;
+    const int64_t least = tile_least_key<OBJ>(st, dw, c_dram, cap);
+    const int64_t key = fused ? fused_least_key<OBJ>(st, x1, rho, mask, c_dram, cap)
+                              : unfused_least_key<OBJ>(st, x1, x2, pass, mask, c_dram, cap);
+    return least <= key;
+}
+bool bounds_hold(const DimWords& dw, int64_t x1, int64_t x2, bool fused, int64_t rho, uint64_t seed) {
+    return bound_holds<MMEE_OBJ_ENERGY>(dw, x1, x2, fused, rho, seed) && bound_holds<MMEE_OBJ_LATENCY>(dw, x1, x2, fused, rho, seed + 1) &&
+           bound_holds<MMEE_OBJ_EDP>(dw, x1, x2, fused, rho, seed + 2) && bound_holds<MMEE_OBJ_ENERGY_LCAP>(dw, x1, x2, fused, rho, seed + 3) &&
+           bound_holds<MMEE_OBJ_LATENCY_ECAP>(dw, x1, x2, fused, rho, seed + 4);
+}
+
+}  // namespace
+
+// Every `stride`-th tiling of a problem: the rows of all its blocks that fit, all of them and the kept ones, every block's least words
+// and needs, and the tiling's bounds on keys and needs.  Returns MMEE_OK, or MMEE_ERR_CHECK with the tiling in *at where two of them
+// differ or a bound is above what it bounds.
 extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, const mmee_objective_t* o, uint32_t stride, uint64_t* at) {
     using namespace mmee;
     Plan p;
@@ -30,6 +64,9 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
         }
         for (int i = 0; i < kSizeSlots; ++i) tb.size[i] = sat_size(size_words(p.dim, tb.b + 4, i));
         uint64_t rows = 0, rows_kept = 0, want = 0, want_kept = 0;
+        // (no row needs less buffer: every operand at L3)
+        const int one = sat_add(tb.size[S_ik], tb.size[S_kl]), two = sat_add(tb.size[S_lj], tb.size[S_ij]);
+        const int least_need = sat_add(tb.size[S_il], one > two ? one : two);
         const int c0 = (p.fuse_mask & 1u) ? 0 : 4, c1 = modes ? 5 : 4;
         for (int ab = 0; ab < 9; ++ab) {
             rows += count_rows(tb.size, ab, c0, c1, modes, cap, all, any);
@@ -44,6 +81,9 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
                 want += n;
                 fused_words<true>(tb, p.order[s], dw, c, cap, any, y, need2);
                 if (x != y || (x < kNoRow && need != need2)) return MMEE_ERR_CHECK;
+                if (x < kNoRow && (need < least_need ||
+                                   !bounds_hold(dw, x, 0, true, p.order[s].recompute[c] ? tb.b[LOOP_J] : 1, tiling * 97 + s * 3 + c)))
+                    return MMEE_ERR_CHECK;
                 fused_words<false>(tb, p.order[s], dw, c, cap, any, y, need2);
                 if (x != y) return MMEE_ERR_CHECK;
                 fused_class<true, false>(tb, p.order[s], dw, c, cap, masks.fused[s][c], any, n, x, need);
@@ -54,6 +94,7 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
             want += (uint64_t)n * modes;
             unfused_words<true>(tb, p.order[s], dw, cap, y, y2, need2);
             if (x != y || x2 != y2 || (x < kNoRow && need != need2)) return MMEE_ERR_CHECK;
+            if (x < kNoRow && (need < least_need || !bounds_hold(dw, x, x2, false, 1, tiling * 97 + s * 3 + 50))) return MMEE_ERR_CHECK;
             unfused_words<false>(tb, p.order[s], dw, cap, y, y2, need2);
             if (x != y || x2 != y2) return MMEE_ERR_CHECK;
             unfused_nests<true, false>(tb, p.order[s], dw, cap, fit1, fit2, n, x, x2, need);

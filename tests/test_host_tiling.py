@@ -1,5 +1,5 @@
-"""How the search counts a tiling's rows and finds its blocks' least words, compiled for the CPU, against the same by blocks and
-classes of levels, which test_host_math.py checks against the oracle's rows."""
+"""How the search counts a tiling's rows, finds its blocks' least words and bounds its keys, compiled for the CPU, against the same
+by blocks and classes of levels, which test_host_math.py checks against the oracle's rows."""
 import ctypes as C
 import os
 import subprocess
