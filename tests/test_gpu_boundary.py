@@ -580,3 +580,113 @@ def test_fronts_in_a_context_with_a_part_of_the_sms():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", PART_SCRIPT], cwd=root, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0 and "same records" in r.stdout, r.stdout + r.stderr
+
+
+def _raw(buf):
+    return buf.cpu().numpy().tobytes()
+
+
+def _problems_that_follow():
+    """Searches of one CTA and of all, with lists of one and of sixteen, each with its records found by a search of its own, the small
+    one's checked against the oracle (the large one's answers are the stored ones of test_gpu_parity)."""
+    out = []
+    small, large = mi.random_tiny_problem(3), mi.config4()
+    for cfg, k in ((small, 1), (small, 16), (large, 1), (large, 16)):
+        obj = dict(cfg["searches"][0], topk=k)
+        if cfg is small:
+            obj = shrink_to(cfg, obj, 2_000_000)
+        best, top = mm.result_buffer(1), mm.result_buffer(k)
+        with Handle(cfg, obj) as h:
+            mm.mmee_search(h, best, top)
+            torch.cuda.synchronize()
+        if cfg is small:
+            want = oracle.search(oracle.make_problem(cfg["workload"], cfg["arch"], obj))
+            assert [r.idx for r in mm.read_results(top, k) if r.idx != mm.NO_INDEX] == [r.idx for r in want.topk]
+        out.append((cfg, obj, (_raw(best), _raw(top))))
+    return out
+
+
+def test_many_searches_in_a_row_into_buffers_of_their_own():
+    """More searches one after the other than a handle has scratches, with nothing between them, on one handle and on two in
+    alternation: every one's records."""
+    jobs = _problems_that_follow()
+    for pair in [[j] for j in jobs] + [[jobs[0], jobs[2]], [jobs[1], jobs[3]], [jobs[1], jobs[2]], [jobs[0], jobs[0]]]:
+        handles = [mm.mmee_create(c["workload"], c["arch"], o) for c, o, _ in pair]
+        runs = [(i % len(pair), mm.result_buffer(1), mm.result_buffer(pair[i % len(pair)][1]["topk"])) for i in range(24)]
+        torch.cuda.synchronize()
+        for _ in range(10):
+            for i, b, t in runs:
+                b.zero_()
+                t.zero_()
+            for i, b, t in runs:
+                mm.mmee_search(handles[i], b, t)
+            torch.cuda.synchronize()
+            for n, (i, b, t) in enumerate(runs):
+                assert (_raw(b), _raw(t)) == pair[i][2], n
+        for h in handles:
+            mm.mmee_destroy(h)
+
+
+def test_captured_searches_among_launched_ones():
+    """Searches of one handle on a stream, behind other work, while another stream's capture records searches of the same handle in
+    between: the launched ones' records, then those of the captured graph, launched several times."""
+    eager, side = torch.cuda.Stream(), torch.cuda.Stream()
+    for cfg, obj, want in _problems_that_follow()[:3]:
+        h = mm.mmee_create(cfg["workload"], cfg["arch"], obj)
+        outs = [[(mm.result_buffer(1), mm.result_buffer(obj["topk"])) for _ in range(24)] for _ in range(2)]
+        launched, captured = [], []
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(eager):
+            torch.cuda._sleep(2_000_000)                # about a millisecond
+        with torch.cuda.stream(side):
+            graph.capture_begin(capture_error_mode="relaxed")
+        for turn, n in enumerate((2, 1, 3, 2, 1, 1, 4, 3, 2, 5, 6, 6)):
+            for _ in range(n):
+                done, stream, left = (captured, side, outs[1]) if turn % 2 else (launched, eager, outs[0])
+                b, t = left[len(done)]
+                mm.mmee_search(h, b, t, stream=stream)
+                done.append((b, t))
+        with torch.cuda.stream(side):
+            graph.capture_end()
+        torch.cuda.synchronize()
+        assert all((_raw(b), _raw(t)) == want for b, t in launched)
+        for _ in range(3):
+            for b, t in captured:
+                b.zero_()
+                t.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all((_raw(b), _raw(t)) == want for b, t in captured)
+        for b, t in launched:
+            b.zero_()
+            t.zero_()
+        graph.replay()
+        for b, t in launched:
+            mm.mmee_search(h, b, t)
+        torch.cuda.synchronize()
+        assert all((_raw(b), _raw(t)) == want for b, t in launched + captured)
+        del graph
+        mm.mmee_destroy(h)
+
+
+def test_handles_that_take_over_the_workspace_of_a_call_with_host_records():
+    """A call with host records returns before its kernel has ended, and its handle may be released: the next handle takes the same
+    workspace and searches on another stream at once."""
+    jobs = _problems_that_follow()[:3]
+    stream = torch.cuda.Stream()
+    outs = [(mm.result_buffer(1), mm.result_buffer(jobs[n % 3][1]["topk"])) for n in range(60)]
+    torch.cuda.synchronize()
+    for n, (b, t) in enumerate(outs):
+        cfg, obj, want = jobs[n % 3]
+        mm.mmee_solve_host(*[(jobs[(n + 1) % 3][0][key]) for key in ("workload", "arch")], jobs[(n + 1) % 3][1])
+        h = mm.mmee_create(cfg["workload"], cfg["arch"], obj)
+        best, top = mm.mmee_search_host(h, want_topk=True, topk=obj["topk"])
+        assert (bytes(best), b"".join(bytes(r) for r in top)) == want
+        mm.mmee_destroy(h)
+        h = mm.mmee_create(cfg["workload"], cfg["arch"], obj)
+        for _ in range(5):
+            mm.mmee_search(h, b, t, stream=stream)
+        stream.synchronize()
+        mm.mmee_destroy(h)
+        assert (_raw(b), _raw(t)) == want

@@ -699,3 +699,37 @@ def test_energy_latency_front_equals_alternating_capped_searches(dims, pe, gb_by
         cap = r.l_key - 1
     got = [bytes(r) for r in mm.mmee_pareto_front(w, arch, base, 4096)]
     assert got == want and len(want) == points
+
+
+@pytest.mark.parametrize("order_set,fuse_mask,tilings,objective,least_live", [
+    (mi.ORD_NORECOMP2, mi.FUSE_ALL, (4000, 13000), mi.OBJ_ENERGY, 24),
+    (mi.ORD_ALL6, mi.FUSE_SEPARATE, (3000, 16500), mi.OBJ_LATENCY, 40)])
+def test_several_tilings_to_a_warp_best_first(order_set, fuse_mask, tilings, objective, least_live):
+    """Three and five tilings to a warp's lanes, and more of them per CTA than its warps evaluate at once, so that the most promising
+    go first and the others only where their bound may enter: the sixteen best and the best one of a range, every record the
+    oracle's; and the best one among the rows that pruning keeps."""
+    cfg = dict(name="per_warp", workload=mi.workload(1, 1, 1, 240, 240, 24, 12, 1),
+               arch=mi.arch(4, 8, 1, 8000, 0, 3, 50.0, 6.0, 1.0, 1.0))
+    obj = mi.objective(objective, 16, order_set=order_set, fuse_mask=fuse_mask)
+    obj.update(t_begin=tilings[0], t_end=tilings[1])
+    best, found = check_search(cfg, obj)
+    one, _, stats = gpu_search(cfg, dict(obj, topk=1))
+    assert_same_record(one, best)
+    assert one.n_feasible == best.n_feasible and stats.grid * least_live < tilings[1] - tilings[0]
+    pruned, _, _ = gpu_search(cfg, dict(obj, topk=1, row_pruning=1))
+    assert_same_record(pruned, best)
+
+
+@pytest.mark.parametrize("objective", [mi.OBJ_ENERGY, mi.OBJ_EDP])
+def test_one_optimum_over_several_passes_equals_the_best_of_its_parts(objective):
+    """63 504 tilings, two passes of every CTA: the optimum and the number of mappings that fit are those of three parts, each within
+    one pass, with all rows and with the kept ones."""
+    cfg = [c for c in mi.beyond_attention_configs() if c["name"] == "conv_chain_cc1"][0]
+    for pruning in (0, 1):
+        obj = dict(cfg["searches"][0], objective=objective, topk=1, row_pruning=pruning)
+        whole, _, _ = gpu_search(cfg, obj)
+        parts = [gpu_search(cfg, dict(obj, t_begin=lo, t_end=hi))[0] for lo, hi in ((0, 11111), (11111, 40000), (40000, 63504))]
+        key = lambda r: (r.edp_key if objective == mi.OBJ_EDP else r.e_key, r.idx)
+        assert whole.n_feasible == sum(r.n_feasible for r in parts)
+        assert_same_record(whole, min((r for r in parts if r.idx != mm.NO_INDEX), key=key))
+        assert_same_record(whole, oracle.evaluate(oracle.make_problem(cfg["workload"], cfg["arch"], obj), whole.idx))
