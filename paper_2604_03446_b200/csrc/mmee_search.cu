@@ -1300,26 +1300,26 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
                 for (uint32_t i = (uint32_t)warp * per; i < n_tiles; i += per * (uint32_t)kWarps)
                     evaluate(i + sub < n_tiles ? i + sub : i, sub < per && i + sub < n_tiles);
             } else if (!m0 && (MULTI || warp < kWarps / 2)) {
-                const uint32_t first = (uint32_t)warp, every = MULTI ? (uint32_t)kWarps : (uint32_t)kWarps / 2u;
+                // (by the bound as a float, then by the index: where many bounds are the same, as those of the latency often are, the
+                // lowest index is the best; which come first changes no result)
+                const uint32_t every = MULTI ? (uint32_t)kWarps : (uint32_t)kWarps / 2u, own = (uint32_t)warp + (uint32_t)lane * every;
+                uint32_t rank = 0xffffffffu, number = 0xffffffffu;
+                if (own < n_tiles) {
+                    rank = __float_as_uint(__ll2float_rn(sh.tile[own].least));
+                    number = sh.tile[own].t << 5 | (uint32_t)lane;
+                }
                 uint32_t slot = 0;
                 bool valid = false;
                 for (uint32_t i = 0; i < per; ++i) {
-                    int64_t lk = kInfKey;
-                    uint64_t li = UINT64_MAX;
-                    uint32_t mine = 0;
-                    for (uint32_t at = first + (uint32_t)lane * every; at < n_tiles; at += 32u * every) {
-                        const uint32_t s = at;
-                        const int64_t key = sh.tile[s].least;
-                        if (!sh.done[s] && pair_less(key, sh.tile[s].t, lk, li)) { lk = key; li = sh.tile[s].t; mine = s; }
+                    const uint32_t least = __reduce_min_sync(kFull, rank);
+                    const uint32_t first = __reduce_min_sync(kFull, rank == least ? number : 0xffffffffu);
+                    if (least == 0xffffffffu) break;
+                    const uint32_t src = first & 31u;
+                    if ((uint32_t)lane == src) {
+                        rank = 0xffffffffu;
+                        sh.done[own] = 1;
                     }
-                    const uint64_t own = li;
-                    warp_min_pair(lk, li);
-                    if (li == UINT64_MAX) break;
-                    const int src = __ffs(__ballot_sync(kFull, own == li)) - 1;
-                    const uint32_t s = __shfl_sync(kFull, mine, src);
-                    if (lane == 0) sh.done[s] = 1;
-                    __syncwarp();
-                    if (sub >= i) slot = s;
+                    if (sub >= i) slot = (uint32_t)warp + src * every;
                     if (sub == i) valid = true;
                 }
                 evaluate(slot, valid);
