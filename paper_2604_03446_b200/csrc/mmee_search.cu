@@ -1081,7 +1081,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             const bool valid = i < units;
             const uint32_t ab = valid ? i / n_tiles : 0u;
             const uint32_t n = count_rows(sh.tile[valid ? i - ab * n_tiles : 0u].size, (int)ab, (int)c0, (int)c1,
-                                          p.row_pruning ? 1u : unfused_modes, capc, sh.weights, [&](bool v) { return any(v && valid); });
+                                          p.row_pruning ? 1u : unfused_modes, capc, sh.weights, n_orders == 2u, [&](bool v) { return any(v && valid); });
             if (valid) my_rows += n;
         }
     };

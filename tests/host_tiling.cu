@@ -69,8 +69,8 @@ extern "C" int host_tilings(const mmee_workload_t* w, const mmee_arch_t* a, cons
         const int least_need = sat_add(tb.size[S_il], one > two ? one : two);
         const int c0 = (p.fuse_mask & 1u) ? 0 : 4, c1 = modes ? 5 : 4;
         for (int ab = 0; ab < 9; ++ab) {
-            rows += count_rows(tb.size, ab, c0, c1, modes, cap, all, any);
-            for (int c = c0; c < c1; ++c) rows_kept += count_rows(tb.size, ab, c, c + 1, 1u, cap, kept, any);
+            rows += count_rows(tb.size, ab, c0, c1, modes, cap, all, p.n_orders == 2, any);
+            for (int c = c0; c < c1; ++c) rows_kept += count_rows(tb.size, ab, c, c + 1, 1u, cap, kept, p.n_orders == 2, any);
         }
         for (uint32_t s = 0; s < p.n_orders; ++s) {
             uint32_t n, fit1, fit2;
