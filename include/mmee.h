@@ -162,7 +162,7 @@ typedef struct mmee_handle mmee_handle_t;
  * the query vectors of every (order, operand, level) (Section V-E, Section VI-A "offline"
  * enumeration), quantises the energies and bounds the largest possible key.
  *   workload, arch, objective : HOST, read only during the call.
- *   out                       : HOST, receives the handle.  The handle holds 0.16 MB of DEVICE scratch on the
+ *   out                       : HOST, receives the handle.  The handle holds 0.32 MB of DEVICE scratch on the
  *                               device that is current at the call and 11 KB of pinned host memory, taken from
  *                               the library's idle workspaces (see mmee_trim) or allocated.
  * Errors: MMEE_ERR_ARG, _OVERFLOW, _QUANTUM, _RANGE (more than MMEE_MAX_DIVISORS divisors), _CUDA.
@@ -202,7 +202,7 @@ int mmee_destroy(mmee_handle_t* handle);
 
 /*
  * mmee_trim -- free the idle workspaces.  Device scratch and pinned host memory of released handles and one-shot calls
- * stay with the library for the next handle on the same device, at most eight of them (0.16 MB of device memory and
+ * stay with the library for the next handle on the same device, at most eight of them (0.32 MB of device memory and
  * 11 KB of pinned host memory each); no two handles or calls share one.  Handles in use are not affected.  A kept workspace
  * belongs to the CUDA context it was made in and is dropped when that has ended (cudaDeviceReset): no call is needed before
  * a reset, but handles must not be used after it, only destroyed.

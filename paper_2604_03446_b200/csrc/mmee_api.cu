@@ -47,10 +47,11 @@ int cuda_status(cudaError_t e) {
     return MMEE_ERR_CUDA;
 }
 
-// Two CTAs per SM (118 registers a thread, no spills) beat three (80, spilled) and four (64): GQA latency 13.0, 13.7 and
-// 15.1 us, BERT energy 9.4, 10.4 and 12.6, convolution chain top-16 52, 58 and 65.  One slot is left free: a search that follows another starts while that one's
-// last CTA finalizes, and a CTA that had to wait for its slot would begin its work only then (BERT energy, one search
-// after the other: 16.4 us with all slots taken, 11.6 us with one left; GQA latency 20.1 and 13.7).
+// Two CTAs per SM (108 to 128 registers a thread, no spills) beat three (80, spilled) and four (64); when the items still counted
+// their rows: GQA latency 13.0, 13.7 and 15.1 us, BERT energy 9.4, 10.4 and 12.6, convolution chain top-16 52, 58 and 65.  One slot
+// is left free: a search that follows another starts while that one's last CTA finalizes, and a CTA that had to wait for its slot
+// would begin its work only then (BERT energy, one search after the other: 16.4 us with all slots taken, 11.6 us with one left; GQA
+// latency 20.1 and 13.7).
 int max_search_ctas(int device, uint32_t* out) {
     int sm_count = 0;      // attribute query: cudaGetDeviceProperties costs milliseconds
     const cudaError_t e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device);

@@ -1193,7 +1193,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             const uint32_t n_tiles = sh.n_live;
             if (tid == 0) my_live += n_tiles;
 
-            // ---- the least keys: first of the tilings whose least_of is smallest among a warp's own, by half of the warps for a single
+            // ---- the least keys: first of the tilings whose bound (tile_least_key) is smallest among a warp's own, by half of the warps for a single
             // optimum (the others count meanwhile), by all for the k best
             const bool all_at_once = ARRAYS || CHAIN || n_tiles <= per * (uint32_t)kWarps;
             if (CHAIN) {
