@@ -42,8 +42,8 @@ ALG_OPS_PER_ROW = {0: 2.0, 1: 2.0, 2: 2.0}
 LANES_PER_SM = 64          # 4 sub-partitions x 16 lanes: width of the integer-ALU pipe, the busiest pipe of these kernels
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, recorded from the ncu captures summarised under
 # profiles/ (not measured in this run); workload -> objective -> bytes.  None where no capture backs it.
-NCU_DRAM_BYTES_PER_LAUNCH = {"gqa": {1: 121088, 2: 127232}, "llama": {0: 162304, 1: 139776},
-                             "bert": {0: 120832, 1: 121344}}
+NCU_DRAM_BYTES_PER_LAUNCH = {"gqa": {1: 138240, 2: 148480}, "llama": {0: 153600, 1: 154624},
+                             "bert": {0: 134912, 1: 139264}}
 
 
 WORKLOADS = {"tiny": mi.config1, "bert": mi.config2, "llama": mi.config3, "gqa": mi.config4}
