@@ -430,10 +430,11 @@ __device__ __forceinline__ void load_shared(const Plan& p, uint32_t pe_rows, uin
 }
 
 // The weights of the rows, by all threads of a CTA: those of the orders, on their way when this returns (await_weights), or one for
-// every row that pruning keeps.
+// every row that pruning keeps (PRUNED: where there may be such).
+template <bool PRUNED>
 __device__ __forceinline__ void start_weights(const Plan& p, Shared& sh) {
     constexpr int kWords = sizeof(CountWeights) / 4;
-    if (p.row_pruning) {
+    if (PRUNED && p.row_pruning) {
         // (a warp's 32 weights are one 16-byte word of the parameters: lanes that read different words there wait for one another)
         const uint4* packed = reinterpret_cast<const uint4*>(p.kept_weights);
 #pragma unroll
@@ -936,14 +937,14 @@ template <int OBJ, int MODE>
 __global__ void __launch_bounds__(kSearchThreads, 2)
 search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHeader* __restrict__ head, Partial* __restrict__ partials,
               mmee_result_t* __restrict__ out_best, mmee_result_t* __restrict__ out_topk) {
-    constexpr bool MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain, ARRAYS = MODE == kModeArrays;
+    constexpr bool SINGLE = MODE == kModeSingle, MULTI = MODE == kModeMulti, CHAIN = MODE == kModeChain, ARRAYS = MODE == kModeArrays;
     constexpr bool FRONT = CHAIN && OBJ == MMEE_OBJ_ENERGY_LCAP;      // least (energy, latency) under a bound on the latency
     constexpr bool STAIRS = CHAIN && OBJ == MMEE_OBJ_ENERGY;          // least (energy, block, buffer need) under a capacity
     static_assert(FRONT || STAIRS || !CHAIN, "only the searches of the Pareto fronts are chained");
     __shared__ Shared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (!shape.hold) release_next_kernel();
-    if (!CHAIN || blockIdx.x < shape.grid) start_weights(p, sh);
+    if (!CHAIN || blockIdx.x < shape.grid) start_weights<SINGLE>(p, sh);
     load_shared(p, p.pe_rows, p.pe_cols, sh);
     // Array shapes: the stationary-pair terms of shape y and tiling slot i at [y * chunk + i], behind the tilings' tables;
     // the warps' best items of shape y in sh.tops[.][y].
@@ -1069,7 +1070,8 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
     auto evaluate = [&](uint32_t slot, bool valid) { evaluate_with(slot, valid, sh.tile[slot].st); };
 
     // How many rows fit: units of one (A, B) of a tiling.  (Units of one (A, B, C) where those of a CTA fill no more than half of its
-    // lanes: no gain, 768 tilings for k = 3 39.1 us and 38.9 without, tiny power-of-two tilings 7.15 and 7.14.)
+    // lanes: no gain, 768 tilings for k = 3 39.1 us and 38.9 without, tiny power-of-two tilings 7.15 and 7.14.  Code of their own for two
+    // orders only where a single optimum is searched: it costs the others, which gain nothing, up to 2 % by its length alone.)
     auto count_fitting = [&](uint32_t n_tiles) {
         const uint32_t c0 = fused_items ? 0u : 4u, c1 = unfused_modes ? 5u : 4u, units = 9u * n_tiles;
         while (true) {
@@ -1081,7 +1083,7 @@ search_kernel(const __grid_constant__ Plan p, const LaunchShape shape, SearchHea
             const bool valid = i < units;
             const uint32_t ab = valid ? i / n_tiles : 0u;
             const uint32_t n = count_rows(sh.tile[valid ? i - ab * n_tiles : 0u].size, (int)ab, (int)c0, (int)c1,
-                                          p.row_pruning ? 1u : unfused_modes, capc, sh.weights, n_orders == 2u, [&](bool v) { return any(v && valid); });
+                                          SINGLE && p.row_pruning ? 1u : unfused_modes, capc, sh.weights, SINGLE && n_orders == 2u, [&](bool v) { return any(v && valid); });
             if (valid) my_rows += n;
         }
     };
